@@ -204,15 +204,19 @@ int mhd_set_fusion(mhd_t *m, int on);
  * take the freezing speeds' square roots from the hardware approximation (a
  * few ulp; the faster choice on each path), so the two paths agree to FP32
  * rounding, not bitwise (the magnetic sweeps bitwise); on = 0 always uses
- * register loads.  Ensembles, pencils shorter than 16 cells and boxes that do
+ * register loads.  With on = 1, boxes whose pencils are few or short, and x
+ * sweeps of boxes that the row sweeps do not take, run tile sweeps instead: a
+ * block holds its pencils' whole stencil on chip and each thread updates 4
+ * cells, with bitwise the result of the sweep they replace.  Ensembles, pencils shorter than 16 cells and boxes that do
  * not qualify use register loads.  If staged data does not arrive within the
  * bounded wait (about half a second), the block records the failure and
  * stops; mhd_cfl_dt then returns MHD_E_TIMEOUT until the next mhd_set_state.
  * MHD_E_ARG unless on is 0 or 1, or for an FP64 box. */
 int mhd_set_tma(mhd_t *m, int on);
 
-/* Number of sweeps (fluid and magnetic) this box has launched TMA-staged so
- * far.  MHD_E_ARG for NULL. */
+/* Number of sweeps (fluid and magnetic) this box has launched so far that
+ * qualify for staging, TMA-staged or as the tile sweep that replaces it.
+ * MHD_E_ARG for NULL. */
 int mhd_tma_sweeps(const mhd_t *m, long long *count);
 
 /* Optional floor on the gas pressure (not in the paper; 0 = off, the
@@ -270,7 +274,8 @@ int mhd_fill_ghosts(mhd_t *m);
  * thread (more parallelism for small boxes, 8 cells of warm-up re-read per
  * piece).  Each seg_d must be a multiple of 4 that divides n_d; 0 restores
  * the automatic choice.  The arithmetic of every cell is the same for any
- * segmentation, so results are bitwise independent of it. */
+ * segmentation, so results are bitwise independent of it.  An axis with a
+ * given segment length always marches (no tile sweeps, see mhd_set_tma). */
 int mhd_set_segments(mhd_t *m, int seg_x, int seg_y, int seg_z);
 
 /* How x sweeps read the state: 1 = directly (over whole x rows staged in
@@ -278,8 +283,9 @@ int mhd_set_segments(mhd_t *m, int seg_x, int seg_y, int seg_z);
  * warp stages 8-cell row pieces of its 32 pencils), 2 = through a copy with x
  * and y exchanged (all 8 fields transposed once before a group of x sweeps
  * and once after; consecutive steps share one group, so a run of steps costs
- * two transposes per step), 0 = automatic: 1 where both row sweeps qualify,
- * else 2 once the state exceeds 64 MiB, else 1.  3 = the paper's data flow,
+ * two transposes per step), 0 = automatic: 1 with mhd_set_tma on (row or tile
+ * sweeps) unless the freezing speed is per pencil, else 2 once the state
+ * exceeds 64 MiB, else 1.  3 = the paper's data flow,
  * as an ablation: every sweep runs along the contiguous axis of a copy
  * transposed so that its axis is fastest (x<->y around the y sweeps, x<->z
  * around the z sweeps; six transposes per step); needs every extent a

@@ -369,7 +369,7 @@ mhd_ens_t* mhd_ens_create(int nbox, const int* dims3, double gamma) {
   const mhd::Box big = mhd::make_box((int)std::min<long long>(biggest, 1 << 30), 1, 1);
   const int nblk = mhd::diag_blocks(big);
   cudaError_t ce;
-  if ((ce = mhd::prepare_mag_kernels()) != cudaSuccess ||
+  if ((ce = mhd::prepare_sweep_kernels()) != cudaSuccess ||
       (ce = cudaMalloc(&e->arena, sizeof(float) * (size_t)off * 16)) != cudaSuccess ||
       (ce = cudaMalloc(&e->boxes_d, sizeof(mhd::EnsBox) * nbox)) != cudaSuccess ||
       (ce = cudaMalloc(&e->tau, sizeof(float) * nbox)) != cudaSuccess ||

@@ -91,6 +91,7 @@ struct mhd_s {
   double time64 = 0.0;
   cudaStream_t stream = nullptr;
   int seg[3];
+  bool seg_set[3] = {false, false, false};  // segments given by mhd_set_segments
   int sms = 0;          // multiprocessors of the device (segment choice)
   // tracing: event pairs around launches (see mhd_profile)
   std::vector<cudaEvent_t> ev;
@@ -110,17 +111,13 @@ struct mhd_s {
 
 namespace {
 
-// x sweeps run directly along x when both row sweeps take the box (whole
-// x rows staged in shared memory: nx a multiple of 128 up to 1024, ny a
-// multiple of the magnetic tile's rows (4, or 2 for rows longer than 512),
-// tensor-copy staging on, a freezing speed of its own per cell); otherwise
-// they go through the exchanged layout once the state no longer fits in L2
-// (the pencil sweeps along x read 32 different lines per warp and position,
-// which only L2 can absorb).
+// x sweeps run directly along x (row or tile sweeps) wherever staged sweeps
+// are on and the freezing speed is one of its own per cell; otherwise they go
+// through the exchanged layout once the state no longer fits in L2 (the pencil
+// sweeps along x read 32 different lines per warp and position, which only L2
+// can absorb).
 int auto_xpath(const mhd_s* m) {
-  const bool rows = m->tma && m->fast != 2 && m->n[0] % 128 == 0 && m->n[0] <= 1024 &&
-                    m->n[1] % (m->n[0] <= 512 ? 4 : 2) == 0 && m->n[2] >= 2;
-  if (rows) return 1;
+  if (m->tma && m->fast != 2) return 1;
   return m->N * 32LL > (64LL << 20) ? 2 : 1;
 }
 
@@ -194,6 +191,56 @@ int choose_seg(const mhd_s* m, int d) {
     }
   }
   return best;
+}
+
+// Estimated microseconds of a y or z sweep, from measured times: a marching
+// sweep takes (positions a thread marches) x (time per position), the latter
+// growing with the blocks that share an SM (0.5 us for one fluid block of 4
+// warps, 0.98 us for 4; 0.36 to 0.56 us for one or two magnetic blocks; the
+// fused magnetic pair 0.55 to 0.87 us); a tile sweep takes a time per cell
+// once it fills the chip (21 ps fluid, 19 ps magnetic).  Measured at 96^3:
+// fluid 21 us tile, 31 us marching, magnetic 21 and 27; at 128^3: 44 and 39,
+// 39 and 25.
+double march_us(const mhd_s* m, int d, bool mag, int passes) {
+  const int nA = m->n[d == 0 ? 1 : 0], nO = m->n[d == 2 ? 1 : 2];
+  const int W = mag ? mhd::kMagWarps : 4, resident = mag ? 2 : 4;
+  const double blocks = (double)((nA + 31) / 32) * ((nO + W - 1) / W) * (m->n[d] / m->seg[d]) /
+                        (m->sms > 0 ? m->sms : 152);  // per SM
+  const double b = std::min(blocks, (double)resident), waves = std::max(1.0, blocks / resident);
+  if (!mag) return (m->seg[d] + 7) * (0.5 + 0.03 * b * b) * waves;
+  return passes == 2 ? (m->seg[d] + 14) * (0.55 + 0.16 * b) * waves : (m->seg[d] + 7) * (0.36 + 0.1 * b) * waves;
+}
+double tile_us(const mhd_s* m, bool mag) { return 2.5 + (mag ? 19e-6 : 21e-6) * (double)m->N; }
+
+// Tile sweep or not, along axis d of a box in the plain layout: 0, or the tile
+// argument of FluidArgs / MagArgs.  Along y and z by the estimates above.
+// Along x the row sweeps win wherever they take the fluid (128^3: 31 us
+// against 36), and the magnetic one for large boxes (128^3: 49 us rows, 31 us
+// tile; 256^3: 129 and 196; 512 x 64 x 64: 25 and 31; 512 x 8 x 8: 25 and 8);
+// every other box takes the tile sweep (496^3: 6.1 ms of x sweeps per step against 6.7 ms
+// with transposes and marching).
+int tile_choice(const mhd_s* m, int d, bool mag, int passes) {
+  if (!m->tma || m->fast == 2 || m->xpath == 3 || m->layout || m->seg_set[d]) return 0;
+  // magnetic tiles of 8 x 2 pencils where there are few (32^3: 64 tiles, 10 us
+  // against 15 us) and along x (128^3: 31 against 33 us), else 16 x 4
+  const int shape = d == 0 || m->N <= 150000 ? 1 : 2;
+  if (d == 0) {
+    const bool rows = m->n[0] % 128 == 0 && m->n[0] <= 1024;
+    if (!mag) return rows ? 0 : 128;
+    const bool mag_rows = rows && m->n[1] % mhd::mag_row_tile(m->n[0]) == 0 && m->n[2] >= 2;
+    return mag_rows && m->N > (m->n[0] > 256 ? 1000000 : 4200000) ? 0 : shape;
+  }
+  if (mag && passes == 2 && m->n[d] > mhd::kMTileWhole) return 0;
+  if (tile_us(m, mag) * (passes == 2 ? 1.3 : 1.0) >= march_us(m, d, mag, passes)) return 0;
+  return mag ? shape : (m->n[d] > 64 ? 256 : 128);
+}
+
+// Whether the two magnetic z sweeps in the middle of a step run as one
+// launch: two tile sweeps may beat the fused marching pair on pencils too long
+// for the fused tile sweep (96^3: 2 x 21 us against 41 us, 64^3: 2 x 12 and 34).
+bool fuse_z_pair(const mhd_s* m) {
+  if (m->n[2] <= mhd::kMTileWhole || !tile_choice(m, 2, true, 1)) return true;
+  return 2.0 * tile_us(m, true) >= march_us(m, 2, true, 2);
 }
 
 // Bracket the launches issued by `body` with an event pair when tracing.
@@ -385,6 +432,7 @@ int fluid(mhd_s* m, int d, bool rate) {
   a.tma = m->tma;
   a.err = &m->sc->err;
   a.tma_used = &staged;
+  a.tile = tile_choice(m, d, false, 1);
   if (m->fast == 2) {  // per-pencil freezing speeds before the sweep
     a.pencil_c = m->pencil_c;
     if ((rc = traced(m, MHD_K_CONTROL, [&] {
@@ -423,6 +471,7 @@ int magnetic(mhd_s* m, int d, int passes = 1) {
   a.tma = m->tma;
   a.err = &m->sc->err;
   a.tma_used = &staged;
+  a.tile = tile_choice(m, d, true, passes);
   rc = traced(m, MHD_K_MAG_X + d, [&] {
     CK(mhd::launch_mag(ka, a, m->stream));
     return MHD_OK;
@@ -449,7 +498,7 @@ int full_step(mhd_s* m) {
     if ((rc = magnetic(m, d))) return rc;
   }
   if ((rc = fluid(m, 2, false))) return rc;
-  if (m->fuse && m->xpath != 3 && !any_bc(m)) {
+  if (m->fuse && m->xpath != 3 && !any_bc(m) && fuse_z_pair(m)) {
     if ((rc = magnetic(m, 2, 2))) return rc;
   } else {
     if ((rc = magnetic(m, 2))) return rc;
@@ -638,7 +687,7 @@ mhd_t* mhd_create(int nx, int ny, int nz, double gamma) {
   m->box.n[1] = ny;
   m->box.n[2] = nz;
   m->box = mhd::make_box(nx, ny, nz);
-  cudaError_t e = mhd::prepare_mag_kernels();
+  cudaError_t e = mhd::prepare_sweep_kernels();
   if (e != cudaSuccess) {
     cuda_fail(e, "kernel attributes");
     delete m;
@@ -966,7 +1015,10 @@ int mhd_set_segments(mhd_t* m, int seg_x, int seg_y, int seg_z) {
   for (int d = 0; d < 3; d++)
     if (seg[d] != 0 && (seg[d] < 4 || seg[d] % 4 != 0 || m->n[d] % seg[d] != 0))
       return fail(MHD_E_ARG, "segment length must be a multiple of 4 dividing n_d");
-  for (int d = 0; d < 3; d++) m->seg[d] = seg[d] ? seg[d] : choose_seg(m, d);
+  for (int d = 0; d < 3; d++) {
+    m->seg[d] = seg[d] ? seg[d] : choose_seg(m, d);
+    m->seg_set[d] = seg[d] != 0;
+  }
   return MHD_OK;
 }
 

@@ -398,4 +398,17 @@ struct MagPipe {
   }
 };
 
+// The constraint on b_D from the two transverse edge-flux differences,
+// applied in the order of the local frame (first transverse axis first), each
+// rounded once: b + k_A (fA1 - fA0) + k_O (fO1 - fO0).
+__device__ __forceinline__ float constrain(float b, float kA, float fa0, float fa1, float kO, float fo0,
+                                          float fo1, bool a_first) {
+  if (a_first) {
+    b = __fmaf_rn(kA, __fsub_rn(fa1, fa0), b);
+    return __fmaf_rn(kO, __fsub_rn(fo1, fo0), b);
+  }
+  b = __fmaf_rn(kO, __fsub_rn(fo1, fo0), b);
+  return __fmaf_rn(kA, __fsub_rn(fa1, fa0), b);
+}
+
 }  // namespace mhd

@@ -12,6 +12,10 @@
 namespace mhd {
 
 constexpr int kMagWarps = 8;  // interior rows of a magnetic-sweep tile
+// Rows per tile of the magnetic row sweep: 4 for rows of up to 512 cells (5
+// groups of nx/4 threads, 640 threads), 2 for 1024 cells (3 groups of 256
+// threads, 768).
+__host__ __device__ constexpr int mag_row_tile(int nx) { return nx <= 512 ? 4 : 2; }
 
 // One box of an ensemble: physical extents, first cell in the concatenated
 // field arrays (a multiple of 32), and pencil segment length per axis.
@@ -35,6 +39,55 @@ struct EnsArgs {
   int phys_axis = 0;
 };
 
+// Split of a fluid tile sweep (sweep_tile.cuh) along a pencil of nD cells for
+// blocks of `threads` threads: td threads of 4 cells per pencil, np pencils
+// per block, segs segments of `out` positions.  `whole`: one segment that is
+// the whole periodic pencil; otherwise a segment has one thread of halo cells
+// at each end.  At least 8 pencils per block (32-byte sectors of neighbouring
+// pencils); used on the host for grids and work lists.
+constexpr int kTileThreads = 256;
+constexpr int kTileCells = 4;  // cells per thread
+struct FluidTile {
+  int td, np, segs, out;
+  bool whole;
+};
+__host__ __device__ inline FluidTile fluid_tile_split(int axis, int nD, int threads) {
+  constexpr int K = kTileCells;
+  FluidTile s;
+  const int tmax = threads / (axis == 0 ? 2 : 8);
+  s.whole = nD % K == 0 && nD / K <= tmax;
+  if (s.whole) {
+    s.segs = 1;
+    s.out = nD;
+    s.td = nD / K;
+  } else {
+    const int most = K * (tmax - 2);
+    s.segs = (nD + most - 1) / most;
+    s.out = ((nD + s.segs - 1) / s.segs + 3) / 4 * 4;
+    s.segs = (nD + s.out - 1) / s.out;
+    s.td = s.out / K + 2;
+  }
+  s.np = threads / s.td;
+  if (s.np > 4) s.np &= ~3;
+  return s;
+}
+// Split of a magnetic tile sweep along a pencil of nD cells: segs segments
+// of `out` positions (a multiple of 4 unless whole), whole pencils of up to
+// kMTileWhole cells.
+constexpr int kMTileWhole = 40, kMTileOut = 32;
+struct MagTile {
+  int segs, out;
+  bool whole;
+};
+__host__ __device__ inline MagTile mag_tile_split(int nD) {
+  MagTile s;
+  s.whole = nD <= kMTileWhole;
+  s.segs = s.whole ? 1 : (nD + kMTileOut - 1) / kMTileOut;
+  s.out = s.whole ? nD : ((nD + s.segs - 1) / s.segs + 3) / 4 * 4;
+  s.segs = (nD + s.out - 1) / s.out;
+  return s;
+}
+
 struct FluidArgs {
   const float* in[8];  // current fields
   float* out[8];       // destinations of fields 0..4 (others unused)
@@ -56,6 +109,7 @@ struct FluidArgs {
   int tma = 0;              // 1: stage chunks with tensor-tile copies where the sweep qualifies
   unsigned* err = nullptr;  // set to 1 (atomicOr) if a staged chunk did not arrive within the bound
   int* tma_used = nullptr;  // host: set to 1 when the launch was TMA-staged
+  int tile = 0;             // > 0: tile sweep with blocks of up to that many threads
 };
 
 // Tensor maps of a TMA-staged fluid sweep (kernel axes 1 and 2), dimensions
@@ -81,6 +135,7 @@ struct FluidMaps {
 // shorter than 16 cells) or the driver's encoder is unavailable.  Lane and
 // row extents need not fill the 32 x 4 tiles.
 bool make_fluid_maps(int axis, const FluidArgs& a, FluidMaps* m);
+bool fluid_chunks_qualify(int axis, const FluidArgs& a);  // the box's part of that
 
 struct MagArgs {
   const float* in[8];
@@ -95,6 +150,8 @@ struct MagArgs {
   int tma = 0;              // 1: stage chunks with tensor-tile copies where the sweep qualifies
   unsigned* err = nullptr;  // set to 1 (atomicOr) if a staged chunk did not arrive within the bound
   int* tma_used = nullptr;  // host: set to 1 when the launch was TMA-staged
+  int tile = 0;             // 1: tile sweep
+  int tile_out = 0;         // ensemble tile launches: largest `out` of any box (shared memory)
 };
 
 // Ghost layers of a non-periodic axis (boundary.cu): kernel axis `axis` of
@@ -256,6 +313,8 @@ template <int LIM>
 cudaError_t launch_mag_t(int axis, const MagArgs& a, cudaStream_t s);
 template <int LIM>
 cudaError_t prepare_mag_t();
+template <int LIM, int FRZ>
+cudaError_t prepare_fluid_t();
 extern template cudaError_t launch_fluid_t<0, 0>(int, bool, const FluidArgs&, cudaStream_t);
 extern template cudaError_t launch_fluid_t<1, 0>(int, bool, const FluidArgs&, cudaStream_t);
 extern template cudaError_t launch_fluid_t<2, 0>(int, bool, const FluidArgs&, cudaStream_t);
@@ -264,11 +323,15 @@ extern template cudaError_t launch_fluid_t<0, 2>(int, bool, const FluidArgs&, cu
 extern template cudaError_t launch_mag_t<0>(int, const MagArgs&, cudaStream_t);
 extern template cudaError_t launch_mag_t<1>(int, const MagArgs&, cudaStream_t);
 extern template cudaError_t launch_mag_t<2>(int, const MagArgs&, cudaStream_t);
+extern template cudaError_t prepare_fluid_t<0, 0>();
+extern template cudaError_t prepare_fluid_t<1, 0>();
+extern template cudaError_t prepare_fluid_t<2, 0>();
+extern template cudaError_t prepare_fluid_t<0, 1>();
 extern template cudaError_t prepare_mag_t<0>();
 extern template cudaError_t prepare_mag_t<1>();
 extern template cudaError_t prepare_mag_t<2>();
 // one-time per-device kernel attributes (call on the current device before launching)
-cudaError_t prepare_mag_kernels();
+cudaError_t prepare_sweep_kernels();
 // Tensor maps of a TMA-staged magnetic sweep (kernel axes 1 and 2), dimensions
 // ordered (lane axis A, row axis O, sweep axis D): rho, m_D, b_A, b_O, b_D
 // over the 32 x 8 tile (32 x 8 x 4), rho, m_D, b_O one row (32 x 1 x 4) and
@@ -282,6 +345,7 @@ struct MagMaps {
 // false if the box does not qualify (lane extent not a multiple of 32, row
 // extent not a multiple of 8, unaligned fields) or the encoder is unavailable
 bool make_mag_maps(int axis, const MagArgs& a, MagMaps* m);
+bool mag_chunks_qualify(int axis, const MagArgs& a);  // the box's part of that
 // cells [lo, hi) per kernel axis (the interior of a box with ghost layers)
 struct CellRange {
   int lo[3], hi[3];

@@ -25,14 +25,21 @@ constexpr int kMapCache = 16;
 
 }  // namespace
 
-bool make_fluid_maps(int axis, const FluidArgs& a, FluidMaps* out) {
-  if (axis != 1 && axis != 2) return false;
+bool fluid_chunks_qualify(int axis, const FluidArgs& a) {
+  if (!a.tma || a.ens.items || (axis != 1 && axis != 2)) return false;
   const Box& b = a.box;
-  const int A = 0, O = (axis == 2) ? 1 : 2, D = axis, T1 = (D + 1) % 3, T2 = (D + 2) % 3;
+  const int A = 0, O = (axis == 2) ? 1 : 2, D = axis;
   if (b.stride[A] != 1 || b.n[D] < 16) return false;
   if ((b.stride[O] * 4) % 16 || (b.stride[D] * 4) % 16) return false;
   for (int q = 0; q < 8; q++)
     if (reinterpret_cast<uintptr_t>(a.in[q]) % 16) return false;
+  return true;
+}
+
+bool make_fluid_maps(int axis, const FluidArgs& a, FluidMaps* out) {
+  if (!fluid_chunks_qualify(axis, a)) return false;
+  const Box& b = a.box;
+  const int A = 0, O = (axis == 2) ? 1 : 2, D = axis, T1 = (D + 1) % 3, T2 = (D + 2) % 3;
   MapKey key;
   std::memset(&key, 0, sizeof key);
   for (int q = 0; q < 8; q++) key.f[q] = a.in[q];
@@ -73,6 +80,7 @@ bool make_fluid_maps(int axis, const FluidArgs& a, FluidMaps* out) {
 }
 
 template cudaError_t launch_fluid_t<0, 0>(int, bool, const FluidArgs&, cudaStream_t);
+template cudaError_t prepare_fluid_t<0, 0>();
 
 cudaError_t launch_fluid(int axis, bool rate, const FluidArgs& a, cudaStream_t s) {
   if (a.fast == 1) return launch_fluid_t<0, 1>(axis, rate, a, s);

@@ -27,6 +27,7 @@
 #include "mhd_device.cuh"
 #include "mhd_launch.h"
 #include "sweep_row.cuh"
+#include "sweep_tile.cuh"
 #include "tma.cuh"
 
 namespace mhd {
@@ -414,6 +415,15 @@ cudaError_t launch_fluid_t(int axis, bool rate, const FluidArgs& a, cudaStream_t
   if (a.ens.items) grid = dim3(a.nblocks, 1, 1);
   const bool small = a.box.n[axis] < 16;
   const bool floor = a.p_floor > 0.f;
+  if (a.tile) {
+    // the square root of the sweep that would run otherwise: a cell's result
+    // does not depend on which sweep takes it
+    if (fluid_chunks_qualify(axis, a) || (axis == 0 && fluid_rows_qualify(a))) {
+      if (a.tma_used) *a.tma_used = 1;
+      return launch_fluid_tile<LIM, FRZ, true>(axis, rate, a, s);
+    }
+    return launch_fluid_tile<LIM, FRZ, false>(axis, rate, a, s);
+  }
   if (axis == 0 && fluid_rows_qualify(a)) {  // x sweeps over whole staged rows
     if (a.tma_used) *a.tma_used = 1;
     return launch_fluid_rows<LIM, FRZ>(rate, a, s);
@@ -446,6 +456,14 @@ cudaError_t launch_fluid_t(int axis, bool rate, const FluidArgs& a, cudaStream_t
   FLUID_CASE(2, false) FLUID_CASE(2, true)
 #undef FLUID_CASE
   return cudaGetLastError();
+}
+
+// The tile kernels' shared-memory limits (once per device, before any launch).
+template <int LIM, int FRZ>
+cudaError_t prepare_fluid_t() {
+  cudaError_t e = prepare_fluid_tile<LIM, FRZ, true>();
+  if (e == cudaSuccess) e = prepare_fluid_tile<LIM, FRZ, false>();
+  return e;
 }
 
 }  // namespace mhd

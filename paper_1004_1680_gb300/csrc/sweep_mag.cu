@@ -25,15 +25,22 @@ constexpr int kMagMapCache = 16;
 
 }  // namespace
 
-bool make_mag_maps(int axis, const MagArgs& a, MagMaps* out) {
-  if (axis != 1 && axis != 2) return false;
+bool mag_chunks_qualify(int axis, const MagArgs& a) {
+  if (!a.tma || a.ens.items || (axis != 1 && axis != 2)) return false;
   const Box& b = a.box;
   const int A = 0, O = (axis == 2) ? 1 : 2, D = axis;
   if (b.stride[A] != 1 || b.n[A] % 32 || b.n[O] % kMagWarps || b.n[D] < 16) return false;
   if ((b.stride[O] * 4) % 16 || (b.stride[D] * 4) % 16) return false;
-  const float* f[5] = {a.in[RHO], a.in[MX + D], a.in[BX + A], a.in[BX + O], a.in[BX + D]};
-  for (const float* p : f)
+  for (const float* p : {a.in[RHO], a.in[MX + D], a.in[BX + A], a.in[BX + O], a.in[BX + D]})
     if (reinterpret_cast<uintptr_t>(p) % 16) return false;
+  return true;
+}
+
+bool make_mag_maps(int axis, const MagArgs& a, MagMaps* out) {
+  if (!mag_chunks_qualify(axis, a)) return false;
+  const Box& b = a.box;
+  const int A = 0, O = (axis == 2) ? 1 : 2, D = axis;
+  const float* f[5] = {a.in[RHO], a.in[MX + D], a.in[BX + A], a.in[BX + O], a.in[BX + D]};
   MagMapKey key;
   std::memset(&key, 0, sizeof key);
   for (int q = 0; q < 8; q++) key.f[q] = a.in[q];
@@ -76,8 +83,12 @@ bool make_mag_maps(int axis, const MagArgs& a, MagMaps* out) {
 template cudaError_t launch_mag_t<0>(int, const MagArgs&, cudaStream_t);
 template cudaError_t prepare_mag_t<0>();
 
-cudaError_t prepare_mag_kernels() {
+cudaError_t prepare_sweep_kernels() {
   cudaError_t e = prepare_mag_t<0>();
+  if (e == cudaSuccess) e = prepare_fluid_t<0, 0>();
+  if (e == cudaSuccess) e = prepare_fluid_t<1, 0>();
+  if (e == cudaSuccess) e = prepare_fluid_t<2, 0>();
+  if (e == cudaSuccess) e = prepare_fluid_t<0, 1>();
   if (e == cudaSuccess) e = prepare_mag_t<1>();
   if (e == cudaSuccess) e = prepare_mag_t<2>();
   return e;

@@ -27,22 +27,10 @@
 #include "mhd_device.cuh"
 #include "mhd_launch.h"
 #include "sweep_row.cuh"
+#include "sweep_tile.cuh"
 #include "tma.cuh"
 
 namespace mhd {
-
-// The constraint on b_D from the two transverse edge-flux differences,
-// applied in the order of the local frame (first transverse axis first), each
-// rounded once: b + k_A (fA1 - fA0) + k_O (fO1 - fO0).
-__device__ __forceinline__ float constrain(float b, float kA, float fa0, float fa1, float kO, float fo0,
-                                          float fo1, bool a_first) {
-  if (a_first) {
-    b = __fmaf_rn(kA, __fsub_rn(fa1, fa0), b);
-    return __fmaf_rn(kO, __fsub_rn(fo1, fo0), b);
-  }
-  b = __fmaf_rn(kO, __fsub_rn(fo1, fo0), b);
-  return __fmaf_rn(kA, __fsub_rn(fa1, fa0), b);
-}
 
 template <int D>
 struct MagAxes {
@@ -709,6 +697,7 @@ cudaError_t prepare_mag_t() {
       e = cudaFuncSetAttribute(mag_sweep_tma_kernel<2, 2, LIM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)kMagTmaSmem);
   }
+  if (e == cudaSuccess) e = prepare_mag_tile<LIM>();
   return e;
 }
 
@@ -719,6 +708,10 @@ cudaError_t launch_mag_t(int axis, const MagArgs& a, cudaStream_t s) {
   dim3 grid((a.box.n[A] + 31) / 32, (a.box.n[O] + kMagWarps - 1) / kMagWarps, a.box.n[axis] / a.seg);
   if (a.ens.items) grid = dim3(a.nblocks, 1, 1);  // one block per work item
   const bool small = a.box.n[axis] < 16;
+  if (a.tile) {
+    if (a.tma_used && (mag_chunks_qualify(axis, a) || (axis == 0 && mag_rows_qualify(a)))) *a.tma_used = 1;
+    return launch_mag_tile<LIM>(axis, a, s);
+  }
   if (axis == 0 && mag_rows_qualify(a)) {  // x sweeps over whole staged rows
     if (a.tma_used) *a.tma_used = 1;
     return launch_mag_rows<LIM>(a, s);

@@ -343,9 +343,6 @@ __global__ void __launch_bounds__(kRowMaxThreads, 2) fluid_row_kernel(const __gr
 // barrier).  The exchanges along a row wait for the row's own warps only (a
 // named barrier per group); a group may run up to a step ahead of the
 // others, which the double-buffered v and E_y rows allow.
-// Rows per tile: 4 for rows of up to 512 cells (5 groups of nx/4 threads,
-// 640 threads), 2 for 1024 cells (3 groups of 256 threads, 768).
-__host__ __device__ constexpr int mag_row_tile(int nx) { return nx <= 512 ? 4 : 2; }
 // Row slots of a staged plane for a tile of R rows: rho and m_x of rows
 // j0-1 .. j0+R, b_x of the tile, b_y of rows j0 .. j0+R, b_z of the tile.
 template <int R>

@@ -1,0 +1,673 @@
+// Tile sweeps (Section II.B), FP32: sweeps along any axis in which a block
+// holds its pencils' whole stencil on chip and every thread updates 4
+// consecutive cells, for boxes (and ensembles of boxes) whose pencils are too
+// few or too short for the marching sweeps.
+//
+// A marching thread carries its pencil through one position after another:
+// about 0.5 us per position of dependent arithmetic and loads, 39 positions
+// for a 32-cell pencil, however idle the chip is.  Here the positions of a
+// pencil are spread over threads, all loads of a sweep go out at once and the
+// chain is that of 4 cells, with three exchanges between neighbouring threads
+// (fluid) or two passes over shared memory (magnetic).  Time per step, marching
+// -> tile: 32^3 302 -> 78 us, 64^3 308 -> 111, 96^3 432 -> 217, 236 x 150 x 98
+// (x sweeps without transposes) 1043 -> 800 us.  Small boxes are bound by the
+// launches (about 2.5 us each) and one chain of loads, arithmetic and stores
+// (2 to 5 us); once the chip is full a fluid tile sweep runs at 17 (x) or 21 ps
+// per cell, twice the marching sweep's 8.3 ps on a 512^3 box, because each
+// block waits for its loads before it computes: the dispatch (tile_choice in
+// mhd_api.cu) leaves large boxes to the marching and row sweeps.
+//
+// The arithmetic of a cell is that of FluidPipe and MagPipe (mhd_device.cuh),
+// operation for operation, so a tile sweep gives bitwise the result of the
+// register-load marching sweep (FSQ = false), and agrees with it to FP32
+// rounding with the hardware square root (FSQ = true, as in the staged
+// sweeps).
+#pragma once
+#include "mhd_device.cuh"
+#include "mhd_launch.h"
+#include "sweep_row.cuh"
+#include "tma.cuh"
+
+namespace mhd {
+
+// Periodic image of a position anywhere (a modulo only where one period is
+// not enough: pencils of a few cells).
+__device__ __forceinline__ int wrap_any(int i, int n) {
+  i = i < 0 ? i + n : i;
+  i = i >= n ? i - n : i;
+  return (unsigned)i < (unsigned)n ? i : wrapi(i, n);
+}
+
+// ---------------------------------------------------------------------------
+// Fluid tile sweep.  A block takes `np` consecutive pencils (row order of the
+// other two axes, the contiguous one fastest) and `out` positions of them,
+// `td` threads of 4 cells along each pencil.  Pencils of a multiple of 4
+// cells that fit in the block are taken whole (`whole`: the end threads are
+// neighbours across the periodic wrap); others in segments with one thread of
+// 4 halo cells at each end (3 are needed), which stores nothing.
+// (FluidTile and fluid_tile_split are declared in mhd_launch.h: the host
+// builds grids and work lists with the same split.)
+constexpr int kTileSlots = 6;  // exchanged V5 values per thread (slot 0 is used twice)
+
+__host__ __device__ constexpr size_t fluid_tile_smem(int threads) {
+  return (size_t)threads * (5 * 16 + kTileSlots * 20);  // U of the 4 cells, the slots
+}
+
+// 128 registers: 2 blocks of 256 threads (or 4 of 128) per SM.  4 cells per
+// thread: with 2 the exchanges cost more than the extra warps hide (128^3
+// along y 57 us against 44).
+template <int D, bool RATE, bool FLOOR, int LIM, int FRZ, bool FSQ>
+__global__ void __launch_bounds__(kTileThreads, 2) fluid_tile_kernel(const __grid_constant__ FluidArgs a) {
+  static_assert(FRZ != 2, "the per-pencil freezing speed keeps the pencil sweeps");
+  constexpr int K = kTileCells;
+  constexpr int A = (D == 0) ? 1 : 0, O = (D == 2) ? 1 : 2, T1 = (D + 1) % 3, T2 = (D + 2) % 3;
+  extern __shared__ float4 tile_dyn[];
+  const BlockGeom G = block_geom(a.ens, a.box, a.seg, a.tau, a.rate);
+  const int nA = G.box.n[A], nO = G.box.n[O], nD = G.box.n[D];
+  const int T = blockDim.x, tid = threadIdx.x;
+  const FluidTile s = fluid_tile_split(D, nD, a.tile);
+  const int np = s.np, td = s.td;
+  // thread -> (pencil of the block, group of 4 cells): along x the groups of a
+  // pencil are neighbouring threads (16 contiguous bytes each), else the
+  // pencils are
+  const int pp = D == 0 ? tid / td : tid % np, l = D == 0 ? tid - pp * td : tid / np;
+  const int P = G.bx * np + pp;
+  const bool live = pp < np && l < td && P < nA * nO;
+  RowSlots X;
+  X.A = tile_dyn;
+  X.E = reinterpret_cast<float*>(X.A + kTileSlots * T);
+  X.T = T;
+  float4* park = reinterpret_cast<float4*>(X.E + kTileSlots * T) + tid;  // U, [field][thread]
+  const int lm = l > 0 ? l - 1 : (s.whole ? td - 1 : 0), lp = l + 1 < td ? l + 1 : (s.whole ? 0 : l);
+  const int im = D == 0 ? tid + lm - l : tid + (lm - l) * np, ip = D == 0 ? tid + lp - l : tid + (lp - l) * np;
+
+  const float gamma = a.gamma;
+  const float c_full = G.tau * G.box.ih[D];  // tau / h_D
+  const float c_half = 0.5f * c_full;
+  const int pb = P / nA, pa = P - pb * nA;
+  const int sA = (int)G.box.stride[A], sO = (int)G.box.stride[O], sD = (int)G.box.stride[D];
+  const unsigned base = (unsigned)(pa * sA + pb * sO);
+  // the first of the thread's cells, before wrapping
+  const int p0 = G.bz * s.out + K * (l - (s.whole ? 0 : 1));
+
+  V5 f1[K + 1];  // flux1 at p0-1/2 .. p0+7/2
+  V5 FR3, FL0;
+  B3 B[K];
+  if (live) {
+    // every load of the sweep, before the first use
+    const float* __restrict__ f[8];
+#pragma unroll
+    for (int q = 0; q < 8; q++) f[q] = a.in[q] + G.off;
+    const unsigned baseA1 = base + (unsigned)((pa + 1 == nA ? 1 - nA : 1) * sA);  // pencil +1 along A
+    const unsigned baseO1 = base + (unsigned)((pb + 1 == nO ? 1 - nO : 1) * sO);  // pencil +1 along O
+    const unsigned baseT1 = (T1 == A) ? baseA1 : baseO1, baseT2 = (T2 == A) ? baseA1 : baseO1;
+    constexpr int kField[5] = {RHO, MX + D, MX + T1, MX + T2, EN};
+    float u[5][K], bd[K + 1], b1[K], b1n[K], b2[K], b2n[K];
+    if constexpr (D == 0) {
+      const unsigned c = base + (unsigned)wrap_any(p0, nD);  // p0 and nx are multiples of 4
+      auto ld4 = [](const float* p, float (&d)[K]) {
+        const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+#pragma unroll
+        for (int j = 0; j < K; j++) d[j] = (&v.x)[j];
+      };
+      const unsigned w = c - base;
+#pragma unroll
+      for (int q = 0; q < 5; q++) ld4(f[kField[q]] + c, u[q]);
+      float t[K];
+      ld4(f[BX + D] + c, t);
+#pragma unroll
+      for (int j = 0; j < K; j++) bd[j] = t[j];
+      bd[K] = __ldg(f[BX + D] + base + (unsigned)wrap_any(p0 + K, nD));
+      ld4(f[BX + T1] + c, b1);
+      ld4(f[BX + T1] + (baseT1 + w), b1n);
+      ld4(f[BX + T2] + c, b2);
+      ld4(f[BX + T2] + (baseT2 + w), b2n);
+    } else {
+      unsigned off[K + 1];
+#pragma unroll
+      for (int j = 0; j <= K; j++) off[j] = (unsigned)(wrap_any(p0 + j, nD) * sD);
+#pragma unroll
+      for (int j = 0; j < K; j++) {
+#pragma unroll
+        for (int q = 0; q < 5; q++) u[q][j] = __ldg(f[kField[q]] + (base + off[j]));
+        bd[j] = __ldg(f[BX + D] + (base + off[j]));
+        b1[j] = __ldg(f[BX + T1] + (base + off[j]));
+        b1n[j] = __ldg(f[BX + T1] + (baseT1 + off[j]));
+        b2[j] = __ldg(f[BX + T2] + (base + off[j]));
+        b2n[j] = __ldg(f[BX + T2] + (baseT2 + off[j]));
+      }
+      bd[K] = __ldg(f[BX + D] + (base + off[K]));
+    }
+    // U waits in the thread's own shared memory between its three uses
+#pragma unroll
+    for (int q = 0; q < 5; q++) {
+      float4 v;
+#pragma unroll
+      for (int j = 0; j < K; j++) (&v.x)[j] = u[q][j];
+      park[q * T] = v;
+    }
+    // stage 1: first-order fluxes
+    V5 FRp;
+#pragma unroll
+    for (int j = 0; j < K; j++) {
+      B[j] = {{face_mean(bd[j], bd[j + 1]), face_mean(b1[j], b1n[j]), face_mean(b2[j], b2n[j])}};
+      const V5 U = {make_float2(u[0][j], u[1][j]), make_float2(u[2][j], u[3][j]), u[4][j]};
+      V5 FR, FL;
+      split_flux<FRZ, FSQ>(U, B[j].v[0], make_float2(B[j].v[1], B[j].v[2]), gamma, FR, FL);
+      if (j == 0) FL0 = FL;
+      else f1[j] = v5_sub(FRp, FL);
+      FRp = FR;
+    }
+    FR3 = FRp;
+    X.put(0, tid, FR3);
+    X.put(1, tid, FL0);
+  }
+  __syncthreads();
+  V5 Rh[K], Lh[K];
+  auto parked = [&](V5 (&U)[K]) {
+    float4 v[5];
+#pragma unroll
+    for (int q = 0; q < 5; q++) v[q] = park[q * T];
+#pragma unroll
+    for (int j = 0; j < K; j++)
+      U[j] = {make_float2((&v[0].x)[j], (&v[1].x)[j]), make_float2((&v[2].x)[j], (&v[3].x)[j]), (&v[4].x)[j]};
+  };
+  if (live) {
+    f1[0] = v5_sub(X.get(0, im), FL0);          // FR(p0-1) - FL(p0)
+    f1[K] = v5_sub(FR3, X.get(1, ip));  // FR(p0+3) - FL(p0+4)
+    V5 U[K];
+    parked(U);
+#pragma unroll
+    for (int j = 0; j < K; j++) {
+      const V5 Uh = v5_fma(-c_half, v5_sub(f1[j + 1], f1[j]), U[j]);
+      // stage 2
+      split_flux<FRZ, FSQ>(Uh, B[j].v[0], make_float2(B[j].v[1], B[j].v[2]), gamma, Rh[j], Lh[j]);
+    }
+    X.put(2, tid, Rh[K - 1]);
+    X.put(3, tid, Rh[0]);
+    X.put(4, tid, Lh[0]);
+    X.put(5, tid, Lh[1]);
+  }
+  __syncthreads();
+  V5 F2[K];
+  if (live) {
+    // interface j+1/2: Rh(j-1..j+1), Lh(j..j+2)
+    auto flux2 = [&](int j, const V5& Rl, const V5& Rr, const V5& L1, const V5& L2) {
+      const V5 right = v5_add(Rh[j], half_limited5<LIM>(v5_sub(Rh[j], Rl), v5_sub(Rr, Rh[j])));
+      const V5 left = v5_sub(L1, half_limited5<LIM>(v5_sub(L1, Lh[j]), v5_sub(L2, L1)));
+      return v5_sub(right, left);
+    };
+    const V5 Rp = X.get(3, ip), Lp0 = X.get(4, ip), Lp1 = X.get(5, ip);
+    F2[K - 1] = flux2(K - 1, Rh[K - 2], Rp, Lp0, Lp1);
+    X.put(0, tid, F2[K - 1]);
+    F2[2] = flux2(2, Rh[1], Rh[3], Lh[3], Lp0);
+    F2[1] = flux2(1, Rh[0], Rh[2], Lh[2], Lh[3]);
+    F2[0] = flux2(0, X.get(2, im), Rh[1], Lh[1], Lh[2]);
+  }
+  __syncthreads();
+  float rmax = 0.f;
+  // cells of this block's own positions (halo threads and the cells past the
+  // pencil's end store nothing)
+  const int pend = min(nD, (G.bz + 1) * s.out);
+  if (live && p0 >= G.bz * s.out && p0 < pend) {
+    float* __restrict__ o[5];
+    constexpr int kField[5] = {RHO, MX + D, MX + T1, MX + T2, EN};
+#pragma unroll
+    for (int q = 0; q < 5; q++) o[q] = a.out[kField[q]] + G.off;
+    V5 U[K];
+    parked(U);
+    const V5 Fm = X.get(0, im);
+    const bool rate_pencil =
+        RATE && pa >= a.rate_lo[A] && pa < a.rate_hi[A] && pb >= a.rate_lo[O] && pb < a.rate_hi[O];
+    float r[K][5];
+#pragma unroll
+    for (int j = 0; j < K; j++) {
+      const V5 v = v5_fma(-c_full, v5_sub(F2[j], j ? F2[j ? j - 1 : 0] : Fm), U[j]);
+      r[j][0] = v.p0.x;
+      r[j][1] = v.p0.y;
+      r[j][2] = v.p1.x;
+      r[j][3] = v.p1.y;
+      r[j][4] = v.e;
+      if (FLOOR) r[j][4] = floored_energy(r[j], B[j].v, gamma, a.p_floor);
+      const int p = p0 + j;
+      if (RATE && rate_pencil && p < pend && p >= a.rate_lo[D] && p < a.rate_hi[D]) {
+        float m[3], bg[3];
+        m[D] = r[j][1]; m[T1] = r[j][2]; m[T2] = r[j][3];
+        bg[D] = B[j].v[0]; bg[T1] = B[j].v[1]; bg[T2] = B[j].v[2];
+        rmax = fmaxf(rmax, cell_rate(r[j][0], m, r[j][4], bg, gamma, G.box.ih));
+      }
+    }
+    if constexpr (D == 0) {
+#pragma unroll
+      for (int q = 0; q < 5; q++) {
+        float4 v;
+#pragma unroll
+        for (int j = 0; j < K; j++) (&v.x)[j] = r[j][q];
+        *reinterpret_cast<float4*>(o[q] + (base + (unsigned)p0)) = v;
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < K; j++)
+        if (p0 + j < pend)
+#pragma unroll
+          for (int q = 0; q < 5; q++) o[q][base + (unsigned)((p0 + j) * sD)] = r[j][q];
+    }
+  }
+  if (RATE) {
+    for (int k = 16; k > 0; k >>= 1) rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, k));
+    if ((tid & 31) == 0 && rmax > 0.f) atomicMax(G.rate, __float_as_uint(rmax));
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Magnetic tile sweep.  A block takes a tile of LX (lane axis A) x R (row
+// axis O) pencils and `out` positions of them, and holds in shared memory,
+// with the positions' halo at each end (periodic images):
+//   v  = m_D / rho of the tile's pencils and of the ones next to them,
+//   q  = the advected fields of the tile's edge-flux rows: b_A of columns
+//        0 .. LX (LX: the halo column) and b_O of rows 0 .. R,
+//   bD = b_D of the tile's pencils.
+// All of it arrives by asynchronous copies, issued at once.  Then every
+// (edge-flux row, group of 4 edges) is one independent task: 9 cells of q and
+// of the two v rows give the 4 limited edge fluxes f, with the half step of
+// 3 cells at the group's ends repeated by both neighbours (which needs no
+// exchange between threads).  After a barrier the cells are finished from f.
+template <int LX, int R>
+struct MTile {
+  static constexpr int VC = LX + 2, V = (R + 2) * VC;      // v slots of a plane
+  static constexpr int QA = R * (LX + 1), Q = QA + (R + 1) * LX;  // edge-flux rows: b_A, then b_O
+  static constexpr int C = LX * R;                          // cells of a plane
+  static constexpr int T = C >= 64 ? 256 : 128;             // threads
+  // v slots of edge-flux row ts's pencil (low) and of the one across its faces (high half)
+  static __device__ __forceinline__ void rows(int ts, int& own, int& nbr) {
+    if (ts < QA) {
+      const int row = ts / (LX + 1), col = ts - row * (LX + 1);
+      own = (row + 1) * VC + col + 1;
+      nbr = own - 1;
+    } else {
+      const int o = ts - QA, row = o / LX, col = o - row * LX;
+      own = (row + 1) * VC + col + 1;
+      nbr = own - VC;
+    }
+  }
+};
+__host__ __device__ constexpr int mag_tile_halo(int D) { return D == 0 ? 4 : 3; }  // 4: 16-byte loads along x
+// positions held per slot: `out`, the halos and what the last group of edges
+// may touch past them; along x an odd number of 16-byte pieces (bank conflicts)
+__host__ __device__ constexpr int mag_tile_positions(int D, int out) {
+  const int n = out + 2 * mag_tile_halo(D) + 4;
+  return D == 0 ? (n + 3) / 8 * 8 + 4 : n;
+}
+template <int LX, int R>
+__host__ __device__ constexpr size_t mag_tile_smem(int D, int out) {
+  return sizeof(float) * (MTile<LX, R>::V + 2 * MTile<LX, R>::Q + MTile<LX, R>::C) * mag_tile_positions(D, out);
+}
+
+__device__ __forceinline__ void copy4_async(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy16_async(float* dst, const float* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// The 4 limited edge fluxes of a group from 9 cells of q and face velocity u
+// (MagPipe's arithmetic): edge k lies between cells k + 2 and k + 3.
+template <int LIM>
+__device__ __forceinline__ void edge_fluxes(const float (&q)[9], const float (&u)[9], float c_half, float (&f)[4]) {
+  float ub[8], g[8], h[7], d[6];
+#pragma unroll
+  for (int k = 0; k < 8; k++) {
+    ub[k] = __fmul_rn(0.5f, __fadd_rn(u[k], u[k + 1]));
+    g[k] = __fmul_rn(ub[k], ub[k] >= 0.f ? q[k] : q[k + 1]);
+  }
+#pragma unroll
+  for (int k = 0; k < 7; k++) h[k] = __fmaf_rn(-c_half, __fsub_rn(g[k + 1], g[k]), q[k + 1]);
+#pragma unroll
+  for (int k = 0; k < 6; k++) d[k] = __fsub_rn(h[k + 1], h[k]);
+#pragma unroll
+  for (int k = 0; k < 4; k++) {
+    const float w = ub[k + 2];
+    const bool pos = w >= 0.f;
+    const float lim = half_limited<LIM>(pos ? d[k] : d[k + 1], pos ? d[k + 1] : d[k + 2]);
+    f[k] = __fmul_rn(w, pos ? __fadd_rn(h[k + 1], lim) : __fsub_rn(h[k + 2], lim));
+  }
+}
+
+// Along y and z: planes of slots, one per position.  NP = 2 (whole pencils
+// only): two sweeps with the same step; the first one's result stays in
+// shared memory.
+template <int D, int LX, int R, int LIM, int NP>
+__global__ void __launch_bounds__(MTile<LX, R>::T) mag_tile_kernel(const __grid_constant__ MagArgs a) {
+  static_assert(D != 0, "x sweeps use mag_tile_x_kernel");
+  constexpr int A = 0, O = (D == 2) ? 1 : 2, T1 = (D + 1) % 3;
+  using M = MTile<LX, R>;
+  constexpr int H = mag_tile_halo(D), T = M::T;
+  extern __shared__ __align__(16) float mt_dyn[];
+  const BlockGeom G = block_geom(a.ens, a.box, a.seg, a.tau, nullptr);
+  const int nA = G.box.n[A], nO = G.box.n[O], nD = G.box.n[D];
+  const MagTile sp = mag_tile_split(nD);
+  const int a0 = G.bx * LX, b0 = G.by * R;
+  const int s0 = G.bz * sp.out, S = min(sp.out, nD - s0);  // this block's positions s0 .. s0 + S - 1
+  const int PN = mag_tile_positions(D, sp.out);
+  float* sv = mt_dyn;
+  float* sq = sv + M::V * PN;
+  float* sf = sq + M::Q * PN;
+  float* sb = sf + M::Q * PN;
+  const int tid = threadIdx.x;
+  const int sA = (int)G.box.stride[A], sO = (int)G.box.stride[O], sD = (int)G.box.stride[D];
+
+  // slot (row, col) of the (R+2) x (LX+2) plane is the pencil (b0 + row - 1,
+  // a0 + col - 1), periodic; the corners are not needed.  A thread keeps its
+  // slot and walks the positions; rho waits in sf.
+  {
+    constexpr int kSlots = M::V <= 64 ? 64 : 128, kStep = T / kSlots;
+    static_assert(M::V <= kSlots && T % kSlots == 0 && M::Q >= M::V, "slots of a plane");
+    const int slot = tid % kSlots;
+    const int row = slot / M::VC, col = slot - row * M::VC;
+    const bool rin = row >= 1 && row <= R, cin = col >= 1 && col <= LX;
+    if (slot < M::V && (rin || cin)) {
+      const unsigned pb = (unsigned)(wrap_any(a0 + col - 1, nA) * sA + wrap_any(b0 + row - 1, nO) * sO);
+      const float* rho = a.in[RHO] + G.off + pb;
+      const float* md = a.in[MX + D] + G.off + pb;
+      const float* bA = a.in[BX + A] + G.off + pb;
+      const float* bO = a.in[BX + O] + G.off + pb;
+      const float* bD = a.in[BX + D] + G.off + pb;
+      const bool hasA = rin && col >= 1, hasO = cin && row >= 1, own = rin && cin;
+      float* qa = sq + (row - 1) * (LX + 1) + col - 1;
+      float* qo = sq + M::QA + (row - 1) * LX + col - 1;
+      float* qd = sb + (row - 1) * LX + col - 1;
+      for (int p = tid / kSlots; p < S + 2 * H; p += kStep) {
+        const unsigned c = (unsigned)(wrap_any(s0 - H + p, nD) * sD);
+        copy4_async(sv + p * M::V + slot, md + c);
+        copy4_async(sf + p * M::V + slot, rho + c);
+        if (hasA) copy4_async(qa + p * M::Q, bA + c);
+        if (hasO) copy4_async(qo + p * M::Q, bO + c);
+        if (own) copy4_async(qd + p * M::C, bD + c);
+      }
+      copies_wait();
+      for (int p = tid / kSlots; p < S + 2 * H; p += kStep)
+        sv[p * M::V + slot] = v_div(sv[p * M::V + slot], sf[p * M::V + slot]);
+    }
+  }
+  const float tau = G.tau;
+  const float c_full = tau * G.box.ih[D];  // tau / h_D
+  const float c_half = 0.5f * c_full;
+  const float kA = tau * G.box.ih[A];      // tau / h_A
+  const float kO = tau * G.box.ih[O];      // tau / h_O
+  // edge e lies between local cells e - 1 and e: edges 0 .. S are needed; of a
+  // whole pencil 1 .. S (edge 0 is edge S)
+  const int e0 = sp.whole ? 1 : 0;
+  const int groups = (S + 1 - e0 + 3) / 4;
+#pragma unroll 1
+  for (int pass = 0; pass < NP; pass++) {
+    __syncthreads();
+    for (int t = tid; t < M::Q * groups; t += T) {
+      const int g = t / M::Q, ts = t - g * M::Q;
+      const int e = e0 + 4 * g;  // edges e .. e + 3; cells e - 3 .. e + 5
+      int vo, vn;
+      M::rows(ts, vo, vn);
+      const float* pv = sv + vo + (e - 3 + H) * M::V;
+      const float* pn = sv + vn + (e - 3 + H) * M::V;
+      const float* pq = sq + ts + (e - 3 + H) * M::Q;
+      float q[9], u[9], f[4];
+#pragma unroll
+      for (int k = 0; k < 9; k++) {
+        q[k] = pq[k * M::Q];
+        u[k] = __fmul_rn(0.5f, __fadd_rn(pv[k * M::V], pn[k * M::V]));  // v_D on the face
+      }
+      edge_fluxes<LIM>(q, u, c_half, f);
+#pragma unroll
+      for (int k = 0; k < 4; k++) sf[ts + (e + k) * M::Q] = f[k];
+    }
+    __syncthreads();
+    if (pass + 1 == NP) {
+      // finish the tile's cells
+      float* __restrict__ oA = a.out[A] + G.off;
+      float* __restrict__ oO = a.out[O] + G.off;
+      float* __restrict__ oD = a.out[D] + G.off;
+      static_assert(T % M::C == 0, "a thread keeps its pencil");
+      const int c = tid % M::C, row = c / LX, col = c - row * LX;
+      if (a0 + col < nA && b0 + row < nO) {
+        const int qa = row * (LX + 1) + col, qo = M::QA + row * LX + col;
+        const unsigned ob = (unsigned)((a0 + col) * sA + (b0 + row) * sO + s0 * sD);
+        for (int p = tid / M::C; p < S; p += T / M::C) {
+          const float* fl = sf + (sp.whole && p == 0 ? S : p) * M::Q;  // the edge below cell p
+          const float* fh = sf + (p + 1) * M::Q;
+          const float* qp = sq + (p + H) * M::Q;
+          const float fa0 = fl[qa], fo0 = fl[qo];
+          const unsigned o = ob + (unsigned)(p * sD);
+          oA[o] = __fmaf_rn(-c_full, __fsub_rn(fh[qa], fa0), qp[qa]);
+          oO[o] = __fmaf_rn(-c_full, __fsub_rn(fh[qo], fo0), qp[qo]);
+          oD[o] = constrain(sb[c + (p + H) * M::C], kA, fa0, fl[qa + 1], kO, fo0, fl[qo + LX], T1 == A);
+        }
+      }
+    } else {
+      // the first pass's result back into shared memory (whole pencils): the
+      // edge-flux rows' fields with their periodic images, and b_D
+      for (int t = tid; t < M::Q * S; t += T) {
+        const int p = t / M::Q, ts = t - p * M::Q;
+        float* z = sq + ts + H * M::Q;
+        const float v = __fmaf_rn(-c_full, __fsub_rn(sf[ts + (p + 1) * M::Q], sf[ts + (p == 0 ? S : p) * M::Q]),
+                                  z[p * M::Q]);
+        z[p * M::Q] = v;
+        if (p < H) z[(p + S) * M::Q] = v;
+        if (p >= S - H) z[(p - S) * M::Q] = v;
+      }
+      for (int t = tid; t < M::C * S; t += T) {
+        const int p = t / M::C, c = t - p * M::C, row = c / LX, col = c - row * LX;
+        const float* fl = sf + (p == 0 ? S : p) * M::Q;
+        const int qa = row * (LX + 1) + col, qo = M::QA + row * LX + col;
+        float* z = sb + c + (p + H) * M::C;
+        *z = constrain(*z, kA, fl[qa], fl[qa + 1], kO, fl[qo], fl[qo + LX], T1 == A);
+      }
+    }
+  }
+}
+
+// Along x: a slot's positions are contiguous, everything moves in 16-byte
+// pieces (4 positions; an odd number of pieces per slot keeps the slots of a
+// quarter warp in different banks).
+template <int LX, int R, int LIM>
+__global__ void __launch_bounds__(MTile<LX, R>::T) mag_tile_x_kernel(const __grid_constant__ MagArgs a) {
+  using M = MTile<LX, R>;
+  constexpr int H = mag_tile_halo(0), T = M::T;
+  extern __shared__ __align__(16) float mt_dyn[];
+  const BlockGeom G = block_geom(a.ens, a.box, a.seg, a.tau, nullptr);
+  const int nA = G.box.n[1], nO = G.box.n[2], nD = G.box.n[0];
+  const MagTile sp = mag_tile_split(nD);
+  const int a0 = G.bx * LX, b0 = G.by * R;
+  const int s0 = G.bz * sp.out, S = min(sp.out, nD - s0);  // multiples of 4
+  const int PN = mag_tile_positions(0, sp.out);
+  float* sv = mt_dyn;
+  float* sq = sv + M::V * PN;
+  float* sf = sq + M::Q * PN;
+  float* sb = sf + M::Q * PN;
+  const int tid = threadIdx.x;
+  const int sA = (int)G.box.stride[1], sO = (int)G.box.stride[2];
+  auto at4 = [](float* p) -> float4& { return *reinterpret_cast<float4*>(p); };
+
+  const int pieces = (S + 2 * H) / 4;
+  for (int half = 0; half < 2; half++) {  // copies, then v of the thread's own pieces
+    for (int t = tid; t < M::V * pieces; t += T) {
+      const int slot = t / pieces, g = t - slot * pieces;
+      const int row = slot / M::VC, col = slot - row * M::VC;
+      const bool rin = row >= 1 && row <= R, cin = col >= 1 && col <= LX;
+      if (!rin && !cin) continue;
+      float* v = sv + slot * PN + 4 * g;
+      float* r = sf + slot * PN + 4 * g;
+      if (half == 0) {
+        const unsigned c = (unsigned)(wrap_any(a0 + col - 1, nA) * sA + wrap_any(b0 + row - 1, nO) * sO +
+                                      wrap_any(s0 - H + 4 * g, nD)) + (unsigned)G.off;
+        copy16_async(v, a.in[MX] + c);
+        copy16_async(r, a.in[RHO] + c);
+        if (rin && col >= 1) copy16_async(sq + ((row - 1) * (LX + 1) + col - 1) * PN + 4 * g, a.in[BY] + c);
+        if (cin && row >= 1) copy16_async(sq + (M::QA + (row - 1) * LX + col - 1) * PN + 4 * g, a.in[BZ] + c);
+        if (rin && cin) copy16_async(sb + ((row - 1) * LX + col - 1) * PN + 4 * g, a.in[BX] + c);
+      } else {
+        const float4 m4 = at4(v), r4 = at4(r);
+        at4(v) = make_float4(v_div(m4.x, r4.x), v_div(m4.y, r4.y), v_div(m4.z, r4.z), v_div(m4.w, r4.w));
+      }
+    }
+    if (half == 0) copies_wait();
+  }
+  const float tau = G.tau;
+  const float c_full = tau * G.box.ih[0];  // tau / h_x
+  const float c_half = 0.5f * c_full;
+  const float kA = tau * G.box.ih[1];      // tau / h_y
+  const float kO = tau * G.box.ih[2];      // tau / h_z
+  const int e0 = sp.whole ? 1 : 0;         // edges e0 .. S, edge e at position e - e0 of sf
+  const int groups = (S + 1 - e0 + 3) / 4;
+  __syncthreads();
+  for (int t = tid; t < M::Q * groups; t += T) {
+    const int g = t / M::Q, ts = t - g * M::Q;
+    int vo, vn;
+    M::rows(ts, vo, vn);
+    // cells e - 3 .. e + 5, e = e0 + 4 g: positions 4 g + 1 + e0 .. of the
+    // three pieces from 4 g
+    auto cells = [&](float* s, float (&x)[9]) {
+      float w[12];
+#pragma unroll
+      for (int k = 0; k < 3; k++) {
+        const float4 z = at4(s + 4 * k);
+        w[4 * k] = z.x;
+        w[4 * k + 1] = z.y;
+        w[4 * k + 2] = z.z;
+        w[4 * k + 3] = z.w;
+      }
+#pragma unroll
+      for (int k = 0; k < 9; k++) x[k] = e0 ? w[k + 2] : w[k + 1];
+    };
+    float q[9], u[9], un[9], f[4];
+    cells(sv + vo * PN + 4 * g, u);
+    cells(sv + vn * PN + 4 * g, un);
+#pragma unroll
+    for (int k = 0; k < 9; k++) u[k] = __fmul_rn(0.5f, __fadd_rn(u[k], un[k]));  // v_x on the face
+    cells(sq + ts * PN + 4 * g, q);
+    edge_fluxes<LIM>(q, u, c_half, f);
+    at4(sf + ts * PN + 4 * g) = make_float4(f[0], f[1], f[2], f[3]);
+  }
+  __syncthreads();
+  // finish: 4 cells per thread and pencil
+  const int quads = S / 4;
+  for (int t = tid; t < M::C * quads; t += T) {
+    const int c = t / quads, g = t - c * quads;
+    const int row = c / LX, col = c - row * LX;
+    if (a0 + col >= nA || b0 + row >= nO) continue;
+    // edges below the 4 cells and above the last: F[0..4]
+    auto edges = [&](int ts, float (&F)[5]) {
+      float* s = sf + ts * PN;
+      const float4 z = at4(s + 4 * g);
+      if (e0) {
+        F[0] = s[g ? 4 * g - 1 : S - 1];
+        F[1] = z.x, F[2] = z.y, F[3] = z.z, F[4] = z.w;
+      } else {
+        F[0] = z.x, F[1] = z.y, F[2] = z.z, F[3] = z.w;
+        F[4] = s[4 * g + 4];
+      }
+    };
+    const int qa = row * (LX + 1) + col, qo = M::QA + row * LX + col;
+    float fa[5], fo[5], fa1[5], fo1[5], rA[4], rO[4], rD[4];
+    edges(qa, fa);
+    edges(qo, fo);
+    edges(qa + 1, fa1);
+    edges(qo + LX, fo1);
+    const float4 bA = at4(sq + qa * PN + H + 4 * g), bO = at4(sq + qo * PN + H + 4 * g),
+                 bD = at4(sb + c * PN + H + 4 * g);
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      rA[k] = __fmaf_rn(-c_full, __fsub_rn(fa[k + 1], fa[k]), (&bA.x)[k]);
+      rO[k] = __fmaf_rn(-c_full, __fsub_rn(fo[k + 1], fo[k]), (&bO.x)[k]);
+      rD[k] = constrain((&bD.x)[k], kA, fa[k], fa1[k], kO, fo[k], fo1[k], true);
+    }
+    const unsigned o = (unsigned)((a0 + col) * sA + (b0 + row) * sO + s0 + 4 * g) + (unsigned)G.off;
+    at4(a.out[1] + o) = make_float4(rA[0], rA[1], rA[2], rA[3]);
+    at4(a.out[2] + o) = make_float4(rO[0], rO[1], rO[2], rO[3]);
+    at4(a.out[0] + o) = make_float4(rD[0], rD[1], rD[2], rD[3]);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Launches.  A single box takes a block per run of pencils (fluid) or tile
+// (magnetic) and segment; an ensemble one block per work item.
+template <int LIM, int FRZ, bool FSQ>
+cudaError_t launch_fluid_tile(int axis, bool rate, const FluidArgs& a, cudaStream_t s) {
+  if constexpr (FRZ == 2) {
+    return cudaErrorInvalidValue;
+  } else {
+    const int A = (axis == 0) ? 1 : 0, O = (axis == 2) ? 1 : 2;
+    const FluidTile t = fluid_tile_split(axis, a.box.n[axis], a.tile);
+    const int threads = a.ens.items ? a.tile : (t.np * t.td + 31) / 32 * 32;
+    const long long pencils = (long long)a.box.n[A] * a.box.n[O];
+    const dim3 grid = a.ens.items ? dim3(a.nblocks) : dim3((unsigned)((pencils + t.np - 1) / t.np), 1, t.segs);
+    const size_t smem = fluid_tile_smem(threads);
+    const bool floor = a.p_floor > 0.f;
+#define FLUID_TILE_CASE(DD, RR, FF) \
+  if (axis == DD && rate == RR && floor == FF) fluid_tile_kernel<DD, RR, FF, LIM, FRZ, FSQ><<<grid, threads, smem, s>>>(a);
+    FLUID_TILE_CASE(0, false, false) FLUID_TILE_CASE(0, true, false) FLUID_TILE_CASE(0, false, true)
+    FLUID_TILE_CASE(0, true, true) FLUID_TILE_CASE(1, false, false) FLUID_TILE_CASE(1, true, false)
+    FLUID_TILE_CASE(1, false, true) FLUID_TILE_CASE(1, true, true) FLUID_TILE_CASE(2, false, false)
+    FLUID_TILE_CASE(2, true, false) FLUID_TILE_CASE(2, false, true) FLUID_TILE_CASE(2, true, true)
+#undef FLUID_TILE_CASE
+    return cudaGetLastError();
+  }
+}
+
+template <int LIM, int LX, int R>
+cudaError_t launch_mag_tile_shape(int axis, const MagArgs& a, cudaStream_t s) {
+  const int A = (axis == 0) ? 1 : 0, O = (axis == 2) ? 1 : 2;
+  const MagTile t = mag_tile_split(a.box.n[axis]);
+  const dim3 grid = a.ens.items ? dim3(a.nblocks)
+                                : dim3((a.box.n[A] + LX - 1) / LX, (a.box.n[O] + R - 1) / R, t.segs);
+  const size_t smem = mag_tile_smem<LX, R>(axis, a.ens.items ? a.tile_out : t.out);
+  constexpr int T = MTile<LX, R>::T;
+  if (axis == 0) mag_tile_x_kernel<LX, R, LIM><<<grid, T, smem, s>>>(a);
+  else if (axis == 1) mag_tile_kernel<1, LX, R, LIM, 1><<<grid, T, smem, s>>>(a);
+  else if (a.passes == 2) mag_tile_kernel<2, LX, R, LIM, 2><<<grid, T, smem, s>>>(a);
+  else mag_tile_kernel<2, LX, R, LIM, 1><<<grid, T, smem, s>>>(a);
+  return cudaGetLastError();
+}
+
+template <int LIM>
+cudaError_t launch_mag_tile(int axis, const MagArgs& a, cudaStream_t s) {
+  return a.tile == 1 ? launch_mag_tile_shape<LIM, 8, 2>(axis, a, s) : launch_mag_tile_shape<LIM, 16, 4>(axis, a, s);
+}
+
+// Shared-memory limits of the tile kernels, raised once per device before any
+// launch.
+template <int LIM, int FRZ, bool FSQ>
+cudaError_t prepare_fluid_tile() {
+  cudaError_t e = cudaSuccess;
+  const int smem = (int)fluid_tile_smem(kTileThreads);
+  auto set = [&](auto* k) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  };
+#define FLUID_TILE_SET(DD)                                                                                     \
+  set(fluid_tile_kernel<DD, false, false, LIM, FRZ, FSQ>), set(fluid_tile_kernel<DD, true, false, LIM, FRZ, FSQ>), \
+      set(fluid_tile_kernel<DD, false, true, LIM, FRZ, FSQ>), set(fluid_tile_kernel<DD, true, true, LIM, FRZ, FSQ>);
+  FLUID_TILE_SET(0) FLUID_TILE_SET(1) FLUID_TILE_SET(2)
+#undef FLUID_TILE_SET
+  return e;
+}
+
+template <int LIM, int LX, int R>
+cudaError_t prepare_mag_tile_shape() {
+  cudaError_t e = cudaSuccess;
+  auto set = [&](auto* k, int axis) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)mag_tile_smem<LX, R>(axis, kMTileWhole));
+  };
+  set(mag_tile_x_kernel<LX, R, LIM>, 0);
+  set(mag_tile_kernel<1, LX, R, LIM, 1>, 1);
+  set(mag_tile_kernel<2, LX, R, LIM, 1>, 2);
+  set(mag_tile_kernel<2, LX, R, LIM, 2>, 2);
+  return e;
+}
+template <int LIM>
+cudaError_t prepare_mag_tile() {
+  const cudaError_t e = prepare_mag_tile_shape<LIM, 8, 2>();
+  return e == cudaSuccess ? prepare_mag_tile_shape<LIM, 16, 4>() : e;
+}
+
+}  // namespace mhd

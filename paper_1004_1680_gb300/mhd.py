@@ -301,7 +301,8 @@ class Box:
         _check(self.lib.mhd_set_tma(self.h, int(bool(on))))
 
     def tma_sweeps(self) -> int:
-        """Sweeps (fluid and magnetic) this box has launched TMA-staged so far."""
+        """Sweeps (fluid and magnetic) this box has launched so far that qualify for
+        staging (TMA-staged, or as the tile sweep that replaces it)."""
         n = ctypes.c_longlong(0)
         _check(self.lib.mhd_tma_sweeps(self.h, ctypes.byref(n)))
         return int(n.value)
