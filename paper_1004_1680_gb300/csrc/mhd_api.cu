@@ -224,6 +224,10 @@ int tile_choice(const mhd_s* m, int d, bool mag, int passes) {
   // magnetic tiles of 8 x 2 pencils where there are few (32^3: 64 tiles, 10 us
   // against 15 us) and along x (128^3: 31 against 33 us), else 16 x 4
   const int shape = d == 0 || m->N <= 150000 ? 1 : 2;
+  // a launch holds 65535 rows of tiles (the axes' roles as in the sweeps: row
+  // axis z, or y for z sweeps) and as many segments of a pencil
+  if (mag && (m->n[d == 2 ? 1 : 2] > 2 * 65535 || m->n[d] > 24 * 65535)) return 0;
+  if (!mag && m->n[d] > 24 * 65535) return 0;
   if (d == 0) {
     const bool rows = m->n[0] % 128 == 0 && m->n[0] <= 1024;
     if (!mag) return rows ? 0 : 128;
