@@ -140,6 +140,8 @@ struct V5 {
 __device__ __forceinline__ float2 f2(float s) { return make_float2(s, s); }
 // a - b = fma(b, -1, a): the product is exact, so one rounding as in __fsub_rn
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, f2(-1.f), a); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 abs2(float2 a) { return make_float2(fabsf(a.x), fabsf(a.y)); }
 __device__ __forceinline__ V5 v5_sub(const V5& a, const V5& b) {
   return {sub2(a.p0, b.p0), sub2(a.p1, b.p1), __fsub_rn(a.e, b.e)};
 }

@@ -9,7 +9,9 @@
 //     max |div b| and the min pressure, reduced in a fixed order (bitwise
 //     reproducible).
 #include <cfloat>
+#include <cstdint>
 
+#include "fp32_sums.cuh"
 #include "mhd_device.cuh"
 #include "mhd_launch.h"
 
@@ -135,46 +137,12 @@ __device__ __forceinline__ KB kb_merge(KB a, KB b) {
 
 constexpr int kDiagThreads = 256;
 
-// Error-free FP32 transformations (Knuth's TwoSum; the FMA product error):
-// s + e == a + b and p + e == a * b exactly (round to nearest, no overflow).
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  const float bp = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bp)), __fsub_rn(b, bp));
+// Order-preserving integer image of a float (atomic minima and maxima).
+__device__ __forceinline__ int float_key(float x) {
+  const int i = __float_as_int(x);
+  return i < 0 ? i ^ 0x7fffffff : i;
 }
-__device__ __forceinline__ void two_prod(float a, float b, float& p, float& e) {
-  p = __fmul_rn(a, b);
-  e = __fmaf_rn(a, b, -p);
-}
-
-// FP32 window sums without FP64 arithmetic per value (FP64 runs at a small
-// fraction of the FP32 rate on this GPU): three FP32 words h + l + t.  Each
-// value goes into h by TwoSum; its error goes into l by TwoSum; that error
-// into t by a plain add.  With P the largest partial sum of a window of K
-// values, |error of h + l| <= K 2^-24 P, so |t's errors| <= K^3 2^-72 P:
-// 2^-48 P for K = kWin = 256.  Infinities and NaNs make the sum NaN, as in
-// FP64.
-constexpr int kWin = 256;
-struct FWin {
-  float h, l, t;
-};
-
-__device__ __forceinline__ void fwin_add(FWin& w, float x) {
-  float s, e, s2, e2;
-  two_sum(w.h, x, s, e);
-  two_sum(w.l, e, s2, e2);
-  w.h = s;
-  w.l = s2;
-  w.t = __fadd_rn(w.t, e2);
-}
-
-// A lane's windows add up in a plain FP64 sum (a few windows per lane: their
-// roundings stay near 2^-53 of the field's absolute sum); the compensated
-// sum starts at the warps' totals.
-__device__ __forceinline__ void fwin_flush(FWin& w, double& acc) {
-  acc += ((double)w.h + (double)w.l) + (double)w.t;
-  w = FWin{0.f, 0.f, 0.f};
-}
+__device__ __forceinline__ float key_float(int k) { return __int_as_float(k < 0 ? k ^ 0x7fffffff : k); }
 
 // The FP64 values of one cell (the formulas the diagnostics define), out of
 // line: the filters below reach them for a few cells only.
@@ -190,280 +158,407 @@ __device__ __noinline__ double cell_p64(float rho, float m1, float m2, float m3,
   return (gamma - 1.0) * ((double)e - kin - 0.5 * (b0 * b0 + b1 * b1 + b2 * b2));
 }
 
-// Float-float tier of the max |div b| filter (inline: out of line it cost
-// about 15 % on near-tied states, for no fewer registers).  Each
-// difference is exact (TwoSum), times n_d (product error by FMA), summed by
-// TwoSum: |D - div| <= 2^-44 dT, dT = sum |(b_high - b_low) n_d|.  True
-// unless |div| is certainly below thr.
-__device__ __forceinline__ bool div_ff_may_exceed(float bxl, float bxh, float byl, float byh, float bzl,
-                                                  float bzh, float nxf, float nyf, float nzf, float thr) {
-  float s0, e0, s1, e1, s2, e2, p0, q0, p1, q1, p2, q2;
-  two_sum(bxh, -bxl, s0, e0);
-  two_sum(byh, -byl, s1, e1);
-  two_sum(bzh, -bzl, s2, e2);
-  two_prod(s0, nxf, p0, q0);
-  two_prod(s1, nyf, p1, q1);
-  two_prod(s2, nzf, p2, q2);
-  float h01, r01, dh, r2;
-  two_sum(p0, p1, h01, r01);
-  two_sum(h01, p2, dh, r2);
-  const float dl = __fadd_rn(__fadd_rn(__fadd_rn(q0, q1), q2),
-                             __fadd_rn(__fadd_rn(__fmaf_rn(e0, nxf, __fmul_rn(e1, nyf)), __fmul_rn(e2, nzf)),
-                                       __fadd_rn(r01, r2)));
-  const float dT = fabsf(p0) + fabsf(p1) + fabsf(p2);
-  const float dabs = fabsf(__fadd_rn(dh, dl));
-  return !(dabs + (0x1p-22f * dabs + 0x1p-40f * dT + 1e-37f) < thr);  // NaN: true
+// Float-float estimate of |div b| of two cells on packed FP32.  Each difference
+// is exact (TwoSum), times n_d (product error by FMA), summed by TwoSum: the
+// estimate is within 2^-44 dT of div, dT = sum |(b_high - b_low) n_d|; err
+// covers it with a margin of 16.  (An FP32 estimate in front rules nothing
+// out: the field is divergence-free up to rounding, so max |div b| is of the
+// size of that estimate's own error.)
+__device__ __forceinline__ void div_ff2(float2 xl, float2 xh, float2 yl, float2 yh, float2 zl, float2 zh, float2 nx,
+                                        float2 ny, float2 nz, float2& dabs, float2& err, float2& dT) {
+  float2 s0, e0, s1, e1, s2, e2;
+  two_sum2(xh, neg2(xl), s0, e0);
+  two_sum2(yh, neg2(yl), s1, e1);
+  two_sum2(zh, neg2(zl), s2, e2);
+  const float2 p0 = __fmul2_rn(s0, nx), p1 = __fmul2_rn(s1, ny), p2 = __fmul2_rn(s2, nz);
+  const float2 q0 = __ffma2_rn(s0, nx, neg2(p0)), q1 = __ffma2_rn(s1, ny, neg2(p1)), q2 = __ffma2_rn(s2, nz, neg2(p2));
+  float2 h01, r01, dh, r2;
+  two_sum2(p0, p1, h01, r01);
+  two_sum2(h01, p2, dh, r2);
+  float2 dl = __fadd2_rn(__fadd2_rn(q0, q1), q2);
+  dl = __ffma2_rn(e0, nx, __ffma2_rn(e1, ny, __ffma2_rn(e2, nz, dl)));
+  dl = __fadd2_rn(dl, __fadd2_rn(r01, r2));
+  const float2 d = __fadd2_rn(dh, dl);
+  dabs = make_float2(fabsf(d.x), fabsf(d.y));
+  dT = make_float2(fabsf(p0.x) + fabsf(p1.x) + fabsf(p2.x), fabsf(p0.y) + fabsf(p1.y) + fabsf(p2.y));
+  err = __ffma2_rn(f2(0x1p-22f), dabs, __ffma2_rn(f2(0x1p-40f), dT, f2(1e-37f)));
 }
 
-// Float-float tier of the min p filter:
-// |estimate - p| <= 2^-42 (gamma - 1) U.  True unless p certainly exceeds
-// the float-float threshold th + tl.
-__device__ __forceinline__ bool p_ff_may_undercut(float rho, float m1, float m2, float m3, float e, float bxl,
-                                                  float bxh, float byl, float byh, float bzl, float bzh, float rr,
-                                                  float g_hi, float g_lo, float U, float th, float tl) {
-  float a0, ae0, a1, ae1, a2, ae2, sa, ra, sh, rb;
-  two_prod(m1, m1, a0, ae0);
-  two_prod(m2, m2, a1, ae1);
-  two_prod(m3, m3, a2, ae2);
-  two_sum(a0, a1, sa, ra);
-  two_sum(sa, a2, sh, rb);
-  const float sl = __fadd_rn(__fadd_rn(__fadd_rn(ae0, ae1), ae2), __fadd_rn(ra, rb));
-  // an approximate reciprocal rr: k1 within a few ulp of S / rho, the FMA
-  // remainder S - k1 rho then corrects it to about 2^-43 S / rho
-  const float k1 = __fmul_rn(sh, rr);
-  const float k2 = __fmul_rn(__fadd_rn(__fmaf_rn(-k1, rho, sh), sl), rr);  // kin = (k1 + k2) / 2
-  float c0h, c0l, c1h, c1l, c2h, c2l;
-  two_sum(bxl, bxh, c0h, c0l);
-  two_sum(byl, byh, c1h, c1l);
-  two_sum(bzl, bzh, c2h, c2l);  // 2 b_c = c_h + c_l exactly
-  float w0, we0, w1, we1, w2, we2, sw, rw, mh, rm;
-  two_prod(c0h, c0h, w0, we0);
-  two_prod(c1h, c1h, w1, we1);
-  two_prod(c2h, c2h, w2, we2);
-  we0 = __fmaf_rn(2.f * c0h, c0l, we0);
-  we1 = __fmaf_rn(2.f * c1h, c1l, we1);
-  we2 = __fmaf_rn(2.f * c2h, c2l, we2);
-  two_sum(w0, w1, sw, rw);
-  two_sum(sw, w2, mh, rm);  // 4 |b_c|^2 = mh + ml
-  const float ml = __fadd_rn(__fadd_rn(__fadd_rn(we0, we1), we2), __fadd_rn(rw, rm));
-  float d1, de1, d2, de2;
-  two_sum(e, -0.5f * k1, d1, de1);
-  two_sum(d1, -0.125f * mh, d2, de2);
-  const float dlo = __fsub_rn(__fsub_rn(__fadd_rn(de1, de2), 0.5f * k2), 0.125f * ml);
-  float ph, phe;
-  two_prod(g_hi, d2, ph, phe);
-  const float pl = __fadd_rn(phe, __fmaf_rn(g_hi, dlo, __fmul_rn(g_lo, d2)));
-  const float dp = 0x1p-38f * g_hi * U + 1e-37f;
-  return !(__fadd_rn(__fsub_rn(ph, th), __fsub_rn(__fsub_rn(pl, tl), dp)) > 0.f);  // NaN: true
+// Float-float estimate ph + pl of the pressure of two cells on packed FP32,
+// within 2^-42 (gamma - 1) U of p (U below); err covers it with a margin of 16.
+// rr: an approximate reciprocal of rho.
+__device__ __forceinline__ void p_ff2(float2 rho, float2 m1, float2 m2, float2 m3, float2 e, float2 xl, float2 xh,
+                                      float2 yl, float2 yh, float2 zl, float2 zh, float2 rr, float g_hi, float g_lo,
+                                      float2 U, float2& ph, float2& pl, float2& err) {
+  float2 a0, ae0, a1, ae1, a2, ae2, sa, ra, sh, rb;
+  two_prod2(m1, m1, a0, ae0);
+  two_prod2(m2, m2, a1, ae1);
+  two_prod2(m3, m3, a2, ae2);
+  two_sum2(a0, a1, sa, ra);
+  two_sum2(sa, a2, sh, rb);
+  const float2 sl = __fadd2_rn(__fadd2_rn(__fadd2_rn(ae0, ae1), ae2), __fadd2_rn(ra, rb));
+  // k1 within a few ulp of S / rho; the FMA remainder S - k1 rho corrects it
+  // to about 2^-43 S / rho
+  const float2 k1 = __fmul2_rn(sh, rr);
+  const float2 k2 = __fmul2_rn(__fadd2_rn(__ffma2_rn(neg2(k1), rho, sh), sl), rr);  // kin = (k1 + k2) / 2
+  float2 c0h, c0l, c1h, c1l, c2h, c2l;
+  two_sum2(xl, xh, c0h, c0l);
+  two_sum2(yl, yh, c1h, c1l);
+  two_sum2(zl, zh, c2h, c2l);  // 2 b_c = c_h + c_l exactly
+  float2 w0, we0, w1, we1, w2, we2, sw, rw, mh, rm;
+  two_prod2(c0h, c0h, w0, we0);
+  two_prod2(c1h, c1h, w1, we1);
+  two_prod2(c2h, c2h, w2, we2);
+  we0 = __ffma2_rn(__fadd2_rn(c0h, c0h), c0l, we0);
+  we1 = __ffma2_rn(__fadd2_rn(c1h, c1h), c1l, we1);
+  we2 = __ffma2_rn(__fadd2_rn(c2h, c2h), c2l, we2);
+  two_sum2(w0, w1, sw, rw);
+  two_sum2(sw, w2, mh, rm);  // 4 |b_c|^2 = mh + ml
+  const float2 ml = __fadd2_rn(__fadd2_rn(__fadd2_rn(we0, we1), we2), __fadd2_rn(rw, rm));
+  float2 d1, de1, d2, de2;
+  two_sum2(e, __fmul2_rn(f2(-0.5f), k1), d1, de1);
+  two_sum2(d1, __fmul2_rn(f2(-0.125f), mh), d2, de2);
+  float2 dlo = __ffma2_rn(f2(-0.5f), k2, __fadd2_rn(de1, de2));
+  dlo = __ffma2_rn(f2(-0.125f), ml, dlo);
+  float2 phe;
+  two_prod2(f2(g_hi), d2, ph, phe);
+  pl = __fadd2_rn(phe, __ffma2_rn(f2(g_hi), dlo, __fmul2_rn(f2(g_lo), d2)));
+  err = __ffma2_rn(f2(0x1p-38f * g_hi), U, f2(1e-37f));
+}
+
+// n / d for 0 <= n < 2^31 by a multiplication: the quotient rounded down.
+struct FastDiv {
+  unsigned mul, shift, d;
+};
+FastDiv fast_div(unsigned d) {
+  FastDiv f{0, 0, d};
+  while ((1ull << f.shift) < d) f.shift++;
+  f.mul = (unsigned)(((1ull << 32) * ((1ull << f.shift) - d)) / d + 1);
+  return f;
+}
+__device__ __forceinline__ unsigned quotient(unsigned n, const FastDiv& f) {
+  return (unsigned)(((unsigned long long)__umulhi(n, f.mul) + n) >> f.shift);
 }
 
 // One pass over the box: the compensated sums of the 8 fields, max |div b|
 // (the face differences of each cell) and min p, in FP64 as defined by the
-// formulas below.  The extrema are exact FP64 values of those formulas: a
-// cell's FP64 value is only evaluated when a float-float estimate (about 44
-// bits, error bound with a margin of 16 or more) does not rule it out
-// against the warp's running extremum.  Lanes of a warp iterate together
-// over whole x rows (lanes past the row's end add zeros); the FP64 values sit
-// behind warp votes, and the lanes share their new thresholds right after.
-__global__ void __launch_bounds__(kDiagThreads)
+// formulas above.  The extrema are exact FP64 values of those formulas: a
+// cell's FP64 value is only evaluated when an estimate with an error bound
+// (and a margin of 4 or more) does not rule it out against the running
+// extremum.  The estimates sit behind warp votes, a warp's lanes share their
+// new thresholds right after, and the block's warps share theirs through
+// shared memory (a threshold only rules cells out, so the extrema do not
+// depend on when it arrives).
+//
+// A lane takes W = 2 consecutive cells per turn (8-byte loads; nx even and
+// aligned fields) or one, and every operation runs on two cells at once (packed
+// FP32; with 4 cells the windows and values spill).  At 256^3, pressures
+// tied to FP32 rounding (a uniform initial pressure: every cell takes the
+// float-float estimate): 381 -> 255 us, 431 -> 288 instructions per cell,
+// and 512^3 of evolved turbulence 2.12 -> 1.63 ms with the final reduction.
+// Instruction issue and its latencies at 16 warps per SM bound it.  An FP64
+// instruction occupies an SM's pipe for 16 cycles a warp, so the grid is what
+// fits at once (2 blocks per SM: few blocks meet their extremum from
+// nothing), thresholds come from the estimates, the lowest pressure of a lane
+// is evaluated once at the end, and FP64 sums appear once per block or window.
+template <int W>
+__global__ void __launch_bounds__(kDiagThreads, 2)
 diag_partial_kernel(const float* __restrict__ rho, const float* __restrict__ mx,
                     const float* __restrict__ my, const float* __restrict__ mz,
                     const float* __restrict__ en, const float* __restrict__ bx,
-                    const float* __restrict__ by, const float* __restrict__ bz, Box box,
-                    double gamma, double* __restrict__ partial) {
+                    const float* __restrict__ by, const float* __restrict__ bz, int nx, int ny, int nz,
+                    FastDiv row_div, FastDiv ny_div, double gamma, double* __restrict__ partial) {
   const float* f[8] = {rho, mx, my, mz, en, bx, by, bz};
-  const int lane = threadIdx.x & 31;
-  double acc[8];
-  FWin win[8];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  __shared__ int sh_p, sh_div;  // the block's thresholds (float_key)
+  __shared__ double sacc[kDiagThreads / 32][8];
+  __shared__ float2 sw[kDiagThreads / 32][8][3];
+  __shared__ double sx[kDiagThreads / 32][2];
+  FWin2 win[8];
+#pragma unroll
+  for (int q = 0; q < 8; q++) win[q].h = win[q].l = win[q].t = f2(0.f);
+  double divmax = 0.0, pmin = DBL_MAX;
+  float best_h = 3e38f, best_l = 0.f, best_e = 0.f;       // the lane's lowest pressure so far, to be evaluated at the end
+  unsigned best_c = 0;
+  float div_thr = 0.f;                                    // <= the block's running max |div b|
+  float pt_hi = __int_as_float(0x7f800000), pt_lo = 0.f;  // >= the block's running min p
+  const float2 n0 = f2((float)nx), n1 = f2((float)ny), n2 = f2((float)nz);
+  const float g_hi = (float)(gamma - 1.0), g_lo = (float)((gamma - 1.0) - (double)g_hi);
+  if (threadIdx.x == 0) {
+    sh_p = float_key(pt_hi);
+    sh_div = float_key(0.f);
+  }
+  if (lane == 0)
+    for (int q = 0; q < 8; q++) sacc[wid][q] = 0.0;
+  __syncthreads();
+  const unsigned rowlen = (unsigned)nx / W;            // turns of a row
+  const unsigned turns = rowlen * (unsigned)ny * (unsigned)nz;  // < 2^31
+  const unsigned plane = (unsigned)nx * (unsigned)ny;
+  bool seeded = false;
+  int it = 0;
+  // a warp's window words into its FP64 accumulators
+  auto flush = [&] {
+#pragma unroll
+    for (int q = 0; q < 8; q++) {
+      double a0 = 0.0, a1 = 0.0;
+      fwin_flush(win[q], a0, a1);
+      a0 += a1;
+      for (int o = 16; o > 0; o >>= 1) a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+      if (lane == 0) sacc[wid][q] += a0;
+    }
+  };
+  for (unsigned base = (blockIdx.x * kDiagThreads + wid * 32); base < turns; base += gridDim.x * kDiagThreads) {
+    const unsigned g = min(base + lane, turns - 1);
+    const bool valid = base + lane < turns;
+    const unsigned row = quotient(g, row_div), i = (g - row * rowlen) * W, k = quotient(row, ny_div), j = row - k * ny;
+    const unsigned c = row * (unsigned)nx + i;
+    const unsigned cy = j + 1 == (unsigned)ny ? c - (unsigned)(ny - 1) * nx : c + nx;
+    const unsigned cz = k + 1 == (unsigned)nz ? c - (unsigned)(nz - 1) * plane : c + plane;
+    float v[8][2], hy[2], hz[2];
+    auto load = [&](const float* p, float (&d)[2]) {
+      if constexpr (W == 2) {
+        const float2 x = __ldg(reinterpret_cast<const float2*>(p));
+        d[0] = x.x, d[1] = x.y;
+      } else {
+        d[0] = __ldg(p);
+        d[1] = 0.f;
+      }
+    };
+#pragma unroll
+    for (int q = 0; q < 8; q++) load(f[q] + c, v[q]);
+    load(by + cy, hy);
+    load(bz + cz, hz);
+    const float bx_next = __ldg(bx + (i + W == (unsigned)nx ? c - i : c + W));
+    if (!valid)
+#pragma unroll
+      for (int q = 0; q < 8; q++)
+        v[q][0] = v[q][1] = 0.f;
+#pragma unroll
+    for (int q = 0; q < 8; q++) fwin_add(win[q], make_float2(v[q][0], v[q][1]));
+    // high x face of cell e
+    auto hx = [&](int e) { return e + 1 < W ? v[5][1] : bx_next; };
+    auto pair = [&](int q) { return make_float2(v[q][0], v[q][1]); };
+    const float2 xh = make_float2(hx(0), hx(1)), yh = make_float2(hy[0], hy[1]), zh = make_float2(hz[0], hz[1]);
+    // thresholds that other warps have found since
+    div_thr = fmaxf(div_thr, key_float(*reinterpret_cast<volatile int*>(&sh_div)));
+    {
+      const float sp = key_float(*reinterpret_cast<volatile int*>(&sh_p));
+      if (sp < pt_hi) {
+        pt_hi = sp;
+        pt_lo = 0.f;
+      }
+    }
+    // p = (gamma - 1)(e - |m|^2 / (2 rho) - |b_c|^2 / 2), U = |e| + |kin| +
+    // sum ((|b| + |b_high|) / 2)^2 / 2.  FP32: |error| <= 2^-19 (gamma - 1) U.
+    float2 dabs, derr, dT;
+    div_ff2(pair(5), xh, pair(6), yh, pair(7), zh, n0, n1, n2, dabs, derr, dT);
+    const float2 rr = make_float2(fast_rcp(v[0][0]), fast_rcp(v[0][1]));
+    const float2 kin = __fmul2_rn(__ffma2_rn(pair(1), pair(1), __ffma2_rn(pair(2), pair(2), __fmul2_rn(pair(3), pair(3)))),
+                                  __fmul2_rn(f2(0.5f), rr));
+    const float2 bc0 = __fadd2_rn(pair(5), xh), bc1 = __fadd2_rn(pair(6), yh), bc2 = __fadd2_rn(pair(7), zh);  // 2 b_c
+    const float2 b2 = __ffma2_rn(bc0, bc0, __ffma2_rn(bc1, bc1, __fmul2_rn(bc2, bc2)));
+    const float2 a0 = __fadd2_rn(abs2(pair(5)), abs2(xh)), a1 = __fadd2_rn(abs2(pair(6)), abs2(yh)),
+                 a2 = __fadd2_rn(abs2(pair(7)), abs2(zh));
+    const float2 U = __ffma2_rn(f2(0.125f), __ffma2_rn(a0, a0, __ffma2_rn(a1, a1, __fmul2_rn(a2, a2))),
+                                __fadd2_rn(abs2(pair(4)), abs2(kin)));
+    const float2 perr = __ffma2_rn(f2(0x1p-17f * g_hi), U, f2(1e-37f));
+    const float2 p32 = __fmul2_rn(f2(g_hi), sub2(__ffma2_rn(f2(-0.125f), b2, pair(4)), kin));
+    auto el = [](const float2& x, int e) { return e & 1 ? x.y : x.x; };
+    if (!seeded) {  // the block's first thresholds
+      seeded = true;
+#pragma unroll
+      for (int e = 0; e < W; e++) {
+        const float lo = el(dabs, e) - el(derr, e), hi = el(p32, e) + el(perr, e);
+        if (valid && lo > div_thr && lo < 3e38f) div_thr = lo;
+        if (valid && hi < pt_hi && fabsf(hi) < 3e38f) pt_hi = hi, pt_lo = 0.f;
+      }
+      if (div_thr > 0.f) atomicMax(&sh_div, float_key(div_thr));
+      if (fabsf(pt_hi) < 3e38f) atomicMin(&sh_p, float_key(pt_hi));
+      __syncwarp();
+      div_thr = key_float(*reinterpret_cast<volatile int*>(&sh_div));
+      pt_hi = key_float(*reinterpret_cast<volatile int*>(&sh_p));
+    }
+    // cells that the estimates do not rule out; a NaN always goes on, and a
+    // cell whose three differences are zero (uniform fields) has div b = 0
+    const float pt_up = pt_hi + (pt_lo + 0x1p-22f * fabsf(pt_hi));  // >= the threshold, rounded
+    unsigned cd = 0, cp = 0;
+#pragma unroll
+    for (int e = 0; e < W; e++) {
+      if (valid && el(dT, e) != 0.f && !(el(dabs, e) + el(derr, e) < div_thr)) cd |= 1u << e;
+      if (valid && !(__fsub_rn(el(p32, e), el(perr, e)) > pt_up)) cp |= 1u << e;
+    }
+    if (__any_sync(0xffffffffu, cd != 0)) {
+#pragma unroll
+      for (int e = 0; e < W; e++) {
+        if (cd >> e & 1) {
+          const double div = cell_div64(v[5][e], hx(e), v[6][e], hy[e], v[7][e], hz[e], nx, ny, nz);
+          divmax = fmax(divmax, fabs(div));
+          div_thr = fmaxf(div_thr, __double2float_rd(divmax));
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) div_thr = fmaxf(div_thr, __shfl_xor_sync(0xffffffffu, div_thr, o));
+      if (lane == 0) atomicMax(&sh_div, float_key(div_thr));
+    }
+    if (__any_sync(0xffffffffu, cp != 0)) {
+      float2 ph, pl, pe;
+      p_ff2(pair(0), pair(1), pair(2), pair(3), pair(4), pair(5), xh, pair(6), yh, pair(7), zh, rr, g_hi, g_lo, U, ph, pl,
+            pe);
+      // new upper bounds of the minimum: over the lane's cells, then the warp
+      bool lower = false;
+#pragma unroll
+      for (int e = 0; e < W; e++) {
+        const float h = el(ph, e), l = __fadd_ru(el(pl, e), el(pe, e));
+        if ((cp >> e & 1) && fabsf(h) < 1e38f && !(__fadd_rn(__fsub_rn(h, pt_hi), __fsub_rn(l, pt_lo)) >= 0.f)) {
+          pt_hi = h;
+          pt_lo = l;
+          lower = true;
+        }
+      }
+      if (__any_sync(0xffffffffu, lower)) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const float oh = __shfl_xor_sync(0xffffffffu, pt_hi, o), ol = __shfl_xor_sync(0xffffffffu, pt_lo, o);
+          if (__fadd_rn(__fsub_rn(oh, pt_hi), __fsub_rn(ol, pt_lo)) < 0.f) {
+            pt_hi = oh;
+            pt_lo = ol;
+          }
+        }
+        if (lane == 0 && fabsf(pt_hi) < 1e38f) atomicMin(&sh_p, float_key(__fadd_ru(pt_hi, pt_lo)));
+      }
+      // candidates against the new bound: the lane keeps the lowest one for the
+      // end (its FP64 value is needed only if it still stands then); one that
+      // cannot be told from it, or that FP32 cannot hold, is evaluated now
+#pragma unroll
+      for (int e = 0; e < W; e++) {
+        const float h = el(ph, e), l = el(pl, e), er = el(pe, e);
+        const bool far = !(fabsf(h) < 1e38f) || !(fabsf(er) < 1e38f);
+        if ((cp >> e & 1) && (far || !(__fadd_rn(__fsub_rn(h, pt_hi), __fsub_rn(__fsub_rn(l, pt_lo), er)) > 0.f))) {
+          const float diff = __fadd_rn(__fsub_rn(h, best_h), __fsub_rn(l, best_l)), tol = 1.125f * (er + best_e);
+          if (!far && diff < -tol) {
+            best_h = h;
+            best_l = l;
+            best_e = er;
+            best_c = c + e;
+          } else if (far || !(diff > tol)) {
+            pmin = fmin(pmin, cell_p64(v[0][e], v[1][e], v[2][e], v[3][e], v[4][e], v[5][e], hx(e), v[6][e], hy[e],
+                                       v[7][e], hz[e], gamma));
+          }
+        }
+      }
+    }
+    if (++it == kWin) {
+      it = 0;
+      flush();
+    }
+  }
+  // the lanes' kept candidates that the block's final threshold leaves
+  __syncthreads();
+  {
+    const float sp = key_float(sh_p);
+    if (best_h < 3e38f && !(best_h + (best_l - best_e) - 0x1p-22f * fabsf(best_h) > sp)) {
+      const unsigned c = best_c, row = c / (unsigned)nx, i = c - row * nx, k = row / (unsigned)ny, j = row - k * ny;
+      const unsigned cx = i + 1 == (unsigned)nx ? c - i : c + 1;
+      const unsigned cy = j + 1 == (unsigned)ny ? c - (unsigned)(ny - 1) * nx : c + nx;
+      const unsigned cz = k + 1 == (unsigned)nz ? c - (unsigned)(nz - 1) * plane : c + plane;
+      pmin = fmin(pmin, cell_p64(rho[c], mx[c], my[c], mz[c], en[c], bx[c], bx[cx], by[c], by[cy], bz[c], bz[cz], gamma));
+    }
+  }
+  // windows whose block total could leave FP32's range go on in FP64
+  bool large = false;
+#pragma unroll
+  for (int q = 0; q < 8; q++) large = large || !(fabsf(win[q].h.x) + fabsf(win[q].h.y) < 1e35f);
+  if (__syncthreads_or(large)) flush();
+  // the block's totals in a fixed order: the words over the lanes by a shuffle
+  // tree and over the warps in order, in FP32, then in FP64 with the windows
+  // flushed before; one warp per extremum
 #pragma unroll
   for (int q = 0; q < 8; q++) {
-    acc[q] = 0.0;
-    win[q] = FWin{0.f, 0.f, 0.f};
-  }
-  double divmax = 0.0, pmin = DBL_MAX;
-  float div_thr = 0.f;                        // <= the warp's running max |div b|
-  float pt_hi = __int_as_float(0x7f800000), pt_lo = 0.f;  // >= the warp's running min p
-  const float nxf = (float)box.n[0], nyf = (float)box.n[1], nzf = (float)box.n[2];
-  const float g_hi = (float)(gamma - 1.0), g_lo = (float)((gamma - 1.0) - (double)g_hi);
-  // a warp walks whole x rows (no division per cell), 32 cells at a time
-  const int nx = box.n[0], ny = box.n[1], nz = box.n[2];
-  const long long rows = (long long)ny * nz;
-  const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
-  int it = 0;
-  // row r = j + ny k, stepped by nwarps rows without a division per row
-  // (64-bit integer division is emulated in software)
-  long long r = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  int j = (int)(r % ny);
-  long long k = r / ny;
-  const int dj = (int)(nwarps % ny);
-  const long long dk = nwarps / ny;
-  for (; r < rows; r += nwarps) {
-    const long long rowbase = j * box.stride[1] + k * box.stride[2];
-    const long long yoff = (j + 1 < ny) ? box.stride[1] : -(long long)(ny - 1) * box.stride[1];
-    const long long zoff = (k + 1 < nz) ? box.stride[2] : -(long long)(nz - 1) * box.stride[2];
-    // the 11 values of a lane's cell at x = i0 + lane (x is the contiguous
-    // axis, checked at launch); the next chunk's loads go out before this
-    // chunk's arithmetic
-    float nv[11];
-    auto load = [&](int i0, float (&u)[11]) {
-      const int ii = min(i0 + lane, nx - 1);
-      const long long cc = rowbase + ii;
 #pragma unroll
-      for (int q = 0; q < 8; q++) u[q] = __ldg(f[q] + cc);
-      u[8] = __ldg(bx + (ii + 1 < nx ? cc + 1 : cc - (nx - 1)));
-      u[9] = __ldg(by + cc + yoff);
-      u[10] = __ldg(bz + cc + zoff);
-    };
-    load(0, nv);
-    for (int i0 = 0; i0 < nx; i0 += 32, it++) {
-      const bool valid = i0 + lane < nx;
-      float v[8];
-#pragma unroll
-      for (int q = 0; q < 8; q++) v[q] = valid ? nv[q] : 0.f;
-      const float bxh = nv[8], byh = nv[9], bzh = nv[10];
-      if (i0 + 32 < nx) load(i0 + 32, nv);
-#pragma unroll
-      for (int q = 0; q < 8; q++) fwin_add(win[q], v[q]);
-      {
-        // Three tiers, each behind a warp vote (so that a tier is skipped, not
-        // just predicated off, when no lane needs it): an FP32 estimate, a
-        // float-float estimate, the FP64 value.  A lane's cell goes on only if
-        // the tier's error bound (with a margin of 4 or more) cannot rule it out
-        // against the warp's running extremum; a NaN always goes on.
-        //
-        // div b = sum_d (b_high - b_low) n_d.  FP32: |error| <= 2^-22 dT with
-        // dT = sum |(b_high - b_low) n_d|.
-        const float t0 = __fmul_rn(__fsub_rn(bxh, v[5]), nxf), t1 = __fmul_rn(__fsub_rn(byh, v[6]), nyf),
-                    t2 = __fmul_rn(__fsub_rn(bzh, v[7]), nzf);
-        const float d32 = fabsf(t0 + t1 + t2), T32 = fabsf(t0) + fabsf(t1) + fabsf(t2);
-        const bool sdiv = valid && !(d32 + (0x1p-20f * T32 + 1e-37f) < div_thr);
-        if (__any_sync(0xffffffffu, sdiv)) {
-          const bool cand_div = sdiv && div_ff_may_exceed(v[5], bxh, v[6], byh, v[7], bzh, nxf, nyf, nzf, div_thr);
-          if (__any_sync(0xffffffffu, cand_div)) {
-            if (cand_div) {
-              const double div = cell_div64(v[5], bxh, v[6], byh, v[7], bzh, nx, ny, nz);
-              divmax = fmax(divmax, fabs(div));
-              div_thr = fmaxf(div_thr, __double2float_rd(divmax));
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) div_thr = fmaxf(div_thr, __shfl_xor_sync(0xffffffffu, div_thr, o));
-          }
-        }
-        // p = (gamma - 1)(e - |m|^2 / (2 rho) - |b_c|^2 / 2), U = |e| + |kin| +
-        // sum ((|b| + |b_high|) / 2)^2 / 2.  FP32: |error| <= 2^-19 (gamma - 1) U.
-        const float rr = fast_rcp(v[0]);
-        const float kin32 = 0.5f * __fmaf_rn(v[1], v[1], __fmaf_rn(v[2], v[2], __fmul_rn(v[3], v[3]))) * rr;
-        const float bc0 = v[5] + bxh, bc1 = v[6] + byh, bc2 = v[7] + bzh;  // 2 b_c
-        const float p32 = g_hi * (v[4] - kin32 - 0.125f * __fmaf_rn(bc0, bc0, __fmaf_rn(bc1, bc1, __fmul_rn(bc2, bc2))));
-        const float ax = fabsf(v[5]) + fabsf(bxh), ay = fabsf(v[6]) + fabsf(byh), az = fabsf(v[7]) + fabsf(bzh);
-        const float U = fabsf(v[4]) + fabsf(kin32) + 0.125f * (ax * ax + ay * ay + az * az);
-        // skip while p32 - bound exceeds the threshold pt_hi + pt_lo (>= the
-        // warp's min; 2^-22 |pt_hi| covers rounding that sum)
-        const bool sp = valid && !(__fsub_rn(p32, 0x1p-17f * g_hi * U + 1e-37f) >
-                                   pt_hi + (pt_lo + 0x1p-22f * fabsf(pt_hi)));
-        if (__any_sync(0xffffffffu, sp)) {
-          const bool cand_p = sp && p_ff_may_undercut(v[0], v[1], v[2], v[3], v[4], v[5], bxh, v[6], byh, v[7], bzh, rr,
-                                                      g_hi, g_lo, U, pt_hi, pt_lo);
-          if (__any_sync(0xffffffffu, cand_p)) {
-            if (cand_p) {
-              const double p = cell_p64(v[0], v[1], v[2], v[3], v[4], v[5], bxh, v[6], byh, v[7], bzh, gamma);
-              pmin = fmin(pmin, p);
-              // float-float upper bound of pmin (pt_hi + pt_lo >= pmin)
-              if (fabs(pmin) < 1e38) {
-                const float h = __double2float_rn(pmin);
-                pt_hi = h;
-                pt_lo = __double2float_ru(pmin - (double)h);
-              } else {
-                pt_hi = pmin > 0.0 ? __int_as_float(0x7f800000) : -FLT_MAX;
-                pt_lo = 0.f;
-              }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-              const float oh = __shfl_xor_sync(0xffffffffu, pt_hi, o), ol = __shfl_xor_sync(0xffffffffu, pt_lo, o);
-              if (__fadd_rn(__fsub_rn(oh, pt_hi), __fsub_rn(ol, pt_lo)) < 0.f) {
-                pt_hi = oh;
-                pt_lo = ol;
-              }
-            }
-          }
-        }
-      }
-      if (it % kWin == kWin - 1) {
-#pragma unroll
-        for (int q = 0; q < 8; q++) fwin_flush(win[q], acc[q]);
-      }
-    }
-    j += dj;
-    k += dk;
-    if (j >= ny) {
-      j -= ny;
-      k++;
+    for (int o = 16; o > 0; o >>= 1) fwin_merge(win[q], shfl_down2(win[q].h, o), shfl_down2(win[q].l, o), shfl_down2(win[q].t, o));
+    if (lane == 0) {
+      sw[wid][q][0] = win[q].h;
+      sw[wid][q][1] = win[q].l;
+      sw[wid][q][2] = win[q].t;
     }
   }
-#pragma unroll
-  for (int q = 0; q < 8; q++) fwin_flush(win[q], acc[q]);
-  // fixed-order tree: warp shuffles (plain FP64: 5 roundings), then the
-  // warps in order and the blocks in order with compensation
-  __shared__ double sm[kDiagThreads / 32][kDiagSlots];
-  const int wid = threadIdx.x >> 5;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-    for (int q = 0; q < 8; q++) acc[q] += __shfl_down_sync(0xffffffffu, acc[q], o);
     divmax = fmax(divmax, __shfl_down_sync(0xffffffffu, divmax, o));
     pmin = fmin(pmin, __shfl_down_sync(0xffffffffu, pmin, o));
   }
   if (lane == 0) {
-#pragma unroll
-    for (int q = 0; q < 8; q++) {
-      sm[wid][2 * q] = acc[q];
-      sm[wid][2 * q + 1] = 0.0;
-    }
-    sm[wid][16] = divmax;
-    sm[wid][17] = pmin;
+    sx[wid][0] = divmax;
+    sx[wid][1] = pmin;
   }
   __syncthreads();
+  double* out = partial + (long long)blockIdx.x * kDiagSlots;
   if (threadIdx.x < 8) {
     const int q = threadIdx.x;
-    KB t{sm[0][2 * q], sm[0][2 * q + 1]};
-    for (int w = 1; w < kDiagThreads / 32; w++) t = kb_merge(t, KB{sm[w][2 * q], sm[w][2 * q + 1]});
-    partial[(long long)blockIdx.x * kDiagSlots + 2 * q] = t.s;
-    partial[(long long)blockIdx.x * kDiagSlots + 2 * q + 1] = t.c;
-  } else if (threadIdx.x == 8) {
-    double m = sm[0][16];
-    for (int w = 1; w < kDiagThreads / 32; w++) m = fmax(m, sm[w][16]);
-    partial[(long long)blockIdx.x * kDiagSlots + 16] = m;
-  } else if (threadIdx.x == 9) {
-    double m = sm[0][17];
-    for (int w = 1; w < kDiagThreads / 32; w++) m = fmin(m, sm[w][17]);
-    partial[(long long)blockIdx.x * kDiagSlots + 17] = m;
+    FWin2 t{sw[0][q][0], sw[0][q][1], sw[0][q][2]};
+    for (int w = 1; w < kDiagThreads / 32; w++) fwin_merge(t, sw[w][q][0], sw[w][q][1], sw[w][q][2]);
+    double a0 = 0.0, a1 = 0.0;
+    fwin_flush(t, a0, a1);
+    KB s{a0 + a1, 0.0};
+    for (int w = 0; w < kDiagThreads / 32; w++) s = kb_merge(s, KB{sacc[w][q], 0.0});
+    out[2 * q] = s.s;
+    out[2 * q + 1] = s.c;
+  } else if (threadIdx.x == 32) {
+    double m = sx[0][0];
+    for (int w = 1; w < kDiagThreads / 32; w++) m = fmax(m, sx[w][0]);
+    out[16] = m;
+  } else if (threadIdx.x == 64) {
+    double m = sx[0][1];
+    for (int w = 1; w < kDiagThreads / 32; w++) m = fmin(m, sx[w][1]);
+    out[17] = m;
   }
 }
 
-__global__ void diag_final_kernel(const double* __restrict__ partial, int nblk, double hmin,
-                                  double* __restrict__ out) {
-  const int q = threadIdx.x;
-  if (q < 8) {
-    KB t{0.0, 0.0};
-    for (int b = 0; b < nblk; b++)
-      t = kb_merge(t, KB{partial[(long long)b * kDiagSlots + 2 * q], partial[(long long)b * kDiagSlots + 2 * q + 1]});
-    out[q] = t.s + t.c;
-  } else if (q == 8) {
-    double m = 0.0;
-    for (int b = 0; b < nblk; b++) m = fmax(m, partial[(long long)b * kDiagSlots + 16]);
-    out[8] = m * hmin;
-  } else if (q == 9) {
-    double m = DBL_MAX;
-    for (int b = 0; b < nblk; b++) m = fmin(m, partial[(long long)b * kDiagSlots + 17]);
-    out[9] = m;
+// The blocks' partials in a fixed order: a block per quantity, each lane
+// merging every 96th partial (with compensation for the sums), then the lanes
+// by a shuffle tree and the 3 warps in order.  (One lane per quantity over 1216
+// partials took 537 us, a chain of dependent FP64 operations; all quantities
+// on one SM are bound by its FP64 pipe, 23 us.)
+constexpr int kFinalWarps = 3;
+__global__ void __launch_bounds__(32 * kFinalWarps)
+diag_final_kernel(const double* __restrict__ partial, int nblk, double hmin, double* __restrict__ out) {
+  __shared__ double sm[kFinalWarps][2];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, q = blockIdx.x;
+  KB t{0.0, 0.0};
+  double m = q == 9 ? DBL_MAX : 0.0;
+  for (int b = threadIdx.x; b < nblk; b += 32 * kFinalWarps) {
+    const double* p = partial + (long long)b * kDiagSlots;
+    if (q < 8) t = kb_merge(t, KB{p[2 * q], p[2 * q + 1]});
+    else m = q == 8 ? fmax(m, p[16]) : fmin(m, p[17]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    if (q < 8) {
+      t = kb_merge(t, KB{__shfl_down_sync(0xffffffffu, t.s, o), __shfl_down_sync(0xffffffffu, t.c, o)});
+    } else {
+      const double x = __shfl_down_sync(0xffffffffu, m, o);
+      m = q == 8 ? fmax(m, x) : fmin(m, x);
+    }
+  }
+  if (lane == 0) {
+    sm[w][0] = q < 8 ? t.s : m;
+    sm[w][1] = t.c;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    KB s{sm[0][0], sm[0][1]};
+    for (int i = 1; i < kFinalWarps; i++) {
+      if (q < 8) s = kb_merge(s, KB{sm[i][0], sm[i][1]});
+      else s.s = q == 8 ? fmax(s.s, sm[i][0]) : fmin(s.s, sm[i][0]);
+    }
+    out[q] = q < 8 ? s.s + s.c : (q == 8 ? s.s * hmin : s.s);
   }
 }
 
 int diag_blocks(const Box& box) {
   const long long N = (long long)box.n[0] * box.n[1] * box.n[2];
   long long b = (N + 4LL * kDiagThreads - 1) / (4LL * kDiagThreads);
-  if (b > kDiagMaxBlocks) b = kDiagMaxBlocks;
+  if (b > kDiagGrid) b = kDiagGrid;
   if (b < 1) b = 1;
   return (int)b;
 }
@@ -472,11 +567,16 @@ cudaError_t launch_diagnostics(const float* const f[8], const Box& box, double g
                                double* out, cudaStream_t s) {
   if (box.stride[0] != 1) return cudaErrorInvalidValue;
   const int nblk = diag_blocks(box);
-  diag_partial_kernel<<<nblk, kDiagThreads, 0, s>>>(f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7],
-                                                    box, gamma, partial);
+  bool vec = box.n[0] % 2 == 0;
+  for (int q = 0; q < 8; q++) vec = vec && reinterpret_cast<uintptr_t>(f[q]) % 8 == 0;
+  const int W = vec ? 2 : 1;
+  const FastDiv row_div = fast_div(box.n[0] / W), ny_div = fast_div(box.n[1]);
+  auto* kernel = vec ? diag_partial_kernel<2> : diag_partial_kernel<1>;
+  kernel<<<nblk, kDiagThreads, 0, s>>>(f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7], box.n[0], box.n[1], box.n[2],
+                                       row_div, ny_div, gamma, partial);
   int nmax = box.n[0] > box.n[1] ? box.n[0] : box.n[1];
   nmax = nmax > box.n[2] ? nmax : box.n[2];
-  diag_final_kernel<<<1, 32, 0, s>>>(partial, nblk, 1.0 / nmax, out);
+  diag_final_kernel<<<10, 32 * kFinalWarps, 0, s>>>(partial, nblk, 1.0 / nmax, out);
   return cudaGetLastError();
 }
 
