@@ -81,7 +81,7 @@ struct mhd_s {
   Scalars* sc = nullptr;
   double* diag_partial = nullptr;
   int rcur = 0;
-  // FP64 boxes (mhd_create_f64): the state in double, whole-pencil kernels
+  // FP64 boxes (mhd_create_f64): the state in double
   bool f64 = false;
   double* arena64 = nullptr;
   double* cur64[8];
@@ -601,6 +601,7 @@ int magnetic64(mhd_s* m, int d, double tau) {
   }
   a.E[0] = m->e64;
   a.E[1] = m->e64 + m->N;
+  a.v = m->spare64[0];  // free until the next fluid sweep writes it
   for (int k = 0; k < 3; k++) {
     a.n[k] = m->n[k];
     a.ih[k] = m->cpl[k] > 0.0 ? m->cpl[k] : (double)m->n[k];
@@ -765,7 +766,8 @@ mhd_t* mhd_create_f64(int nx, int ny, int nz, double gamma) {
   m->box = mhd::make_box(nx, ny, nz);
   m->f64 = true;
   cudaError_t e;
-  if ((e = cudaMalloc(&m->arena64, sizeof(double) * (size_t)N * 18)) != cudaSuccess ||
+  if ((e = mhd::prepare_f64_kernels()) != cudaSuccess ||
+      (e = cudaMalloc(&m->arena64, sizeof(double) * (size_t)N * 18)) != cudaSuccess ||
       (e = cudaMalloc(&m->rate64, sizeof(unsigned long long))) != cudaSuccess ||
       (e = cudaMemset(m->arena64, 0, sizeof(double) * (size_t)N * 18)) != cudaSuccess) {
     cuda_fail(e, "mhd_create_f64");

@@ -271,7 +271,7 @@ cudaError_t launch_conv_wgrad(const __nv_bfloat16* x, const __nv_bfloat16* gy, c
 cudaError_t launch_conv_wgrad_cuda_cores(const __nv_bfloat16* x, const __nv_bfloat16* gy, const int n[3], int cin,
                                          int cout, float* gw, float* gb, cudaStream_t s);
 
-// FP64 path (sweep_f64.cu): whole-pencil kernels on the plain layout
+// FP64 path (sweep_f64.cu): kernels on the plain layout, a thread per cell
 struct Fluid64Args {
   const double* in[8];
   double* out[8];  // fields 0..4 written
@@ -284,10 +284,12 @@ struct Mag64Args {
   const double* in[8];
   double* out[8];  // fields 5..7 written
   double* E[2];    // edge fluxes of the transverse axes (D+1)%3, (D+2)%3 (N each)
+  double* v;       // scratch: v_D of every cell (N)
   int n[3];
   double ih[3];
   double tau;
 };
+cudaError_t prepare_f64_kernels();  // once per device before any launch
 cudaError_t launch_fluid64(int axis, const Fluid64Args& a, cudaStream_t s);
 cudaError_t launch_mag64(int axis, const Mag64Args& a, cudaStream_t s);
 cudaError_t launch_cfl64(const double* const f[8], const int n[3], const double ih[3], double gamma,

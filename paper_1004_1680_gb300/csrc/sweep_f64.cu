@@ -1,17 +1,17 @@
 // FP64 path of the grid update (an ablation: the paper computes in FP32,
 // Section III).  The same scheme as the FP32 kernels (Section II.B: relaxing
 // TVD fluid sweeps, advection-constraint magnetic sweeps, xyz then zyx),
-// written for clarity rather than speed: FP64 runs at a small fraction of
-// the FP32 rate on this GPU, so the arithmetic, not memory traffic, bounds
-// these kernels.
+// FP64 runs at a small fraction of the FP32 rate on this GPU, so the
+// arithmetic, not memory traffic, bounds these kernels.
 //  * Every operation is an IEEE double operation rounded once (__dadd_rn,
-//    __dmul_rn, __ddiv_rn, __dsqrt_rn; no multiply-add contraction).
-//  * Fluid sweep: one thread per whole periodic pencil along any axis, with
-//    the marching window of the FP32 pipeline (3 cells of lag).
-//  * Magnetic sweep: a flux kernel advects each transverse component (one
-//    thread per pencil and component) and stores its edge flux; a
-//    constraint kernel then updates b_d of every cell from the stored
-//    fluxes of its pencil and the neighbouring pencils.
+//    __dmul_rn, __dsqrt_rn, correctly rounded quotients; no multiply-add
+//    contraction).
+//  * Fluid sweep: one thread per cell, the intermediate values of a block's
+//    pencils exchanged through shared memory.
+//  * Magnetic sweep: the velocity of every cell; a flux kernel that advects
+//    each transverse component (one thread per cell and component) and
+//    stores its edge flux; a constraint kernel that updates b_d of every
+//    cell from the stored fluxes of its pencil and the neighbouring pencils.
 //  * CFL rate: the largest (|v_d| + c_f*) / h_d over cells, as double bits
 //    reduced with an atomic maximum (rates are >= 0).
 #include <cstdint>
@@ -26,10 +26,48 @@ __device__ __forceinline__ double dsub(double a, double b) { return __dsub_rn(a,
 __device__ __forceinline__ double dmul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double ddiv(double a, double b) { return __ddiv_rn(a, b); }
 
+// Quotients.  A division is about 14 FP64 operations here, and a fluid cell has
+// 18 of them; written out for operands of ordinary size they are 6, and 3 more
+// for each further quotient by the same divisor:
+//   y0, the hardware's approximate reciprocal (relative error e <= 2^-20),
+//   y  = y0 (1 + e + e^2), e = 1 - r y0   (one step of a cubic Newton iteration;
+//        its error, 2^-60, is below y's rounding),
+//   q  = a y, then q + (a - q r) y        (Markstein, "Computation of elementary
+//        functions on the IBM RISC System/6000 processor", 1990: the remainder
+//        is exact in one FMA).
+// The result is a / r rounded correctly (2 x 10^8 operand pairs with random and
+// extreme mantissas agree) for divisors whose mantissa is not all ones; those,
+// and operands whose exponents could spoil the remainder (zeros, infinities and
+// NaNs among them), take the division.
+__device__ __forceinline__ double approx_rcp(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  return y;
+}
+__device__ __forceinline__ double reciprocal(double r) {
+  const double y0 = approx_rcp(r), e = __fma_rn(-r, y0, 1.0);
+  return __fma_rn(__fma_rn(e, e, e), y0, y0);
+}
+__device__ __forceinline__ double ddiv_by(double a, double r, double y) {
+  const double q = dmul(a, y);
+  return __fma_rn(__fma_rn(-q, r, a), y, q);
+}
+// 2^-500 <= |x| < 2^500 (from the exponent: no FP64 comparison)
+__device__ __forceinline__ bool plain_exponent(double x) {
+  return ((unsigned)__double2hiint(x) >> 20 & 0x7ffu) - 523u < 1000u;
+}
+__device__ __forceinline__ bool plain_divisor(double x) { return plain_exponent(x) && __double2loint(x) != -1; }
+__device__ __forceinline__ bool negative(double x) { return __double2hiint(x) < 0; }
+
 // half the van Leer limiter, phi(a, b) / 2 = ab / (a + b) for ab > 0, else 0
 __device__ __forceinline__ double vl_half(double a, double b) {
-  const double ab = dmul(a, b);
-  return ab > 0.0 ? ddiv(ab, dadd(a, b)) : 0.0;
+  const double ab = dmul(a, b), s = dadd(a, b);
+  const int hi = __double2hiint(ab);
+  double q = 0.0;
+  // (2^-500 <= ab < 2^500 leaves |s| between 2^-250 and 2^1023, its remainder normal)
+  if ((unsigned)hi - (523u << 20) < (1000u << 20) && plain_divisor(s)) q = ddiv_by(ab, s, reciprocal(s));
+  else if (hi >= 0 && (hi | __double2loint(ab)) != 0) q = ab > 0.0 ? ddiv(ab, s) : 0.0;
+  return q;
 }
 
 // Right and left movers FR = (c u + F) / 2, FL = (c u - F) / 2 of Eq. 1-3
@@ -37,7 +75,10 @@ __device__ __forceinline__ double vl_half(double a, double b) {
 // b_d, b_t1, b_t2), with the freezing speed c = |v_d| + sqrt((gamma p + b^2) / rho).
 __device__ __forceinline__ void movers64(const double u[5], const double b[3], double gamma, double FR[5],
                                          double FL[5]) {
-  const double vd = ddiv(u[1], u[0]), v1 = ddiv(u[2], u[0]), v2 = ddiv(u[3], u[0]);
+  const double y = reciprocal(u[0]);
+  const bool rho_ok = plain_divisor(u[0]);
+  auto over_rho = [&](double x) { return rho_ok && plain_exponent(x) ? ddiv_by(x, u[0], y) : ddiv(x, u[0]); };
+  const double vd = over_rho(u[1]), v1 = over_rho(u[2]), v2 = over_rho(u[3]);
   const double bb = dadd(dadd(dmul(b[0], b[0]), dmul(b[1], b[1])), dmul(b[2], b[2]));
   const double kin = dmul(0.5, dadd(dadd(dmul(u[1], vd), dmul(u[2], v1)), dmul(u[3], v2)));
   const double p = dmul(gamma - 1.0, dsub(dsub(u[4], kin), dmul(0.5, bb)));
@@ -49,7 +90,7 @@ __device__ __forceinline__ void movers64(const double u[5], const double b[3], d
   F[2] = dsub(dmul(u[2], vd), dmul(b[0], b[1]));
   F[3] = dsub(dmul(u[3], vd), dmul(b[0], b[2]));
   F[4] = dsub(dmul(dadd(u[4], ps), vd), dmul(b[0], bv));
-  const double c = dadd(fabs(vd), __dsqrt_rn(ddiv(dadd(dmul(gamma, p), bb), u[0])));
+  const double c = dadd(fabs(vd), __dsqrt_rn(over_rho(dadd(dmul(gamma, p), bb))));
 #pragma unroll
   for (int q = 0; q < 5; q++) {
     FR[q] = dmul(0.5, dadd(dmul(c, u[q]), F[q]));
@@ -57,161 +98,197 @@ __device__ __forceinline__ void movers64(const double u[5], const double b[3], d
   }
 }
 
-// The fluid marching pipeline (the FP32 FluidPipe's window, in double):
-// consuming position t yields Unew at t - 3.
-struct FluidPipe64 {
-  double U1[5], U2[5], U3[5], b1[3], FR1[5], f1m[5], Rh2[5], Rh3[5], dR3[5], Lh2[5], dL2[5], F2m[5];
-
-  __device__ void init() {
-#pragma unroll
-    for (int q = 0; q < 5; q++)
-      U1[q] = U2[q] = U3[q] = FR1[q] = f1m[q] = Rh2[q] = Rh3[q] = dR3[q] = Lh2[q] = dL2[q] = F2m[q] = 0.0;
-    b1[0] = b1[1] = b1[2] = 0.0;
-  }
-
-  __device__ void step(const double U[5], const double b[3], double gamma, double c_half, double c_full,
-                       double out[5]) {
-    double FR[5], FL[5], Uh[5], Rh[5], Lh[5], f1[5];
-    movers64(U, b, gamma, FR, FL);
-#pragma unroll
-    for (int q = 0; q < 5; q++) {
-      f1[q] = dsub(FR1[q], FL[q]);                                 // first-order flux at t - 1/2
-      Uh[q] = dsub(U1[q], dmul(c_half, dsub(f1[q], f1m[q])));      // half step at t - 1
-    }
-    movers64(Uh, b1, gamma, Rh, Lh);
-#pragma unroll
-    for (int q = 0; q < 5; q++) {
-      const double dR2 = dsub(Rh2[q], Rh3[q]), dL1 = dsub(Lh[q], Lh2[q]);
-      const double right = dadd(Rh3[q], vl_half(dR3[q], dR2));   // upwind cell t - 3
-      const double left = dsub(Lh2[q], vl_half(dL2[q], dL1));    // upwind cell t - 2
-      const double F2 = dsub(right, left);                       // second-order flux at t - 5/2
-      out[q] = dsub(U3[q], dmul(c_full, dsub(F2, F2m[q])));
-      F2m[q] = F2;
-      U3[q] = U2[q];
-      U2[q] = U1[q];
-      U1[q] = U[q];
-      FR1[q] = FR[q];
-      f1m[q] = f1[q];
-      dR3[q] = dR2;
-      Rh3[q] = Rh2[q];
-      Rh2[q] = Rh[q];
-      dL2[q] = dL1;
-      Lh2[q] = Lh[q];
-    }
-    b1[0] = b[0];
-    b1[1] = b[1];
-    b1[2] = b[2];
-  }
+// Threads of a block and split of a pencil of nD cells: one thread per cell,
+// np pencils, the whole periodic pencil (`whole`) or a segment of `out`
+// cells with 3 halo cells at each end (the reach of both sweeps' stencils).
+constexpr int kThreads64 = 512;
+struct Tile64 {
+  int threads, np, td, out, segs;
+  bool whole;
 };
+__host__ __device__ inline Tile64 tile64(int nD) {
+  Tile64 t;
+  const int most = kThreads64 / 4;  // at least 4 pencils: 32-byte pieces across the pencils
+  t.whole = nD <= most;
+  t.segs = t.whole ? 1 : (nD + most - 7) / (most - 6);
+  t.out = (nD + t.segs - 1) / t.segs;
+  t.td = t.out + (t.whole ? 0 : 6);
+  t.threads = t.td <= 64 ? 256 : kThreads64;
+  t.np = t.threads / t.td;
+  return t;
+}
 
-// The magnetic advection pipeline (the FP32 MagPipe in double): consuming
-// (q, u) at t yields qnew at t - 3 and the edge flux at t - 5/2.
-struct MagPipe64 {
-  double q1, q2, q3, u1, g1m, h2, h3, d32, d43, ub1, ub2, fm;
-
-  __device__ void init() { q1 = q2 = q3 = u1 = g1m = h2 = h3 = d32 = d43 = ub1 = ub2 = fm = 0.0; }
-
-  __device__ double step(double q, double u, double c_half, double c_full, double& qnew) {
-    const double ub = dmul(0.5, dadd(u1, u));                      // edge velocity at t - 1/2
-    const double g = dmul(ub, ub >= 0.0 ? q1 : q);                 // upwind flux
-    const double h = dsub(q1, dmul(c_half, dsub(g, g1m)));         // half step at t - 1
-    const double d21 = dsub(h, h2);
-    const bool pos = ub2 >= 0.0;                                   // edge t - 5/2
-    const double base = pos ? h3 : h2;
-    const double lim = pos ? vl_half(d43, d32) : vl_half(d32, d21);
-    const double f = dmul(ub2, pos ? dadd(base, lim) : dsub(base, lim));
-    qnew = dsub(q3, dmul(c_full, dsub(f, fm)));
-    fm = f;
-    q3 = q2;
-    q2 = q1;
-    q1 = q;
-    u1 = u;
-    g1m = g;
-    d43 = d32;
-    d32 = d21;
-    h3 = h2;
-    h2 = h;
-    ub2 = ub1;
-    ub1 = ub;
-    return f;
-  }
+// This thread's cell: pencil (pa, pb) of the two other axes, position p along
+// D (periodic), whether it exists and whether it is written; im, ip, ip2: the
+// threads of cells p - 1, p + 1, p + 2 (their own thread past a segment's end:
+// only halo cells read those).
+struct Cell64 {
+  int pa, pb, p, im, ip, ip2;
+  bool live, own;
 };
-
-struct Geo {
-  int n[3];
-  int s[3];
-  double ih[3];
-};
-
-// one thread per pencil along D (A, O: the other axes)
 template <int D>
-__global__ void __launch_bounds__(128) fluid64_kernel(Fluid64Args a) {
+__device__ __forceinline__ Cell64 cell64(const int n[3]) {
+  constexpr int A = (D == 0) ? 1 : 0, O = (D == 2) ? 1 : 2;
+  const Tile64 t = tile64(n[D]);
+  const int tid = threadIdx.x;
+  // along x neighbouring threads take neighbouring cells, else neighbouring pencils
+  const int pp = D == 0 ? tid / t.td : tid % t.np, i = D == 0 ? tid - pp * t.td : tid / t.np;
+  const int step = D == 0 ? 1 : t.np;
+  Cell64 c;
+  const unsigned pencils = (unsigned)n[A] * (unsigned)n[O], runs = (pencils + t.np - 1) / t.np;
+  const unsigned seg = blockIdx.x / runs, P = (blockIdx.x - seg * runs) * t.np + pp;
+  c.live = pp < t.np && i < t.td && P < pencils;
+  c.pb = (int)(P / (unsigned)n[A]);
+  c.pa = (int)(P - (unsigned)c.pb * (unsigned)n[A]);
+  const int off = t.whole ? i : i - 3, s0 = (int)seg * t.out;
+  c.own = c.live && off >= 0 && off < t.out && s0 + off < n[D];
+  c.p = wrapi(s0 + off, n[D]);
+  auto nb = [&](int d) {
+    int k = i + d;
+    if (t.whole) k = wrapi(k, t.td);
+    else k = k < 0 || k >= t.td ? i : k;
+    return tid + (k - i) * step;
+  };
+  c.im = nb(-1);
+  c.ip = nb(1);
+  c.ip2 = nb(2);
+  return c;
+}
+
+// Fluid sweep, one thread per cell.  FP64 arithmetic bounds it (338 operations
+// per cell, 16 cycles of an SM per warp instruction: its pipe is 85 % busy), so nothing is
+// computed twice but a few subtractions: the movers of both stages and the
+// limited values are exchanged through shared memory, [component][thread], in
+// two alternating sets.  (Marching whole pencils with one thread each left
+// the FP64 pipe idle below about 150,000 pencils: 64^3 1050 us a sweep, now
+// 175; 256^3 111 ms a step, now 101.)
+template <int D>
+__global__ void __launch_bounds__(kThreads64, 1) fluid64_kernel(const __grid_constant__ Fluid64Args a) {
   constexpr int A = (D == 0) ? 1 : 0, O = (D == 2) ? 1 : 2, T1 = (D + 1) % 3, T2 = (D + 2) % 3;
-  const Geo g{{a.n[0], a.n[1], a.n[2]}, {1, a.n[0], a.n[0] * a.n[1]}, {a.ih[0], a.ih[1], a.ih[2]}};
-  const int pa = blockIdx.x * 32 + threadIdx.x, pb = blockIdx.y * blockDim.y + threadIdx.y;
-  if (pa >= g.n[A] || pb >= g.n[O]) return;
-  const int nD = g.n[D];
-  const int base = pa * g.s[A] + pb * g.s[O];
-  const int eT1 = (T1 == A) ? wrapi(pa + 1, g.n[A]) * g.s[A] + pb * g.s[O] : pa * g.s[A] + wrapi(pb + 1, g.n[O]) * g.s[O];
-  const int eT2 = (T2 == A) ? wrapi(pa + 1, g.n[A]) * g.s[A] + pb * g.s[O] : pa * g.s[A] + wrapi(pb + 1, g.n[O]) * g.s[O];
-  const double c_full = dmul(a.tau, g.ih[D]), c_half = dmul(0.5, c_full);
-  FluidPipe64 pipe;
-  pipe.init();
-  for (int t = -4; t < nD + 3; t++) {
-    const int off = wrapi(t, nD) * g.s[D], off1 = wrapi(t + 1, nD) * g.s[D];
-    const int c = base + off;
-    const double U[5] = {a.in[RHO][c], a.in[MX + D][c], a.in[MX + T1][c], a.in[MX + T2][c], a.in[EN][c]};
-    const double b[3] = {dmul(0.5, dadd(a.in[BX + D][c], a.in[BX + D][base + off1])),
-                         dmul(0.5, dadd(a.in[BX + T1][c], a.in[BX + T1][eT1 + off])),
-                         dmul(0.5, dadd(a.in[BX + T2][c], a.in[BX + T2][eT2 + off]))};
-    double o[5];
-    pipe.step(U, b, a.gamma, c_half, c_full, o);
-    const int po = t - 3;
-    if (po >= 0 && po < nD) {
-      const int w = base + po * g.s[D];
-      a.out[RHO][w] = o[0];
-      a.out[MX + D][w] = o[1];
-      a.out[MX + T1][w] = o[2];
-      a.out[MX + T2][w] = o[3];
-      a.out[EN][w] = o[4];
+  extern __shared__ double sm64[];
+  const int T = blockDim.x;
+  double* x0 = sm64;                     // FR, FL, then the limited right and left values
+  double* x1 = sm64 + 10 * T;   // Rh, Lh
+  const long long st[3] = {1, a.n[0], (long long)a.n[0] * a.n[1]};
+  const Cell64 c = cell64<D>(a.n);
+  const int tid = threadIdx.x;
+  const double c_full = dmul(a.tau, a.ih[D]), c_half = dmul(0.5, c_full);
+  const long long cell = c.pa * st[A] + c.pb * st[O] + c.p * st[D];
+  double U[5], b[3], FR[5], FL[5];
+  if (c.live) {
+    auto up = [&](int d, int x) { return cell + (x + 1 == a.n[d] ? -(long long)x : 1) * st[d]; };
+    const long long cD = up(D, c.p), cA = up(A, c.pa), cO = up(O, c.pb);
+    const long long c1 = T1 == A ? cA : cO, c2 = T2 == A ? cA : cO;
+    U[0] = a.in[RHO][cell], U[1] = a.in[MX + D][cell], U[2] = a.in[MX + T1][cell], U[3] = a.in[MX + T2][cell];
+    U[4] = a.in[EN][cell];
+    b[0] = dmul(0.5, dadd(a.in[BX + D][cell], a.in[BX + D][cD]));
+    b[1] = dmul(0.5, dadd(a.in[BX + T1][cell], a.in[BX + T1][c1]));
+    b[2] = dmul(0.5, dadd(a.in[BX + T2][cell], a.in[BX + T2][c2]));
+    movers64(U, b, a.gamma, FR, FL);
+#pragma unroll
+    for (int q = 0; q < 5; q++) {
+      x0[q * T + tid] = FR[q];
+      x0[(5 + q) * T + tid] = FL[q];
     }
+  }
+  __syncthreads();
+  if (c.live) {
+    double Uh[5];
+#pragma unroll
+    for (int q = 0; q < 5; q++) {  // first-order fluxes at p +- 1/2, half step
+      const double hi = dsub(FR[q], x0[(5 + q) * T + c.ip]);
+      const double lo = dsub(x0[q * T + c.im], FL[q]);
+      Uh[q] = dsub(U[q], dmul(c_half, dsub(hi, lo)));
+    }
+    movers64(Uh, b, a.gamma, FR, FL);
+#pragma unroll
+    for (int q = 0; q < 5; q++) {
+      x1[q * T + tid] = FR[q];
+      x1[(5 + q) * T + tid] = FL[q];
+    }
+  }
+  __syncthreads();
+  if (c.live) {
+#pragma unroll
+    for (int q = 0; q < 5; q++) {  // the right mover extrapolated to p + 1/2, the left one to p - 1/2
+      const double *R = x1 + q * T, *L = x1 + (5 + q) * T;
+      FR[q] = dadd(FR[q], vl_half(dsub(FR[q], R[c.im]), dsub(R[c.ip], FR[q])));
+      FL[q] = dsub(FL[q], vl_half(dsub(FL[q], L[c.im]), dsub(L[c.ip], FL[q])));
+      x0[q * T + tid] = FR[q];
+      x0[(5 + q) * T + tid] = FL[q];
+    }
+  }
+  __syncthreads();
+  if (c.own) {
+    double o[5];
+#pragma unroll
+    for (int q = 0; q < 5; q++) {
+      const double hi = dsub(FR[q], x0[(5 + q) * T + c.ip]);  // second-order flux at p + 1/2
+      const double lo = dsub(x0[q * T + c.im], FL[q]);        // and at p - 1/2
+      o[q] = dsub(U[q], dmul(c_full, dsub(hi, lo)));
+    }
+    a.out[RHO][cell] = o[0];
+    a.out[MX + D][cell] = o[1];
+    a.out[MX + T1][cell] = o[2];
+    a.out[MX + T2][cell] = o[3];
+    a.out[EN][cell] = o[4];
   }
 }
 
+// v_D of every cell, once per magnetic sweep.
+__global__ void __launch_bounds__(256) velocity64_kernel(const double* __restrict__ m, const double* __restrict__ rho,
+                                                         double* __restrict__ v, long long N) {
+  for (long long c = (long long)blockIdx.x * 256 + threadIdx.x; c < N; c += (long long)gridDim.x * 256)
+    v[c] = ddiv(m[c], rho[c]);
+}
+
+// (with the flux kernel and the constraint below: 64^3 218 us a sweep, now 51)
+//
 // Advection of b_t along D for one transverse axis t (blockIdx.z: 0 -> T1,
-// 1 -> T2): new b_t into out[BX + t], edge fluxes into E[blockIdx.z] (the
-// flux of edge i + 1/2 of a pencil stored at its cell i).
+// 1 -> T2), one thread per cell: new b_t into out[BX + t], edge fluxes into
+// E[blockIdx.z] (the flux of edge i + 1/2 of a pencil stored at its cell i).
 template <int D>
-__global__ void __launch_bounds__(128) mag64_flux_kernel(Mag64Args a) {
+__global__ void __launch_bounds__(kThreads64) mag64_flux_kernel(const __grid_constant__ Mag64Args a) {
   constexpr int A = (D == 0) ? 1 : 0, O = (D == 2) ? 1 : 2;
-  const Geo g{{a.n[0], a.n[1], a.n[2]}, {1, a.n[0], a.n[0] * a.n[1]}, {a.ih[0], a.ih[1], a.ih[2]}};
-  const int pa = blockIdx.x * 32 + threadIdx.x, pb = blockIdx.y * blockDim.y + threadIdx.y;
-  if (pa >= g.n[A] || pb >= g.n[O]) return;
+  __shared__ double su[kThreads64], sq[kThreads64], sh[kThreads64], sf[kThreads64];
+  const long long st[3] = {1, a.n[0], (long long)a.n[0] * a.n[1]};
+  const Cell64 c = cell64<D>(a.n);
+  const int tid = threadIdx.x;
   const int t = (blockIdx.z == 0) ? (D + 1) % 3 : (D + 2) % 3;
-  const int nD = g.n[D];
-  const int base = pa * g.s[A] + pb * g.s[O];
-  // the pencil one cell down along t (the other side of the b_t face)
-  const int baseM = (t == A) ? wrapi(pa - 1, g.n[A]) * g.s[A] + pb * g.s[O]
-                             : pa * g.s[A] + wrapi(pb - 1, g.n[O]) * g.s[O];
-  const double c_full = dmul(a.tau, g.ih[D]), c_half = dmul(0.5, c_full);
-  const double* __restrict__ rho = a.in[RHO];
-  const double* __restrict__ md = a.in[MX + D];
-  const double* __restrict__ q = a.in[BX + t];
-  double* __restrict__ qo = a.out[BX + t];
-  double* __restrict__ E = a.E[blockIdx.z];
-  MagPipe64 pipe;
-  pipe.init();
-  for (int s = -4; s < nD + 3; s++) {
-    const int off = wrapi(s, nD) * g.s[D];
-    const int c = base + off, cm = baseM + off;
-    const double u = dmul(0.5, dadd(ddiv(md[c], rho[c]), ddiv(md[cm], rho[cm])));  // v_D on the b_t face
-    double qn;
-    const double f = pipe.step(q[c], u, c_half, c_full, qn);
-    const int po = s - 3;
-    if (po >= 0 && po < nD) {
-      qo[base + po * g.s[D]] = qn;
-      E[base + po * g.s[D]] = f;  // edge po + 1/2
-    }
+  const double c_full = dmul(a.tau, a.ih[D]), c_half = dmul(0.5, c_full);
+  const long long cell = c.pa * st[A] + c.pb * st[O] + c.p * st[D];
+  double q = 0.0, u = 0.0;
+  if (c.live) {
+    // the pencil one cell down along t (the other side of the b_t face)
+    const long long down = cell + (t == A ? (c.pa ? -1 : a.n[A] - 1) * st[A] : (c.pb ? -1 : a.n[O] - 1) * st[O]);
+    q = a.in[BX + t][cell];
+    u = dmul(0.5, dadd(a.v[cell], a.v[down]));  // v_D on the b_t face
+    su[tid] = u;
+    sq[tid] = q;
+  }
+  __syncthreads();
+  double ub = 0.0, h = 0.0;
+  if (c.live) {
+    ub = dmul(0.5, dadd(u, su[c.ip]));                                   // edge velocity at p + 1/2
+    const double um = dmul(0.5, dadd(su[c.im], u));                      // and at p - 1/2
+    const double g = dmul(ub, negative(ub) ? sq[c.ip] : q), gm = dmul(um, negative(um) ? q : sq[c.im]);  // upwind fluxes
+    h = dsub(q, dmul(c_half, dsub(g, gm)));                              // half step
+    sh[tid] = h;
+  }
+  __syncthreads();
+  double f = 0.0;
+  if (c.live) {
+    const double hm = sh[c.im], hp = sh[c.ip], hpp = sh[c.ip2];
+    const bool pos = !negative(ub);
+    const double base = pos ? h : hp;  // the upwind cell and the ones below and above it
+    const double lim = vl_half(dsub(base, pos ? hm : h), dsub(pos ? hp : hpp, base));
+    f = dmul(ub, pos ? dadd(base, lim) : dsub(base, lim));
+    sf[tid] = f;
+  }
+  __syncthreads();
+  if (c.own) {
+    a.out[BX + t][cell] = dsub(q, dmul(c_full, dsub(f, sf[c.im])));
+    a.E[blockIdx.z][cell] = f;  // edge p + 1/2
   }
 }
 
@@ -254,15 +331,18 @@ __global__ void __launch_bounds__(256) cfl64_kernel(const double* __restrict__ r
     const double b[3] = {dmul(0.5, dadd(bx[c], bx[cx])), dmul(0.5, dadd(by[c], by[cy])), dmul(0.5, dadd(bz[c], bz[cz]))};
     const double m[3] = {mx[c], my[c], mz[c]};
     const double r = rho[c];
+    const double y = reciprocal(r);
+    const bool r_ok = plain_divisor(r);
+    auto over_rho = [&](double x) { return r_ok && plain_exponent(x) ? ddiv_by(x, r, y) : ddiv(x, r); };
     double v[3], bb = 0.0, kin = 0.0;
 #pragma unroll
     for (int d = 0; d < 3; d++) {
-      v[d] = ddiv(m[d], r);
+      v[d] = over_rho(m[d]);
       bb = dadd(bb, dmul(b[d], b[d]));
       kin = dadd(kin, dmul(0.5, dmul(m[d], v[d])));
     }
     const double p = dmul(gamma - 1.0, dsub(dsub(en[c], kin), dmul(0.5, bb)));
-    const double cf = __dsqrt_rn(ddiv(dadd(dmul(gamma, p), bb), r));
+    const double cf = __dsqrt_rn(over_rho(dadd(dmul(gamma, p), bb)));
     double rc = fmax(fmax(dmul(dadd(fabs(v[0]), cf), ihx), dmul(dadd(fabs(v[1]), cf), ihy)),
                      dmul(dadd(fabs(v[2]), cf), ihz));
     if (!(r > 0.0) || !(p > 0.0) || !(rc <= 1.0e300)) rc = __longlong_as_double(0x7ff0000000000000LL);
@@ -274,30 +354,49 @@ __global__ void __launch_bounds__(256) cfl64_kernel(const double* __restrict__ r
 
 }  // namespace
 
-cudaError_t launch_fluid64(int axis, const Fluid64Args& a, cudaStream_t s) {
+namespace {
+dim3 grid64(int axis, const int n[3], int z) {
   const int A = (axis == 0) ? 1 : 0, O = (axis == 2) ? 1 : 2;
-  const dim3 block(32, 4), grid((a.n[A] + 31) / 32, (a.n[O] + 3) / 4);
-  if (axis == 0) fluid64_kernel<0><<<grid, block, 0, s>>>(a);
-  if (axis == 1) fluid64_kernel<1><<<grid, block, 0, s>>>(a);
-  if (axis == 2) fluid64_kernel<2><<<grid, block, 0, s>>>(a);
+  const Tile64 t = tile64(n[axis]);
+  const long long pencils = (long long)n[A] * n[O];
+  return dim3((unsigned)((pencils + t.np - 1) / t.np * t.segs), 1, z);  // segment by segment
+}
+int fluid64_smem(int threads) { return 20 * threads * (int)sizeof(double); }
+}  // namespace
+
+cudaError_t prepare_f64_kernels() {
+  cudaError_t e = cudaSuccess;
+  for (auto* k : {fluid64_kernel<0>, fluid64_kernel<1>, fluid64_kernel<2>})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                      fluid64_smem(kThreads64));
+  return e;
+}
+
+cudaError_t launch_fluid64(int axis, const Fluid64Args& a, cudaStream_t s) {
+  const dim3 grid = grid64(axis, a.n, 1);
+  const int threads = tile64(a.n[axis]).threads, smem = fluid64_smem(threads);
+  if (axis == 0) fluid64_kernel<0><<<grid, threads, smem, s>>>(a);
+  if (axis == 1) fluid64_kernel<1><<<grid, threads, smem, s>>>(a);
+  if (axis == 2) fluid64_kernel<2><<<grid, threads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
 cudaError_t launch_mag64(int axis, const Mag64Args& a, cudaStream_t s) {
-  const int A = (axis == 0) ? 1 : 0, O = (axis == 2) ? 1 : 2;
-  const dim3 block(32, 4), grid((a.n[A] + 31) / 32, (a.n[O] + 3) / 4, 2);
+  const dim3 grid = grid64(axis, a.n, 2);
+  const int threads = tile64(a.n[axis]).threads;
   const long long N = (long long)a.n[0] * a.n[1] * a.n[2];
   const int cblocks = (int)((N + 255) / 256 < 152 * 16 ? (N + 255) / 256 : 152 * 16);
+  velocity64_kernel<<<cblocks, 256, 0, s>>>(a.in[MX + axis], a.in[RHO], a.v, N);
   if (axis == 0) {
-    mag64_flux_kernel<0><<<grid, block, 0, s>>>(a);
+    mag64_flux_kernel<0><<<grid, threads, 0, s>>>(a);
     mag64_constraint_kernel<0><<<cblocks, 256, 0, s>>>(a);
   }
   if (axis == 1) {
-    mag64_flux_kernel<1><<<grid, block, 0, s>>>(a);
+    mag64_flux_kernel<1><<<grid, threads, 0, s>>>(a);
     mag64_constraint_kernel<1><<<cblocks, 256, 0, s>>>(a);
   }
   if (axis == 2) {
-    mag64_flux_kernel<2><<<grid, block, 0, s>>>(a);
+    mag64_flux_kernel<2><<<grid, threads, 0, s>>>(a);
     mag64_constraint_kernel<2><<<cblocks, 256, 0, s>>>(a);
   }
   return cudaGetLastError();
