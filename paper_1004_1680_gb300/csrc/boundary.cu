@@ -22,6 +22,7 @@ namespace mhd {
 // they fit, which avoids emulated 64-bit division per element).
 template <typename I>
 __global__ void __launch_bounds__(256) ghost_fill_kernel(GhostArgs a) {
+  wait_for_previous_in_place();
   const int k = a.axis;
   const I n1 = (I)a.n1;
   const I plane = (I)a.n1 * (I)a.n2;
@@ -84,10 +85,8 @@ cudaError_t launch_ghost_fill(float* const f[8], const Box& box, int axis, int m
   if (blocks > 65535LL * 16) blocks = 65535LL * 16;
   // 32-bit counters while the element count and the last id + stride fit
   if (total + blocks * 256 < (1LL << 32))
-    ghost_fill_kernel<unsigned><<<(unsigned)blocks, 256, 0, s>>>(a);
-  else
-    ghost_fill_kernel<unsigned long long><<<(unsigned)blocks, 256, 0, s>>>(a);
-  return cudaGetLastError();
+    return launch_after(true, ghost_fill_kernel<unsigned>, dim3((unsigned)blocks), dim3(256), 0, s, a);
+  return launch_after(true, ghost_fill_kernel<unsigned long long>, dim3((unsigned)blocks), dim3(256), 0, s, a);
 }
 
 }  // namespace mhd

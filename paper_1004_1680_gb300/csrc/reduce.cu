@@ -78,6 +78,7 @@ cudaError_t launch_cfl_rate(const float* const f[8], const Box& box, float gamma
 
 __global__ void step_control_kernel(const unsigned* rate_cur, unsigned* rate_next, float* tau,
                                     double* time, double cfl, double tau_host) {
+  wait_for_previous();
   double t;
   if (cfl > 0.0) {
     const float r = __uint_as_float(*rate_cur);
@@ -93,8 +94,7 @@ __global__ void step_control_kernel(const unsigned* rate_cur, unsigned* rate_nex
 
 cudaError_t launch_step_control(const unsigned* rate_cur, unsigned* rate_next, float* tau,
                                 double* time, double cfl, double tau_host, cudaStream_t s) {
-  step_control_kernel<<<1, 1, 0, s>>>(rate_cur, rate_next, tau, time, cfl, tau_host);
-  return cudaGetLastError();
+  return launch_after(true, step_control_kernel, dim3(1), dim3(1), 0, s, rate_cur, rate_next, tau, time, cfl, tau_host);
 }
 
 __global__ void ens_control_kernel(const unsigned* rate_cur, unsigned* rate_next, float* tau,

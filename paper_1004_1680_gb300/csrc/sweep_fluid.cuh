@@ -394,6 +394,7 @@ fluid_sweep_kernel(FluidArgs a) {
 template <int D, bool RATE, bool FLOOR, int LIM, int FRZ>
 __global__ void __launch_bounds__(32 * kFluidWarps, 4)
 fluid_sweep_tma_kernel(const __grid_constant__ FluidArgs a, const __grid_constant__ FluidMaps mp) {
+  wait_for_previous();
   fluid_sweep_body<D, RATE, false, FLOOR, LIM, FRZ, true>(a, &mp);
 }
 
@@ -434,12 +435,12 @@ cudaError_t launch_fluid_t(int axis, bool rate, const FluidArgs& a, cudaStream_t
       if (a.tma_used) *a.tma_used = 1;
 #define FLUID_TMA_CASE(DD, RR, FF) \
   if (axis == DD && rate == RR && floor == FF)                                                       \
-    fluid_sweep_tma_kernel<DD, RR, FF, LIM, FRZ><<<tiles, block, 0, s>>>(a, mp);
+    return launch_after(true, fluid_sweep_tma_kernel<DD, RR, FF, LIM, FRZ>, tiles, block, 0, s, a, mp);
       FLUID_TMA_CASE(1, false, false) FLUID_TMA_CASE(1, true, false) FLUID_TMA_CASE(2, false, false)
       FLUID_TMA_CASE(2, true, false) FLUID_TMA_CASE(1, false, true) FLUID_TMA_CASE(1, true, true)
       FLUID_TMA_CASE(2, false, true) FLUID_TMA_CASE(2, true, true)
 #undef FLUID_TMA_CASE
-      return cudaGetLastError();
+      return cudaErrorInvalidValue;
     }
   }
 #define FLUID_CASE(DD, RR)                                                                            \

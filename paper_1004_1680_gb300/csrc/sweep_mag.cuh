@@ -663,6 +663,7 @@ mag_sweep_tma_kernel(const __grid_constant__ MagArgs a, const __grid_constant__ 
   __shared__ MagShared<NP> sh;
   extern __shared__ float mag_dyn[];
   __shared__ alignas(8) unsigned long long tfull[2];
+  wait_for_previous();
   const BlockGeom G = block_geom(a.ens, a.box, a.seg, a.tau, nullptr);
   // the buffers start at the first 128-byte boundary (a tile copy lands on one)
   const float* tb = mag_dyn + ((128u - (smem_u32(mag_dyn) & 127u)) & 127u) / 4;
@@ -728,10 +729,10 @@ cudaError_t launch_mag_t(int axis, const MagArgs& a, cudaStream_t s) {
     MagMaps mp;
     if (a.tma && !a.ens.items && !small && axis != 0 && make_mag_maps(axis, a, &mp)) {
       if (a.tma_used) *a.tma_used = 1;
-      if (axis == 1) mag_sweep_tma_kernel<1, 1, LIM><<<grid, block, kMagTmaSmem, s>>>(a, mp);
-      else if (a.passes == 2) mag_sweep_tma_kernel<2, 2, LIM><<<grid, block, kMagTmaSmem, s>>>(a, mp);
-      else mag_sweep_tma_kernel<2, 1, LIM><<<grid, block, kMagTmaSmem, s>>>(a, mp);
-      return cudaGetLastError();
+      auto* kernel = axis == 1       ? mag_sweep_tma_kernel<1, 1, LIM>
+                     : a.passes == 2 ? mag_sweep_tma_kernel<2, 2, LIM>
+                                     : mag_sweep_tma_kernel<2, 1, LIM>;
+      return launch_after(true, kernel, grid, block, kMagTmaSmem, s, a, mp);
     }
   }
   if (axis == 1) {

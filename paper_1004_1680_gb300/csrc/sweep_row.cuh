@@ -149,6 +149,7 @@ __global__ void __launch_bounds__(kRowMaxThreads, 2) fluid_row_kernel(const __gr
   // on the missing warp's arrivals run out too, within the bound)
   __shared__ alignas(8) unsigned long long xbar[3];
   __shared__ int stop;
+  wait_for_previous();
   const int nx = a.box.n[0], ny = a.box.n[1], nz = a.box.n[2];
   const int T = nx / kRowCells, l = threadIdx.x;
   const int rows = ny * nz;
@@ -462,6 +463,7 @@ __global__ void __launch_bounds__(R == 4 ? 640 : 768, 1) mag_row_kernel(const __
   using M = MRow<R>;
   extern __shared__ __align__(128) float ms_dyn[];
   __shared__ alignas(8) unsigned long long mbarr[2];
+  wait_for_previous();
   const int nx = a.box.n[0], ny = a.box.n[1], nz = a.box.n[2];
   const int T = nx / kRowCells, l = threadIdx.x, g = threadIdx.y;
   const bool halo = g == R;
@@ -693,11 +695,11 @@ cudaError_t launch_fluid_rows(bool rate, const FluidArgs& a, cudaStream_t s) {
   if (rate == RR && floor == FF) {                                                    \
     e = row_grid(fluid_row_kernel<RR, FF, LIM, FRZ>, threads, smem, rows, &grid);     \
     if (e != cudaSuccess) return e;                                                   \
-    fluid_row_kernel<RR, FF, LIM, FRZ><<<grid, threads, smem, s>>>(a);                \
+    return launch_after(true, fluid_row_kernel<RR, FF, LIM, FRZ>, dim3(grid), dim3(threads), smem, s, a); \
   }
     FLUID_ROW_CASE(false, false) FLUID_ROW_CASE(true, false) FLUID_ROW_CASE(false, true) FLUID_ROW_CASE(true, true)
 #undef FLUID_ROW_CASE
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
   }
 }
 
@@ -751,8 +753,7 @@ cudaError_t launch_mag_rows_r(const MagArgs& a, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   const int tiles = ny / R;
   const int L = mag_row_segment(tiles, nz, sms > 0 ? sms : 1);
-  mag_row_kernel<LIM, R><<<tiles * (nz / L), dim3(nx / kRowCells, R + 1), smem, s>>>(a, L);
-  return cudaGetLastError();
+  return launch_after(true, mag_row_kernel<LIM, R>, dim3(tiles * (nz / L)), dim3(nx / kRowCells, R + 1), smem, s, a, L);
 }
 
 template <int LIM>

@@ -62,6 +62,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) fluid_tile_kernel(const __gri
   constexpr int K = kTileCells;
   constexpr int A = (D == 0) ? 1 : 0, O = (D == 2) ? 1 : 2, T1 = (D + 1) % 3, T2 = (D + 2) % 3;
   extern __shared__ float4 tile_dyn[];
+  wait_for_previous();
   const BlockGeom G = block_geom(a.ens, a.box, a.seg, a.tau, a.rate);
   const int nA = G.box.n[A], nO = G.box.n[O], nD = G.box.n[D];
   const int T = blockDim.x, tid = threadIdx.x;
@@ -344,6 +345,7 @@ __global__ void __launch_bounds__(MTile<LX, R>::T) mag_tile_kernel(const __grid_
   using M = MTile<LX, R>;
   constexpr int H = mag_tile_halo(D), T = M::T;
   extern __shared__ __align__(16) float mt_dyn[];
+  wait_for_previous();
   const BlockGeom G = block_geom(a.ens, a.box, a.seg, a.tau, nullptr);
   const int nA = G.box.n[A], nO = G.box.n[O], nD = G.box.n[D];
   const MagTile sp = mag_tile_split(nD);
@@ -473,6 +475,7 @@ __global__ void __launch_bounds__(MTile<LX, R>::T) mag_tile_x_kernel(const __gri
   using M = MTile<LX, R>;
   constexpr int H = mag_tile_halo(0), T = M::T;
   extern __shared__ __align__(16) float mt_dyn[];
+  wait_for_previous();
   const BlockGeom G = block_geom(a.ens, a.box, a.seg, a.tau, nullptr);
   const int nA = G.box.n[1], nO = G.box.n[2], nD = G.box.n[0];
   const MagTile sp = mag_tile_split(nD);
@@ -603,13 +606,14 @@ cudaError_t launch_fluid_tile(int axis, bool rate, const FluidArgs& a, cudaStrea
     const size_t smem = fluid_tile_smem(threads);
     const bool floor = a.p_floor > 0.f;
 #define FLUID_TILE_CASE(DD, RR, FF) \
-  if (axis == DD && rate == RR && floor == FF) fluid_tile_kernel<DD, RR, FF, LIM, FRZ, FSQ><<<grid, threads, smem, s>>>(a);
+  if (axis == DD && rate == RR && floor == FF)                                                        \
+    return launch_after(!a.ens.items, fluid_tile_kernel<DD, RR, FF, LIM, FRZ, FSQ>, grid, dim3(threads), smem, s, a);
     FLUID_TILE_CASE(0, false, false) FLUID_TILE_CASE(0, true, false) FLUID_TILE_CASE(0, false, true)
     FLUID_TILE_CASE(0, true, true) FLUID_TILE_CASE(1, false, false) FLUID_TILE_CASE(1, true, false)
     FLUID_TILE_CASE(1, false, true) FLUID_TILE_CASE(1, true, true) FLUID_TILE_CASE(2, false, false)
     FLUID_TILE_CASE(2, true, false) FLUID_TILE_CASE(2, false, true) FLUID_TILE_CASE(2, true, true)
 #undef FLUID_TILE_CASE
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
   }
 }
 
@@ -621,11 +625,10 @@ cudaError_t launch_mag_tile_shape(int axis, const MagArgs& a, cudaStream_t s) {
                                 : dim3((a.box.n[A] + LX - 1) / LX, (a.box.n[O] + R - 1) / R, t.segs);
   const size_t smem = mag_tile_smem<LX, R>(axis, a.ens.items ? a.tile_out : t.out);
   constexpr int T = MTile<LX, R>::T;
-  if (axis == 0) mag_tile_x_kernel<LX, R, LIM><<<grid, T, smem, s>>>(a);
-  else if (axis == 1) mag_tile_kernel<1, LX, R, LIM, 1><<<grid, T, smem, s>>>(a);
-  else if (a.passes == 2) mag_tile_kernel<2, LX, R, LIM, 2><<<grid, T, smem, s>>>(a);
-  else mag_tile_kernel<2, LX, R, LIM, 1><<<grid, T, smem, s>>>(a);
-  return cudaGetLastError();
+  auto* kernel = axis == 0   ? mag_tile_x_kernel<LX, R, LIM>
+                 : axis == 1 ? mag_tile_kernel<1, LX, R, LIM, 1>
+                             : (a.passes == 2 ? mag_tile_kernel<2, LX, R, LIM, 2> : mag_tile_kernel<2, LX, R, LIM, 1>);
+  return launch_after(!a.ens.items, kernel, grid, dim3(T), smem, s, a);
 }
 
 template <int LIM>
