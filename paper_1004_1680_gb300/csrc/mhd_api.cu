@@ -375,23 +375,16 @@ bool any_bc(const mhd_s* m) { return m->bc[0] || m->bc[1] || m->bc[2]; }
 
 // Refill the ghost layers of the non-periodic axes in the current layout:
 // physical axis a is kernel axis k there, with its normal momentum and face
-// field in slots 1 + k and 5 + k (the exchanges relabel the slots).  Axes in
-// physical order x, y, z.
+// field in slots 1 + k and 5 + k (the exchanges relabel the slots).
 int fill_ghosts(mhd_s* m) {
   if (!any_bc(m)) return MHD_OK;
   const mhd::Box& b = m->layout == 2 ? m->zbox : (m->layout ? m->tbox : m->box);
-  for (int a = 0; a < 3; a++) {
-    if (!m->bc[a]) continue;
-    int k = a;
-    if (m->layout == 1 && a < 2) k = 1 - a;
-    if (m->layout == 2 && a != 1) k = 2 - a;
-    if (int rc = traced(m, MHD_K_CONTROL, [&] {
-          CK(mhd::launch_ghost_fill(m->cur, b, k, m->bc[a], m->stream));
-          return MHD_OK;
-        }))
-      return rc;
-  }
-  return MHD_OK;
+  int mode[3];
+  for (int a = 0; a < 3; a++) mode[kernel_axis_of(m, a)] = m->bc[a];
+  return traced(m, MHD_K_CONTROL, [&] {
+    CK(mhd::launch_ghost_fill(m->cur, b, mode, m->stream));
+    return MHD_OK;
+  });
 }
 
 // CFL rate of the current state into *rate (zeroed first).  With ghost

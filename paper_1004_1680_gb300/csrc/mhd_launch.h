@@ -189,18 +189,17 @@ struct MagArgs {
   int tile_out = 0;         // ensemble tile launches: largest `out` of any box (shared memory)
 };
 
-// Ghost layers of a non-periodic axis (boundary.cu): kernel axis `axis` of
-// the fields as stored in `box`; the normal momentum and face field of that
-// axis are f[1 + axis] and f[5 + axis].
+// Ghost layers of the non-periodic axes (boundary.cu) of the fields as stored
+// in `box`: mode per kernel axis k (0 periodic, 1 outflow, 2 reflecting), whose
+// normal momentum and face field are f[1 + k] and f[5 + k].
 constexpr int kGhost = 4;
 struct GhostArgs {
   float* f[8];
-  int axis;
-  int mode;                  // 1 outflow, 2 reflecting
-  int nk, n1, n2;            // extents: the axis, then the other two (n1 the faster)
-  long long sk, s1, s2;      // their strides
+  int n[3], mode[3];
+  long long stride[3];
+  long long first[4];  // elements of the axes' ghost layers, accumulated
 };
-cudaError_t launch_ghost_fill(float* const f[8], const Box& box, int axis, int mode, cudaStream_t s);
+cudaError_t launch_ghost_fill(float* const f[8], const Box& box, const int mode[3], cudaStream_t s);
 
 struct TransposeArgs {
   const float* in[8];
