@@ -425,13 +425,19 @@ int mhd_ens_set_state(mhd_ens_t* e, int b, const float* const f[8], int on_devic
   if (e->layout) return mhd::set_error(MHD_E_ARG, "mhd_ens_set_state", "internal: exchanged layout");
   const mhd::EnsBox& x = e->boxes[b];
   const size_t bytes = sizeof(float) * (size_t)x.n[0] * x.n[1] * x.n[2];
-  for (int q = 0; q < 8; q++)
-    CKE(cudaMemcpyAsync(e->cur[q] + x.offset, f[q], bytes,
-                        on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, e->stream));
   CKE(cudaMemsetAsync(e->rate[e->rcur] + b, 0, sizeof(unsigned), e->stream));
   CKE(cudaMemsetAsync(e->time + b, 0, sizeof(double), e->stream));
   const float* p[8];
   box_ptrs(e, b, p);
+  if (on_device && mhd::local_fields(reinterpret_cast<const void* const*>(f))) {  // copied and rated in one pass
+    float* out[8];
+    for (int q = 0; q < 8; q++) out[q] = e->cur[q] + x.offset;
+    CKE(mhd::launch_cfl_rate(f, plain_box(x), (float)e->gamma, e->rate[e->rcur] + b, e->stream, nullptr, out));
+    return MHD_OK;
+  }
+  for (int q = 0; q < 8; q++)
+    CKE(cudaMemcpyAsync(e->cur[q] + x.offset, f[q], bytes,
+                        on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, e->stream));
   CKE(mhd::launch_cfl_rate(p, plain_box(x), (float)e->gamma, e->rate[e->rcur] + b, e->stream));
   return MHD_OK;
 }
@@ -443,9 +449,15 @@ int mhd_ens_get_state(const mhd_ens_t* e, int b, float* const f[8], int on_devic
   if (e->layout) return mhd::set_error(MHD_E_ARG, "mhd_ens_get_state", "internal: exchanged layout");
   const mhd::EnsBox& x = e->boxes[b];
   const size_t bytes = sizeof(float) * (size_t)x.n[0] * x.n[1] * x.n[2];
-  for (int q = 0; q < 8; q++)
-    CKE(cudaMemcpyAsync(f[q], e->cur[q] + x.offset, bytes,
-                        on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, e->stream));
+  if (on_device && mhd::local_fields(reinterpret_cast<const void* const*>(f))) {
+    const float* p[8];
+    box_ptrs(e, b, p);
+    CKE(mhd::launch_copy_fields(p, f, (long long)x.n[0] * x.n[1] * x.n[2], e->stream));
+  } else {
+    for (int q = 0; q < 8; q++)
+      CKE(cudaMemcpyAsync(f[q], e->cur[q] + x.offset, bytes,
+                          on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, e->stream));
+  }
   CKE(cudaStreamSynchronize(e->stream));
   return MHD_OK;
 }

@@ -387,19 +387,20 @@ int fill_ghosts(mhd_s* m) {
   });
 }
 
-// CFL rate of the current state into *rate (zeroed first).  With ghost
+// CFL rate of the current state into *rate (zeroed first); with `from` (device
+// fields, no ghost layers) of that state, which is copied in on the way.  With ghost
 // layers the rate covers the interior cells only (a ghost cell next to the
 // periodic wrap pairs faces from both ends of the axis), after a refill.
-int state_rate(mhd_s* m, unsigned* rate) {
+int state_rate(mhd_s* m, unsigned* rate, const float* const from[8] = nullptr) {
   if (int rc = fill_ghosts(m)) return rc;
   const mhd::Box& b = m->layout == 2 ? m->zbox : (m->layout ? m->tbox : m->box);
   mhd::CellRange r;
   for (int a = 0; a < 3; a++) rate_window(m, a, &r.lo[kernel_axis_of(m, a)], &r.hi[kernel_axis_of(m, a)]);
-  CK(cudaMemsetAsync(rate, 0, sizeof(unsigned), m->stream));
+  if (!from) CK(cudaMemsetAsync(rate, 0, sizeof(unsigned), m->stream));
   const float* cf[8];
   field_ptrs(m, cf);
   return traced(m, MHD_K_CONTROL, [&] {
-    CK(mhd::launch_cfl_rate(cf, b, (float)m->gamma, rate, m->stream, &r));
+    CK(mhd::launch_cfl_rate(from ? from : cf, b, (float)m->gamma, rate, m->stream, &r, from ? m->cur : nullptr));
     return MHD_OK;
   });
 }
@@ -835,11 +836,16 @@ int mhd_set_state(mhd_t* m, const float* const f[8], int on_device) {
     std::swap(m->spare[5], m->spare[4 + a]);
     m->layout = 0;
   }
-  for (int q = 0; q < 8; q++)
-    CK(cudaMemcpyAsync(m->cur[q], f[q], bytes,
-                       on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, m->stream));
+  const bool local = on_device && mhd::local_fields(reinterpret_cast<const void* const*>(f));
   CK(cudaMemsetAsync(m->sc, 0, sizeof(Scalars), m->stream));
   m->rcur = 0;
+  if (local && !any_bc(m)) return state_rate(m, &m->sc->rate[0], f);
+  if (local)
+    CK(mhd::launch_copy_fields(f, m->cur, m->N, m->stream));
+  else
+    for (int q = 0; q < 8; q++)
+      CK(cudaMemcpyAsync(m->cur[q], f[q], bytes,
+                         on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, m->stream));
   return state_rate(m, &m->sc->rate[0]);
 }
 
@@ -851,9 +857,15 @@ int mhd_get_state(const mhd_t* m, float* const f[8], int on_device) {
   const size_t bytes = sizeof(float) * (size_t)m->N;
   if (m->layout) return fail(MHD_E_ARG, "internal: state left in the exchanged layout");
   if (int rc = join_pipeline(const_cast<mhd_s*>(m))) return rc;
-  for (int q = 0; q < 8; q++)
-    CK(cudaMemcpyAsync(f[q], m->cur[q], bytes,
-                       on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, m->stream));
+  if (on_device && mhd::local_fields(reinterpret_cast<const void* const*>(f))) {
+    const float* cf[8];
+    field_ptrs(m, cf);
+    CK(mhd::launch_copy_fields(cf, f, m->N, m->stream));
+  } else {
+    for (int q = 0; q < 8; q++)
+      CK(cudaMemcpyAsync(f[q], m->cur[q], bytes,
+                         on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, m->stream));
+  }
   CK(cudaStreamSynchronize(m->stream));
   return MHD_OK;
 }

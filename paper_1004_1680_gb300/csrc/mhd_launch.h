@@ -387,7 +387,14 @@ struct CellRange {
   int lo[3], hi[3];
 };
 cudaError_t launch_cfl_rate(const float* const f[8], const Box& box, float gamma, unsigned* rate,
-                            cudaStream_t s, const CellRange* range = nullptr);
+                            cudaStream_t s, const CellRange* range = nullptr,
+                            float* const copy[8] = nullptr);  // copy: also write the fields there
+struct CopyArgs {
+  const float* in[8];
+  float* out[8];
+};
+cudaError_t launch_copy_fields(const float* const in[8], float* const out[8], long long N, cudaStream_t s);
+bool local_fields(const void* const f[8]);
 // device-side step control: tau = cfl / rate_cur (or the given tau if cfl<0),
 // time += 2 tau, rate_next = 0
 cudaError_t launch_step_control(const unsigned* rate_cur, unsigned* rate_next, float* tau,

@@ -17,11 +17,18 @@
 
 namespace mhd {
 
-__global__ void cfl_rate_kernel(const float* __restrict__ rho, const float* __restrict__ mx,
-                                const float* __restrict__ my, const float* __restrict__ mz,
-                                const float* __restrict__ en, const float* __restrict__ bx,
-                                const float* __restrict__ by, const float* __restrict__ bz, Box box,
-                                float gamma, unsigned* rate, CellRange r) {
+// COPY: also writes the fields to out (a state that arrives is copied and
+// rated in one pass: 64 bytes per cell moved instead of 96, one launch instead
+// of nine).
+struct FieldCopy {
+  float* out[8];
+};
+template <bool COPY>
+__global__ void __launch_bounds__(256) cfl_rate_kernel(const float* __restrict__ rho, const float* __restrict__ mx,
+                                                       const float* __restrict__ my, const float* __restrict__ mz,
+                                                       const float* __restrict__ en, const float* __restrict__ bx,
+                                                       const float* __restrict__ by, const float* __restrict__ bz,
+                                                       Box box, float gamma, unsigned* rate, CellRange r, FieldCopy d) {
   // a warp walks whole x rows, 32 cells at a time; rows are stepped without
   // a division per row or cell (64-bit integer division is emulated)
   const int nx = box.n[0], ny = box.n[1], nz = box.n[2];
@@ -35,18 +42,32 @@ __global__ void cfl_rate_kernel(const float* __restrict__ rho, const float* __re
   const long long dk = nwarps / ny;
   float rmax = 0.f;
   for (; row < rows; row += nwarps) {
-    if (j >= r.lo[1] && j < r.hi[1] && k >= r.lo[2] && k < r.hi[2]) {
+    const bool rated = j >= r.lo[1] && j < r.hi[1] && k >= r.lo[2] && k < r.hi[2];
+    if (rated || COPY) {
       const long long rowbase = j * box.stride[1] + k * box.stride[2];
       const long long yoff = (j + 1 < ny) ? box.stride[1] : -(long long)(ny - 1) * box.stride[1];
       const long long zoff = (k + 1 < nz) ? box.stride[2] : -(long long)(nz - 1) * box.stride[2];
-      for (int i = r.lo[0] + lane; i < r.hi[0]; i += 32) {
+#pragma unroll 2
+      for (int i = (COPY ? 0 : r.lo[0]) + lane; i < (COPY ? nx : r.hi[0]); i += 32) {
         const long long c = rowbase + i;  // x is the contiguous axis (checked at launch)
         float m[3] = {__ldg(mx + c), __ldg(my + c), __ldg(mz + c)};
+        const float b0 = __ldg(bx + c), b1 = __ldg(by + c), b2 = __ldg(bz + c);
+        const float rr = __ldg(rho + c), ee = __ldg(en + c);
         float b[3];
-        b[0] = 0.5f * (__ldg(bx + c) + __ldg(bx + (i + 1 < nx ? c + 1 : c - (nx - 1))));
-        b[1] = 0.5f * (__ldg(by + c) + __ldg(by + c + yoff));
-        b[2] = 0.5f * (__ldg(bz + c) + __ldg(bz + c + zoff));
-        rmax = fmaxf(rmax, cell_rate(__ldg(rho + c), m, __ldg(en + c), b, gamma, box.ih));
+        b[0] = 0.5f * (b0 + __ldg(bx + (i + 1 < nx ? c + 1 : c - (nx - 1))));
+        b[1] = 0.5f * (b1 + __ldg(by + c + yoff));
+        b[2] = 0.5f * (b2 + __ldg(bz + c + zoff));
+        if constexpr (COPY) {
+          d.out[RHO][c] = rr;
+          d.out[MX][c] = m[0];
+          d.out[MY][c] = m[1];
+          d.out[MZ][c] = m[2];
+          d.out[EN][c] = ee;
+          d.out[BX][c] = b0;
+          d.out[BY][c] = b1;
+          d.out[BZ][c] = b2;
+        }
+        if (!COPY || (rated && i >= r.lo[0] && i < r.hi[0])) rmax = fmaxf(rmax, cell_rate(rr, m, ee, b, gamma, box.ih));
       }
     }
     j += dj;
@@ -61,7 +82,7 @@ __global__ void cfl_rate_kernel(const float* __restrict__ rho, const float* __re
 }
 
 cudaError_t launch_cfl_rate(const float* const f[8], const Box& box, float gamma, unsigned* rate,
-                            cudaStream_t s, const CellRange* range) {
+                            cudaStream_t s, const CellRange* range, float* const copy[8]) {
   if (box.stride[0] != 1) return cudaErrorInvalidValue;
   const long long N = (long long)box.n[0] * box.n[1] * box.n[2];
   long long blocks = (N + 255) / 256;
@@ -71,9 +92,69 @@ cudaError_t launch_cfl_rate(const float* const f[8], const Box& box, float gamma
     r.lo[d] = range ? range->lo[d] : 0;
     r.hi[d] = range ? range->hi[d] : box.n[d];
   }
-  cfl_rate_kernel<<<(unsigned)blocks, 256, 0, s>>>(f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7],
-                                                   box, gamma, rate, r);
+  FieldCopy c = {};
+  if (copy)
+    for (int q = 0; q < 8; q++) c.out[q] = copy[q];
+  auto* kernel = copy ? cfl_rate_kernel<true> : cfl_rate_kernel<false>;
+  kernel<<<(unsigned)blocks, 256, 0, s>>>(f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7], box, gamma, rate, r, c);
   return cudaGetLastError();
+}
+
+// The 8 fields of N cells from one place on this device to another, in one
+// launch (8 copies take 8 launches of about 2 us for a small box).  W = 4:
+// 16-byte accesses (aligned fields).
+template <int W>
+__global__ void __launch_bounds__(256) copy_fields_kernel(const __grid_constant__ CopyArgs a, long long N) {
+  const long long n = N / W;
+  const long long step = (long long)gridDim.x * 256;
+  for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += step) {
+    if constexpr (W == 4) {
+      float4 v[8];
+#pragma unroll
+      for (int q = 0; q < 8; q++) v[q] = __ldg(reinterpret_cast<const float4*>(a.in[q]) + i);
+#pragma unroll
+      for (int q = 0; q < 8; q++) reinterpret_cast<float4*>(a.out[q])[i] = v[q];
+    } else {
+#pragma unroll
+      for (int q = 0; q < 8; q++) a.out[q][i] = __ldg(a.in[q] + i);
+    }
+  }
+  if (W == 4 && blockIdx.x == 0 && threadIdx.x < N % 4)
+#pragma unroll
+    for (int q = 0; q < 8; q++) a.out[q][n * 4 + threadIdx.x] = __ldg(a.in[q] + n * 4 + threadIdx.x);
+}
+
+cudaError_t launch_copy_fields(const float* const in[8], float* const out[8], long long N, cudaStream_t s) {
+  CopyArgs a;
+  bool vec = true;
+  for (int q = 0; q < 8; q++) {
+    a.in[q] = in[q];
+    a.out[q] = out[q];
+    vec = vec && reinterpret_cast<uintptr_t>(in[q]) % 16 == 0 && reinterpret_cast<uintptr_t>(out[q]) % 16 == 0;
+  }
+  const long long n = vec ? N / 4 : N;
+  long long blocks = (n + 255) / 256;
+  blocks = blocks < 1 ? 1 : (blocks > 152 * 8 ? 152 * 8 : blocks);
+  if (vec) copy_fields_kernel<4><<<(unsigned)blocks, 256, 0, s>>>(a, N);
+  else copy_fields_kernel<1><<<(unsigned)blocks, 256, 0, s>>>(a, N);
+  return cudaGetLastError();
+}
+
+// Whether kernels of the current device can read and write all 8 fields
+// directly: memory of this device (another device's, or host memory, goes
+// through cudaMemcpyAsync).
+bool local_fields(const void* const f[8]) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  for (int q = 0; q < 8; q++) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, f[q]) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (at.type != cudaMemoryTypeDevice || at.device != dev) return false;
+  }
+  return true;
 }
 
 __global__ void step_control_kernel(const unsigned* rate_cur, unsigned* rate_next, float* tau,
