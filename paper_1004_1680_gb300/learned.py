@@ -58,28 +58,23 @@ class CorrectionNet:
         self.imgT = [mhd.conv_pack(w, transpose=True) for w in self.W]
 
     def forward(self, x: torch.Tensor, n):
-        """x: (cells, 8) BF16 -> y (cells, 8) FP32 and the activations."""
-        acts = [x]
-        h = x
-        for li, (ci, co) in enumerate(LAYERS):
-            last = li == len(LAYERS) - 1
-            hb, hf = mhd.conv3d(h, self.img[li], n, ci, co, bias=self.b[li], relu=not last,
-                                out_bf16=not last, out_f32=last)
-            h = hf if last else hb
-            if not last:
-                acts.append(h)
-        return h, acts
+        """x: (cells, 8) BF16 -> y (cells, 8) FP32 and the activations.  One
+        call of the library for the four layers (call by call, Python takes
+        longer than the GPU on a 64^3 grid)."""
+        cells = n[0] * n[1] * n[2]
+        acts = [x] + [torch.empty((cells, co), dtype=torch.bfloat16, device=x.device) for _, co in LAYERS[:-1]]
+        y = torch.empty((cells, LAYERS[-1][1]), dtype=torch.float32, device=x.device)
+        mhd.cnn_forward(x, self.img, self.b, acts[1:], y, n)
+        return y, acts
 
     def backward(self, gy: torch.Tensor, acts, n):
         """gy: (cells, 8) BF16 gradient of the loss w.r.t. y; fills self.grads."""
-        self.grads = [torch.zeros_like(p) for p in self.params]
-        g = gy
+        sizes = [p.numel() for p in self.params]
+        flat = torch.zeros(sum(sizes), device=gy.device)  # every gradient, cleared at once
+        self.grads = [v.view(p.shape) for v, p in zip(flat.split(sizes), self.params)]
         L = len(LAYERS)
-        for li in range(L - 1, -1, -1):
-            ci, co = LAYERS[li]
-            mhd.conv3d_wgrad(acts[li], g, n, ci, co, self.grads[li].view(-1), self.grads[L + li])
-            if li > 0:
-                g, _ = mhd.conv3d(g, self.imgT[li], n, co, ci, flip=True, mask=acts[li])
+        scratch = [torch.empty_like(acts[1]) for _ in range(2)]
+        mhd.cnn_backward(acts[0], acts[1:], gy, self.imgT, self.grads[:L], self.grads[L:], scratch, n)
 
     def adam(self, lr: float):
         self.step_count += 1

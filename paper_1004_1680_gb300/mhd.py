@@ -134,8 +134,15 @@ def _check(rc: int):
         raise MHDError(rc, _lib.mhd_last_error().decode())
 
 
+_Ptr8 = ctypes.c_void_p * 8
+
+
 def _field_ptrs(t: torch.Tensor):
-    return (ctypes.c_void_p * 8)(*[t[q].data_ptr() for q in range(8)])
+    """The addresses of t[0] .. t[7] (without slicing: 12 us a call)."""
+    if t.shape[0] < 8:
+        raise IndexError("8 fields are needed")
+    base, step = t.data_ptr(), t.stride(0) * t.element_size()
+    return _Ptr8(*range(base, base + 8 * step, step)) if step > 0 else _Ptr8(*[t[q].data_ptr() for q in range(8)])
 
 
 def diagnostics_static(state: torch.Tensor, gamma: float = 5.0 / 3.0, stream=None) -> np.ndarray:
