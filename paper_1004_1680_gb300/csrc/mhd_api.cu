@@ -221,9 +221,9 @@ double tile_us(const mhd_s* m, bool mag) { return 2.5 + (mag ? 19e-6 : 21e-6) * 
 // with transposes and marching).
 int tile_choice(const mhd_s* m, int d, bool mag, int passes) {
   if (!m->tma || m->fast == 2 || m->xpath == 3 || m->layout || m->seg_set[d]) return 0;
-  // magnetic tiles of 8 x 2 pencils where there are few (32^3: 64 tiles, 10 us
-  // against 15 us) and along x (128^3: 31 against 33 us), else 16 x 4
-  const int shape = d == 0 || m->N <= 150000 ? 1 : 2;
+  // magnetic tiles of 8 x 2 pencils (128 threads) where there are few (32^3: 44 us
+  // per step against 53), else 16 x 4 (384 threads; 96^3 181 us against 227)
+  const int shape = m->N <= 60000 ? 1 : 2;
   // a launch holds 65535 rows of tiles (the axes' roles as in the sweeps: row
   // axis z, or y for z sweeps) and as many segments of a pencil
   if (mag && (m->n[d == 2 ? 1 : 2] > 2 * 65535 || m->n[d] > 24 * 65535)) return 0;

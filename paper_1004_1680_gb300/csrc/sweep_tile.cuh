@@ -265,21 +265,235 @@ __global__ void __launch_bounds__(kTileThreads, 2) fluid_tile_kernel(const __gri
 // axis O) pencils and `out` positions of them, and holds in shared memory,
 // with the positions' halo at each end (periodic images):
 //   v  = m_D / rho of the tile's pencils and of the ones next to them,
-//   q  = the advected fields of the tile's edge-flux rows: b_A of columns
-//        0 .. LX (LX: the halo column) and b_O of rows 0 .. R,
-//   bD = b_D of the tile's pencils.
-// All of it arrives by asynchronous copies, issued at once.  Then every
-// (edge-flux row, group of 4 edges) is one independent task: 9 cells of q and
-// of the two v rows give the 4 limited edge fluxes f, with the half step of
+//   b_A of columns 0 .. LX and b_O of rows 0 .. R (LX and R: the halo pencils
+//   whose edge flux the tile's b_D takes), b_D of the tile's pencils.
+// All of it arrives by asynchronous 16-byte copies, issued at once.  Then every
+// (pencil, group of 4 edges) is one independent task: 9 cells of b_A, b_O and
+// the velocities around them give the 4 limited edge fluxes of both fields on
+// packed FP32 (one of the two is unused in a halo pencil), with the half step of
 // 3 cells at the group's ends repeated by both neighbours (which needs no
-// exchange between threads).  After a barrier the cells are finished from f.
+// exchange between threads).  After a barrier the cells are finished from the
+// fluxes.  Along y and z it executes 232 instructions per cell (318 with a task
+// per field and 4-byte copies; the marching sweep 144), and what bounds it is
+// the latency of its phases at the blocks that shared memory lets in: 2 per
+// SM, of 384 threads so that a tile's tasks take two whole rounds (96^3 along
+// y 19.7 -> 16.4 us, a step 217 -> 181 us with the launches overlapped).
 template <int LX, int R>
 struct MTile {
-  static constexpr int VC = LX + 2, V = (R + 2) * VC;      // v slots of a plane
+  static constexpr int T = LX * R >= 64 ? 384 : 128;     // threads
+  static constexpr int Tasks = (R + 1) * (LX + 1) - 1;   // pencils with a flux (not the far corner)
+  static constexpr int C = LX * R;                       // cells of a plane
+};
+__host__ __device__ constexpr int mag_tile_halo(int D) { return D == 0 ? 4 : 3; }  // 4: 16-byte copies along x
+
+// positions held per pencil: `out`, the halos and what the last group of edges
+// may touch past them; along x an odd number of 16-byte pieces
+__host__ __device__ constexpr int mag_tile_positions(int D, int out) {
+  const int n = out + 2 * mag_tile_halo(D) + 4;
+  return D == 0 ? (n + 3) / 8 * 8 + 4 : n;
+}
+
+__device__ __forceinline__ void copy16_async(float* dst, const float* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ float4& at4(float* p) { return *reinterpret_cast<float4*>(p); }
+__device__ __forceinline__ float4 v_div4(const float4& m, const float4& r) {
+  return make_float4(v_div(m.x, r.x), v_div(m.y, r.y), v_div(m.z, r.z), v_div(m.w, r.w));
+}
+
+// The 4 limited edge fluxes of a group from 9 cells of (b_A, b_O) and of their
+// face velocities (MagPipe's arithmetic, each element rounded as there): edge k
+// lies between cells k + 2 and k + 3.
+template <int LIM>
+__device__ __forceinline__ void edge_fluxes2(const float2 (&q)[9], const float2 (&u)[9], float c_half, float2 (&f)[4]) {
+  auto sel = [](float2 w, float2 a, float2 b) { return make_float2(w.x >= 0.f ? a.x : b.x, w.y >= 0.f ? a.y : b.y); };
+  float2 ub[8], g[8], h[7], d[6];
+#pragma unroll
+  for (int k = 0; k < 8; k++) {
+    ub[k] = __fmul2_rn(f2(0.5f), __fadd2_rn(u[k], u[k + 1]));
+    g[k] = __fmul2_rn(ub[k], sel(ub[k], q[k], q[k + 1]));
+  }
+#pragma unroll
+  for (int k = 0; k < 7; k++) h[k] = __ffma2_rn(f2(-c_half), sub2(g[k + 1], g[k]), q[k + 1]);
+#pragma unroll
+  for (int k = 0; k < 6; k++) d[k] = sub2(h[k + 1], h[k]);
+#pragma unroll
+  for (int k = 0; k < 4; k++) {
+    const float2 w = ub[k + 2];
+    const float2 lim = half_limited2<LIM>(sel(w, d[k], d[k + 1]), sel(w, d[k + 1], d[k + 2]));
+    // base + lim upwind from below, base - lim from above (the product is exact)
+    f[k] = __fmul2_rn(w, __ffma2_rn(sel(w, f2(1.f), f2(-1.f)), lim, sel(w, h[k + 1], h[k + 2])));
+  }
+}
+
+// Along y and z: planes of pencils, one per position.  NP = 2 (whole pencils
+// only): two sweeps with the same step; the first one's result stays in
+// shared memory.
+template <int LX, int R>
+struct MPlane {  // offsets of a plane's arrays (floats) and its size
+  static constexpr int VW = LX + 8, V = (R + 2) * VW;  // v: rows -1 .. R, columns -4 .. LX + 3
+  static constexpr int AW = LX + 4, A = R * AW;        // b_A: columns 0 .. LX + 3
+  static constexpr int O = (R + 1) * LX;               // b_O: rows 0 .. R
+  static constexpr int B = LX * R;                     // b_D
+  static constexpr int F = (2 * MTile<LX, R>::Tasks + 3) / 4 * 4;  // (f_A, f_O) of the tasks; first holds rho
+  static constexpr int Size = V + A + O + B + (F > V ? F : V);
+  static constexpr int Pieces = (2 * V + A + O + B) / 4;
+};
+
+template <int D, int LX, int R, int LIM, int NP>
+__global__ void __launch_bounds__(MTile<LX, R>::T) mag_tile_kernel(const __grid_constant__ MagArgs a) {
+  static_assert(D != 0, "x sweeps use mag_tile_x_kernel");
+  constexpr int A = 0, O = (D == 2) ? 1 : 2, T1 = (D + 1) % 3;
+  using M = MTile<LX, R>;
+  using L = MPlane<LX, R>;
+  constexpr int H = mag_tile_halo(D), T = M::T, Sv = L::V, Sa = L::A, So = L::O, Sb = L::B, Sf = L::F > L::V ? L::F : L::V;
+  extern __shared__ __align__(16) float mt_dyn[];
+  wait_for_previous();
+  const BlockGeom G = block_geom(a.ens, a.box, a.seg, a.tau, nullptr);
+  const int nA = G.box.n[A], nO = G.box.n[O], nD = G.box.n[D];
+  const MagTile sp = mag_tile_split(nD);
+  const int a0 = G.bx * LX, b0 = G.by * R;
+  const int s0 = G.bz * sp.out, S = min(sp.out, nD - s0);  // this block's positions s0 .. s0 + S - 1
+  const int PN = mag_tile_positions(D, sp.out);
+  float* sv = mt_dyn;
+  float* sa = sv + Sv * PN;
+  float* so = sa + Sa * PN;
+  float* sb = so + So * PN;
+  float* sf = sb + Sb * PN;
+  const int tid = threadIdx.x;
+  const int sO = (int)G.box.stride[O], sD = (int)G.box.stride[D];
+
+  // A thread keeps its 16-byte piece of the plane and walks the positions.  The
+  // lanes are contiguous and nA a multiple of 4, so pieces never straddle the
+  // periodic wrap; rho waits in sf.
+  {
+    constexpr int kSlots = L::Pieces <= 64 ? 64 : 128, kStep = T / kSlots;
+    static_assert(L::Pieces <= kSlots && T % kSlots == 0, "pieces of a plane");
+    int piece = tid % kSlots;
+    if (piece < L::Pieces) {
+      const float* src;
+      float* dst;
+      int row, col, plane;
+      auto place = [&](float* arr, int size, int width, int r0, int c0, const float* field) {
+        const int q = piece * 4;
+        row = q / width + r0;
+        col = q % width + c0;
+        dst = arr + q;
+        plane = size;
+        src = field;
+      };
+      if (piece < Sv / 4) {
+        place(sv, Sv, L::VW, -1, -4, a.in[MX + D]);
+      } else if ((piece -= Sv / 4) < Sv / 4) {
+        place(sf, Sf, L::VW, -1, -4, a.in[RHO]);
+      } else if ((piece -= Sv / 4) < Sa / 4) {
+        place(sa, Sa, L::AW, 0, 0, a.in[BX + A]);
+      } else if ((piece -= Sa / 4) < So / 4) {
+        place(so, So, LX, 0, 0, a.in[BX + O]);
+      } else {
+        piece -= So / 4;
+        place(sb, Sb, LX, 0, 0, a.in[BX + D]);
+      }
+      src += G.off + (wrap_any(a0 + col, nA) + wrap_any(b0 + row, nO) * sO);
+      for (int p = tid / kSlots; p < S + 2 * H; p += kStep)
+        copy16_async(dst + p * plane, src + (unsigned)(wrap_any(s0 - H + p, nD) * sD));
+    }
+    copies_wait();
+    __syncthreads();
+    constexpr int kQuads = Sv / 4;
+    for (int t = tid; t < kQuads * (S + 2 * H); t += T) {
+      const int p = t / kQuads, q = 4 * (t - p * kQuads);
+      at4(sv + p * Sv + q) = v_div4(at4(sv + p * Sv + q), at4(sf + p * Sf + q));
+    }
+  }
+  const float tau = G.tau;
+  const float c_full = tau * G.box.ih[D];  // tau / h_D
+  const float c_half = 0.5f * c_full;
+  const float kA = tau * G.box.ih[A];      // tau / h_A
+  const float kO = tau * G.box.ih[O];      // tau / h_O
+  // edge e lies between local cells e - 1 and e: edges 0 .. S are needed; of a
+  // whole pencil 1 .. S (edge 0 is edge S)
+  const int e0 = sp.whole ? 1 : 0;
+  const int groups = (S + 1 - e0 + 3) / 4;
+  auto flux = [&](int task, int e) -> float2& { return *reinterpret_cast<float2*>(sf + e * Sf + 2 * task); };
+#pragma unroll 1
+  for (int pass = 0; pass < NP; pass++) {
+    __syncthreads();
+    for (int t = tid; t < M::Tasks * groups; t += T) {
+      const int g = t / M::Tasks, ts = t - g * M::Tasks, row = ts / (LX + 1), col = ts - row * (LX + 1);
+      const int e = e0 + 4 * g;  // edges e .. e + 3; cells e - 3 .. e + 5
+      const float* pv = sv + (e - 3 + H) * Sv + (row + 1) * L::VW + col + 4;
+      const float* pa = sa + (e - 3 + H) * Sa + row * L::AW + col;  // (past the array in row R: unused)
+      const float* po = so + (e - 3 + H) * So + row * LX + col;     // (the next row's in column LX: unused)
+      float2 q[9], u[9], f[4];
+#pragma unroll
+      for (int k = 0; k < 9; k++) {
+        const float v = pv[k * Sv];
+        q[k] = make_float2(pa[k * Sa], po[k * So]);
+        // v_D on the b_A and the b_O face
+        u[k] = __fmul2_rn(f2(0.5f), __fadd2_rn(f2(v), make_float2(pv[k * Sv - 1], pv[k * Sv - L::VW])));
+      }
+      edge_fluxes2<LIM>(q, u, c_half, f);
+#pragma unroll
+      for (int k = 0; k < 4; k++) flux(ts, e + k) = f[k];
+    }
+    __syncthreads();
+    if (pass + 1 == NP) {
+      // finish the tile's cells
+      float* __restrict__ oA = a.out[A] + G.off;
+      float* __restrict__ oO = a.out[O] + G.off;
+      float* __restrict__ oD = a.out[D] + G.off;
+      static_assert(T % M::C == 0, "a thread keeps its pencil");
+      const int c = tid % M::C, row = c / LX, col = c - row * LX, ts = row * (LX + 1) + col;
+      if (a0 + col < nA && b0 + row < nO) {
+        const unsigned ob = (unsigned)((a0 + col) + (b0 + row) * sO + s0 * sD);
+        for (int p = tid / M::C; p < S; p += T / M::C) {
+          const int el = sp.whole && p == 0 ? S : p;  // the edge below cell p
+          const float2 lo = flux(ts, el), hi = flux(ts, p + 1);
+          const unsigned o = ob + (unsigned)(p * sD);
+          oA[o] = __fmaf_rn(-c_full, __fsub_rn(hi.x, lo.x), sa[(p + H) * Sa + row * L::AW + col]);
+          oO[o] = __fmaf_rn(-c_full, __fsub_rn(hi.y, lo.y), so[(p + H) * So + c]);
+          oD[o] = constrain(sb[(p + H) * Sb + c], kA, lo.x, flux(ts + 1, el).x, kO, lo.y, flux(ts + LX + 1, el).y, T1 == A);
+        }
+      }
+    } else {
+      // the first pass's result back into shared memory (whole pencils): the
+      // advected fields with their periodic images, and b_D
+      for (int t = tid; t < M::Tasks * S; t += T) {
+        const int p = t / M::Tasks, ts = t - p * M::Tasks, row = ts / (LX + 1), col = ts - row * (LX + 1);
+        const float2 lo = flux(ts, p == 0 ? S : p), hi = flux(ts, p + 1);
+        auto update = [&](float* z, int plane, float fl, float fh) {
+          const float v = __fmaf_rn(-c_full, __fsub_rn(fh, fl), z[p * plane]);
+          z[p * plane] = v;
+          if (p < H) z[(p + S) * plane] = v;
+          if (p >= S - H) z[(p - S) * plane] = v;
+        };
+        if (row < R) update(sa + H * Sa + row * L::AW + col, Sa, lo.x, hi.x);
+        if (col < LX) update(so + H * So + row * LX + col, So, lo.y, hi.y);
+        if (row < R && col < LX) {
+          float* z = sb + (p + H) * Sb + row * LX + col;
+          const int el = p == 0 ? S : p;
+          *z = constrain(*z, kA, lo.x, flux(ts + 1, el).x, kO, lo.y, flux(ts + LX + 1, el).y, T1 == A);
+        }
+      }
+    }
+  }
+}
+
+// Along x: a pencil's positions are contiguous, everything moves in 16-byte
+// pieces of 4 positions (an odd number of pieces per pencil keeps the pencils
+// of a quarter warp in different banks).  A task is one field's edge flux: the
+// packed pairs of the other axes, whose operands come from separate 16-byte
+// reads here, executed as many instructions (358 per cell against 354) and ran
+// slower (128^3: 33 us against 31).
+template <int LX, int R>
+struct MRows {
+  static constexpr int VC = LX + 2, V = (R + 2) * VC;      // pencils of v: rows -1 .. R, columns -1 .. LX
   static constexpr int QA = R * (LX + 1), Q = QA + (R + 1) * LX;  // edge-flux rows: b_A, then b_O
-  static constexpr int C = LX * R;                          // cells of a plane
-  static constexpr int T = C >= 64 ? 256 : 128;             // threads
-  // v slots of edge-flux row ts's pencil (low) and of the one across its faces (high half)
+  static constexpr int C = LX * R;
+  static constexpr int Size = V + 2 * Q + C;
+  // v pencils of edge-flux row ts's pencil and of the one across its faces
   static __device__ __forceinline__ void rows(int ts, int& own, int& nbr) {
     if (ts < QA) {
       const int row = ts / (LX + 1), col = ts - row * (LX + 1);
@@ -292,25 +506,6 @@ struct MTile {
     }
   }
 };
-__host__ __device__ constexpr int mag_tile_halo(int D) { return D == 0 ? 4 : 3; }  // 4: 16-byte loads along x
-// positions held per slot: `out`, the halos and what the last group of edges
-// may touch past them; along x an odd number of 16-byte pieces (bank conflicts)
-__host__ __device__ constexpr int mag_tile_positions(int D, int out) {
-  const int n = out + 2 * mag_tile_halo(D) + 4;
-  return D == 0 ? (n + 3) / 8 * 8 + 4 : n;
-}
-template <int LX, int R>
-__host__ __device__ constexpr size_t mag_tile_smem(int D, int out) {
-  return sizeof(float) * (MTile<LX, R>::V + 2 * MTile<LX, R>::Q + MTile<LX, R>::C) * mag_tile_positions(D, out);
-}
-
-__device__ __forceinline__ void copy4_async(float* dst, const float* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void copy16_async(float* dst, const float* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // The 4 limited edge fluxes of a group from 9 cells of q and face velocity u
 // (MagPipe's arithmetic): edge k lies between cells k + 2 and k + 3.
@@ -335,145 +530,10 @@ __device__ __forceinline__ void edge_fluxes(const float (&q)[9], const float (&u
   }
 }
 
-// Along y and z: planes of slots, one per position.  NP = 2 (whole pencils
-// only): two sweeps with the same step; the first one's result stays in
-// shared memory.
-template <int D, int LX, int R, int LIM, int NP>
-__global__ void __launch_bounds__(MTile<LX, R>::T) mag_tile_kernel(const __grid_constant__ MagArgs a) {
-  static_assert(D != 0, "x sweeps use mag_tile_x_kernel");
-  constexpr int A = 0, O = (D == 2) ? 1 : 2, T1 = (D + 1) % 3;
-  using M = MTile<LX, R>;
-  constexpr int H = mag_tile_halo(D), T = M::T;
-  extern __shared__ __align__(16) float mt_dyn[];
-  wait_for_previous();
-  const BlockGeom G = block_geom(a.ens, a.box, a.seg, a.tau, nullptr);
-  const int nA = G.box.n[A], nO = G.box.n[O], nD = G.box.n[D];
-  const MagTile sp = mag_tile_split(nD);
-  const int a0 = G.bx * LX, b0 = G.by * R;
-  const int s0 = G.bz * sp.out, S = min(sp.out, nD - s0);  // this block's positions s0 .. s0 + S - 1
-  const int PN = mag_tile_positions(D, sp.out);
-  float* sv = mt_dyn;
-  float* sq = sv + M::V * PN;
-  float* sf = sq + M::Q * PN;
-  float* sb = sf + M::Q * PN;
-  const int tid = threadIdx.x;
-  const int sA = (int)G.box.stride[A], sO = (int)G.box.stride[O], sD = (int)G.box.stride[D];
-
-  // slot (row, col) of the (R+2) x (LX+2) plane is the pencil (b0 + row - 1,
-  // a0 + col - 1), periodic; the corners are not needed.  A thread keeps its
-  // slot and walks the positions; rho waits in sf.
-  {
-    constexpr int kSlots = M::V <= 64 ? 64 : 128, kStep = T / kSlots;
-    static_assert(M::V <= kSlots && T % kSlots == 0 && M::Q >= M::V, "slots of a plane");
-    const int slot = tid % kSlots;
-    const int row = slot / M::VC, col = slot - row * M::VC;
-    const bool rin = row >= 1 && row <= R, cin = col >= 1 && col <= LX;
-    if (slot < M::V && (rin || cin)) {
-      const unsigned pb = (unsigned)(wrap_any(a0 + col - 1, nA) * sA + wrap_any(b0 + row - 1, nO) * sO);
-      const float* rho = a.in[RHO] + G.off + pb;
-      const float* md = a.in[MX + D] + G.off + pb;
-      const float* bA = a.in[BX + A] + G.off + pb;
-      const float* bO = a.in[BX + O] + G.off + pb;
-      const float* bD = a.in[BX + D] + G.off + pb;
-      const bool hasA = rin && col >= 1, hasO = cin && row >= 1, own = rin && cin;
-      float* qa = sq + (row - 1) * (LX + 1) + col - 1;
-      float* qo = sq + M::QA + (row - 1) * LX + col - 1;
-      float* qd = sb + (row - 1) * LX + col - 1;
-      for (int p = tid / kSlots; p < S + 2 * H; p += kStep) {
-        const unsigned c = (unsigned)(wrap_any(s0 - H + p, nD) * sD);
-        copy4_async(sv + p * M::V + slot, md + c);
-        copy4_async(sf + p * M::V + slot, rho + c);
-        if (hasA) copy4_async(qa + p * M::Q, bA + c);
-        if (hasO) copy4_async(qo + p * M::Q, bO + c);
-        if (own) copy4_async(qd + p * M::C, bD + c);
-      }
-      copies_wait();
-      for (int p = tid / kSlots; p < S + 2 * H; p += kStep)
-        sv[p * M::V + slot] = v_div(sv[p * M::V + slot], sf[p * M::V + slot]);
-    }
-  }
-  const float tau = G.tau;
-  const float c_full = tau * G.box.ih[D];  // tau / h_D
-  const float c_half = 0.5f * c_full;
-  const float kA = tau * G.box.ih[A];      // tau / h_A
-  const float kO = tau * G.box.ih[O];      // tau / h_O
-  // edge e lies between local cells e - 1 and e: edges 0 .. S are needed; of a
-  // whole pencil 1 .. S (edge 0 is edge S)
-  const int e0 = sp.whole ? 1 : 0;
-  const int groups = (S + 1 - e0 + 3) / 4;
-#pragma unroll 1
-  for (int pass = 0; pass < NP; pass++) {
-    __syncthreads();
-    for (int t = tid; t < M::Q * groups; t += T) {
-      const int g = t / M::Q, ts = t - g * M::Q;
-      const int e = e0 + 4 * g;  // edges e .. e + 3; cells e - 3 .. e + 5
-      int vo, vn;
-      M::rows(ts, vo, vn);
-      const float* pv = sv + vo + (e - 3 + H) * M::V;
-      const float* pn = sv + vn + (e - 3 + H) * M::V;
-      const float* pq = sq + ts + (e - 3 + H) * M::Q;
-      float q[9], u[9], f[4];
-#pragma unroll
-      for (int k = 0; k < 9; k++) {
-        q[k] = pq[k * M::Q];
-        u[k] = __fmul_rn(0.5f, __fadd_rn(pv[k * M::V], pn[k * M::V]));  // v_D on the face
-      }
-      edge_fluxes<LIM>(q, u, c_half, f);
-#pragma unroll
-      for (int k = 0; k < 4; k++) sf[ts + (e + k) * M::Q] = f[k];
-    }
-    __syncthreads();
-    if (pass + 1 == NP) {
-      // finish the tile's cells
-      float* __restrict__ oA = a.out[A] + G.off;
-      float* __restrict__ oO = a.out[O] + G.off;
-      float* __restrict__ oD = a.out[D] + G.off;
-      static_assert(T % M::C == 0, "a thread keeps its pencil");
-      const int c = tid % M::C, row = c / LX, col = c - row * LX;
-      if (a0 + col < nA && b0 + row < nO) {
-        const int qa = row * (LX + 1) + col, qo = M::QA + row * LX + col;
-        const unsigned ob = (unsigned)((a0 + col) * sA + (b0 + row) * sO + s0 * sD);
-        for (int p = tid / M::C; p < S; p += T / M::C) {
-          const float* fl = sf + (sp.whole && p == 0 ? S : p) * M::Q;  // the edge below cell p
-          const float* fh = sf + (p + 1) * M::Q;
-          const float* qp = sq + (p + H) * M::Q;
-          const float fa0 = fl[qa], fo0 = fl[qo];
-          const unsigned o = ob + (unsigned)(p * sD);
-          oA[o] = __fmaf_rn(-c_full, __fsub_rn(fh[qa], fa0), qp[qa]);
-          oO[o] = __fmaf_rn(-c_full, __fsub_rn(fh[qo], fo0), qp[qo]);
-          oD[o] = constrain(sb[c + (p + H) * M::C], kA, fa0, fl[qa + 1], kO, fo0, fl[qo + LX], T1 == A);
-        }
-      }
-    } else {
-      // the first pass's result back into shared memory (whole pencils): the
-      // edge-flux rows' fields with their periodic images, and b_D
-      for (int t = tid; t < M::Q * S; t += T) {
-        const int p = t / M::Q, ts = t - p * M::Q;
-        float* z = sq + ts + H * M::Q;
-        const float v = __fmaf_rn(-c_full, __fsub_rn(sf[ts + (p + 1) * M::Q], sf[ts + (p == 0 ? S : p) * M::Q]),
-                                  z[p * M::Q]);
-        z[p * M::Q] = v;
-        if (p < H) z[(p + S) * M::Q] = v;
-        if (p >= S - H) z[(p - S) * M::Q] = v;
-      }
-      for (int t = tid; t < M::C * S; t += T) {
-        const int p = t / M::C, c = t - p * M::C, row = c / LX, col = c - row * LX;
-        const float* fl = sf + (p == 0 ? S : p) * M::Q;
-        const int qa = row * (LX + 1) + col, qo = M::QA + row * LX + col;
-        float* z = sb + c + (p + H) * M::C;
-        *z = constrain(*z, kA, fl[qa], fl[qa + 1], kO, fl[qo], fl[qo + LX], T1 == A);
-      }
-    }
-  }
-}
-
-// Along x: a slot's positions are contiguous, everything moves in 16-byte
-// pieces (4 positions; an odd number of pieces per slot keeps the slots of a
-// quarter warp in different banks).
 template <int LX, int R, int LIM>
 __global__ void __launch_bounds__(MTile<LX, R>::T) mag_tile_x_kernel(const __grid_constant__ MagArgs a) {
-  using M = MTile<LX, R>;
-  constexpr int H = mag_tile_halo(0), T = M::T;
+  using M = MRows<LX, R>;
+  constexpr int H = mag_tile_halo(0), T = MTile<LX, R>::T;
   extern __shared__ __align__(16) float mt_dyn[];
   wait_for_previous();
   const BlockGeom G = block_geom(a.ens, a.box, a.seg, a.tau, nullptr);
@@ -488,28 +548,35 @@ __global__ void __launch_bounds__(MTile<LX, R>::T) mag_tile_x_kernel(const __gri
   float* sb = sf + M::Q * PN;
   const int tid = threadIdx.x;
   const int sA = (int)G.box.stride[1], sO = (int)G.box.stride[2];
-  auto at4 = [](float* p) -> float4& { return *reinterpret_cast<float4*>(p); };
-
-  const int pieces = (S + 2 * H) / 4;
-  for (int half = 0; half < 2; half++) {  // copies, then v of the thread's own pieces
-    for (int t = tid; t < M::V * pieces; t += T) {
-      const int slot = t / pieces, g = t - slot * pieces;
+  // (pencil, piece) pairs, stepped without a division per piece; a thread
+  // forms v of the pieces it has copied itself
+  const int pieces = (S + 2 * H) / 4, dslot = T / pieces, dpiece = T - dslot * pieces;
+  const int slot0 = tid / pieces, piece0 = tid - slot0 * pieces;
+  for (int half = 0; half < 2; half++) {
+    int slot = slot0, g = piece0;
+    while (slot < M::V) {
       const int row = slot / M::VC, col = slot - row * M::VC;
       const bool rin = row >= 1 && row <= R, cin = col >= 1 && col <= LX;
-      if (!rin && !cin) continue;
-      float* v = sv + slot * PN + 4 * g;
-      float* r = sf + slot * PN + 4 * g;
-      if (half == 0) {
-        const unsigned c = (unsigned)(wrap_any(a0 + col - 1, nA) * sA + wrap_any(b0 + row - 1, nO) * sO +
-                                      wrap_any(s0 - H + 4 * g, nD)) + (unsigned)G.off;
-        copy16_async(v, a.in[MX] + c);
-        copy16_async(r, a.in[RHO] + c);
-        if (rin && col >= 1) copy16_async(sq + ((row - 1) * (LX + 1) + col - 1) * PN + 4 * g, a.in[BY] + c);
-        if (cin && row >= 1) copy16_async(sq + (M::QA + (row - 1) * LX + col - 1) * PN + 4 * g, a.in[BZ] + c);
-        if (rin && cin) copy16_async(sb + ((row - 1) * LX + col - 1) * PN + 4 * g, a.in[BX] + c);
-      } else {
-        const float4 m4 = at4(v), r4 = at4(r);
-        at4(v) = make_float4(v_div(m4.x, r4.x), v_div(m4.y, r4.y), v_div(m4.z, r4.z), v_div(m4.w, r4.w));
+      if (rin || cin) {
+        float* v = sv + slot * PN + 4 * g;
+        float* r = sf + slot * PN + 4 * g;
+        if (half == 0) {
+          const unsigned c = (unsigned)(wrap_any(a0 + col - 1, nA) * sA + wrap_any(b0 + row - 1, nO) * sO +
+                                        wrap_any(s0 - H + 4 * g, nD)) + (unsigned)G.off;
+          copy16_async(v, a.in[MX] + c);
+          copy16_async(r, a.in[RHO] + c);
+          if (rin && col >= 1) copy16_async(sq + ((row - 1) * (LX + 1) + col - 1) * PN + 4 * g, a.in[BY] + c);
+          if (cin && row >= 1) copy16_async(sq + (M::QA + (row - 1) * LX + col - 1) * PN + 4 * g, a.in[BZ] + c);
+          if (rin && cin) copy16_async(sb + ((row - 1) * LX + col - 1) * PN + 4 * g, a.in[BX] + c);
+        } else {
+          at4(v) = v_div4(at4(v), at4(r));
+        }
+      }
+      slot += dslot;
+      g += dpiece;
+      if (g >= pieces) {
+        g -= pieces;
+        slot++;
       }
     }
     if (half == 0) copies_wait();
@@ -588,6 +655,11 @@ __global__ void __launch_bounds__(MTile<LX, R>::T) mag_tile_x_kernel(const __gri
     at4(a.out[2] + o) = make_float4(rO[0], rO[1], rO[2], rO[3]);
     at4(a.out[0] + o) = make_float4(rD[0], rD[1], rD[2], rD[3]);
   }
+}
+
+template <int LX, int R>
+__host__ __device__ constexpr size_t mag_tile_smem(int D, int out) {
+  return sizeof(float) * (D == 0 ? MRows<LX, R>::Size : MPlane<LX, R>::Size) * mag_tile_positions(D, out);
 }
 
 // ---------------------------------------------------------------------------
