@@ -9,6 +9,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <map>
 #include <new>
 #include <utility>
 #include <vector>
@@ -17,6 +18,8 @@
 #include "mhd_launch.h"
 
 namespace {
+
+constexpr int kMinSeg = 28;  // cells of a pencil segment at least (7 of warm-up)
 
 thread_local char g_err[512] = "";
 
@@ -90,7 +93,7 @@ struct mhd_s {
   unsigned long long* rate64 = nullptr;  // CFL rate (double bits)
   double time64 = 0.0;
   cudaStream_t stream = nullptr;
-  int seg[3];
+  int seg[3][3];        // per axis: segment length of its fluid, magnetic and fused magnetic sweeps
   bool seg_set[3] = {false, false, false};  // segments given by mhd_set_segments
   int sms = 0;          // multiprocessors of the device (segment choice)
   // tracing: event pairs around launches (see mhd_profile)
@@ -149,68 +152,97 @@ void rate_window(const mhd_s* m, int p, int* lo, int* hi) {
   *hi = std::min(m->bc[p] ? m->n[p] - mhd::kGhost : m->n[p], m->own_hi[p]);
 }
 
-// Segment length along each axis.  Splitting pencils into segments adds 7
-// cells of warm-up per segment but gives the GPU more threads.  First split
-// until the pencil segments give about one full wave of threads (152 x 1024:
-// enough warps to hide latency); then, since a sweep runs ceil(n_A/32) x
-// ceil(n_O/W) blocks per segment of every pencil (W = 4 rows for the fluid
-// sweep, 8 for the magnetic one), take among that and further splits (at
-// least 32 cells, multiples of 8) the one that minimises (warm-up work) /
-// sqrt(last-wave efficiency) summed over the two sweeps, with the resident
-// blocks per SM of each kernel (fluid 4, magnetic 2).
-int choose_seg(const mhd_s* m, int d) {
-  const int nd = m->n[d];
-  const long long pencils = m->N / nd;
-  const long long want = 152LL * 1024;
-  int first = nd;
-  while (pencils * (nd / first) < want && first % 8 == 0 && first / 2 >= 32 && nd % (first / 2) == 0)
-    first /= 2;
-  const int nA = m->n[d == 0 ? 1 : 0], nO = m->n[d == 2 ? 1 : 2];
-  const double sms = m->sms > 0 ? m->sms : 152;
-  auto cost = [&](int seg) {
-    double c = 0.0;
-    const int rows[2] = {4, mhd::kMagWarps}, resident[2] = {4, 2};
-    for (int k = 0; k < 2; k++) {
-      const double blocks = (double)((nA + 31) / 32) * ((nO + rows[k] - 1) / rows[k]) * (nd / seg);
-      const double waves = blocks / (sms * resident[k]);
-      // a partial last wave costs less than its idle fraction (the SMs that
-      // run it go faster alone): its weight enters as a square root, which
-      // matches measured sweeps at 256^3, 512^3 and 1024^3
-      c += (double)(seg + 7) / seg * std::sqrt(std::ceil(waves) / waves);
-    }
-    return c;
+// Segment length of a marching sweep along axis d (kind 0: fluid, 1: magnetic,
+// 2: the fused magnetic pair).  A segment costs `warm` cells of warm-up, a
+// sweep runs `tiles` blocks per segment (32 lanes x W rows of pencils) and an
+// SM holds `resident` of them; the blocks are launched segment by segment, and
+// the last segment of a pencil may be shorter.  What costs is a last wave that
+// leaves most of the chip idle: with lengths that divide the pencil only,
+// 160^3 took 67 us per fluid sweep and 49 per magnetic one, 56 and 35 with
+// 56 + 56 + 48 cells (200 and 100 blocks a segment for 608 and 304 places).
+//
+// Magnetic sweeps: k nearly equal segments, the k with the least (cells
+// marched) x sqrt(idle share of the last wave) - within 1 % of the best
+// length at 128^3 .. 512^3; a long and a short segment, which the fluid sweep
+// prefers, loses up to 25 % (224^3: 80 us with 3 x 76, 104 with 156 + 68).
+// Fluid sweeps: any length; the blocks are placed on the chip's slots in
+// launch order, a stretch during which b blocks are on an SM counts
+// 0.6 + 0.4 (b - 1) / 3 per cell, and a tenth of the last block's length is
+// added (blocks do not end together: short last ones fill the gaps).  Within
+// 1.1 % of the best length on average (3 % at most, 256^3 and 384^3), e.g.
+// 200^3 139 -> 117 us with 140 + 60 cells, 256^3 196 -> 188 with 228 + 28
+// (equal segments: 190), 512^3 1312 -> 1288.
+int choose_seg(const mhd_s* m, int d, int kind) {
+  const int nd = m->n[d], nA = m->n[d == 0 ? 1 : 0], nO = m->n[d == 2 ? 1 : 2];
+  const int W = kind ? mhd::kMagWarps : 4, resident = kind ? 2 : 4, warm = kind == 2 ? 14 : 7;
+  const int sms = m->sms > 0 ? m->sms : 152;
+  const double tiles = (double)((nA + 31) / 32) * ((nO + W - 1) / W), slots = (double)sms * resident;
+  auto magnetic_cost = [&](int seg) {
+    const int k = (nd + seg - 1) / seg;
+    const double waves = tiles * k / slots;
+    return k * (double)(seg + warm) * std::sqrt(std::ceil(waves) / waves);
   };
-  int best = first;
-  double best_cost = cost(first);
-  for (int seg = first; seg % 8 == 0 && seg / 2 >= 32 && nd % (seg / 2) == 0;) {
-    seg /= 2;
-    const double c = cost(seg);
+  auto fluid_cost = [&](int seg) {
+    const int rest = nd % seg;
+    const double work = ((nd / seg) * (double)(seg + warm) + (rest ? rest + warm : 0)) * tiles / slots;
+    const double last = 0.1 * ((rest ? rest : seg) + warm);
+    if (tiles * (nd / seg) > 64 * slots) return work + last;
+    const double length[2] = {(double)(seg + warm), (double)(rest + warm)};
+    double left[2] = {tiles * (nd / seg), rest ? tiles : 0.0};
+    std::map<double, double> running;  // cells marched at the finish -> blocks
+    double now = 0.0, cost = 0.0, active = 0.0;
+    for (;;) {
+      for (int q = 0; q < 2; q++) {  // the short ones start once every long one has
+        const double c = q && left[0] > 0.0 ? 0.0 : std::min(slots - active, left[q]);
+        if (c <= 0.0) continue;
+        running[now + length[q]] += c;
+        active += c;
+        left[q] -= c;
+      }
+      if (running.empty()) return std::max(work, cost) + last;
+      const auto first = running.begin();
+      cost += (first->first - now) * (0.6 + 0.4 / 3.0 * (std::ceil(active / sms) - 1.0));
+      now = first->first;
+      active -= first->second;
+      running.erase(first);
+    }
+  };
+  int best = nd;
+  double best_cost = kind ? magnetic_cost(nd) : fluid_cost(nd);
+  auto candidate = [&](int seg) {  // (multiples of 4: x chunks start 16-byte aligned)
+    seg = (seg + 3) / 4 * 4;
+    if (seg < kMinSeg || seg >= nd) return;
+    const double c = kind ? magnetic_cost(seg) : fluid_cost(seg);
     if (c < best_cost * 0.999) {
       best = seg;
       best_cost = c;
     }
-  }
+  };
+  for (int k = 2; nd / k >= kMinSeg - 3; k += 1 + k / 16) candidate((nd + k - 1) / k);
+  if (!kind)
+    for (int f = 17; f < 32; f++) candidate((int)((long long)nd * f / 32));  // a long and a short one
   return best;
 }
 
-// Estimated microseconds of a y or z sweep, from measured times: a marching
-// sweep takes (positions a thread marches) x (time per position), the latter
-// growing with the blocks that share an SM (0.5 us for one fluid block of 4
-// warps, 0.98 us for 4; 0.36 to 0.56 us for one or two magnetic blocks; the
-// fused magnetic pair 0.55 to 0.87 us); a tile sweep takes a time per cell
-// once it fills the chip (21 ps fluid, 19 ps magnetic).  Measured at 96^3:
-// fluid 21 us tile, 31 us marching, magnetic 21 and 27; at 128^3: 44 and 39,
-// 39 and 25.
+// Estimated microseconds of a y or z sweep within a step, from measured times:
+// a marching sweep takes 3 us and (positions a thread marches) x (time per
+// position), the latter growing with the blocks that share an SM (0.5 us for
+// one fluid block of 4 warps, 0.98 us for 4; 0.46 and 0.56 us for one or two
+// magnetic blocks; the fused magnetic pair 0.71 and 0.87 us); a tile sweep
+// takes a time per cell once it fills the chip (21 ps fluid, 19 ps magnetic;
+// its launch overlaps the sweep before).  Measured alone at 96^3: fluid 21 us
+// tile, 31 us marching, magnetic 18 and 21 (a step 182 us with both tiles, 204
+// with marching magnetic sweeps); at 128^3: 44 and 39, 39 and 25.
 double march_us(const mhd_s* m, int d, bool mag, int passes) {
   const int nA = m->n[d == 0 ? 1 : 0], nO = m->n[d == 2 ? 1 : 2];
-  const int W = mag ? mhd::kMagWarps : 4, resident = mag ? 2 : 4;
-  const double blocks = (double)((nA + 31) / 32) * ((nO + W - 1) / W) * (m->n[d] / m->seg[d]) /
+  const int W = mag ? mhd::kMagWarps : 4, resident = mag ? 2 : 4, seg = m->seg[d][mag ? passes : 0];
+  const double blocks = (double)((nA + 31) / 32) * ((nO + W - 1) / W) * (double)m->n[d] / seg /
                         (m->sms > 0 ? m->sms : 152);  // per SM
-  const double b = std::min(blocks, (double)resident), waves = std::max(1.0, blocks / resident);
-  if (!mag) return (m->seg[d] + 7) * (0.5 + 0.03 * b * b) * waves;
-  return passes == 2 ? (m->seg[d] + 14) * (0.55 + 0.16 * b) * waves : (m->seg[d] + 7) * (0.36 + 0.1 * b) * waves;
+  const double b = std::min(std::ceil(blocks), (double)resident), waves = std::max(1.0, blocks / resident);
+  if (!mag) return 3.0 + (seg + 7) * (0.5 + 0.03 * b * b) * waves;
+  return 3.0 + (passes == 2 ? (seg + 14) * (0.55 + 0.16 * b) : (seg + 7) * (0.36 + 0.1 * b)) * waves;
 }
-double tile_us(const mhd_s* m, bool mag) { return 2.5 + (mag ? 19e-6 : 21e-6) * (double)m->N; }
+double tile_us(const mhd_s* m, bool mag) { return (mag ? 19e-6 : 21e-6) * (double)m->N; }
 
 // Tile sweep or not, along axis d of a box in the plain layout: 0, or the tile
 // argument of FluidArgs / MagArgs.  Along y and z by the estimates above.
@@ -421,7 +453,7 @@ int fluid(mhd_s* m, int d, bool rate) {
   a.p_floor = m->p_floor;
   a.tau = &m->sc->tau;
   a.rate = rate ? &m->sc->rate[1 - m->rcur] : nullptr;
-  a.seg = m->seg[d];
+  a.seg = m->seg[d][0];
   a.lim = m->lim;
   a.fast = m->fast;
   for (int p = 0; p < 3; p++)  // the fused rate covers the interior, own cells
@@ -462,7 +494,7 @@ int magnetic(mhd_s* m, int d, int passes = 1) {
   for (int q = 0; q < 3; q++) a.out[q] = m->spare[5 + q];
   a.box = *box;
   a.tau = &m->sc->tau;
-  a.seg = m->seg[d];
+  a.seg = m->seg[d][passes];
   a.lim = m->lim;
   a.passes = passes;
   int staged = 0;
@@ -733,7 +765,8 @@ mhd_t* mhd_create(int nx, int ny, int nz, double gamma) {
     delete m;
     return nullptr;
   }
-  for (int d = 0; d < 3; d++) m->seg[d] = choose_seg(m, d);
+  for (int d = 0; d < 3; d++)
+    for (int k = 0; k < 3; k++) m->seg[d][k] = choose_seg(m, d, k);
   return m;
 }
 
@@ -1027,7 +1060,7 @@ int mhd_set_segments(mhd_t* m, int seg_x, int seg_y, int seg_z) {
     if (seg[d] != 0 && (seg[d] < 4 || seg[d] % 4 != 0 || m->n[d] % seg[d] != 0))
       return fail(MHD_E_ARG, "segment length must be a multiple of 4 dividing n_d");
   for (int d = 0; d < 3; d++) {
-    m->seg[d] = seg[d] ? seg[d] : choose_seg(m, d);
+    for (int k = 0; k < 3; k++) m->seg[d][k] = seg[d] ? seg[d] : choose_seg(m, d, k);
     m->seg_set[d] = seg[d] != 0;
   }
   return MHD_OK;

@@ -182,10 +182,10 @@ __device__ __forceinline__ void fluid_sweep_body(const FluidArgs& a, const Fluid
   const float c_full = tau * G.box.ih[D];  // tau / h_D
   const float c_half = 0.5f * c_full;    // tau / (2 h_D)
   const int s0 = G.bz * G.seg;
-  const int s1 = s0 + G.seg;
+  const int s1 = min(nD, s0 + G.seg);  // the last segment may be shorter
   // positions s0-4 .. s1+2 feed outputs s0 .. s1-1 (3 cells of lag, 1 extra
   // warm-up cell so that x chunks start 16-byte aligned)
-  const int nchunk = (G.seg + 7 + CH - 1) / CH;
+  const int nchunk = (s1 - s0 + 7 + CH - 1) / CH;
 
   // staged chunks: this thread's element of a field, and the element of its
   // neighbour pencil along A and along O: the next lane / row of the block,
@@ -406,11 +406,12 @@ cudaError_t launch_fluid_t(int axis, bool rate, const FluidArgs& a, cudaStream_t
   dim3 block(32, kFluidWarps);
   // tiles of 32 x kFluidWarps pencils (TMA-staged and x sweeps) or runs of
   // 32 kFluidWarps consecutive pencils (register-load y and z sweeps)
-  const dim3 tiles((a.box.n[A] + 31) / 32, (a.box.n[O] + kFluidWarps - 1) / kFluidWarps, a.box.n[axis] / a.seg);
+  const int segs = (a.box.n[axis] + a.seg - 1) / a.seg;
+  const dim3 tiles((a.box.n[A] + 31) / 32, (a.box.n[O] + kFluidWarps - 1) / kFluidWarps, segs);
   dim3 grid = axis == 0 ? tiles
                         : dim3((unsigned)(((long long)a.box.n[A] * a.box.n[O] + 32 * kFluidWarps - 1) /
                                           (32 * kFluidWarps)),
-                               1, a.box.n[axis] / a.seg);
+                               1, segs);
   // ensemble launches: one block per work item; `small` must hold for every
   // box of the launch (the host passes the smallest extent in a.box)
   if (a.ens.items) grid = dim3(a.nblocks, 1, 1);

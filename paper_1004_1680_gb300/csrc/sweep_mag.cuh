@@ -144,10 +144,10 @@ mag_sweep_kernel(MagArgs a) {
   const float kA = tau * G.box.ih[X::A];       // tau / h_A
   const float kO = tau * G.box.ih[X::O];       // tau / h_O
   const int s0 = G.bz * G.seg;
-  const int s1 = s0 + G.seg;
+  const int s1 = min(nD, s0 + G.seg);  // the last segment may be shorter
   // positions s0-4 .. s1+2 feed outputs s0 .. s1-1 (3 cells of lag, 1 extra
   // warm-up cell so that x chunks start 16-byte aligned)
-  const int nchunk = (G.seg + 7 + CH - 1) / CH;
+  const int nchunk = (s1 - s0 + 7 + CH - 1) / CH;
   // slots read by the tile: fO rows 0..cntO (row cntO = halo row), fA columns
   // 0..cntA (column cntA = halo column); idle lanes of a partial tile must not
   // overwrite a halo slot
@@ -401,11 +401,11 @@ __device__ __forceinline__ void mag_pipe_role(const MagArgs& a, const BlockGeom&
   const float kA = tau * G.box.ih[X::A];       // tau / h_A
   const float kO = tau * G.box.ih[X::O];       // tau / h_O
   const int s0 = G.bz * G.seg;
-  const int s1 = s0 + G.seg;
+  const int s1 = min(nD, s0 + G.seg);  // the last segment may be shorter
   // each pass lags its input by 3 positions: positions s0-4NP .. s1+3NP-1
   // feed outputs s0 .. s1-1 (one extra warm-up cell per pass, as in the
   // staged x kernel)
-  const int nchunk = (G.seg + 7 * NP + CH - 1) / CH;
+  const int nchunk = (s1 - s0 + 7 * NP + CH - 1) / CH;
   constexpr int kLag = 3 * NP;                 // final b_t at t - kLag, final b_D at face t - kLag + 1
 
   MagPipe<LIM> pA, pO;      // first pass
@@ -706,7 +706,8 @@ template <int LIM>
 cudaError_t launch_mag_t(int axis, const MagArgs& a, cudaStream_t s) {
   const int A = (axis == 0) ? 1 : 0, O = (axis == 2) ? 1 : 2;
   dim3 block(32, kMagWarps + 2);
-  dim3 grid((a.box.n[A] + 31) / 32, (a.box.n[O] + kMagWarps - 1) / kMagWarps, a.box.n[axis] / a.seg);
+  dim3 grid((a.box.n[A] + 31) / 32, (a.box.n[O] + kMagWarps - 1) / kMagWarps,
+            (a.box.n[axis] + a.seg - 1) / a.seg);
   if (a.ens.items) grid = dim3(a.nblocks, 1, 1);  // one block per work item
   const bool small = a.box.n[axis] < 16;
   if (a.tile) {
