@@ -221,6 +221,7 @@ int fluid(mhd_ens_s* e, int d, bool rate, cudaStream_t s) {
   a.box.n[ka] = e->fluid[d].minext;  // selects the short-axis kernel if any box needs it
   a.gamma = (float)e->gamma;
   a.p_floor = e->p_floor;
+  a.e_floor = a.p_floor / (a.gamma - 1.f);
   a.tau = e->tau;
   a.rate = nullptr;
   a.seg = 1;

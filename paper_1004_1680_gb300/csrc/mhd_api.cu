@@ -451,6 +451,7 @@ int fluid(mhd_s* m, int d, bool rate) {
   a.box = *box;
   a.gamma = (float)m->gamma;
   a.p_floor = m->p_floor;
+  a.e_floor = a.p_floor / (a.gamma - 1.f);
   a.tau = &m->sc->tau;
   a.rate = rate ? &m->sc->rate[1 - m->rcur] : nullptr;
   a.seg = m->seg[d][0];

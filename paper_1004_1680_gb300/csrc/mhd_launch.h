@@ -129,6 +129,7 @@ struct FluidArgs {
   Box box;
   float gamma;
   float p_floor = 0.f; // optional floor on the gas pressure of the output (0: off)
+  float e_floor = 0.f; // its internal energy, p_floor / (gamma - 1)
   const float* tau;    // device scalar: step of this sweep
   unsigned* rate;      // fused CFL rate accumulator (float bits), or nullptr
   int seg;             // pencil segment length along the sweep axis

@@ -223,6 +223,7 @@ __device__ __forceinline__ void fluid_sweep_body(const FluidArgs& a, const Fluid
     pipe.c2 = __ldg(a.pencil_c + (long long)nA * nO + pc);
   }
   float bc2[3] = {0.f, 0.f, 0.f}, bc3[3] = {0.f, 0.f, 0.f};  // b_c at t-1, t-2 (RATE only)
+  float b2w1 = 0.f, b2w2 = 0.f, b2w3 = 0.f;  // |b|^2 at t-1, t-2, t-3 (FLOOR only: fewer registers than b_c)
   float rmax = 0.f;
   const bool rate_pencil = RATE && pa >= a.rate_lo[X::A] && pa < a.rate_hi[X::A] && pb >= a.rate_lo[X::O] &&
                            pb < a.rate_hi[X::O];
@@ -302,6 +303,8 @@ __device__ __forceinline__ void fluid_sweep_body(const FluidArgs& a, const Fluid
     // steady chunks store without a per-position test (1.135 -> 1.108 ms
     // at 512^3).
     auto positions = [&](const bool all) {
+      unsigned low = 0;  // FLOOR: the chunk's cells whose energy may be below the floor
+      float b2c[CH];
 #pragma unroll
       for (int j = 0; j < CH; j++) {
         float o[5], Uj[5], Bj[3];
@@ -336,7 +339,8 @@ __device__ __forceinline__ void fluid_sweep_body(const FluidArgs& a, const Fluid
         const int po = t - 3;  // position of the finished cell
         if (all || (active && po >= s0 && po < s1)) {
           const unsigned cell = ub + (unsigned)(po * sD);  // po is inside [s0, s1)
-          if (FLOOR) o[4] = floored_energy(o, bc3, gamma, a.p_floor);  // optional (b_c of this cell is bc3)
+          if (FLOOR && RATE) o[4] = floored_energy(o, b2w3, a.e_floor);  // (b2w3: |b|^2 of this cell)
+          if (FLOOR && !RATE && !above_floor(o, b2w3, a.e_floor)) low |= 1 << j;
           o_rho[cell] = o[0];
           o_md[cell] = o[1];
           o_m1[cell] = o[2];
@@ -351,12 +355,25 @@ __device__ __forceinline__ void fluid_sweep_body(const FluidArgs& a, const Fluid
             rmax = fmaxf(rmax, cell_rate(o[0], m, o[4], bg, gamma, G.box.ih));
           }
         }
-        if (RATE || FLOOR) {  // window of b_c: bc2 = b_c(t-1), bc3 = b_c(t-2) for the next step
+        if (FLOOR) {  // |b|^2 at t-1, t-2, t-3 for the next step
+          b2c[j] = b2w3;
+          b2w3 = b2w2;
+          b2w2 = b2w1;
+          b2w1 = square3(Bj);
+        }
+        if (RATE) {  // window of b_c: bc2 = b_c(t-1), bc3 = b_c(t-2) for the next step
           bc3[0] = bc2[0]; bc3[1] = bc2[1]; bc3[2] = bc2[2];
           bc2[0] = bprev0; bc2[1] = bprev1; bc2[2] = bprev2;
         }
       }
-  
+      if (FLOOR && !RATE && low) {
+        for (int j = 0; j < CH; j++) {
+          if (!(low >> j & 1)) continue;
+          const unsigned cell = ub + (unsigned)((p0 + j - 3) * sD);
+          const float o[5] = {o_rho[cell], o_md[cell], o_m1[cell], o_m2[cell], o_en[cell]};
+          o_en[cell] = floored_energy(o, b2c[j], a.e_floor);
+        }
+      }
     };
     if (TMA && full_tile && p0 >= s0 + 3 && p0 < s1)
       positions(true);

@@ -281,6 +281,7 @@ __global__ void __launch_bounds__(kRowMaxThreads, 2) fluid_row_kernel(const __gr
     const long long ro = (long long)y * nx + (long long)z * nx * ny + x0;
     const bool rate_row = RATE && y >= a.rate_lo[1] && y < a.rate_hi[1] && z >= a.rate_lo[2] && z < a.rate_hi[2];
     float o[kRowCells][5];
+    bool clear = true;  // FLOOR: every cell above the floor
     row_state(sb, nx, x0, U);
     auto finish = [&](int j, const V5& fl) {
       const V5 v = v5_fma(-c_full, v5_sub(F2[j], fl), U[j]);
@@ -289,14 +290,20 @@ __global__ void __launch_bounds__(kRowMaxThreads, 2) fluid_row_kernel(const __gr
       o[j][2] = v.p1.x;
       o[j][3] = v.p1.y;
       o[j][4] = v.e;
-      if (FLOOR) o[j][4] = floored_energy(o[j], B[j].v, gamma, a.p_floor);
-      if (RATE && rate_row && x0 + j >= a.rate_lo[0] && x0 + j < a.rate_hi[0])
-        rmax = fmaxf(rmax, cell_rate(o[j][0], &o[j][1], o[j][4], B[j].v, gamma, a.box.ih));
+      if (FLOOR) clear &= above_floor(o[j], square3(B[j].v), a.e_floor);
     };
 #pragma unroll
     for (int j = 1; j < kRowCells; j++) finish(j, F2[j - 1]);
     if (!wait_ok(smem_u32(&xbar[2]), it & 1)) break;
     finish(0, X.get(6, lm));  // F2(4l-1/2)
+    if (FLOOR && !clear)
+#pragma unroll
+      for (int j = 0; j < kRowCells; j++) o[j][4] = floored_energy(o[j], square3(B[j].v), a.e_floor);
+    if (RATE && rate_row)
+#pragma unroll
+      for (int j = 0; j < kRowCells; j++)
+        if (x0 + j >= a.rate_lo[0] && x0 + j < a.rate_hi[0])
+          rmax = fmaxf(rmax, cell_rate(o[j][0], &o[j][1], o[j][4], B[j].v, gamma, a.box.ih));
 #pragma unroll
     for (int q = 0; q < 5; q++)
       *reinterpret_cast<float4*>(a.out[q] + ro) = make_float4(o[0][q], o[1][q], o[2][q], o[3][q]);

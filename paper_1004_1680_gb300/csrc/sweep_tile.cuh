@@ -221,6 +221,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) fluid_tile_kernel(const __gri
     const bool rate_pencil =
         RATE && pa >= a.rate_lo[A] && pa < a.rate_hi[A] && pb >= a.rate_lo[O] && pb < a.rate_hi[O];
     float r[K][5];
+    bool clear = true;  // FLOOR: every cell above the floor
 #pragma unroll
     for (int j = 0; j < K; j++) {
       const V5 v = v5_fma(-c_full, v5_sub(F2[j], j ? F2[j ? j - 1 : 0] : Fm), U[j]);
@@ -229,15 +230,22 @@ __global__ void __launch_bounds__(kTileThreads, 2) fluid_tile_kernel(const __gri
       r[j][2] = v.p1.x;
       r[j][3] = v.p1.y;
       r[j][4] = v.e;
-      if (FLOOR) r[j][4] = floored_energy(r[j], B[j].v, gamma, a.p_floor);
-      const int p = p0 + j;
-      if (RATE && rate_pencil && p < pend && p >= a.rate_lo[D] && p < a.rate_hi[D]) {
-        float m[3], bg[3];
-        m[D] = r[j][1]; m[T1] = r[j][2]; m[T2] = r[j][3];
-        bg[D] = B[j].v[0]; bg[T1] = B[j].v[1]; bg[T2] = B[j].v[2];
-        rmax = fmaxf(rmax, cell_rate(r[j][0], m, r[j][4], bg, gamma, G.box.ih));
-      }
+      if (FLOOR) clear &= above_floor(r[j], square3(B[j].v), a.e_floor);
     }
+    if (FLOOR && !clear)
+#pragma unroll
+      for (int j = 0; j < K; j++) r[j][4] = floored_energy(r[j], square3(B[j].v), a.e_floor);
+    if (RATE && rate_pencil)
+#pragma unroll
+      for (int j = 0; j < K; j++) {
+        const int p = p0 + j;
+        if (p < pend && p >= a.rate_lo[D] && p < a.rate_hi[D]) {
+          float m[3], bg[3];
+          m[D] = r[j][1]; m[T1] = r[j][2]; m[T2] = r[j][3];
+          bg[D] = B[j].v[0]; bg[T1] = B[j].v[1]; bg[T2] = B[j].v[2];
+          rmax = fmaxf(rmax, cell_rate(r[j][0], m, r[j][4], bg, gamma, G.box.ih));
+        }
+      }
     if constexpr (D == 0) {
 #pragma unroll
       for (int q = 0; q < 5; q++) {
