@@ -393,8 +393,9 @@ int mhd_ens_diagnostics(mhd_ens_t *e, double *out);
 int mhd_ens_set_pressure_floor(mhd_ens_t *e, double p_floor);
 
 /* Tiling of the ensemble launches: x path (1 direct, 2 exchanged layout; see
- * mhd_set_xpath) and pencil segment divisor (1, 2 or 4: each pencil of a box
- * is marched by that many threads when its length allows). */
+ * mhd_set_xpath) and pencil segment divisor (2 or 4: each pencil of a box is
+ * marched by that many threads when its length allows; 1: the library chooses
+ * the segments, longer or shorter ones for the whole ensemble). */
 int mhd_ens_set_tuning(mhd_ens_t *e, int xpath, int segdiv);
 
 /* Pick the fastest tiling by timing two steps of each candidate on a copy of

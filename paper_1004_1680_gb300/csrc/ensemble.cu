@@ -12,9 +12,11 @@
 // The per-box arithmetic is exactly that of a single box run with the same
 // x path and segments, so an ensemble member is bitwise equal to the same box
 // run alone.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <mutex>
 #include <new>
@@ -119,37 +121,124 @@ int upload(WorkList* l, const std::vector<int4>& items, int minext) {
   return MHD_OK;
 }
 
-// Segment lengths and work lists for the current x path and divisor.
-int build_lists(mhd_ens_s* e) {
-  for (auto& b : e->boxes) {
-    for (int d = 0; d < 3; d++) {
-      int seg = b.n[d];
-      if (e->segdiv > 1 && b.n[d] % (4 * e->segdiv) == 0 && b.n[d] / e->segdiv >= 16)
-        seg = b.n[d] / e->segdiv;
-      b.seg[d] = seg;
+// Blocks per segment of a box in a sweep of kernel axis ka (n: extents as the
+// kernel sees them): fluid y and z kernel axes take runs of 32 W consecutive
+// pencils (the kernel's row-order mapping), the others tiles of 32 x W.
+struct Tiles {
+  int x, y;
+};
+Tiles sweep_tiles(int kind, int ka, const int n[3]) {
+  const int A = (ka == 0) ? 1 : 0, O = (ka == 2) ? 1 : 2, W = kind ? mhd::kMagWarps : 4;
+  if (kind == 0 && ka != 0) return {(n[A] * n[O] + 32 * W - 1) / (32 * W), 1};
+  return {(n[A] + 31) / 32, (n[O] + W - 1) / W};
+}
+
+// Nearly equal segments of a pencil of n cells, about `want` cells each
+// (multiples of 4: x chunks start 16-byte aligned).
+int even_segment(int n, int want) {
+  const int k = std::max(1, (n + want / 2) / want);
+  return std::min(n, ((n + k - 1) / k + 3) / 4 * 4);
+}
+
+// Segment length aimed at for one sweep of all boxes.  The blocks are launched
+// longest first; the length with the earliest end on the chip's places wins,
+// a stretch with b blocks per SM counting 0.6 + 0.4 (b - 1) / 3 per cell (fluid,
+// 4 places) or 0.8 + 0.2 (b - 1) (magnetic, 2 places), and `warm` cells of
+// warm-up per segment.  Whole pencils left most of the chip idle at the end of
+// a launch: a step of 32 boxes of 32 .. 96 cells a side took 1260 us with them,
+// 1120 with halves and 1084 with these; of 3 boxes 490, 293 and 234.
+int segment_target(const mhd_ens_s* e, int kind, int d, int layout, int sms) {
+  const int ka = kernel_axis(layout, d), resident = kind ? 2 : 4, warm = kind && d == 2 ? 14 : 7;
+  const long long slots = (long long)sms * resident;
+  int longest = 0;
+  for (auto& b : e->boxes) longest = std::max(longest, b.n[d]);
+  int best = longest;
+  double best_end = 0.0;
+  for (int want = longest; want >= 24; want -= std::max(4, want / 12)) {
+    std::map<int, long long, std::greater<int>> jobs;  // cells marched -> blocks
+    double work = 0.0;
+    for (auto& b : e->boxes) {
+      const int n[3] = {layout ? b.n[1] : b.n[0], layout ? b.n[0] : b.n[1], b.n[2]};
+      const Tiles t = sweep_tiles(kind, ka, n);
+      const int seg = even_segment(b.n[d], want), rest = b.n[d] % seg;
+      jobs[seg + warm] += (long long)t.x * t.y * (b.n[d] / seg);
+      if (rest) jobs[rest + warm] += (long long)t.x * t.y;
+      work += (double)t.x * t.y * (b.n[d] + warm * (b.n[d] / seg + (rest > 0)));
+    }
+    std::map<int, long long> running;  // cell at which they end -> blocks
+    long long active = 0;
+    int now = 0;
+    double end = 0.0;
+    if (work > 64.0 * longest * slots) {  // the end of the launch hardly counts
+      end = work / slots;
+    } else {
+      auto next = jobs.begin();
+      for (;;) {
+        while (next != jobs.end() && active < slots) {
+          const long long c = std::min(slots - active, next->second);
+          running[now + next->first] += c;
+          active += c;
+          if ((next->second -= c) == 0) ++next;
+        }
+        if (running.empty()) break;
+        const auto first = running.begin();
+        const double b = std::ceil((double)active / sms) - 1.0;
+        end += (first->first - now) * (kind ? 0.8 + 0.2 * b : 0.6 + 0.4 / 3.0 * b);
+        now = first->first;
+        active -= first->second;
+        running.erase(first);
+      }
+      end = std::max(end, work / slots);
+    }
+    if (best_end == 0.0 || end < best_end * 0.999) {
+      best = want;
+      best_end = end;
     }
   }
+  return best;
+}
+
+// Segment lengths and work lists for the current x path and divisor (1: the
+// lengths of segment_target; 2, 4: that many segments where they divide).
+int build_lists(mhd_ens_s* e) {
+  int dev = 0, sms = 0;
+  CKE(cudaGetDevice(&dev));
+  CKE(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  for (int kind = 0; kind < 2; kind++)
+    for (int d = 0; d < 3; d++) {
+      const int want = e->segdiv > 1 ? 0 : segment_target(e, kind, d, sweep_layout(e, d), sms);
+      for (auto& b : e->boxes) {
+        int seg = b.n[d];
+        if (e->segdiv == 1)
+          seg = even_segment(b.n[d], want);
+        else if (b.n[d] % (4 * e->segdiv) == 0 && b.n[d] / e->segdiv >= 16)
+          seg = b.n[d] / e->segdiv;
+        b.seg[kind][d] = seg;
+      }
+    }
   CKE(cudaMemcpy(e->boxes_d, e->boxes.data(), sizeof(mhd::EnsBox) * e->nbox, cudaMemcpyHostToDevice));
   for (int kind = 0; kind < 2; kind++) {
-    const int W = kind == 0 ? 4 : mhd::kMagWarps;  // rows per block: fluid, magnetic
     for (int d = 0; d < 3; d++) {
       const int L = sweep_layout(e, d), ka = kernel_axis(L, d);
-      const int A = (ka == 0) ? 1 : 0, O = (ka == 2) ? 1 : 2;
       std::vector<int4> items;
       int minext = 1 << 30;
       for (int bi = 0; bi < e->nbox; bi++) {
         const mhd::EnsBox& b = e->boxes[bi];
-        int n[3] = {L ? b.n[1] : b.n[0], L ? b.n[0] : b.n[1], b.n[2]};
+        const int n[3] = {L ? b.n[1] : b.n[0], L ? b.n[0] : b.n[1], b.n[2]};
         minext = std::min(minext, n[ka]);
-        // fluid y and z kernel axes: runs of 32 W consecutive pencils (the
-        // kernel's row-order mapping); otherwise tiles of 32 x W pencils
-        const bool runs = kind == 0 && ka != 0;
-        const int gx = runs ? (n[A] * n[O] + 32 * W - 1) / (32 * W) : (n[A] + 31) / 32;
-        const int gy = runs ? 1 : (n[O] + W - 1) / W, gz = n[ka] / b.seg[d];
+        const Tiles t = sweep_tiles(kind, ka, n);
+        const int gz = (n[ka] + b.seg[kind][d] - 1) / b.seg[kind][d];
         for (int z = 0; z < gz; z++)
-          for (int y = 0; y < gy; y++)
-            for (int x = 0; x < gx; x++) items.push_back(make_int4(bi, x, y, z));
+          for (int y = 0; y < t.y; y++)
+            for (int x = 0; x < t.x; x++) items.push_back(make_int4(bi, x, y, z));
       }
+      // the longest blocks first, otherwise in box order
+      auto length = [&](const int4& it) {
+        const mhd::EnsBox& b = e->boxes[it.x];
+        return std::min(b.seg[kind][d], b.n[d] - it.w * b.seg[kind][d]);
+      };
+      std::stable_sort(items.begin(), items.end(),
+                       [&](const int4& p, const int4& q) { return length(p) > length(q); });
       int rc = upload(kind == 0 ? &e->fluid[d] : &e->mag[d], items, minext);
       if (rc) return rc;
     }
@@ -170,13 +259,14 @@ int build_lists(mhd_ens_s* e) {
   return MHD_OK;
 }
 
-mhd::EnsArgs ens_args(const mhd_ens_s* e, const WorkList& l, int layout, int d, unsigned* rate) {
+mhd::EnsArgs ens_args(const mhd_ens_s* e, const WorkList& l, int layout, int kind, int d, unsigned* rate) {
   mhd::EnsArgs a;
   a.items = l.d;
   a.boxes = e->boxes_d;
   a.tau_arr = e->tau;
   a.rate_arr = rate;
   a.layout = layout;
+  a.kind = kind;
   a.phys_axis = d;
   return a;
 }
@@ -188,7 +278,7 @@ int exchange(mhd_ens_s* e, cudaStream_t s) {
     a.out[q] = e->spare[q];
   }
   a.n[0] = a.n[1] = a.n[2] = 32;
-  a.ens = ens_args(e, e->trans[e->layout], e->layout, 0, nullptr);
+  a.ens = ens_args(e, e->trans[e->layout], e->layout, 0, 0, nullptr);
   a.nblocks = e->trans[e->layout].n;
   CKE(mhd::launch_transpose01(a, s));
   static const int relabel[8] = {0, 2, 1, 3, 4, 6, 5, 7};
@@ -225,7 +315,7 @@ int fluid(mhd_ens_s* e, int d, bool rate, cudaStream_t s) {
   a.tau = e->tau;
   a.rate = nullptr;
   a.seg = 1;
-  a.ens = ens_args(e, e->fluid[d], e->layout, d, rate ? e->rate[1 - e->rcur] : nullptr);
+  a.ens = ens_args(e, e->fluid[d], e->layout, 0, d, rate ? e->rate[1 - e->rcur] : nullptr);
   a.nblocks = e->fluid[d].n;
   CKE(mhd::launch_fluid(ka, rate, a, s));
   for (int q = 0; q < 5; q++) std::swap(e->cur[q], e->spare[q]);
@@ -245,7 +335,7 @@ int magnetic(mhd_ens_s* e, int d, cudaStream_t s, int passes = 1) {
   a.box.n[ka] = e->mag[d].minext;
   a.tau = e->tau;
   a.seg = 1;
-  a.ens = ens_args(e, e->mag[d], e->layout, d, nullptr);
+  a.ens = ens_args(e, e->mag[d], e->layout, 1, d, nullptr);
   a.nblocks = e->mag[d].n;
   a.passes = passes;
   CKE(mhd::launch_mag(ka, a, s));

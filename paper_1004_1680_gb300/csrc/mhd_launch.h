@@ -18,12 +18,13 @@ constexpr int kMagWarps = 8;  // interior rows of a magnetic-sweep tile
 __host__ __device__ constexpr int mag_row_tile(int nx) { return nx <= 512 ? 4 : 2; }
 
 // One box of an ensemble: physical extents, first cell in the concatenated
-// field arrays (a multiple of 32), and pencil segment length per axis.
+// field arrays (a multiple of 32), and pencil segment length per axis of its
+// fluid and magnetic sweeps (the last segment of a pencil may be shorter).
 struct EnsBox {
   int n[3];
   int offset;
-  int seg[3];
-  int pad;
+  int seg[2][3];
+  int pad[2];
 };
 
 // Ensemble launches (items != nullptr): block b of the grid works on
@@ -36,6 +37,7 @@ struct EnsArgs {
   const float* tau_arr = nullptr;
   unsigned* rate_arr = nullptr;
   int layout = 0;
+  int kind = 0;  // 0: fluid sweep, 1: magnetic
   int phys_axis = 0;
 };
 
@@ -257,7 +259,7 @@ __device__ __forceinline__ BlockGeom block_geom(const EnsArgs& e, const Box& box
     g.bx = it.y;
     g.by = it.z;
     g.bz = it.w;
-    g.seg = eb.seg[e.phys_axis];
+    g.seg = eb.seg[e.kind][e.phys_axis];
     g.off = eb.offset;
     g.tau = tau ? e.tau_arr[it.x] : 0.f;
     g.rate = e.rate_arr ? e.rate_arr + it.x : nullptr;

@@ -53,3 +53,29 @@ def test_ragged_segments_match_whole_pencils(mhd, dims, cfg):
         b.close()
     assert torch.isfinite(out[0]).all()
     assert torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("xpath", [1, 2])
+def test_ragged_ensemble_segments_match_single_boxes(mhd, xpath):
+    """Members of very different extents: one segment length for all leaves
+    whole pencils, equal segments and short last ones."""
+    dims = [(36, 20, 44), (84, 40, 36), (8, 4, 12), (48, 52, 100), (120, 12, 20), (32, 32, 31)]
+    states = [to_gpu(ic.turbulence(d, seed=90 + i, dtype=torch.float64, kmin=1.0, kmax=2.0, mach=0.6))
+              for i, d in enumerate(dims)]
+    ens = mhd.Ensemble(dims, gamma=G)
+    ens.set_tuning(xpath, 1)
+    ens.set_pressure_floor(1e-3)
+    for i, x in enumerate(states):
+        ens.set_state(i, x)
+    ens.run(2, 0.7)
+    for i, (d, x) in enumerate(zip(dims, states)):
+        b = mhd.Box(*d, gamma=G)
+        b.set_tma(False)
+        b.set_xpath(xpath)
+        b.set_segments(*(n if n % 4 == 0 else 0 for n in d))
+        b.set_pressure_floor(1e-3)
+        b.set_state(x)
+        b.run(2, 0.7)
+        assert torch.equal(ens.get_state(i), b.get_state()), d
+        b.close()
+    ens.close()
