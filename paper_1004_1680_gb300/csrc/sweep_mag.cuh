@@ -309,8 +309,6 @@ __device__ __forceinline__ void mag_pipe_role(const MagArgs& a, const BlockGeom&
   constexpr bool kEarly = D == 1;  // next chunk's loads before the current chunk's arithmetic
   using X = MagAxes<D>;
   constexpr int CH = kMagCH;
-  constexpr bool kA_ = ROLE != kRoleHaloRow;  // advects b_A (flux along A)
-  constexpr bool kO_ = ROLE != kRoleHaloCol;  // advects b_O (flux along O)
   const int lane = threadIdx.x, w = threadIdx.y;
   const int nA = G.box.n[X::A], nO = G.box.n[X::O], nD = G.box.n[D];
   const int a0 = G.bx * 32, b0 = G.by * kMagWarps;
@@ -408,13 +406,14 @@ __device__ __forceinline__ void mag_pipe_role(const MagArgs& a, const BlockGeom&
   const int nchunk = (s1 - s0 + 7 * NP + CH - 1) / CH;
   constexpr int kLag = 3 * NP;                 // final b_t at t - kLag, final b_D at face t - kLag + 1
 
-  MagPipe<LIM> pA, pO;      // first pass
-  MagPipe<LIM> qA, qO;      // second pass (NP == 2)
-  pA.init();
-  pO.init();
-  qA.init();
-  qO.init();
-  float uA1 = 0.f, uA2 = 0.f, uA3 = 0.f, uO1 = 0.f, uO2 = 0.f, uO3 = 0.f;  // face velocities at t-1..t-3
+  // first and second pass (NP == 2) of an interior pencil and of a halo pencil
+  MagPipe2<LIM, TMA && NP == 1> p2_, q2_;
+  MagPipe<LIM> p1_, q1_;
+  p2_.init();
+  q2_.init();
+  p1_.init();
+  q1_.init();
+  float2 u1 = f2(0.f), u2 = f2(0.f), u3 = f2(0.f);  // face velocities at t-1 .. t-3 (halo pencils: .x)
   float bD1 = 0.f, bD2 = 0.f;  // raw b_D at t-1, t-2
   float bP1 = 0.f, bP2 = 0.f, bP3 = 0.f;  // b_D after the first pass at faces t-3, t-4, t-5
 
@@ -541,45 +540,68 @@ __device__ __forceinline__ void mag_pipe_role(const MagArgs& a, const BlockGeom&
 #pragma unroll
       for (int j = 0; j < CH; j++) {
         const float vj = cv[j];
-        float nA_new = 0.f, nO_new = 0.f;
-        if constexpr (kA_) {  // flux along A: interior and halo column
-          const float uA = __fmul_rn(0.5f, __fadd_rn(vj, sh.v[buf][j][vAr][vAc]));
-          const float fa = pA.step(cq2[j], uA, c_half, c_full, nA_new);
-          if (wr_col) sh.fA[0][buf][j][row][col] = fa;
-          if constexpr (NP == 2) {
-            float q2;
-            const float fa2 = qA.step(nA_new, uA3, c_half, c_full, q2);
-            if (wr_col) sh.fA[1][buf][j][row][col] = fa2;
-            nA_new = q2;
-            uA3 = uA2;
-            uA2 = uA1;
-            uA1 = uA;
+        if constexpr (ROLE == kRoleInterior) {  // both fluxes
+          float2 qn;
+          if constexpr (TMA) {  // both fluxes at once
+            const float2 u = decltype(p2_)::mean(vj, sh.v[buf][j][vAr][vAc], sh.v[buf][j][vOr][vOc]);
+            float2 f = p2_.step(make_float2(cq2[j], cq3[j]), u, c_half, c_full, qn);
+            if (wr_col) sh.fA[0][buf][j][row][col] = f.x;
+            if (wr_row) sh.fO[0][buf][j][row][col] = f.y;
+            if constexpr (NP == 2) {
+              f = q2_.step(qn, u3, c_half, c_full, qn);
+              if (wr_col) sh.fA[1][buf][j][row][col] = f.x;
+              if (wr_row) sh.fO[1][buf][j][row][col] = f.y;
+              u3 = u2;
+              u2 = u1;
+              u1 = u;
+            }
+          } else {  // one after the other: fewer live registers (200^3, fused pair: 134 us against 158)
+            const float uA = face_mean(vj, sh.v[buf][j][vAr][vAc]);
+            float f = p2_.A.step(cq2[j], uA, c_half, c_full, qn.x);
+            if (wr_col) sh.fA[0][buf][j][row][col] = f;
+            if constexpr (NP == 2) {
+              f = q2_.A.step(qn.x, u3.x, c_half, c_full, qn.x);
+              if (wr_col) sh.fA[1][buf][j][row][col] = f;
+              u3.x = u2.x;
+              u2.x = u1.x;
+              u1.x = uA;
+            }
+            const float uO = face_mean(vj, sh.v[buf][j][vOr][vOc]);
+            f = p2_.O.step(cq3[j], uO, c_half, c_full, qn.y);
+            if (wr_row) sh.fO[0][buf][j][row][col] = f;
+            if constexpr (NP == 2) {
+              f = q2_.O.step(qn.y, u3.y, c_half, c_full, qn.y);
+              if (wr_row) sh.fO[1][buf][j][row][col] = f;
+              u3.y = u2.y;
+              u2.y = u1.y;
+              u1.y = uO;
+            }
           }
-        }
-        if constexpr (kO_) {  // flux along O: interior and halo row
-          const float qin = (ROLE == kRoleInterior) ? cq3[j] : cq2[j];
-          const float uO = __fmul_rn(0.5f, __fadd_rn(vj, sh.v[buf][j][vOr][vOc]));
-          const float fo = pO.step(qin, uO, c_half, c_full, nO_new);
-          if (wr_row) sh.fO[0][buf][j][row][col] = fo;
-          if constexpr (NP == 2) {
-            float q2;
-            const float fo2 = qO.step(nO_new, uO3, c_half, c_full, q2);
-            if (wr_row) sh.fO[1][buf][j][row][col] = fo2;
-            nO_new = q2;
-            uO3 = uO2;
-            uO2 = uO1;
-            uO1 = uO;
-          }
-        }
-        if constexpr (ROLE == kRoleInterior) {
           bDold[j] = bD2;  // b_D at position t-2, the face of edge t-5/2
           bD2 = bD1;
           bD1 = cq4[j];
           const int po = p0 + j - kLag;
           if (all || (interior && po >= s0 && po < s1)) {
             const unsigned cell = ib + (unsigned)(po * sD);  // po is inside [s0, s1)
-            o_bA[cell] = nA_new;
-            o_bO[cell] = nO_new;
+            o_bA[cell] = qn.x;
+            o_bO[cell] = qn.y;
+          }
+        } else {  // halo column: the flux along A; halo row: along O
+          constexpr bool kCol = ROLE == kRoleHaloCol;
+          const bool wr = kCol ? wr_col : wr_row;
+          auto put = [&](int pass, float f) {
+            if (!wr) return;
+            if constexpr (kCol) sh.fA[pass][buf][j][row][col] = f;
+            else sh.fO[pass][buf][j][row][col] = f;
+          };
+          const float u = __fmul_rn(0.5f, __fadd_rn(vj, kCol ? sh.v[buf][j][vAr][vAc] : sh.v[buf][j][vOr][vOc]));
+          float qn;
+          put(0, p1_.step(cq2[j], u, c_half, c_full, qn));
+          if constexpr (NP == 2) {
+            put(1, q1_.step(qn, u3.x, c_half, c_full, qn));
+            u3.x = u2.x;
+            u2.x = u1.x;
+            u1.x = u;
           }
         }
       }
