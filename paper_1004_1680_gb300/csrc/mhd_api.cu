@@ -245,12 +245,14 @@ double march_us(const mhd_s* m, int d, bool mag, int passes) {
 double tile_us(const mhd_s* m, bool mag) { return (mag ? 19e-6 : 21e-6) * (double)m->N; }
 
 // Tile sweep or not, along axis d of a box in the plain layout: 0, or the tile
-// argument of FluidArgs / MagArgs.  Along y and z by the estimates above.
-// Along x the row sweeps win wherever they take the fluid (128^3: 31 us
-// against 36), and the magnetic one for large boxes (128^3: 49 us rows, 31 us
-// tile; 256^3: 129 and 196; 512 x 64 x 64: 25 and 31; 512 x 8 x 8: 25 and 8);
-// every other box takes the tile sweep (496^3: 6.1 ms of x sweeps per step against 6.7 ms
-// with transposes and marching).
+// argument of FluidArgs / MagArgs (-1: the magnetic row sweep).  Along y and z by the estimates above.
+// Along x the fluid row sweep wins wherever rows are whole warps of threads
+// (128^3: 31 us against 36; rows with idle lanes lose: 160^3 96 against 64).  The
+// magnetic row sweep (-1) takes any row of up to 1024 cells, by its estimate
+// against 15 ps per cell of the tile sweep (tile and rows in us: 96^3 17 and 19,
+// 112^3 26 and 21, 128^3 31 and 22, 200^3 112 and 78, 236 x 150 x 98 53 and 38,
+// 256^3 196 and 121, 320^3 405 and 338, 420 x 300 x 200 322 and 216, 512 x 8 x 8
+// 8 and 25).
 int tile_choice(const mhd_s* m, int d, bool mag, int passes) {
   if (!m->tma || m->fast == 2 || m->xpath == 3 || m->layout || m->seg_set[d]) return 0;
   // magnetic tiles of 8 x 2 pencils (128 threads) where there are few (32^3: 44 us
@@ -263,8 +265,8 @@ int tile_choice(const mhd_s* m, int d, bool mag, int passes) {
   if (d == 0) {
     const bool rows = m->n[0] % 128 == 0 && m->n[0] <= 1024;
     if (!mag) return rows ? 0 : 128;
-    const bool mag_rows = rows && m->n[1] % mhd::mag_row_tile(m->n[0]) == 0 && m->n[2] >= 2;
-    return mag_rows && m->N > (m->n[0] > 256 ? 1000000 : 4200000) ? 0 : shape;
+    const bool fits = m->n[0] <= 1024 && m->n[2] >= 2;
+    return fits && mhd::mag_rows_us(m->n, m->sms > 0 ? m->sms : 152) < 15e-6 * (double)m->N ? -1 : shape;
   }
   if (mag && passes == 2 && m->n[d] > mhd::kMTileWhole) return 0;
   if (tile_us(m, mag) * (passes == 2 ? 1.3 : 1.0) >= march_us(m, d, mag, passes)) return 0;

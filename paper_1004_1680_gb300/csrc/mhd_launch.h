@@ -16,6 +16,8 @@ constexpr int kMagWarps = 8;  // interior rows of a magnetic-sweep tile
 // groups of nx/4 threads, 640 threads), 2 for 1024 cells (3 groups of 256
 // threads, 768).
 __host__ __device__ constexpr int mag_row_tile(int nx) { return nx <= 512 ? 4 : 2; }
+// Estimated microseconds of the magnetic row sweep of a box (sweep_mag.cu).
+double mag_rows_us(const int n[3], int sms);
 
 // One box of an ensemble: physical extents, first cell in the concatenated
 // field arrays (a multiple of 32), and pencil segment length per axis of its

@@ -732,7 +732,11 @@ cudaError_t launch_mag_t(int axis, const MagArgs& a, cudaStream_t s) {
             (a.box.n[axis] + a.seg - 1) / a.seg);
   if (a.ens.items) grid = dim3(a.nblocks, 1, 1);  // one block per work item
   const bool small = a.box.n[axis] < 16;
-  if (a.tile) {
+  if (a.tile < 0 && axis == 0 && mag_rows_possible(a)) {
+    if (a.tma_used && mag_rows_qualify(a)) *a.tma_used = 1;
+    return launch_mag_rows<LIM>(a, s);
+  }
+  if (a.tile > 0) {
     if (a.tma_used && (mag_chunks_qualify(axis, a) || (axis == 0 && mag_rows_qualify(a)))) *a.tma_used = 1;
     return launch_mag_tile<LIM>(axis, a, s);
   }
