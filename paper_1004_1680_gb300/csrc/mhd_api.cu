@@ -410,13 +410,15 @@ bool any_bc(const mhd_s* m) { return m->bc[0] || m->bc[1] || m->bc[2]; }
 // Refill the ghost layers of the non-periodic axes in the current layout:
 // physical axis a is kernel axis k there, with its normal momentum and face
 // field in slots 1 + k and 5 + k (the exchanges relabel the slots).
-int fill_ghosts(mhd_s* m) {
+// `parts`: the fields written since the last fill (a fluid sweep writes rho, m and
+// e, a magnetic one b; filling the others again would store what they hold).
+int fill_ghosts(mhd_s* m, int parts = mhd::kGhostAll) {
   if (!any_bc(m)) return MHD_OK;
   const mhd::Box& b = m->layout == 2 ? m->zbox : (m->layout ? m->tbox : m->box);
   int mode[3];
   for (int a = 0; a < 3; a++) mode[kernel_axis_of(m, a)] = m->bc[a];
   return traced(m, MHD_K_CONTROL, [&] {
-    CK(mhd::launch_ghost_fill(m->cur, b, mode, m->stream));
+    CK(mhd::launch_ghost_fill(m->cur, b, mode, parts, m->stream));
     return MHD_OK;
   });
 }
@@ -439,12 +441,12 @@ int state_rate(mhd_s* m, unsigned* rate, const float* const from[8] = nullptr) {
   });
 }
 
-int fluid(mhd_s* m, int d, bool rate) {
+int fluid(mhd_s* m, int d, bool rate, int stale = mhd::kGhostAll) {
   const mhd::Box* box;
   int ka;
   int rc = sweep_frame(m, d, &box, &ka);
   if (rc) return rc;
-  if ((rc = fill_ghosts(m))) return rc;
+  if ((rc = fill_ghosts(m, stale))) return rc;
   mhd::FluidArgs a;
   for (int q = 0; q < 8; q++) {
     a.in[q] = m->cur[q];
@@ -486,12 +488,12 @@ int fluid(mhd_s* m, int d, bool rate) {
 
 // passes = 2: two magnetic sweeps along d with the same step in one launch
 // (bitwise equal to two launches; kernel axis 2 only, the caller checks).
-int magnetic(mhd_s* m, int d, int passes = 1) {
+int magnetic(mhd_s* m, int d, int passes = 1, int stale = mhd::kGhostAll) {
   const mhd::Box* box;
   int ka;
   int rc = sweep_frame(m, d, &box, &ka);
   if (rc) return rc;
-  if ((rc = fill_ghosts(m))) return rc;
+  if ((rc = fill_ghosts(m, stale))) return rc;
   mhd::MagArgs a;
   for (int q = 0; q < 8; q++) a.in[q] = m->cur[q];
   for (int q = 0; q < 3; q++) a.out[q] = m->spare[5 + q];
@@ -525,22 +527,23 @@ int magnetic(mhd_s* m, int d, int passes = 1) {
 // result), unless the z sweep runs along the contiguous axis (x path 3) or
 // ghost layers must be refilled between them.
 int full_step(mhd_s* m) {
+  constexpr int F = mhd::kGhostFluid, B = mhd::kGhostField;  // what the sweep before has written
   int rc;
   for (int d = 0; d < 2; d++) {
-    if ((rc = fluid(m, d, false))) return rc;
-    if ((rc = magnetic(m, d))) return rc;
+    if ((rc = fluid(m, d, false, d == 0 ? mhd::kGhostAll : B))) return rc;
+    if ((rc = magnetic(m, d, 1, F))) return rc;
   }
-  if ((rc = fluid(m, 2, false))) return rc;
+  if ((rc = fluid(m, 2, false, B))) return rc;
   if (m->fuse && m->xpath != 3 && !any_bc(m) && fuse_z_pair(m)) {
-    if ((rc = magnetic(m, 2, 2))) return rc;
+    if ((rc = magnetic(m, 2, 2, F))) return rc;
   } else {
-    if ((rc = magnetic(m, 2))) return rc;
-    if ((rc = magnetic(m, 2))) return rc;
+    if ((rc = magnetic(m, 2, 1, F))) return rc;
+    if ((rc = magnetic(m, 2, 1, B))) return rc;
   }
-  if ((rc = fluid(m, 2, false))) return rc;
+  if ((rc = fluid(m, 2, false, B))) return rc;
   for (int d = 1; d >= 0; d--) {
-    if ((rc = magnetic(m, d))) return rc;
-    if ((rc = fluid(m, d, d == 0))) return rc;
+    if ((rc = magnetic(m, d, 1, F))) return rc;
+    if ((rc = fluid(m, d, d == 0, B))) return rc;
   }
   m->rcur ^= 1;
   return MHD_OK;

@@ -198,13 +198,15 @@ struct MagArgs {
 // in `box`: mode per kernel axis k (0 periodic, 1 outflow, 2 reflecting), whose
 // normal momentum and face field are f[1 + k] and f[5 + k].
 constexpr int kGhost = 4;
+enum { kGhostFluid = 1, kGhostField = 2, kGhostAll = 3 };  // rho, m, e; b
 struct GhostArgs {
   float* f[8];
+  int parts;  // the fields to fill
   int n[3], mode[3];
   long long stride[3];
-  long long first[4];  // elements of the axes' ghost layers, accumulated
+  long long first[4];  // elements (or groups of them) of the axes' ghost layers, accumulated
 };
-cudaError_t launch_ghost_fill(float* const f[8], const Box& box, const int mode[3], cudaStream_t s);
+cudaError_t launch_ghost_fill(float* const f[8], const Box& box, const int mode[3], int parts, cudaStream_t s);
 
 struct TransposeArgs {
   const float* in[8];
