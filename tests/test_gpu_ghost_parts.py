@@ -44,7 +44,7 @@ def mapped(u, modes):
 
 @pytest.mark.parametrize("modes", [("periodic", "outflow", "reflecting"), ("reflecting", "outflow", "periodic"),
                                    ("outflow", "reflecting", "outflow"), ("reflecting", "periodic", "periodic")])
-@pytest.mark.parametrize("dims", [(20, 17, 24), (36, 16, 13)])
+@pytest.mark.parametrize("dims", [(20, 17, 24), (36, 16, 13), (12, 12, 16), (72, 70, 66)])
 def test_fill_and_step(mhd, modes, dims):
     x = to_gpu(ic.turbulence(dims, seed=3, dtype=torch.float64, kmin=1.0, kmax=2.0, mach=0.6))
     boxes = [mhd.Box(*dims, gamma=G) for _ in range(2)]
