@@ -107,6 +107,13 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
          ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(hi)) << 16);
 }
 
+// Programmatic dependent launch of kernels that take tensor memory: a block may
+// become resident while the kernel before it drains, but allocates only after
+// that kernel has completed, and lets its own dependent launch only once every
+// block has its columns: two kernels never compete for them.
+__device__ __forceinline__ void wait_before_tmem() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void launch_after_tmem() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
@@ -202,6 +209,7 @@ __global__ void __launch_bounds__(256, 1) conv3d_tc_kernel(ConvArgs a) {
   uint64_t* wfull = ofree + kRing;  // the weight image has landed
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(wfull + 1);
   const uint32_t tmem_cols = (uint32_t)(NACC * kRing * npad);  // 128 .. 512, a power of two
+  wait_before_tmem();
 
   const int nx = a.n[0], ny = a.n[1], nz = a.n[2];
   const int tiles_x = nx / kTX, tiles_y = ny / TY;
@@ -269,6 +277,7 @@ __global__ void __launch_bounds__(256, 1) conv3d_tc_kernel(ConvArgs a) {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  launch_after_tmem();
   const uint32_t tmem = *tmem_slot;
 
   bool ok = true;
@@ -654,6 +663,7 @@ __global__ void __launch_bounds__(8 * TY + 32, 1) conv_wgrad_tc_kernel(WgradArgs
   uint64_t* empty = full + NS;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(empty + NS);
   uint8_t* stages = smem + W::BASE;
+  wait_before_tmem();
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_slot)),
@@ -671,6 +681,7 @@ __global__ void __launch_bounds__(8 * TY + 32, 1) conv_wgrad_tc_kernel(WgradArgs
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  launch_after_tmem();
   const uint32_t tmem = *tmem_slot;
 
   const int nx = a.n[0], ny = a.n[1];
@@ -920,13 +931,9 @@ cudaError_t launch_wgrad_tc(const __nv_bfloat16* x, const __nv_bfloat16* gy, con
   a.err = err;
   const size_t smem = wgrad_smem_bytes<TY>();
   constexpr int threads = WgradTile<TY>::NTHR;
-  if (cout == 32)
-    cin == 32 ? conv_wgrad_tc_kernel<TY, true, true><<<grid, threads, smem, s>>>(a)
-              : conv_wgrad_tc_kernel<TY, true, false><<<grid, threads, smem, s>>>(a);
-  else
-    cin == 32 ? conv_wgrad_tc_kernel<TY, false, true><<<grid, threads, smem, s>>>(a)
-              : conv_wgrad_tc_kernel<TY, false, false><<<grid, threads, smem, s>>>(a);
-  return cudaGetLastError();
+  auto* kernel = cout == 32 ? (cin == 32 ? conv_wgrad_tc_kernel<TY, true, true> : conv_wgrad_tc_kernel<TY, true, false>)
+                            : (cin == 32 ? conv_wgrad_tc_kernel<TY, false, true> : conv_wgrad_tc_kernel<TY, false, false>);
+  return launch_after(true, kernel, dim3(grid), dim3(threads), smem, s, a);
 }
 }  // namespace
 
@@ -1038,8 +1045,7 @@ cudaError_t launch_variant(const ConvArgs& a, cudaStream_t s) {
   }
   const long long tiles = (long long)(a.n[0] / kTX) * (a.n[1] / TY) * a.n[2];
   const unsigned grid = (unsigned)(tiles < cap ? tiles : cap);
-  conv3d_tc_kernel<G, TY><<<grid, 256, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_after(true, conv3d_tc_kernel<G, TY>, dim3(grid), dim3(256), smem, s, a);
 }
 }  // namespace
 

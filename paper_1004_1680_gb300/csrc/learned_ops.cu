@@ -163,6 +163,7 @@ __device__ __forceinline__ void load_cell(const float* __restrict__ y, int c, fl
 }
 
 __global__ void normalize_kernel(CP8 s, int N, F8 mu, F8 isig, __nv_bfloat16* x, bool vec) {
+  wait_for_previous();
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < N; c += gridDim.x * blockDim.x) {
     float v[8];
 #pragma unroll
@@ -223,6 +224,7 @@ __device__ __forceinline__ void block_totals(FWin2 (&w)[NP], int n, double* sums
 // Box totals of d_q = s_q y_q (q < 5), for the mean removal.
 __global__ void __launch_bounds__(kSumThreads) project_sums_kernel(const float* __restrict__ y, int N, F8 sc,
                                                                    double* sums, bool vec) {
+  wait_for_previous();
   FWin2 w[3];
   for (int k = 0; k < 3; k++) w[k].h = w[k].l = w[k].t = f2(0.f);
   for (int c = blockIdx.x * kSumThreads + threadIdx.x; c < N; c += gridDim.x * kSumThreads) {
@@ -248,6 +250,7 @@ __global__ void __launch_bounds__(kSumThreads) project_sums_kernel(const float* 
 // took 28 us on a 64^3 grid).
 __global__ void __launch_bounds__(256) project_kernel(const float* __restrict__ y, int nx, int ny, int nz, F8 sc,
                                                       P8 d, const double* __restrict__ sums, bool vec) {
+  wait_for_previous();
   __shared__ float mean[5];
   const int N = nx * ny * nz;
   if (threadIdx.x < 5) mean[threadIdx.x] = (float)(sums[threadIdx.x] / N);
@@ -288,6 +291,7 @@ struct LossWeights {
   double w2[8];
 };
 __global__ void __launch_bounds__(kSumThreads) loss_kernel(CP8 d, CP8 t, int N, LossWeights w, double* loss, P8 g) {
+  wait_for_previous();
   __shared__ double tot[8];
   if (threadIdx.x < 8) tot[threadIdx.x] = 0.0;
   FWin2 s[4];
@@ -333,6 +337,7 @@ __global__ void __launch_bounds__(kSumThreads) loss_kernel(CP8 d, CP8 t, int N, 
 }
 
 __global__ void __launch_bounds__(kSumThreads) grad_sums_kernel(CP8 g, int N, double* sums) {
+  wait_for_previous();
   FWin2 w[3];
   for (int k = 0; k < 3; k++) w[k].h = w[k].l = w[k].t = f2(0.f);
   for (int c = blockIdx.x * kSumThreads + threadIdx.x; c < N; c += gridDim.x * kSumThreads) {
@@ -352,6 +357,7 @@ __global__ void __launch_bounds__(kSumThreads) grad_sums_kernel(CP8 g, int N, do
 __global__ void __launch_bounds__(256) project_backward_kernel(CP8 g, int nx, int ny, int nz, F8 sc,
                                                                const double* __restrict__ sums, __nv_bfloat16* gy,
                                                                bool vec) {
+  wait_for_previous();
   __shared__ float mean[5];
   const int N = nx * ny * nz;
   if (threadIdx.x < 5) mean[threadIdx.x] = (float)(sums[threadIdx.x] / N);
@@ -381,6 +387,7 @@ __global__ void __launch_bounds__(256) project_backward_kernel(CP8 g, int nx, in
 // magnetic energy), e is raised to that bound.  The faces are read
 // uncorrected and corrected on the fly; pass 2 writes them.
 __global__ void __launch_bounds__(256) add_cells_kernel(P8 s, CP8 d, int nx, int ny, int nz, int* nclip) {
+  wait_for_previous_in_place();
   const int N = nx * ny * nz;
   int clipped = 0;
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < N; c += gridDim.x * blockDim.x) {
@@ -430,6 +437,7 @@ __global__ void __launch_bounds__(256) add_cells_kernel(P8 s, CP8 d, int nx, int
 
 // pass 2: faces b += d_b (divergence-free, never scaled)
 __global__ void add_field_kernel(P8 s, CP8 d, int N) {
+  wait_for_previous_in_place();
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < N; c += gridDim.x * blockDim.x)
     for (int q = 5; q < 8; q++) s.p[q][c] += d.p[q][c];
 }
@@ -518,8 +526,8 @@ int mhd_cnn_normalize(int nx, int ny, int nz, const float* const s[8], const flo
                       void* x_bf16, void* stream) {
   if (bad_ptrs(s) || !mu || !inv_sigma || !x_bf16) return set_error(MHD_E_ARG, "mhd_cnn_normalize", "null argument");
   const int N = nx * ny * nz;
-  normalize_kernel<<<blocks(N), 256, 0, (cudaStream_t)stream>>>(cp8(s), N, f8(mu, 8), f8(inv_sigma, 8),
-                                                                static_cast<__nv_bfloat16*>(x_bf16), vec16(x_bf16));
+  launch_after(true, normalize_kernel, dim3(blocks(N)), dim3(256), 0, (cudaStream_t)stream, cp8(s), N, f8(mu, 8),
+               f8(inv_sigma, 8), static_cast<__nv_bfloat16*>(x_bf16), vec16(x_bf16));
   return check_launch("mhd_cnn_normalize");
 }
 
@@ -530,8 +538,10 @@ int mhd_cnn_project(int nx, int ny, int nz, const float* y, const float scale[6]
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e = cudaMemsetAsync(sums, 0, sizeof(double) * 5, s);
   if (e != cudaSuccess) return set_error(MHD_E_CUDA, "mhd_cnn_project", cudaGetErrorString(e));
-  project_sums_kernel<<<sum_blocks(N), kSumThreads, 0, s>>>(y, N, f8(scale, 6), sums, vec16(y));
-  project_kernel<<<blocks(N), 256, 0, s>>>(y, nx, ny, nz, f8(scale, 6), p8(d), sums, vec16(y));
+  launch_after(true, project_sums_kernel, dim3(sum_blocks(N)), dim3(kSumThreads), 0, s, y, N, f8(scale, 6), sums,
+               vec16(y));
+  launch_after(true, project_kernel, dim3(blocks(N)), dim3(256), 0, s, y, nx, ny, nz, f8(scale, 6), p8(d),
+               static_cast<const double*>(sums), vec16(y));
   return check_launch("mhd_cnn_project");
 }
 
@@ -552,7 +562,7 @@ int mhd_cnn_loss(int nx, int ny, int nz, const float* const d[8], const float* c
     lw.scale[q] = (float)std::ldexp(1.0, ex);
     lw.w2[q] = std::ldexp((double)weight[q], -2 * ex);
   }
-  loss_kernel<<<sum_blocks(N), kSumThreads, 0, s>>>(cp8(d), cp8(t), N, lw, loss, p8(g));
+  launch_after(true, loss_kernel, dim3(sum_blocks(N)), dim3(kSumThreads), 0, s, cp8(d), cp8(t), N, lw, loss, p8(g));
   return check_launch("mhd_cnn_loss");
 }
 
@@ -564,9 +574,9 @@ int mhd_cnn_project_backward(int nx, int ny, int nz, const float* const g[8], co
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e = cudaMemsetAsync(sums, 0, sizeof(double) * 5, s);
   if (e != cudaSuccess) return set_error(MHD_E_CUDA, "mhd_cnn_project_backward", cudaGetErrorString(e));
-  grad_sums_kernel<<<sum_blocks(N), kSumThreads, 0, s>>>(cp8(g), N, sums);
-  project_backward_kernel<<<blocks(N), 256, 0, s>>>(cp8(g), nx, ny, nz, f8(scale, 6), sums,
-                                                    static_cast<__nv_bfloat16*>(gy_bf16), vec16(gy_bf16));
+  launch_after(true, grad_sums_kernel, dim3(sum_blocks(N)), dim3(kSumThreads), 0, s, cp8(g), N, sums);
+  launch_after(true, project_backward_kernel, dim3(blocks(N)), dim3(256), 0, s, cp8(g), nx, ny, nz, f8(scale, 6),
+               static_cast<const double*>(sums), static_cast<__nv_bfloat16*>(gy_bf16), vec16(gy_bf16));
   return check_launch("mhd_cnn_project_backward");
 }
 
@@ -577,8 +587,8 @@ int mhd_correct(int nx, int ny, int nz, float* const s[8], const float* const d[
     if (!s[q]) return set_error(MHD_E_ARG, "mhd_correct", "null field");
   const int N = nx * ny * nz;
   cudaStream_t st = (cudaStream_t)stream;
-  add_cells_kernel<<<blocks(N), 256, 0, st>>>(p8(s), cp8(d), nx, ny, nz, nclip);
-  add_field_kernel<<<blocks(N), 256, 0, st>>>(p8(s), cp8(d), N);
+  launch_after(true, add_cells_kernel, dim3(blocks(N)), dim3(256), 0, st, p8(s), cp8(d), nx, ny, nz, nclip);
+  launch_after(true, add_field_kernel, dim3(blocks(N)), dim3(256), 0, st, p8(s), cp8(d), N);
   return check_launch("mhd_correct");
 }
 
