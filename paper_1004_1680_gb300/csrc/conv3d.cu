@@ -129,6 +129,10 @@ struct ConvRing {
   static constexpr int SLOT = G * PLANE;              // one z plane of the halo
   static constexpr int NSLOT = 6;
   static constexpr int NACC = TY / 16;                // 128-row accumulators per tile
+  // warps: MMA issue (0, 1), copies (2, 3), epilogue (4 per accumulator), more copies (NXC)
+  static constexpr int NXC = G == 4 ? 0 : 2;
+  static constexpr int NTHR = 32 * (4 + 4 * NACC + NXC);
+  static constexpr int NL = 64 + 32 * NXC;
 };
 
 // The block's contiguous run of tiles, z fastest: tile t is column t / nz
@@ -160,8 +164,7 @@ __device__ __forceinline__ void load_plane(uint8_t* slot, const __nv_bfloat16* _
 }
 
 // G = cin / 8 channel groups, tiles of 8 x TY x 1 cells (TY / 16 accumulators
-// of 128 rows).  Persistent, 256 threads, warp-specialised, z taps packed
-// along N:
+// of 128 rows).  Persistent, warp-specialised, z taps packed along N:
 //  * The block's run of tiles (z fastest) splits into column segments: L
 //    consecutive tiles of one 8 x TY column at z = z0 .. z0 + L - 1.  A
 //    segment reads its input planes P = z0 - 1 .. z0 + L once each, in
@@ -177,10 +180,16 @@ __device__ __forceinline__ void load_plane(uint8_t* slot, const __nv_bfloat16* _
 //    The first K step that reaches an output plane (input plane = output
 //    plane + 1 - j3 with j3 = 0) writes its block with accumulate off.
 //  * Output plane z is complete once input plane z + 1 has been added.
-// Roles: warps 0 .. NACC-1, lane 0: the MMAs of accumulator q; warps 2, 3:
-// copy input planes into the ring (cp.async); warps 4..7: epilogue of the
-// completed output planes (tcgen05.ld, bias, ReLU or the ReLU mask, BF16 /
-// FP32 stores).  mbarriers: input slot full (copying threads) / empty (a
+// Roles: warps 0 .. NACC-1, lane 0: the MMAs of accumulator q; warps 2, 3 (and
+// the last two for 8 input channels): copy input planes into the ring (cp.async); warps 4 .. 4 NACC
+// + 3, four per accumulator: epilogue of the completed output planes
+// (tcgen05.ld, bias, ReLU or the ReLU mask, BF16 / FP32 stores).  A block has
+// its SM to itself, so what bounds it is the instruction stream of single
+// warps (tensor pipe 6 % busy): with two copying warps and four epilogue
+// warps for both accumulators 8 -> 32 channels at 64^3 took 20 us and now takes
+// 17.6, 32 -> 32 24 and 23.8, input gradients 24 .. 27.5 and 20.5 .. 24.  With 32
+// input channels the MMAs' reads of shared memory bound it (18 K steps of 7 KB per
+// plane and accumulator) and two more copying warps only got in the way: 24.9.  mbarriers: input slot full (copying threads) / empty (a
 // tcgen05.commit after the plane's MMAs); output slot full (a commit after
 // the output plane's last MMA) / free (the epilogue warps).  The weights
 // (packed once by conv_pack) are copied into shared memory once per block.
@@ -190,10 +199,10 @@ __device__ __forceinline__ void load_plane(uint8_t* slot, const __nv_bfloat16* _
 constexpr int kRing = 8;  // output-plane slots per accumulator
 
 template <int G, int TY>
-__global__ void __launch_bounds__(256, 1) conv3d_tc_kernel(ConvArgs a) {
+__global__ void __launch_bounds__(ConvRing<G, TY>::NTHR, 3 - ConvRing<G, TY>::NACC) conv3d_tc_kernel(ConvArgs a) {
   using R = ConvRing<G, TY>;
   constexpr int NS = R::NSLOT, NACC = R::NACC;
-  constexpr int NL = 64;  // copying threads
+  constexpr int NL = R::NL;  // copying threads
   extern __shared__ __align__(1024) uint8_t smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int npad = a.npad;
@@ -253,7 +262,7 @@ __global__ void __launch_bounds__(256, 1) conv3d_tc_kernel(ConvArgs a) {
   // zero pad cells; the packed weight image (once per block) comes in one
   // bulk asynchronous copy that the MMA threads wait for, while the copying
   // warps start on the input planes
-  for (int i = tid; i < NS * G * 4; i += 256)
+  for (int i = tid; i < NS * G * 4; i += R::NTHR)
     *reinterpret_cast<uint4*>(ring + (i / 4) * R::PLANE + (kHX * R::HY + i % 4) * 16) = make_uint4(0u, 0u, 0u, 0u);
   if (tid < 32) sBias[tid] = (a.bias && tid < a.cout) ? __ldg(a.bias + tid) : 0.f;
   if (warp == 0) {
@@ -269,7 +278,7 @@ __global__ void __launch_bounds__(256, 1) conv3d_tc_kernel(ConvArgs a) {
     }
     for (int i = 0; i < kRing; i++) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(ofull + i)), "r"(NACC) : "memory");
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;" ::"r"(smem_addr(ofree + i)) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(ofree + i)), "r"(4 * NACC) : "memory");
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -387,9 +396,9 @@ __global__ void __launch_bounds__(256, 1) conv3d_tc_kernel(ConvArgs a) {
       }
     }
     ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-  } else if (warp == 2 || warp == 3) {
+  } else if (warp == 2 || warp == 3 || warp >= 4 + 4 * NACC) {
     // ---- copies: input plane k goes to slot k % NS ---------------------------
-    const int lt = tid - 64;
+    const int lt = warp < 4 ? tid - 64 : tid - 32 * (4 + 4 * NACC) + 64;
     int k = 0;
     for (int i0 = 0; i0 < run.count && ok;) {
       int L = 1;
@@ -413,8 +422,8 @@ __global__ void __launch_bounds__(256, 1) conv3d_tc_kernel(ConvArgs a) {
       asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(full + (k - 1) % NS)) : "memory");
     }
   } else if (warp >= 4) {
-    // ---- epilogue: TMEM lanes 32 (warp - 4) + lane = GEMM row -------------
-    const int ew = warp - 4, row = 32 * ew + lane;
+    // ---- epilogue: TMEM lanes 32 (warp % 4) + lane = GEMM row of accumulator q
+    const int ew = warp & 3, row = 32 * ew + lane, q = (warp - 4) >> 2;
     const int co_n = a.cout;
     for (int g = 0; g < run.count; g++) {
       const int c = run.col(g), z0 = run.z(g);
@@ -422,23 +431,18 @@ __global__ void __launch_bounds__(256, 1) conv3d_tc_kernel(ConvArgs a) {
       // the saved activations that mask this plane, on their way while the plane
       // is computed (read after it, their latency was most of an input
       // gradient's excess over a forward layer: 32 -> 32 at 64^3 40 us, now 28)
-      uint4 mk[NACC][4];
+      const int cell = (x0 + (row & 7)) + nx * ((y0 + 16 * q + (row >> 3)) + ny * z0);
+      uint4 mk[4];
       if (a.mask) {
 #pragma unroll
-        for (int q = 0; q < NACC; q++) {
-          const int cell = (x0 + (row & 7)) + nx * ((y0 + 16 * q + (row >> 3)) + ny * z0);
-#pragma unroll
-          for (int c8 = 0; c8 < 4; c8++)
-            if (c8 < co_n / 8) mk[q][c8] = load16(a.mask + (size_t)cell * co_n + c8 * 8);
-        }
+        for (int c8 = 0; c8 < 4; c8++)
+          if (c8 < co_n / 8) mk[c8] = load16(a.mask + (size_t)cell * co_n + c8 * 8);
       }
       ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(ofull + g % kRing), (g / kRing) & 1));
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int slot = kRing - 1 - (g % kRing);
-#pragma unroll
-      for (int q = 0; q < NACC; q++) {
-        const int cell = (x0 + (row & 7)) + nx * ((y0 + 16 * q + (row >> 3)) + ny * z0);
+      {
         const uint32_t taddr = tmem + ((uint32_t)(32 * ew) << 16) + (uint32_t)((q * kRing + slot) * npad);
         float acc[32];
         uint32_t r[16];
@@ -466,7 +470,7 @@ __global__ void __launch_bounds__(256, 1) conv3d_tc_kernel(ConvArgs a) {
             if (a.relu) v[j] = fmaxf(v[j], 0.f);
           }
           if (a.mask) {
-            const uint32_t mw[4] = {mk[q][c8].x, mk[q][c8].y, mk[q][c8].z, mk[q][c8].w};
+            const uint32_t mw[4] = {mk[c8].x, mk[c8].y, mk[c8].z, mk[c8].w};
 #pragma unroll
             for (int j = 0; j < 8; j++) {
               const float m = __bfloat162float(__ushort_as_bfloat16((unsigned short)(mw[j / 2] >> (16 * (j & 1)))));
@@ -1029,7 +1033,8 @@ cudaError_t launch_variant(const ConvArgs& a, cudaStream_t s) {
       int sms = 0, per_sm = 0;
       e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
       if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, conv3d_tc_kernel<G, TY>, 256, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, conv3d_tc_kernel<G, TY>, ConvRing<G, TY>::NTHR,
+                                                          smem);
       if (e != cudaSuccess) return e;
       // resident blocks of an SM share its 512 TMEM columns
       const int tmem_cap = 512 / (ConvRing<G, TY>::NACC * kRing * a.npad);
@@ -1045,7 +1050,7 @@ cudaError_t launch_variant(const ConvArgs& a, cudaStream_t s) {
   }
   const long long tiles = (long long)(a.n[0] / kTX) * (a.n[1] / TY) * a.n[2];
   const unsigned grid = (unsigned)(tiles < cap ? tiles : cap);
-  return launch_after(true, conv3d_tc_kernel<G, TY>, dim3(grid), dim3(256), smem, s, a);
+  return launch_after(true, conv3d_tc_kernel<G, TY>, dim3(grid), dim3(ConvRing<G, TY>::NTHR), smem, s, a);
 }
 }  // namespace
 
