@@ -87,7 +87,7 @@ inline cudaError_t launch_after(bool early, void (*kernel)(P...), dim3 grid, dim
 // per block, segs segments of `out` positions.  `whole`: one segment that is
 // the whole periodic pencil; otherwise a segment has one thread of halo cells
 // at each end.  At least 8 pencils per block (32-byte sectors of neighbouring
-// pencils); used on the host for grids and work lists.
+// pencils); used on the host for grids.
 constexpr int kTileThreads = 256;
 constexpr int kTileCells = 4;  // cells per thread
 struct FluidTile {
@@ -195,7 +195,6 @@ struct MagArgs {
   unsigned* err = nullptr;  // set to 1 (atomicOr) if a staged chunk did not arrive within the bound
   int* tma_used = nullptr;  // host: set to 1 when the launch was TMA-staged
   int tile = 0;             // 1: tile sweep
-  int tile_out = 0;         // ensemble tile launches: largest `out` of any box (shared memory)
 };
 
 // Ghost layers of the non-periodic axes (boundary.cu) of the fields as stored

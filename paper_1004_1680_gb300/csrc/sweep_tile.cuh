@@ -1,7 +1,7 @@
 // Tile sweeps (Section II.B), FP32: sweeps along any axis in which a block
 // holds its pencils' whole stencil on chip and every thread updates 4
-// consecutive cells, for boxes (and ensembles of boxes) whose pencils are too
-// few or too short for the marching sweeps.
+// consecutive cells, for boxes whose pencils are too few or too short for the
+// marching sweeps.
 //
 // A marching thread carries its pencil through one position after another:
 // about 0.5 us per position of dependent arithmetic and loads, 39 positions
@@ -10,12 +10,15 @@
 // chain is that of 4 cells, with three exchanges between neighbouring threads
 // (fluid) or two passes over shared memory (magnetic).  Time per step, marching
 // -> tile: 32^3 302 -> 78 us, 64^3 308 -> 111, 96^3 432 -> 217, 236 x 150 x 98
-// (x sweeps without transposes) 1043 -> 800 us.  Small boxes are bound by the
+// (x sweeps without transposes) 1043 -> 800 us (all sweeps by tiles, before
+// the later changes; now 43, 91, 179 and 571).  Small boxes are bound by the
 // launches (about 2.5 us each) and one chain of loads, arithmetic and stores
 // (2 to 5 us); once the chip is full a fluid tile sweep runs at 17 (x) or 21 ps
-// per cell, twice the marching sweep's 8.3 ps on a 512^3 box, because each
-// block waits for its loads before it computes: the dispatch (tile_choice in
-// mhd_api.cu) leaves large boxes to the marching and row sweeps.
+// per cell, twice the marching sweep's 8.3 ps on a 512^3 box: its phases are
+// separated by barriers at 16 warps per SM (resident blocks that copy the next
+// tile's fields ahead only added instructions: 200^3 along x 141 -> 167 us).
+// The dispatch (tile_choice in mhd_api.cu) leaves large boxes to the marching
+// and row sweeps.
 //
 // The arithmetic of a cell is that of FluidPipe and MagPipe (mhd_device.cuh),
 // operation for operation, so a tile sweep gives bitwise the result of the
@@ -46,7 +49,7 @@ __device__ __forceinline__ int wrap_any(int i, int n) {
 // neighbours across the periodic wrap); others in segments with one thread of
 // 4 halo cells at each end (3 are needed), which stores nothing.
 // (FluidTile and fluid_tile_split are declared in mhd_launch.h: the host
-// builds grids and work lists with the same split.)
+// builds the grid with the same split.)
 constexpr int kTileSlots = 6;  // exchanged V5 values per thread (slot 0 is used twice)
 
 __host__ __device__ constexpr size_t fluid_tile_smem(int threads) {
@@ -671,8 +674,7 @@ __host__ __device__ constexpr size_t mag_tile_smem(int D, int out) {
 }
 
 // ---------------------------------------------------------------------------
-// Launches.  A single box takes a block per run of pencils (fluid) or tile
-// (magnetic) and segment; an ensemble one block per work item.
+// Launches: a block per run of pencils (fluid) or tile (magnetic) and segment.
 template <int LIM, int FRZ, bool FSQ>
 cudaError_t launch_fluid_tile(int axis, bool rate, const FluidArgs& a, cudaStream_t s) {
   if constexpr (FRZ == 2) {
@@ -680,14 +682,14 @@ cudaError_t launch_fluid_tile(int axis, bool rate, const FluidArgs& a, cudaStrea
   } else {
     const int A = (axis == 0) ? 1 : 0, O = (axis == 2) ? 1 : 2;
     const FluidTile t = fluid_tile_split(axis, a.box.n[axis], a.tile);
-    const int threads = a.ens.items ? a.tile : (t.np * t.td + 31) / 32 * 32;
+    const int threads = (t.np * t.td + 31) / 32 * 32;
     const long long pencils = (long long)a.box.n[A] * a.box.n[O];
-    const dim3 grid = a.ens.items ? dim3(a.nblocks) : dim3((unsigned)((pencils + t.np - 1) / t.np), 1, t.segs);
+    const dim3 grid((unsigned)((pencils + t.np - 1) / t.np), 1, t.segs);
     const size_t smem = fluid_tile_smem(threads);
     const bool floor = a.p_floor > 0.f;
 #define FLUID_TILE_CASE(DD, RR, FF) \
   if (axis == DD && rate == RR && floor == FF)                                                        \
-    return launch_after(!a.ens.items, fluid_tile_kernel<DD, RR, FF, LIM, FRZ, FSQ>, grid, dim3(threads), smem, s, a);
+    return launch_after(true, fluid_tile_kernel<DD, RR, FF, LIM, FRZ, FSQ>, grid, dim3(threads), smem, s, a);
     FLUID_TILE_CASE(0, false, false) FLUID_TILE_CASE(0, true, false) FLUID_TILE_CASE(0, false, true)
     FLUID_TILE_CASE(0, true, true) FLUID_TILE_CASE(1, false, false) FLUID_TILE_CASE(1, true, false)
     FLUID_TILE_CASE(1, false, true) FLUID_TILE_CASE(1, true, true) FLUID_TILE_CASE(2, false, false)
@@ -701,14 +703,13 @@ template <int LIM, int LX, int R>
 cudaError_t launch_mag_tile_shape(int axis, const MagArgs& a, cudaStream_t s) {
   const int A = (axis == 0) ? 1 : 0, O = (axis == 2) ? 1 : 2;
   const MagTile t = mag_tile_split(a.box.n[axis]);
-  const dim3 grid = a.ens.items ? dim3(a.nblocks)
-                                : dim3((a.box.n[A] + LX - 1) / LX, (a.box.n[O] + R - 1) / R, t.segs);
-  const size_t smem = mag_tile_smem<LX, R>(axis, a.ens.items ? a.tile_out : t.out);
+  const dim3 grid((a.box.n[A] + LX - 1) / LX, (a.box.n[O] + R - 1) / R, t.segs);
+  const size_t smem = mag_tile_smem<LX, R>(axis, t.out);
   constexpr int T = MTile<LX, R>::T;
   auto* kernel = axis == 0   ? mag_tile_x_kernel<LX, R, LIM>
                  : axis == 1 ? mag_tile_kernel<1, LX, R, LIM, 1>
                              : (a.passes == 2 ? mag_tile_kernel<2, LX, R, LIM, 2> : mag_tile_kernel<2, LX, R, LIM, 1>);
-  return launch_after(!a.ens.items, kernel, grid, dim3(T), smem, s, a);
+  return launch_after(true, kernel, grid, dim3(T), smem, s, a);
 }
 
 template <int LIM>
