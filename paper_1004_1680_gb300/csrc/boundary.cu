@@ -37,8 +37,8 @@ namespace mhd {
 // ghosts of the contiguous axis are left to that axis's threads.
 template <typename I, int V>
 __global__ void __launch_bounds__(256) ghost_fill_kernel(const __grid_constant__ GhostArgs a) {
-  wait_for_previous_in_place();
   const I total = (I)a.first[3];
+  bool waited = false;  // the first element's indexes are formed while the sweep before still runs
   for (I id = (I)blockIdx.x * blockDim.x + threadIdx.x; id < total; id += (I)gridDim.x * blockDim.x) {
     // the ghost layers of axis k: elements (groups of V cells for k > 0)
     // first[k] .. first[k + 1] - 1
@@ -93,6 +93,12 @@ __global__ void __launch_bounds__(256) ghost_fill_kernel(const __grid_constant__
       cell += (long long)s * a.stride[d];
       face[d] = (long long)(f - s) * a.stride[d];
     }
+    if (!waited) {
+      int moves = di != cell;
+      settled(moves, x[0]);
+      wait_for_previous_in_place();
+      waited = true;
+    }
 #pragma unroll
     for (int q = 0; q < 8; q++) {
       if (!(a.parts & (q >= 5 ? kGhostField : kGhostFluid))) continue;
@@ -109,6 +115,7 @@ __global__ void __launch_bounds__(256) ghost_fill_kernel(const __grid_constant__
       }
     }
   }
+  if (!waited) wait_for_previous_in_place();
 }
 
 cudaError_t launch_ghost_fill(float* const f[8], const Box& box, const int mode[3], int parts, cudaStream_t s) {

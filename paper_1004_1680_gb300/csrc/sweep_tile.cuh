@@ -11,7 +11,7 @@
 // (fluid) or two passes over shared memory (magnetic).  Time per step, marching
 // -> tile: 32^3 302 -> 78 us, 64^3 308 -> 111, 96^3 432 -> 217, 236 x 150 x 98
 // (x sweeps without transposes) 1043 -> 800 us (all sweeps by tiles, before
-// the later changes; now 43, 91, 179 and 571).  Small boxes are bound by the
+// the later changes; now 41, 86, 174 and 567).  Small boxes are bound by the
 // launches (about 2.5 us each) and one chain of loads, arithmetic and stores
 // (2 to 5 us); once the chip is full a fluid tile sweep runs at 17 (x) or 21 ps
 // per cell, twice the marching sweep's 8.3 ps on a 512^3 box: its phases are
@@ -65,9 +65,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) fluid_tile_kernel(const __gri
   constexpr int K = kTileCells;
   constexpr int A = (D == 0) ? 1 : 0, O = (D == 2) ? 1 : 2, T1 = (D + 1) % 3, T2 = (D + 2) % 3;
   extern __shared__ float4 tile_dyn[];
-  wait_for_previous();
-  const BlockGeom G = block_geom(a.ens, a.box, a.seg, a.tau, a.rate);
-  const int nA = G.box.n[A], nO = G.box.n[O], nD = G.box.n[D];
+  const int nA = a.box.n[A], nO = a.box.n[O], nD = a.box.n[D];
   const int T = blockDim.x, tid = threadIdx.x;
   const FluidTile s = fluid_tile_split(D, nD, a.tile);
   const int np = s.np, td = s.td;
@@ -75,7 +73,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) fluid_tile_kernel(const __gri
   // pencil are neighbouring threads (16 contiguous bytes each), else the
   // pencils are
   const int pp = D == 0 ? tid / td : tid % np, l = D == 0 ? tid - pp * td : tid / np;
-  const int P = G.bx * np + pp;
+  const int P = blockIdx.x * np + pp;
   const bool live = pp < np && l < td && P < nA * nO;
   RowSlots X;
   X.A = tile_dyn;
@@ -85,14 +83,24 @@ __global__ void __launch_bounds__(kTileThreads, 2) fluid_tile_kernel(const __gri
   const int lm = l > 0 ? l - 1 : (s.whole ? td - 1 : 0), lp = l + 1 < td ? l + 1 : (s.whole ? 0 : l);
   const int im = D == 0 ? tid + lm - l : tid + (lm - l) * np, ip = D == 0 ? tid + lp - l : tid + (lp - l) * np;
 
-  const float gamma = a.gamma;
-  const float c_full = G.tau * G.box.ih[D];  // tau / h_D
-  const float c_half = 0.5f * c_full;
   const int pb = P / nA, pa = P - pb * nA;
-  const int sA = (int)G.box.stride[A], sO = (int)G.box.stride[O], sD = (int)G.box.stride[D];
-  const unsigned base = (unsigned)(pa * sA + pb * sO);
+  const int sA = (int)a.box.stride[A], sO = (int)a.box.stride[O], sD = (int)a.box.stride[D];
+  unsigned base = (unsigned)(pa * sA + pb * sO);
+  unsigned baseA1 = base + (unsigned)((pa + 1 == nA ? 1 - nA : 1) * sA);  // pencil +1 along A
+  unsigned baseO1 = base + (unsigned)((pb + 1 == nO ? 1 - nO : 1) * sO);  // pencil +1 along O
   // the first of the thread's cells, before wrapping
-  const int p0 = G.bz * s.out + K * (l - (s.whole ? 0 : 1));
+  int p0 = blockIdx.z * s.out + K * (l - (s.whole ? 0 : 1));
+  unsigned off[K + 1];  // of the cells p0 .. p0+4 along the pencil
+#pragma unroll
+  for (int j = 0; j <= K; j++) {
+    off[j] = (D == 0 && j > 0 && j < K) ? 0u : (unsigned)(wrap_any(p0 + j, nD) * sD);
+    settle(off[j]);
+  }
+  settled(base, baseA1, baseO1, p0);
+  wait_for_previous();
+  const float gamma = a.gamma;
+  const float c_full = *a.tau * a.box.ih[D];  // tau / h_D
+  const float c_half = 0.5f * c_full;
 
   V5 f1[K + 1];  // flux1 at p0-1/2 .. p0+7/2
   V5 FR3, FL0;
@@ -101,14 +109,12 @@ __global__ void __launch_bounds__(kTileThreads, 2) fluid_tile_kernel(const __gri
     // every load of the sweep, before the first use
     const float* __restrict__ f[8];
 #pragma unroll
-    for (int q = 0; q < 8; q++) f[q] = a.in[q] + G.off;
-    const unsigned baseA1 = base + (unsigned)((pa + 1 == nA ? 1 - nA : 1) * sA);  // pencil +1 along A
-    const unsigned baseO1 = base + (unsigned)((pb + 1 == nO ? 1 - nO : 1) * sO);  // pencil +1 along O
+    for (int q = 0; q < 8; q++) f[q] = a.in[q];
     const unsigned baseT1 = (T1 == A) ? baseA1 : baseO1, baseT2 = (T2 == A) ? baseA1 : baseO1;
     constexpr int kField[5] = {RHO, MX + D, MX + T1, MX + T2, EN};
     float u[5][K], bd[K + 1], b1[K], b1n[K], b2[K], b2n[K];
     if constexpr (D == 0) {
-      const unsigned c = base + (unsigned)wrap_any(p0, nD);  // p0 and nx are multiples of 4
+      const unsigned c = base + off[0];  // p0 and nx are multiples of 4
       auto ld4 = [](const float* p, float (&d)[K]) {
         const float4 v = __ldg(reinterpret_cast<const float4*>(p));
 #pragma unroll
@@ -121,15 +127,12 @@ __global__ void __launch_bounds__(kTileThreads, 2) fluid_tile_kernel(const __gri
       ld4(f[BX + D] + c, t);
 #pragma unroll
       for (int j = 0; j < K; j++) bd[j] = t[j];
-      bd[K] = __ldg(f[BX + D] + base + (unsigned)wrap_any(p0 + K, nD));
+      bd[K] = __ldg(f[BX + D] + (base + off[K]));
       ld4(f[BX + T1] + c, b1);
       ld4(f[BX + T1] + (baseT1 + w), b1n);
       ld4(f[BX + T2] + c, b2);
       ld4(f[BX + T2] + (baseT2 + w), b2n);
     } else {
-      unsigned off[K + 1];
-#pragma unroll
-      for (int j = 0; j <= K; j++) off[j] = (unsigned)(wrap_any(p0 + j, nD) * sD);
 #pragma unroll
       for (int j = 0; j < K; j++) {
 #pragma unroll
@@ -212,12 +215,12 @@ __global__ void __launch_bounds__(kTileThreads, 2) fluid_tile_kernel(const __gri
   float rmax = 0.f;
   // cells of this block's own positions (halo threads and the cells past the
   // pencil's end store nothing)
-  const int pend = min(nD, (G.bz + 1) * s.out);
-  if (live && p0 >= G.bz * s.out && p0 < pend) {
+  const int first = blockIdx.z * s.out, pend = min(nD, first + s.out);
+  if (live && p0 >= first && p0 < pend) {
     float* __restrict__ o[5];
     constexpr int kField[5] = {RHO, MX + D, MX + T1, MX + T2, EN};
 #pragma unroll
-    for (int q = 0; q < 5; q++) o[q] = a.out[kField[q]] + G.off;
+    for (int q = 0; q < 5; q++) o[q] = a.out[kField[q]];
     V5 U[K];
     parked(U);
     const V5 Fm = X.get(0, im);
@@ -246,7 +249,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) fluid_tile_kernel(const __gri
           float m[3], bg[3];
           m[D] = r[j][1]; m[T1] = r[j][2]; m[T2] = r[j][3];
           bg[D] = B[j].v[0]; bg[T1] = B[j].v[1]; bg[T2] = B[j].v[2];
-          rmax = fmaxf(rmax, cell_rate(r[j][0], m, r[j][4], bg, gamma, G.box.ih));
+          rmax = fmaxf(rmax, cell_rate(r[j][0], m, r[j][4], bg, gamma, a.box.ih));
         }
       }
     if constexpr (D == 0) {
@@ -267,7 +270,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) fluid_tile_kernel(const __gri
   }
   if (RATE) {
     for (int k = 16; k > 0; k >>= 1) rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, k));
-    if ((tid & 31) == 0 && rmax > 0.f) atomicMax(G.rate, __float_as_uint(rmax));
+    if ((tid & 31) == 0 && rmax > 0.f) atomicMax(a.rate, __float_as_uint(rmax));
   }
 }
 
@@ -360,12 +363,10 @@ __global__ void __launch_bounds__(MTile<LX, R>::T) mag_tile_kernel(const __grid_
   using L = MPlane<LX, R>;
   constexpr int H = mag_tile_halo(D), T = M::T, Sv = L::V, Sa = L::A, So = L::O, Sb = L::B, Sf = L::F > L::V ? L::F : L::V;
   extern __shared__ __align__(16) float mt_dyn[];
-  wait_for_previous();
-  const BlockGeom G = block_geom(a.ens, a.box, a.seg, a.tau, nullptr);
-  const int nA = G.box.n[A], nO = G.box.n[O], nD = G.box.n[D];
+  const int nA = a.box.n[A], nO = a.box.n[O], nD = a.box.n[D];
   const MagTile sp = mag_tile_split(nD);
-  const int a0 = G.bx * LX, b0 = G.by * R;
-  const int s0 = G.bz * sp.out, S = min(sp.out, nD - s0);  // this block's positions s0 .. s0 + S - 1
+  const int a0 = (int)blockIdx.x * LX, b0 = (int)blockIdx.y * R;
+  const int s0 = (int)blockIdx.z * sp.out, S = min(sp.out, nD - s0);  // this block's positions s0 .. s0 + S - 1
   const int PN = mag_tile_positions(D, sp.out);
   float* sv = mt_dyn;
   float* sa = sv + Sv * PN;
@@ -373,7 +374,7 @@ __global__ void __launch_bounds__(MTile<LX, R>::T) mag_tile_kernel(const __grid_
   float* sb = so + So * PN;
   float* sf = sb + Sb * PN;
   const int tid = threadIdx.x;
-  const int sO = (int)G.box.stride[O], sD = (int)G.box.stride[D];
+  const int sO = (int)a.box.stride[O], sD = (int)a.box.stride[D];
 
   // A thread keeps its 16-byte piece of the plane and walks the positions.  The
   // lanes are contiguous and nA a multiple of 4, so pieces never straddle the
@@ -406,9 +407,14 @@ __global__ void __launch_bounds__(MTile<LX, R>::T) mag_tile_kernel(const __grid_
         piece -= So / 4;
         place(sb, Sb, LX, 0, 0, a.in[BX + D]);
       }
-      src += G.off + (wrap_any(a0 + col, nA) + wrap_any(b0 + row, nO) * sO);
+      int at = wrap_any(a0 + col, nA) + wrap_any(b0 + row, nO) * sO;
+      settled(at, plane);
+      src += at;
+      wait_for_previous();
       for (int p = tid / kSlots; p < S + 2 * H; p += kStep)
         copy16_async(dst + p * plane, src + (unsigned)(wrap_any(s0 - H + p, nD) * sD));
+    } else {
+      wait_for_previous();
     }
     copies_wait();
     __syncthreads();
@@ -418,11 +424,11 @@ __global__ void __launch_bounds__(MTile<LX, R>::T) mag_tile_kernel(const __grid_
       at4(sv + p * Sv + q) = v_div4(at4(sv + p * Sv + q), at4(sf + p * Sf + q));
     }
   }
-  const float tau = G.tau;
-  const float c_full = tau * G.box.ih[D];  // tau / h_D
+  const float tau = *a.tau;
+  const float c_full = tau * a.box.ih[D];  // tau / h_D
   const float c_half = 0.5f * c_full;
-  const float kA = tau * G.box.ih[A];      // tau / h_A
-  const float kO = tau * G.box.ih[O];      // tau / h_O
+  const float kA = tau * a.box.ih[A];      // tau / h_A
+  const float kO = tau * a.box.ih[O];      // tau / h_O
   // edge e lies between local cells e - 1 and e: edges 0 .. S are needed; of a
   // whole pencil 1 .. S (edge 0 is edge S)
   const int e0 = sp.whole ? 1 : 0;
@@ -452,9 +458,9 @@ __global__ void __launch_bounds__(MTile<LX, R>::T) mag_tile_kernel(const __grid_
     __syncthreads();
     if (pass + 1 == NP) {
       // finish the tile's cells
-      float* __restrict__ oA = a.out[A] + G.off;
-      float* __restrict__ oO = a.out[O] + G.off;
-      float* __restrict__ oD = a.out[D] + G.off;
+      float* __restrict__ oA = a.out[A];
+      float* __restrict__ oO = a.out[O];
+      float* __restrict__ oD = a.out[D];
       static_assert(T % M::C == 0, "a thread keeps its pencil");
       const int c = tid % M::C, row = c / LX, col = c - row * LX, ts = row * (LX + 1) + col;
       if (a0 + col < nA && b0 + row < nO) {
@@ -546,23 +552,23 @@ __global__ void __launch_bounds__(MTile<LX, R>::T) mag_tile_x_kernel(const __gri
   using M = MRows<LX, R>;
   constexpr int H = mag_tile_halo(0), T = MTile<LX, R>::T;
   extern __shared__ __align__(16) float mt_dyn[];
-  wait_for_previous();
-  const BlockGeom G = block_geom(a.ens, a.box, a.seg, a.tau, nullptr);
-  const int nA = G.box.n[1], nO = G.box.n[2], nD = G.box.n[0];
+  const int nA = a.box.n[1], nO = a.box.n[2], nD = a.box.n[0];
   const MagTile sp = mag_tile_split(nD);
-  const int a0 = G.bx * LX, b0 = G.by * R;
-  const int s0 = G.bz * sp.out, S = min(sp.out, nD - s0);  // multiples of 4
+  const int a0 = (int)blockIdx.x * LX, b0 = (int)blockIdx.y * R;
+  const int s0 = (int)blockIdx.z * sp.out, S = min(sp.out, nD - s0);  // multiples of 4
   const int PN = mag_tile_positions(0, sp.out);
   float* sv = mt_dyn;
   float* sq = sv + M::V * PN;
   float* sf = sq + M::Q * PN;
   float* sb = sf + M::Q * PN;
   const int tid = threadIdx.x;
-  const int sA = (int)G.box.stride[1], sO = (int)G.box.stride[2];
+  const int sA = (int)a.box.stride[1], sO = (int)a.box.stride[2];
   // (pencil, piece) pairs, stepped without a division per piece; a thread
   // forms v of the pieces it has copied itself
-  const int pieces = (S + 2 * H) / 4, dslot = T / pieces, dpiece = T - dslot * pieces;
-  const int slot0 = tid / pieces, piece0 = tid - slot0 * pieces;
+  const int pieces = (S + 2 * H) / 4;
+  int dslot = T / pieces, dpiece = T - dslot * pieces, slot0 = tid / pieces, piece0 = tid - slot0 * pieces;
+  settled(dslot, dpiece, slot0, piece0);
+  wait_for_previous();
   for (int half = 0; half < 2; half++) {
     int slot = slot0, g = piece0;
     while (slot < M::V) {
@@ -573,7 +579,7 @@ __global__ void __launch_bounds__(MTile<LX, R>::T) mag_tile_x_kernel(const __gri
         float* r = sf + slot * PN + 4 * g;
         if (half == 0) {
           const unsigned c = (unsigned)(wrap_any(a0 + col - 1, nA) * sA + wrap_any(b0 + row - 1, nO) * sO +
-                                        wrap_any(s0 - H + 4 * g, nD)) + (unsigned)G.off;
+                                        wrap_any(s0 - H + 4 * g, nD));
           copy16_async(v, a.in[MX] + c);
           copy16_async(r, a.in[RHO] + c);
           if (rin && col >= 1) copy16_async(sq + ((row - 1) * (LX + 1) + col - 1) * PN + 4 * g, a.in[BY] + c);
@@ -592,11 +598,11 @@ __global__ void __launch_bounds__(MTile<LX, R>::T) mag_tile_x_kernel(const __gri
     }
     if (half == 0) copies_wait();
   }
-  const float tau = G.tau;
-  const float c_full = tau * G.box.ih[0];  // tau / h_x
+  const float tau = *a.tau;
+  const float c_full = tau * a.box.ih[0];  // tau / h_x
   const float c_half = 0.5f * c_full;
-  const float kA = tau * G.box.ih[1];      // tau / h_y
-  const float kO = tau * G.box.ih[2];      // tau / h_z
+  const float kA = tau * a.box.ih[1];      // tau / h_y
+  const float kO = tau * a.box.ih[2];      // tau / h_z
   const int e0 = sp.whole ? 1 : 0;         // edges e0 .. S, edge e at position e - e0 of sf
   const int groups = (S + 1 - e0 + 3) / 4;
   __syncthreads();
@@ -661,7 +667,7 @@ __global__ void __launch_bounds__(MTile<LX, R>::T) mag_tile_x_kernel(const __gri
       rO[k] = __fmaf_rn(-c_full, __fsub_rn(fo[k + 1], fo[k]), (&bO.x)[k]);
       rD[k] = constrain((&bD.x)[k], kA, fa[k], fa1[k], kO, fo[k], fo1[k], true);
     }
-    const unsigned o = (unsigned)((a0 + col) * sA + (b0 + row) * sO + s0 + 4 * g) + (unsigned)G.off;
+    const unsigned o = (unsigned)((a0 + col) * sA + (b0 + row) * sO + s0 + 4 * g);
     at4(a.out[1] + o) = make_float4(rA[0], rA[1], rA[2], rA[3]);
     at4(a.out[2] + o) = make_float4(rO[0], rO[1], rO[2], rO[3]);
     at4(a.out[0] + o) = make_float4(rD[0], rD[1], rD[2], rD[3]);
