@@ -692,10 +692,11 @@ cudaError_t launch_fluid_tile(int axis, bool rate, const FluidArgs& a, cudaStrea
     const long long pencils = (long long)a.box.n[A] * a.box.n[O];
     const dim3 grid((unsigned)((pencils + t.np - 1) / t.np), 1, t.segs);
     const size_t smem = fluid_tile_smem(threads);
+    const bool shared = all_shared(pencils * a.box.n[axis]);
     const bool floor = a.p_floor > 0.f;
 #define FLUID_TILE_CASE(DD, RR, FF) \
   if (axis == DD && rate == RR && floor == FF)                                                        \
-    return launch_after(true, fluid_tile_kernel<DD, RR, FF, LIM, FRZ, FSQ>, grid, dim3(threads), smem, s, a);
+    return launch_after(true, shared, fluid_tile_kernel<DD, RR, FF, LIM, FRZ, FSQ>, grid, dim3(threads), smem, s, a);
     FLUID_TILE_CASE(0, false, false) FLUID_TILE_CASE(0, true, false) FLUID_TILE_CASE(0, false, true)
     FLUID_TILE_CASE(0, true, true) FLUID_TILE_CASE(1, false, false) FLUID_TILE_CASE(1, true, false)
     FLUID_TILE_CASE(1, false, true) FLUID_TILE_CASE(1, true, true) FLUID_TILE_CASE(2, false, false)
@@ -715,7 +716,8 @@ cudaError_t launch_mag_tile_shape(int axis, const MagArgs& a, cudaStream_t s) {
   auto* kernel = axis == 0   ? mag_tile_x_kernel<LX, R, LIM>
                  : axis == 1 ? mag_tile_kernel<1, LX, R, LIM, 1>
                              : (a.passes == 2 ? mag_tile_kernel<2, LX, R, LIM, 2> : mag_tile_kernel<2, LX, R, LIM, 1>);
-  return launch_after(true, kernel, grid, dim3(T), smem, s, a);
+  return launch_after(true, all_shared((long long)a.box.n[0] * a.box.n[1] * a.box.n[2]), kernel, grid, dim3(T), smem, s,
+                      a);
 }
 
 template <int LIM>
