@@ -142,8 +142,8 @@ cudaError_t launch_ghost_fill(float* const f[8], const Box& box, const int mode[
   const bool narrow = total + blocks * 256 < (1LL << 32);
   auto* kernel = narrow ? (wide ? ghost_fill_kernel<unsigned, 4> : ghost_fill_kernel<unsigned, 1>)
                         : (wide ? ghost_fill_kernel<unsigned long long, 4> : ghost_fill_kernel<unsigned long long, 1>);
-  const bool shared = all_shared((long long)box.n[0] * box.n[1] * box.n[2]);
-  return launch_after(true, shared, kernel, dim3((unsigned)blocks), dim3(256), 0, s, a);
+  const int split = shared_split((long long)box.n[0] * box.n[1] * box.n[2]);
+  return launch_after(true, split, kernel, dim3((unsigned)blocks), dim3(256), 0, s, a);
 }
 
 }  // namespace mhd

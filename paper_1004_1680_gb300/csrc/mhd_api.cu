@@ -256,9 +256,9 @@ double tile_us(const mhd_s* m, bool mag) { return (mag ? 19e-6 : 21e-6) * (doubl
 int tile_choice(const mhd_s* m, int d, bool mag, int passes) {
   if (!m->tma || m->fast == 2 || m->xpath == 3 || m->layout || m->seg_set[d]) return 0;
   // magnetic tiles of 8 x 2 pencils (128 threads) where there are few (32^3: 41 us
-  // per step against 48, 40^3 49 and 63), else 16 x 4 (384 threads; 64^3 86 us
-  // against 102, 96^3 174 and 212)
-  const int shape = m->N <= 64000 ? 1 : 2;
+  // per step against 49, 48^3 50 and 57), else 16 x 4 (384 threads; 52^3 65 us
+  // against 67, 64^3 68 and 77, 96^3 174 and 212)
+  const int shape = m->N <= 120000 ? 1 : 2;
   // a launch holds 65535 rows of tiles (the axes' roles as in the sweeps: row
   // axis z, or y for z sweeps) and as many segments of a pencil
   if (mag && (m->n[d == 2 ? 1 : 2] > 2 * 65535 || m->n[d] > 24 * 65535)) return 0;
@@ -598,7 +598,7 @@ int run_steps(mhd_s* m, int nsteps, double cfl) {
   for (int s = 0; s < nsteps; s++) {
     int rc = traced(m, MHD_K_CONTROL, [&] {
       CK(mhd::launch_step_control(&m->sc->rate[m->rcur], &m->sc->rate[1 - m->rcur], &m->sc->tau,
-                                  &m->sc->time, cfl, 0.0, mhd::all_shared(m->N), m->stream));
+                                  &m->sc->time, cfl, 0.0, mhd::shared_split(m->N), m->stream));
       return MHD_OK;
     });
     if (!rc) rc = full_step(m);
@@ -942,7 +942,7 @@ int mhd_step(mhd_t* m, double dt_full) {
   if (int rc = join_pipeline(m)) return rc;
   int rc = traced(m, MHD_K_CONTROL, [&] {
     CK(mhd::launch_step_control(&m->sc->rate[m->rcur], &m->sc->rate[1 - m->rcur], &m->sc->tau,
-                                &m->sc->time, -1.0, 0.5 * dt_full, mhd::all_shared(m->N), m->stream));
+                                &m->sc->time, -1.0, 0.5 * dt_full, mhd::shared_split(m->N), m->stream));
     return MHD_OK;
   });
   if (!rc) rc = full_step(m);

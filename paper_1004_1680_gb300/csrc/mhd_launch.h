@@ -79,16 +79,18 @@ __device__ __forceinline__ void wait_for_previous_in_place() { asm volatile("gri
 // Launch a kernel that begins with one of the two; `early` = false gives an
 // ordinary launch (the wait then has nothing to wait for).
 //
-// `shared`: all of an SM's memory as shared memory where there is a choice.  A
-// kernel that asks for another split than the one before cannot start beside it,
-// and in small boxes that beginning is most of a sweep: 36^3 53.4 -> 45.5 us per
-// step, 40^3 76.6 -> 49, 48^3 69.7 -> 61.7 with one split for the fluid and the
-// magnetic tiles.  Larger boxes need L1 for the neighbour pencils that a fluid
-// tile loads (56^3 80 -> 85, 96^3 174 -> 194), the smallest, whose tiles need
-// little of it, nothing (32^3 40.9 -> 41.4): `all_shared`.
-inline bool all_shared(long long cells) { return cells > 40000 && cells <= 150000; }
+// `split`: the share of an SM's memory (in percent) to be shared memory, 0 for the
+// driver's choice.  A kernel that asks for another split than the one before
+// cannot start beside it, and in small boxes that beginning is a good part of a
+// sweep; left alone, the fluid tiles get 132 KB, the magnetic ones 196.  132 KB
+// hold a block of 16 x 4 magnetic tiles or four fluid blocks (64^3 86 -> 68 us
+// per step, 48^3 70 -> 57, 40^3 61 -> 48, 128 x 64 x 32 82 -> 64), 164 KB two
+// magnetic blocks, which larger boxes need (68^3 115 -> 95, 72^3 119 -> 97; with
+// 132 KB 105 and 108).  Beyond that a sweep takes so long that its beginning
+// counts less than L1 or a second block (76^3 111 either way, 96^3 174 and 184).
+inline int shared_split(long long cells) { return cells <= 280000 ? 50 : (cells <= 450000 ? 65 : 0); }
 template <class... P>
-inline cudaError_t launch_after(bool early, bool shared, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+inline cudaError_t launch_after(bool early, int split, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
                                 cudaStream_t s, P... args) {
   cudaLaunchConfig_t c = {};
   c.gridDim = grid;
@@ -100,9 +102,9 @@ inline cudaError_t launch_after(bool early, bool shared, void (*kernel)(P...), d
     at[c.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[c.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
   }
-  if (shared) {
+  if (split) {
     at[c.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-    at[c.numAttrs++].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+    at[c.numAttrs++].val.sharedMemCarveout = (unsigned)split;
   }
   c.attrs = at;
   return cudaLaunchKernelEx(&c, kernel, args...);
@@ -110,7 +112,7 @@ inline cudaError_t launch_after(bool early, bool shared, void (*kernel)(P...), d
 template <class... P>
 inline cudaError_t launch_after(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                                 P... args) {
-  return launch_after(early, false, kernel, grid, block, smem, s, args...);
+  return launch_after(early, 0, kernel, grid, block, smem, s, args...);
 }
 
 // Split of a fluid tile sweep (sweep_tile.cuh) along a pencil of nD cells for
@@ -439,7 +441,7 @@ bool local_fields(const void* const f[8]);
 // device-side step control: tau = cfl / rate_cur (or the given tau if cfl<0),
 // time += 2 tau, rate_next = 0
 cudaError_t launch_step_control(const unsigned* rate_cur, unsigned* rate_next, float* tau,
-                                double* time, double cfl, double tau_host, bool shared, cudaStream_t s);
+                                double* time, double cfl, double tau_host, int split, cudaStream_t s);
 // set the device sweep step to a host value (no time advance)
 cudaError_t launch_set_tau(float* tau, double value, cudaStream_t s);
 // FP64 diagnostics: per-block partials into `partial` (nblk*kDiagSlots

@@ -174,8 +174,8 @@ __global__ void step_control_kernel(const unsigned* rate_cur, unsigned* rate_nex
 }
 
 cudaError_t launch_step_control(const unsigned* rate_cur, unsigned* rate_next, float* tau,
-                                double* time, double cfl, double tau_host, bool shared, cudaStream_t s) {
-  return launch_after(true, shared, step_control_kernel, dim3(1), dim3(1), 0, s, rate_cur, rate_next, tau, time, cfl, tau_host);
+                                double* time, double cfl, double tau_host, int split, cudaStream_t s) {
+  return launch_after(true, split, step_control_kernel, dim3(1), dim3(1), 0, s, rate_cur, rate_next, tau, time, cfl, tau_host);
 }
 
 __global__ void ens_control_kernel(const unsigned* rate_cur, unsigned* rate_next, float* tau,

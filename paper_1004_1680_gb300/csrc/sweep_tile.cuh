@@ -11,7 +11,7 @@
 // (fluid) or two passes over shared memory (magnetic).  Time per step, marching
 // -> tile: 32^3 302 -> 78 us, 64^3 308 -> 111, 96^3 432 -> 217, 236 x 150 x 98
 // (x sweeps without transposes) 1043 -> 800 us (all sweeps by tiles, before
-// the later changes; now 41, 86, 174 and 567).  Small boxes are bound by the
+// the later changes; now 41, 68, 174 and 567).  Small boxes are bound by the
 // launches (about 2.5 us each) and one chain of loads, arithmetic and stores
 // (2 to 5 us); once the chip is full a fluid tile sweep runs at 17 (x) or 21 ps
 // per cell, twice the marching sweep's 8.3 ps on a 512^3 box: its phases are
@@ -692,11 +692,11 @@ cudaError_t launch_fluid_tile(int axis, bool rate, const FluidArgs& a, cudaStrea
     const long long pencils = (long long)a.box.n[A] * a.box.n[O];
     const dim3 grid((unsigned)((pencils + t.np - 1) / t.np), 1, t.segs);
     const size_t smem = fluid_tile_smem(threads);
-    const bool shared = all_shared(pencils * a.box.n[axis]);
+    const int split = shared_split(pencils * a.box.n[axis]);
     const bool floor = a.p_floor > 0.f;
 #define FLUID_TILE_CASE(DD, RR, FF) \
   if (axis == DD && rate == RR && floor == FF)                                                        \
-    return launch_after(true, shared, fluid_tile_kernel<DD, RR, FF, LIM, FRZ, FSQ>, grid, dim3(threads), smem, s, a);
+    return launch_after(true, split, fluid_tile_kernel<DD, RR, FF, LIM, FRZ, FSQ>, grid, dim3(threads), smem, s, a);
     FLUID_TILE_CASE(0, false, false) FLUID_TILE_CASE(0, true, false) FLUID_TILE_CASE(0, false, true)
     FLUID_TILE_CASE(0, true, true) FLUID_TILE_CASE(1, false, false) FLUID_TILE_CASE(1, true, false)
     FLUID_TILE_CASE(1, false, true) FLUID_TILE_CASE(1, true, true) FLUID_TILE_CASE(2, false, false)
@@ -716,7 +716,7 @@ cudaError_t launch_mag_tile_shape(int axis, const MagArgs& a, cudaStream_t s) {
   auto* kernel = axis == 0   ? mag_tile_x_kernel<LX, R, LIM>
                  : axis == 1 ? mag_tile_kernel<1, LX, R, LIM, 1>
                              : (a.passes == 2 ? mag_tile_kernel<2, LX, R, LIM, 2> : mag_tile_kernel<2, LX, R, LIM, 1>);
-  return launch_after(true, all_shared((long long)a.box.n[0] * a.box.n[1] * a.box.n[2]), kernel, grid, dim3(T), smem, s,
+  return launch_after(true, shared_split((long long)a.box.n[0] * a.box.n[1] * a.box.n[2]), kernel, grid, dim3(T), smem, s,
                       a);
 }
 
