@@ -12,6 +12,8 @@
 //    each transverse component (one thread per cell and component) and
 //    stores its edge flux; a constraint kernel that updates b_d of every
 //    cell from the stored fluxes of its pencil and the neighbouring pencils.
+//  * Launched with programmatic dependent launch (24 launches a step: 16^3 292 ->
+//    243 us, 64^3 1416 -> 1358).
 //  * CFL rate: the largest (|v_d| + c_f*) / h_d over cells, as double bits
 //    reduced with an atomic maximum (rates are >= 0).
 #include <cstdint>
@@ -164,6 +166,7 @@ __device__ __forceinline__ Cell64 cell64(const int n[3]) {
 // 175; 256^3 111 ms a step, now 101.)
 template <int D>
 __global__ void __launch_bounds__(kThreads64, 1) fluid64_kernel(const __grid_constant__ Fluid64Args a) {
+  wait_for_previous();
   constexpr int A = (D == 0) ? 1 : 0, O = (D == 2) ? 1 : 2, T1 = (D + 1) % 3, T2 = (D + 2) % 3;
   extern __shared__ double sm64[];
   const int T = blockDim.x;
@@ -238,6 +241,7 @@ __global__ void __launch_bounds__(kThreads64, 1) fluid64_kernel(const __grid_con
 // v_D of every cell, once per magnetic sweep.
 __global__ void __launch_bounds__(256) velocity64_kernel(const double* __restrict__ m, const double* __restrict__ rho,
                                                          double* __restrict__ v, long long N) {
+  wait_for_previous();
   for (long long c = (long long)blockIdx.x * 256 + threadIdx.x; c < N; c += (long long)gridDim.x * 256)
     v[c] = ddiv(m[c], rho[c]);
 }
@@ -249,6 +253,7 @@ __global__ void __launch_bounds__(256) velocity64_kernel(const double* __restric
 // E[blockIdx.z] (the flux of edge i + 1/2 of a pencil stored at its cell i).
 template <int D>
 __global__ void __launch_bounds__(kThreads64) mag64_flux_kernel(const __grid_constant__ Mag64Args a) {
+  wait_for_previous();
   constexpr int A = (D == 0) ? 1 : 0, O = (D == 2) ? 1 : 2;
   __shared__ double su[kThreads64], sq[kThreads64], sh[kThreads64], sf[kThreads64];
   const long long st[3] = {1, a.n[0], (long long)a.n[0] * a.n[1]};
@@ -297,6 +302,7 @@ __global__ void __launch_bounds__(kThreads64) mag64_flux_kernel(const __grid_con
 // b_D += tau/h_t (E_t(pencil + e_t) - E_t(pencil)), t = T1 then T2.
 template <int D>
 __global__ void __launch_bounds__(256) mag64_constraint_kernel(Mag64Args a) {
+  wait_for_previous();
   const int N = a.n[0] * a.n[1] * a.n[2];
   const int s[3] = {1, a.n[0], a.n[0] * a.n[1]};
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < N; c += gridDim.x * blockDim.x) {
@@ -323,6 +329,7 @@ __global__ void __launch_bounds__(256) cfl64_kernel(const double* __restrict__ r
                                                     const double* __restrict__ by, const double* __restrict__ bz,
                                                     int nx, int ny, int nz, double ihx, double ihy, double ihz,
                                                     double gamma, unsigned long long* rate) {
+  wait_for_previous();
   const int N = nx * ny * nz;
   double rmax = 0.0;
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < N; c += gridDim.x * blockDim.x) {
@@ -375,10 +382,8 @@ cudaError_t prepare_f64_kernels() {
 cudaError_t launch_fluid64(int axis, const Fluid64Args& a, cudaStream_t s) {
   const dim3 grid = grid64(axis, a.n, 1);
   const int threads = tile64(a.n[axis]).threads, smem = fluid64_smem(threads);
-  if (axis == 0) fluid64_kernel<0><<<grid, threads, smem, s>>>(a);
-  if (axis == 1) fluid64_kernel<1><<<grid, threads, smem, s>>>(a);
-  if (axis == 2) fluid64_kernel<2><<<grid, threads, smem, s>>>(a);
-  return cudaGetLastError();
+  auto* kernel = axis == 0 ? fluid64_kernel<0> : (axis == 1 ? fluid64_kernel<1> : fluid64_kernel<2>);
+  return launch_after(true, kernel, grid, dim3(threads), smem, s, a);
 }
 
 cudaError_t launch_mag64(int axis, const Mag64Args& a, cudaStream_t s) {
@@ -386,20 +391,14 @@ cudaError_t launch_mag64(int axis, const Mag64Args& a, cudaStream_t s) {
   const int threads = tile64(a.n[axis]).threads;
   const long long N = (long long)a.n[0] * a.n[1] * a.n[2];
   const int cblocks = (int)((N + 255) / 256 < 152 * 16 ? (N + 255) / 256 : 152 * 16);
-  velocity64_kernel<<<cblocks, 256, 0, s>>>(a.in[MX + axis], a.in[RHO], a.v, N);
-  if (axis == 0) {
-    mag64_flux_kernel<0><<<grid, threads, 0, s>>>(a);
-    mag64_constraint_kernel<0><<<cblocks, 256, 0, s>>>(a);
-  }
-  if (axis == 1) {
-    mag64_flux_kernel<1><<<grid, threads, 0, s>>>(a);
-    mag64_constraint_kernel<1><<<cblocks, 256, 0, s>>>(a);
-  }
-  if (axis == 2) {
-    mag64_flux_kernel<2><<<grid, threads, 0, s>>>(a);
-    mag64_constraint_kernel<2><<<cblocks, 256, 0, s>>>(a);
-  }
-  return cudaGetLastError();
+  auto* flux = axis == 0 ? mag64_flux_kernel<0> : (axis == 1 ? mag64_flux_kernel<1> : mag64_flux_kernel<2>);
+  auto* constraint =
+      axis == 0 ? mag64_constraint_kernel<0> : (axis == 1 ? mag64_constraint_kernel<1> : mag64_constraint_kernel<2>);
+  cudaError_t e = launch_after(true, velocity64_kernel, dim3(cblocks), dim3(256), 0, s,
+                               static_cast<const double*>(a.in[MX + axis]), static_cast<const double*>(a.in[RHO]), a.v, N);
+  if (e == cudaSuccess) e = launch_after(true, flux, grid, dim3(threads), 0, s, a);
+  if (e == cudaSuccess) e = launch_after(true, constraint, dim3(cblocks), dim3(256), 0, s, a);
+  return e;
 }
 
 cudaError_t launch_cfl64(const double* const f[8], const int n[3], const double ih[3], double gamma,
