@@ -442,7 +442,8 @@ int state_rate(mhd_s* m, unsigned* rate, const float* const from[8] = nullptr) {
   });
 }
 
-int fluid(mhd_s* m, int d, bool rate, int stale = mhd::kGhostAll) {
+// `begin`: the sweep is the first of a step.
+int fluid(mhd_s* m, int d, bool rate, int stale = mhd::kGhostAll, const mhd::StepControl* begin = nullptr) {
   const mhd::Box* box;
   int ka;
   int rc = sweep_frame(m, d, &box, &ka);
@@ -469,6 +470,17 @@ int fluid(mhd_s* m, int d, bool rate, int stale = mhd::kGhostAll) {
   a.err = &m->sc->err;
   a.tma_used = &staged;
   a.tile = tile_choice(m, d, false, 1);
+  // (the FP64 quotient at the head of every block costs large boxes more than
+  // the launch: 200^3 136 -> 157 us for that sweep)
+  if (begin && a.tile > 0 && ka == 0 && !rate && m->N <= 1000000) {
+    a.control = *begin;
+  } else if (begin) {
+    if ((rc = traced(m, MHD_K_CONTROL, [&] {
+           CK(mhd::launch_step_control(*begin, mhd::shared_split(m->N), m->stream));
+           return MHD_OK;
+         })))
+      return rc;
+  }
   if (m->fast == 2) {  // per-pencil freezing speeds before the sweep
     a.pencil_c = m->pencil_c;
     if ((rc = traced(m, MHD_K_CONTROL, [&] {
@@ -527,11 +539,19 @@ int magnetic(mhd_s* m, int d, int passes = 1, int stale = mhd::kGhostAll) {
 // same step and run as one launch when fusion is on (bitwise the same
 // result), unless the z sweep runs along the contiguous axis (x path 3) or
 // ghost layers must be refilled between them.
-int full_step(mhd_s* m) {
+// cfl, tau_host: the step's timestep (StepControl).
+int full_step(mhd_s* m, double cfl, double tau_host) {
   constexpr int F = mhd::kGhostFluid, B = mhd::kGhostField;  // what the sweep before has written
+  mhd::StepControl begin;
+  begin.rate = &m->sc->rate[m->rcur];
+  begin.rate_next = &m->sc->rate[1 - m->rcur];
+  begin.tau = &m->sc->tau;
+  begin.time = &m->sc->time;
+  begin.cfl = cfl;
+  begin.tau_host = tau_host;
   int rc;
   for (int d = 0; d < 2; d++) {
-    if ((rc = fluid(m, d, false, d == 0 ? mhd::kGhostAll : B))) return rc;
+    if ((rc = fluid(m, d, false, d == 0 ? mhd::kGhostAll : B, d == 0 ? &begin : nullptr))) return rc;
     if ((rc = magnetic(m, d, 1, F))) return rc;
   }
   if ((rc = fluid(m, 2, false, B))) return rc;
@@ -596,13 +616,7 @@ int make_pipeline(mhd_s* m) {
 
 int run_steps(mhd_s* m, int nsteps, double cfl) {
   for (int s = 0; s < nsteps; s++) {
-    int rc = traced(m, MHD_K_CONTROL, [&] {
-      CK(mhd::launch_step_control(&m->sc->rate[m->rcur], &m->sc->rate[1 - m->rcur], &m->sc->tau,
-                                  &m->sc->time, cfl, 0.0, mhd::shared_split(m->N), m->stream));
-      return MHD_OK;
-    });
-    if (!rc) rc = full_step(m);
-    if (rc) return rc;
+    if (int rc = full_step(m, cfl, 0.0)) return rc;
   }
   return ensure_layout(m, 0);  // consecutive steps share their x-sweep layout
 }
@@ -940,12 +954,7 @@ int mhd_step(mhd_t* m, double dt_full) {
     return MHD_OK;
   }
   if (int rc = join_pipeline(m)) return rc;
-  int rc = traced(m, MHD_K_CONTROL, [&] {
-    CK(mhd::launch_step_control(&m->sc->rate[m->rcur], &m->sc->rate[1 - m->rcur], &m->sc->tau,
-                                &m->sc->time, -1.0, 0.5 * dt_full, mhd::shared_split(m->N), m->stream));
-    return MHD_OK;
-  });
-  if (!rc) rc = full_step(m);
+  const int rc = full_step(m, -1.0, 0.5 * dt_full);
   return rc ? rc : ensure_layout(m, 0);
 }
 

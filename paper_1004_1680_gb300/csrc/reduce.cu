@@ -157,25 +157,13 @@ bool local_fields(const void* const f[8]) {
   return true;
 }
 
-__global__ void step_control_kernel(const unsigned* rate_cur, unsigned* rate_next, float* tau,
-                                    double* time, double cfl, double tau_host) {
+__global__ void step_control_kernel(StepControl c) {
   wait_for_previous();
-  double t;
-  if (cfl > 0.0) {
-    const float r = __uint_as_float(*rate_cur);
-    t = (r > 0.f && r <= FLT_MAX) ? cfl / (double)r : 0.0;  // invalid state: stand still
-  } else {
-    t = tau_host;
-  }
-  const float tf = (float)t;
-  *tau = tf;
-  *time += 2.0 * (double)tf;
-  *rate_next = 0u;
+  step_begin(c, step_tau(c));
 }
 
-cudaError_t launch_step_control(const unsigned* rate_cur, unsigned* rate_next, float* tau,
-                                double* time, double cfl, double tau_host, int split, cudaStream_t s) {
-  return launch_after(true, split, step_control_kernel, dim3(1), dim3(1), 0, s, rate_cur, rate_next, tau, time, cfl, tau_host);
+cudaError_t launch_step_control(const StepControl& c, int split, cudaStream_t s) {
+  return launch_after(true, split, step_control_kernel, dim3(1), dim3(1), 0, s, c);
 }
 
 __global__ void ens_control_kernel(const unsigned* rate_cur, unsigned* rate_next, float* tau,

@@ -99,8 +99,16 @@ __global__ void __launch_bounds__(kTileThreads, 2) fluid_tile_kernel(const __gri
   settled(base, baseA1, baseO1, p0);
   wait_for_previous();
   const float gamma = a.gamma;
-  const float c_full = *a.tau * a.box.ih[D];  // tau / h_D
-  const float c_half = 0.5f * c_full;
+  const bool begins = D == 0 && !RATE && a.control.rate;
+  __shared__ float own_tau;
+  float tau = 0.f;
+  if (!begins) {
+    tau = *a.tau;
+  } else if (tid == 0) {
+    tau = step_tau(a.control);
+    own_tau = tau;
+    if (blockIdx.x == 0 && blockIdx.z == 0) step_begin(a.control, tau);
+  }
 
   V5 f1[K + 1];  // flux1 at p0-1/2 .. p0+7/2
   V5 FR3, FL0;
@@ -170,6 +178,9 @@ __global__ void __launch_bounds__(kTileThreads, 2) fluid_tile_kernel(const __gri
     X.put(1, tid, FL0);
   }
   __syncthreads();
+  if (begins) tau = own_tau;
+  const float c_full = tau * a.box.ih[D];  // tau / h_D
+  const float c_half = 0.5f * c_full;
   V5 Rh[K], Lh[K];
   auto parked = [&](V5 (&U)[K]) {
     float4 v[5];
