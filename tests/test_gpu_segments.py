@@ -79,3 +79,28 @@ def test_ragged_ensemble_segments_match_single_boxes(mhd, xpath):
         assert torch.equal(ens.get_state(i), b.get_state()), d
         b.close()
     ens.close()
+
+
+@pytest.mark.parametrize("nx,exchanged", [(132, True), (128, False)], ids=["ragged_rows", "whole_rows"])
+def test_given_x_segments_choose_the_x_path(mhd, nx, exchanged):
+    """A given segment length of x keeps tile sweeps off: beyond 2,097,152 cells
+    rows that are not whole go through the exchanged copy, whole ones along x,
+    and the automatic choice is bitwise the requested one."""
+    dims = (nx, 132, 128)
+    x = to_gpu(ic.turbulence(dims, seed=7, dtype=torch.float64, kmin=1.0, kmax=2.0, mach=0.6))
+    out = []
+    for path in (0, 2 if exchanged else 1):
+        b = mhd.Box(*dims, gamma=G)
+        b.set_segments(nx, 0, 0)
+        b.set_xpath(path)
+        b.set_state(x)
+        b.profile(200)
+        b.run(1, 0.7)
+        assert (b.profile_read()["transpose"][0] > 0) == exchanged
+        out.append(b.get_state().clone())
+        b.set_segments(0, 0, 0)  # tiles are open again: along x unless requested otherwise
+        b.profile(200)
+        b.run(1, 0.7)
+        assert (b.profile_read()["transpose"][0] > 0) == (path == 2)
+        b.close()
+    assert torch.equal(out[0], out[1])
