@@ -13,9 +13,10 @@ namespace mhd {
 
 constexpr int kMagWarps = 8;  // interior rows of a magnetic-sweep tile
 // Rows per tile of the magnetic row sweep: 4 for rows of up to 512 cells (5
-// groups of nx/4 threads, 640 threads), 2 for 1024 cells (3 groups of 256
-// threads, 768).
-__host__ __device__ constexpr int mag_row_tile(int nx) { return nx <= 512 ? 4 : 2; }
+// groups of nx/4 threads, 640 threads), 3 below 640 (4 groups of 160, 640 again:
+// two rows leave 480 threads on an SM; sweep of 528^3 1.73 -> 1.24 ms, of 560 x
+// 300 x 200 412 -> 279 us), 2 up to 1024 cells (3 groups of 256 threads, 768).
+__host__ __device__ constexpr int mag_row_tile(int nx) { return nx <= 512 ? 4 : (nx < 640 ? 3 : 2); }
 // Estimated microseconds of the magnetic row sweep of a box (sweep_mag.cu).
 double mag_rows_us(const int n[3], int sms);
 

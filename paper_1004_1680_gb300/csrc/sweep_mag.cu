@@ -29,9 +29,11 @@ constexpr int kMagMapCache = 16;
 // the SM (measured: 1.75 us at 480 threads, 1.9 .. 2.2 at 640; tiles of two
 // rows, whose kernel has fewer registers, 3.3 at 768).
 double mag_rows_us(const int n[3], int sms) {
-  const bool four = mag_row_tile(n[0]) == 4;
-  const MagRowPlan p = four ? mag_row_plan<4>(n[0], n[1], n[2], sms) : mag_row_plan<2>(n[0], n[1], n[2], sms);
-  return p.waves * (p.L + 2) * (0.7 + 2.2e-3 * p.threads) * (four ? 1.0 : 1.4);
+  const int rows = mag_row_tile(n[0]);
+  const MagRowPlan p = rows == 4   ? mag_row_plan<4>(n[0], n[1], n[2], sms)
+                       : rows == 3 ? mag_row_plan<3>(n[0], n[1], n[2], sms)
+                                   : mag_row_plan<2>(n[0], n[1], n[2], sms);
+  return p.waves * (p.L + 2) * (0.7 + 2.2e-3 * p.threads) * (rows > 2 ? 1.0 : 1.4);
 }
 
 bool mag_chunks_qualify(int axis, const MagArgs& a) {

@@ -475,7 +475,7 @@ struct RowAdvect {
 // they read in the block's shared memory; they write only padding (the rows of v
 // and E_y are as long as the group) or nothing.
 template <int LIM, int R, bool RAG>
-__global__ void __launch_bounds__(R == 4 ? 640 : 768, 1) mag_row_kernel(const __grid_constant__ MagArgs a, int L) {
+__global__ void __launch_bounds__(R >= 3 ? 640 : 768, 1) mag_row_kernel(const __grid_constant__ MagArgs a, int L) {
   using M = MRow<R>;
   extern __shared__ __align__(128) float ms_dyn[];
   __shared__ alignas(8) unsigned long long mbarr[2];
@@ -793,7 +793,8 @@ cudaError_t launch_mag_rows_r(const MagArgs& a, cudaStream_t s) {
 
 template <int LIM>
 cudaError_t launch_mag_rows(const MagArgs& a, cudaStream_t s) {
-  return mag_row_tile(a.box.n[0]) == 4 ? launch_mag_rows_r<LIM, 4>(a, s) : launch_mag_rows_r<LIM, 2>(a, s);
+  const int rows = mag_row_tile(a.box.n[0]);
+  return rows == 4 ? launch_mag_rows_r<LIM, 4>(a, s) : rows == 3 ? launch_mag_rows_r<LIM, 3>(a, s) : launch_mag_rows_r<LIM, 2>(a, s);
 }
 
 }  // namespace mhd

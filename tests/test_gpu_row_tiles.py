@@ -40,3 +40,9 @@ def test_ragged_rows_match_the_register_sweep(mhd, dims, limiter):
         b.close()
     assert not torch.equal(out[0], x)
     assert torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("dims", [(516, 67, 60), (572, 99, 61), (636, 64, 64)])
+def test_tiles_of_three_rows_match_the_register_sweep(mhd, dims):
+    """Rows of 513 to 639 cells: a last tile of one row, of three and again of one."""
+    test_ragged_rows_match_the_register_sweep(mhd, dims, "vanleer")
