@@ -50,7 +50,10 @@ struct EnsArgs {
 // before its first access to device memory, until the kernels before it in the
 // stream have completed and their writes are visible.  It lets its own
 // dependent launch only after that wait, so at most two sweeps are on the chip
-// and no block of a third can have cached what the second one writes.
+// and no block of a third can have cached what the second one writes.  Nor may
+// the second one itself: a kernel that lets the next one in reads nothing that
+// it writes, other than past L1 (step_begin, the floor of the marching sweeps);
+// kernels that update in place let it in when they have completed.
 // (The network's kernels as well: the gradients of one 64^3 pair, 18 launches,
 // 342 -> 306 us.  Not the ensembles' launches, which a graph replays: 3 boxes 234
 // us per step, 314 with it; the blocks of a small launch, let in early, pile up

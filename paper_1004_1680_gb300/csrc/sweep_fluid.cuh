@@ -366,11 +366,15 @@ __device__ __forceinline__ void fluid_sweep_body(const FluidArgs& a, const Fluid
           bc2[0] = bprev0; bc2[1] = bprev1; bc2[2] = bprev2;
         }
       }
+      // The cells are read back past L1 (__ldcg): the next kernel is already let
+      // in, and a 32-byte piece that a row shares with another block's (rows of 236
+      // cells) must not stay in L1 as it was before that block stored its part.
       if (FLOOR && !RATE && low) {
         for (int j = 0; j < CH; j++) {
           if (!(low >> j & 1)) continue;
           const unsigned cell = ub + (unsigned)((p0 + j - 3) * sD);
-          const float o[5] = {o_rho[cell], o_md[cell], o_m1[cell], o_m2[cell], o_en[cell]};
+          const float o[5] = {__ldcg(o_rho + cell), __ldcg(o_md + cell), __ldcg(o_m1 + cell), __ldcg(o_m2 + cell),
+                              __ldcg(o_en + cell)};
           o_en[cell] = floored_energy(o, b2c[j], a.e_floor);
         }
       }
