@@ -494,8 +494,8 @@ __global__ void __launch_bounds__(MTile<LX, R>::T) mag_tile_kernel(const __grid_
         auto update = [&](float* z, int plane, float fl, float fh) {
           const float v = __fmaf_rn(-c_full, __fsub_rn(fh, fl), z[p * plane]);
           z[p * plane] = v;
-          if (p < H) z[(p + S) * plane] = v;
-          if (p >= S - H) z[(p - S) * plane] = v;
+          for (int m = p + S; m < S + H; m += S) z[m * plane] = v;  // (a pencil of 1 or 2 cells has several images)
+          for (int m = p - S; m >= -H; m -= S) z[m * plane] = v;
         };
         if (row < R) update(sa + H * Sa + row * L::AW + col, Sa, lo.x, hi.x);
         if (col < LX) update(so + H * So + row * LX + col, So, lo.y, hi.y);
