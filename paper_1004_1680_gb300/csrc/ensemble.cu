@@ -77,6 +77,7 @@ struct mhd_ens_s {
   int xpath = 2;
   int segdiv = 1;
   float p_floor = 0.f;
+  int device = 0;  // the device that holds the arena
   float* tau = nullptr;
   unsigned* rate[2] = {nullptr, nullptr};
   double* time = nullptr;
@@ -460,7 +461,7 @@ mhd_ens_t* mhd_ens_create(int nbox, const int* dims3, double gamma) {
   const mhd::Box big = mhd::make_box((int)std::min<long long>(biggest, 1 << 30), 1, 1);
   const int nblk = mhd::diag_blocks(big);
   cudaError_t ce;
-  if ((ce = mhd::prepare_sweep_kernels()) != cudaSuccess ||
+  if ((ce = cudaGetDevice(&e->device)) != cudaSuccess || (ce = mhd::prepare_sweep_kernels()) != cudaSuccess ||
       (ce = cudaMalloc(&e->arena, sizeof(float) * (size_t)off * 16)) != cudaSuccess ||
       (ce = cudaMalloc(&e->boxes_d, sizeof(mhd::EnsBox) * nbox)) != cudaSuccess ||
       (ce = cudaMalloc(&e->tau, sizeof(float) * nbox)) != cudaSuccess ||
@@ -520,7 +521,7 @@ int mhd_ens_set_state(mhd_ens_t* e, int b, const float* const f[8], int on_devic
   CKE(cudaMemsetAsync(e->time + b, 0, sizeof(double), e->stream));
   const float* p[8];
   box_ptrs(e, b, p);
-  if (on_device && mhd::local_fields(reinterpret_cast<const void* const*>(f))) {  // copied and rated in one pass
+  if (on_device && mhd::local_fields(reinterpret_cast<const void* const*>(f), e->device)) {  // copied and rated in one pass
     float* out[8];
     for (int q = 0; q < 8; q++) out[q] = e->cur[q] + x.offset;
     CKE(mhd::launch_cfl_rate(f, plain_box(x), (float)e->gamma, e->rate[e->rcur] + b, e->stream, nullptr, out));
@@ -540,7 +541,7 @@ int mhd_ens_get_state(const mhd_ens_t* e, int b, float* const f[8], int on_devic
   if (e->layout) return mhd::set_error(MHD_E_ARG, "mhd_ens_get_state", "internal: exchanged layout");
   const mhd::EnsBox& x = e->boxes[b];
   const size_t bytes = sizeof(float) * (size_t)x.n[0] * x.n[1] * x.n[2];
-  if (on_device && mhd::local_fields(reinterpret_cast<const void* const*>(f))) {
+  if (on_device && mhd::local_fields(reinterpret_cast<const void* const*>(f), e->device)) {
     const float* p[8];
     box_ptrs(e, b, p);
     CKE(mhd::launch_copy_fields(p, f, (long long)x.n[0] * x.n[1] * x.n[2], e->stream));

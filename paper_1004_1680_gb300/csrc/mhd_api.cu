@@ -95,7 +95,8 @@ struct mhd_s {
   cudaStream_t stream = nullptr;
   int seg[3][3];        // per axis: segment length of its fluid, magnetic and fused magnetic sweeps
   bool seg_set[3] = {false, false, false};  // segments given by mhd_set_segments
-  int sms = 0;          // multiprocessors of the device (segment choice)
+  int device = 0;       // the device that holds the arena
+  int sms = 0;          // its multiprocessors (segment choice)
   // tracing: event pairs around launches (see mhd_profile)
   std::vector<cudaEvent_t> ev;
   std::vector<int> ev_kind;
@@ -772,11 +773,8 @@ mhd_t* mhd_create(int nx, int ny, int nz, double gamma) {
   m->zbox.stride[2] = (long long)nz * ny;
   set_geometry(m);
   m->xpath = auto_xpath(m);
-  {
-    int dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess)
-      cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, dev);
-  }
+  if (cudaGetDevice(&m->device) == cudaSuccess)
+    cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, m->device);
   const int nblk = mhd::diag_blocks(m->box);
   if ((e = cudaMalloc(&m->sc, sizeof(Scalars))) != cudaSuccess ||
       (e = cudaMalloc(&m->diag_partial, sizeof(double) * mhd::kDiagSlots * nblk)) != cudaSuccess ||
@@ -893,7 +891,7 @@ int mhd_set_state(mhd_t* m, const float* const f[8], int on_device) {
     std::swap(m->spare[5], m->spare[4 + a]);
     m->layout = 0;
   }
-  const bool local = on_device && mhd::local_fields(reinterpret_cast<const void* const*>(f));
+  const bool local = on_device && mhd::local_fields(reinterpret_cast<const void* const*>(f), m->device);
   CK(cudaMemsetAsync(m->sc, 0, sizeof(Scalars), m->stream));
   m->rcur = 0;
   if (local && !any_bc(m)) return state_rate(m, &m->sc->rate[0], f);
@@ -914,7 +912,7 @@ int mhd_get_state(const mhd_t* m, float* const f[8], int on_device) {
   const size_t bytes = sizeof(float) * (size_t)m->N;
   if (m->layout) return fail(MHD_E_ARG, "internal: state left in the exchanged layout");
   if (int rc = join_pipeline(const_cast<mhd_s*>(m))) return rc;
-  if (on_device && mhd::local_fields(reinterpret_cast<const void* const*>(f))) {
+  if (on_device && mhd::local_fields(reinterpret_cast<const void* const*>(f), m->device)) {
     const float* cf[8];
     field_ptrs(m, cf);
     CK(mhd::launch_copy_fields(cf, f, m->N, m->stream));

@@ -471,7 +471,16 @@ struct CopyArgs {
   float* out[8];
 };
 cudaError_t launch_copy_fields(const float* const in[8], float* const out[8], long long N, cudaStream_t s);
-bool local_fields(const void* const f[8]);
+// Whether a kernel on the current device `dev` can copy between a box of device
+// `home` and 8 fields, field q on device device_of(q) (-1: host or managed
+// memory): only where all of it is memory of that device.
+template <class DeviceOf>
+inline bool all_on_device(int dev, int home, DeviceOf device_of) {
+  bool local = dev == home;
+  for (int q = 0; q < 8 && local; q++) local = device_of(q) == dev;
+  return local;
+}
+bool local_fields(const void* const f[8], int home);
 // device-side step control: tau = cfl / rate_cur (or the given tau if cfl<0),
 // time += 2 tau, rate_next = 0
 cudaError_t launch_step_control(const StepControl& c, int split, cudaStream_t s);

@@ -140,21 +140,20 @@ cudaError_t launch_copy_fields(const float* const in[8], float* const out[8], lo
   return cudaGetLastError();
 }
 
-// Whether kernels of the current device can read and write all 8 fields
-// directly: memory of this device (another device's, or host memory, goes
-// through cudaMemcpyAsync).
-bool local_fields(const void* const f[8]) {
+// Whether a kernel of the current device can copy between a box that lives on
+// device `home` and the 8 fields directly (another device's memory, or the
+// host's, goes through cudaMemcpyAsync).
+bool local_fields(const void* const f[8], int home) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
-  for (int q = 0; q < 8; q++) {
+  return all_on_device(dev, home, [&](int q) {
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, f[q]) != cudaSuccess) {
       cudaGetLastError();
-      return false;
+      return -1;
     }
-    if (at.type != cudaMemoryTypeDevice || at.device != dev) return false;
-  }
-  return true;
+    return at.type == cudaMemoryTypeDevice ? at.device : -1;
+  });
 }
 
 __global__ void step_control_kernel(StepControl c) {
