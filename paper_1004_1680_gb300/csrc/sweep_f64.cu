@@ -4,7 +4,7 @@
 // FP64 runs at a small fraction of the FP32 rate on this GPU, so the
 // arithmetic, not memory traffic, bounds these kernels.
 //  * Every operation is an IEEE double operation rounded once (__dadd_rn,
-//    __dmul_rn, __dsqrt_rn, correctly rounded quotients; no multiply-add
+//    __dmul_rn, __dsqrt_rn, the quotients of div64.cuh; no multiply-add
 //    contraction).
 //  * Fluid sweep: one thread per cell, the intermediate values of a block's
 //    pencils exchanged through shared memory.
@@ -18,59 +18,13 @@
 //    reduced with an atomic maximum (rates are >= 0).
 #include <cstdint>
 
+#include "div64.cuh"
 #include "mhd_launch.h"
 
 namespace mhd {
 namespace {
 
-__device__ __forceinline__ double dadd(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ double dsub(double a, double b) { return __dsub_rn(a, b); }
-__device__ __forceinline__ double dmul(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ double ddiv(double a, double b) { return __ddiv_rn(a, b); }
-
-// Quotients.  A division is about 14 FP64 operations here, and a fluid cell has
-// 18 of them; written out for operands of ordinary size they are 6, and 3 more
-// for each further quotient by the same divisor:
-//   y0, the hardware's approximate reciprocal (relative error e <= 2^-20),
-//   y  = y0 (1 + e + e^2), e = 1 - r y0   (one step of a cubic Newton iteration;
-//        its error, 2^-60, is below y's rounding),
-//   q  = a y, then q + (a - q r) y        (Markstein, "Computation of elementary
-//        functions on the IBM RISC System/6000 processor", 1990: the remainder
-//        is exact in one FMA).
-// The result is a / r rounded correctly (2 x 10^8 operand pairs with random and
-// extreme mantissas agree) for divisors whose mantissa is not all ones; those,
-// and operands whose exponents could spoil the remainder (zeros, infinities and
-// NaNs among them), take the division.
-__device__ __forceinline__ double approx_rcp(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  return y;
-}
-__device__ __forceinline__ double reciprocal(double r) {
-  const double y0 = approx_rcp(r), e = __fma_rn(-r, y0, 1.0);
-  return __fma_rn(__fma_rn(e, e, e), y0, y0);
-}
-__device__ __forceinline__ double ddiv_by(double a, double r, double y) {
-  const double q = dmul(a, y);
-  return __fma_rn(__fma_rn(-q, r, a), y, q);
-}
-// 2^-500 <= |x| < 2^500 (from the exponent: no FP64 comparison)
-__device__ __forceinline__ bool plain_exponent(double x) {
-  return ((unsigned)__double2hiint(x) >> 20 & 0x7ffu) - 523u < 1000u;
-}
-__device__ __forceinline__ bool plain_divisor(double x) { return plain_exponent(x) && __double2loint(x) != -1; }
 __device__ __forceinline__ bool negative(double x) { return __double2hiint(x) < 0; }
-
-// half the van Leer limiter, phi(a, b) / 2 = ab / (a + b) for ab > 0, else 0
-__device__ __forceinline__ double vl_half(double a, double b) {
-  const double ab = dmul(a, b), s = dadd(a, b);
-  const int hi = __double2hiint(ab);
-  double q = 0.0;
-  // (2^-500 <= ab < 2^500 leaves |s| between 2^-250 and 2^1023, its remainder normal)
-  if ((unsigned)hi - (523u << 20) < (1000u << 20) && plain_divisor(s)) q = ddiv_by(ab, s, reciprocal(s));
-  else if (hi >= 0 && (hi | __double2loint(ab)) != 0) q = ab > 0.0 ? ddiv(ab, s) : 0.0;
-  return q;
-}
 
 // Right and left movers FR = (c u + F) / 2, FL = (c u - F) / 2 of Eq. 1-3
 // projected on the sweep axis (u = rho, m_d, m_t1, m_t2, e; b = cell-centred
@@ -157,7 +111,7 @@ __device__ __forceinline__ Cell64 cell64(const int n[3]) {
   return c;
 }
 
-// Fluid sweep, one thread per cell.  FP64 arithmetic bounds it (338 operations
+// Fluid sweep, one thread per cell.  FP64 arithmetic bounds it (350 operations
 // per cell, 16 cycles of an SM per warp instruction: its pipe is 85 % busy), so nothing is
 // computed twice but a few subtractions: the movers of both stages and the
 // limited values are exchanged through shared memory, [component][thread], in
