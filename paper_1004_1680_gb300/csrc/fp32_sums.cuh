@@ -24,6 +24,14 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 // Two fields at a time, on packed FP32 (each element rounded as the scalar
 // operation would round it): 13 instructions for two values.
 constexpr int kWin = 256;
+// Grid of the kernels whose threads add their share of n < 2^31 values into one
+// window each (block_totals): enough blocks to read at full rate and few FP64
+// atomics, but no thread with more than kWin values (beyond 39.8 M).
+constexpr int kSumThreads = 256;
+inline int sum_blocks(long long n) {
+  const long long all = (n + kSumThreads - 1) / kSumThreads, most = 152 * 4, least = (all + kWin - 1) / kWin;
+  return (int)(all < 1 ? 1 : (all < most ? all : (least > most ? least : most)));
+}
 struct FWin2 {
   float2 h, l, t;
 };

@@ -178,7 +178,6 @@ __global__ void normalize_kernel(CP8 s, int N, F8 mu, F8 isig, __nv_bfloat16* x,
 // (An FP64 sum and shuffle tree per warp and an atomic per warp took 58 us on
 // a 64^3 grid.)  A block with infinities or sums near the end of FP32's range
 // takes the threads' FP64 totals `exact(q)` instead.
-constexpr int kSumThreads = 256;
 template <int NP, class Exact>
 __device__ __forceinline__ void block_totals(FWin2 (&w)[NP], int n, double* sums, Exact exact) {
   __shared__ float2 sm[kSumThreads / 32][NP][3];
@@ -227,7 +226,7 @@ __global__ void __launch_bounds__(kSumThreads) project_sums_kernel(const float* 
   wait_for_previous();
   FWin2 w[3];
   for (int k = 0; k < 3; k++) w[k].h = w[k].l = w[k].t = f2(0.f);
-  for (int c = blockIdx.x * kSumThreads + threadIdx.x; c < N; c += gridDim.x * kSumThreads) {
+  for (unsigned c = blockIdx.x * kSumThreads + threadIdx.x; c < (unsigned)N; c += gridDim.x * kSumThreads) {
     float v[8];
     load_cell(y, c, v, vec);
     fwin_add(w[0], make_float2(__fmul_rn(sc.v[0], v[0]), __fmul_rn(sc.v[1], v[1])));
@@ -236,7 +235,7 @@ __global__ void __launch_bounds__(kSumThreads) project_sums_kernel(const float* 
   }
   block_totals(w, 5, sums, [&](int q) {
     double a = 0.0;
-    for (int c = blockIdx.x * kSumThreads + threadIdx.x; c < N; c += gridDim.x * kSumThreads)
+    for (unsigned c = blockIdx.x * kSumThreads + threadIdx.x; c < (unsigned)N; c += gridDim.x * kSumThreads)
       a += __fmul_rn(sc.v[q], y[(size_t)c * 8 + q]);
     return a;
   });
@@ -297,7 +296,7 @@ __global__ void __launch_bounds__(kSumThreads) loss_kernel(CP8 d, CP8 t, int N, 
   FWin2 s[4];
   for (int k = 0; k < 4; k++) s[k].h = s[k].l = s[k].t = f2(0.f);
   bool small = false;  // a square whose error word would underflow
-  for (int c = blockIdx.x * kSumThreads + threadIdx.x; c < N; c += gridDim.x * kSumThreads) {
+  for (unsigned c = blockIdx.x * kSumThreads + threadIdx.x; c < (unsigned)N; c += gridDim.x * kSumThreads) {
 #pragma unroll
     for (int k = 0; k < 4; k++) {
       const float2 diff = make_float2(d.p[2 * k][c] - t.p[2 * k][c], d.p[2 * k + 1][c] - t.p[2 * k + 1][c]);
@@ -322,7 +321,7 @@ __global__ void __launch_bounds__(kSumThreads) loss_kernel(CP8 d, CP8 t, int N, 
   __syncthreads();
   block_totals(s, 8, tot, [&](int q) {
     double a = 0.0;
-    for (int c = blockIdx.x * kSumThreads + threadIdx.x; c < N; c += gridDim.x * kSumThreads) {
+    for (unsigned c = blockIdx.x * kSumThreads + threadIdx.x; c < (unsigned)N; c += gridDim.x * kSumThreads) {
       const double x = (double)(d.p[q][c] - t.p[q][c]) * w.scale[q];
       a += x * x;
     }
@@ -340,14 +339,14 @@ __global__ void __launch_bounds__(kSumThreads) grad_sums_kernel(CP8 g, int N, do
   wait_for_previous();
   FWin2 w[3];
   for (int k = 0; k < 3; k++) w[k].h = w[k].l = w[k].t = f2(0.f);
-  for (int c = blockIdx.x * kSumThreads + threadIdx.x; c < N; c += gridDim.x * kSumThreads) {
+  for (unsigned c = blockIdx.x * kSumThreads + threadIdx.x; c < (unsigned)N; c += gridDim.x * kSumThreads) {
     fwin_add(w[0], make_float2(g.p[0][c], g.p[1][c]));
     fwin_add(w[1], make_float2(g.p[2][c], g.p[3][c]));
     fwin_add(w[2], make_float2(g.p[4][c], 0.f));
   }
   block_totals(w, 5, sums, [&](int q) {
     double a = 0.0;
-    for (int c = blockIdx.x * kSumThreads + threadIdx.x; c < N; c += gridDim.x * kSumThreads) a += g.p[q][c];
+    for (unsigned c = blockIdx.x * kSumThreads + threadIdx.x; c < (unsigned)N; c += gridDim.x * kSumThreads) a += g.p[q][c];
     return a;
   });
 }
@@ -457,13 +456,6 @@ __global__ void adam_kernel(float* p, const float* g, float* m, float* v, int n,
 int blocks(long long n) {
   long long b = (n + 255) / 256;
   return (int)(b > 152 * 32 ? 152 * 32 : (b < 1 ? 1 : b));
-}
-
-// grid of the kernels that end in block_totals: enough blocks to read at full
-// rate, few FP64 atomics
-int sum_blocks(long long n) {
-  const long long b = (n + kSumThreads - 1) / kSumThreads;
-  return (int)(b > 152 * 4 ? 152 * 4 : (b < 1 ? 1 : b));
 }
 
 bool vec16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }

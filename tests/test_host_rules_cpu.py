@@ -1,5 +1,6 @@
 """Host-side rules of the library, compiled from its headers into a small program
-that needs no GPU: which copies a kernel may make."""
+that needs no GPU: which copies a kernel may make, and how many values a thread
+adds into one window of FP32 words."""
 import os
 import subprocess
 
@@ -9,12 +10,16 @@ from paper_1004_1680_gb300 import build
 
 PROGRAM = r"""
 #include <cstdio>
+#include "fp32_sums.cuh"
 #include "mhd_launch.h"
 int main() {
   // fields on device a (all but field 5) and b (field 5), current device, the box's device
   const int cases[][4] = {{0, 0, 0, 0}, {1, 1, 1, 0}, {1, 1, 0, 1}, {0, 0, 1, 0}, {0, 1, 0, 0}, {-1, -1, 0, 0}, {0, -1, 0, 0}};
   for (auto& c : cases)
     std::printf("local %d\n", (int)mhd::all_on_device(c[2], c[3], [&](int q) { return q == 5 ? c[1] : c[0]; }));
+  for (long long n : {0LL, 1LL, 255LL, 256LL, 257LL, 155648LL, 155649LL, 262144LL, 39845888LL, 39845889LL, 39911425LL,
+                      134217728LL, 2147483647LL})
+    std::printf("sums %lld %d %d %d\n", n, mhd::sum_blocks(n), mhd::kSumThreads, mhd::kWin);
   return 0;
 }
 """
@@ -35,3 +40,13 @@ def test_fields_are_copied_by_a_kernel_only_on_the_boxs_own_device(printed):
     agreeing does not help: the kernel would read another device's memory), a
     field elsewhere, or host memory."""
     assert [ln for ln in printed if ln.startswith("local")] == [f"local {v}" for v in (1, 0, 0, 0, 0, 0, 0)]
+
+
+def test_no_thread_adds_more_values_than_a_window_holds(printed):
+    """The error bound of the FP32 words is for windows of kWin values."""
+    rows = [tuple(int(v) for v in ln.split()[1:]) for ln in printed if ln.startswith("sums")]
+    assert len(rows) == 13
+    for n, blocks, threads, win in rows:
+        assert blocks >= 1 and -(-n // (blocks * threads)) <= win
+    grid = {r[0]: r[1] for r in rows}  # one grid from 155,648 values to 39.8 M
+    assert grid[262144] == grid[39845888] == 608 and grid[2147483647] == 32768
