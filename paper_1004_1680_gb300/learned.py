@@ -70,7 +70,8 @@ class CorrectionNet:
     def backward(self, gy: torch.Tensor, acts, n):
         """gy: (cells, 8) BF16 gradient of the loss w.r.t. y; fills self.grads."""
         sizes = [p.numel() for p in self.params]
-        flat = torch.zeros(sum(sizes), device=gy.device)  # every gradient, cleared at once
+        # every gradient, cleared at once (in the parameters' type: the library adds FP32)
+        flat = torch.zeros(sum(sizes), dtype=self.params[0].dtype, device=gy.device)
         self.grads = [v.view(p.shape) for v, p in zip(flat.split(sizes), self.params)]
         L = len(LAYERS)
         scratch = [torch.empty_like(acts[1]) for _ in range(2)]
