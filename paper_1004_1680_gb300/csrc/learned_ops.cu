@@ -516,7 +516,7 @@ int mhd_restrict(int nx, int ny, int nz, int r, const float* const fine[8], floa
       if (reinterpret_cast<uintptr_t>(fine[q]) % bytes) return false;
     return true;
   };
-  const int grid = (int)std::min<long long>((N + 127) / 128, 152 * 64);
+  const int grid = (int)std::max<long long>(1, std::min<long long>((N + 127) / 128, 152 * 64));  // (1: no cells)
   cudaStream_t st = (cudaStream_t)stream;
   if (r == 4 && aligned(16)) restrict_kernel<4><<<grid, 128, 0, st>>>(cp8(fine), nx, ny, nz, r, p8(coarse));
   else if (r == 2 && aligned(8)) restrict_kernel<2><<<grid, 128, 0, st>>>(cp8(fine), nx, ny, nz, r, p8(coarse));
