@@ -229,12 +229,16 @@ int choose_seg(const mhd_s* m, int d, int kind) {
 }
 
 // Estimated microseconds of a y or z sweep within a step, from measured times:
-// a marching sweep takes 3 us and (positions a thread marches) x (time per
+// a marching sweep takes its launch (below) and (positions a thread marches) x (time per
 // position), the latter growing with the blocks that share an SM (0.5 us for
 // one fluid block of 4 warps, 0.98 us for 4; 0.46 and 0.56 us for one or two
 // magnetic blocks; the fused magnetic pair 0.71 and 0.87 us); a tile sweep
 // takes a time per cell once it fills the chip (21 ps fluid, 19 ps magnetic;
-// its launch overlaps the sweep before).  Measured alone at 96^3: fluid 21 us
+// its launch overlaps the sweep before), for every position that it computes:
+// short pencils that are not a multiple of 4 cells cost several times their
+// cells (sums of the two z sweeps of a step at 1024 x 1024 x n, tile and marching:
+// n = 1 349 and 166 us, 2 356 and 242, 5 426 and 255, 9 582 and 337, but 4 123 and
+// 247, 8 228 and 330).  Measured alone at 96^3: fluid 21 us
 // tile, 31 us marching, magnetic 18 and 21 (a step 182 us with both tiles, 204
 // with marching magnetic sweeps); at 128^3: 44 and 39, 39 and 25.
 double march_us(const mhd_s* m, int d, bool mag, int passes) {
@@ -243,10 +247,23 @@ double march_us(const mhd_s* m, int d, bool mag, int passes) {
   const double blocks = (double)((nA + 31) / 32) * ((nO + W - 1) / W) * (double)m->n[d] / seg /
                         (m->sms > 0 ? m->sms : 152);  // per SM
   const double b = std::min(std::ceil(blocks), (double)resident), waves = std::max(1.0, blocks / resident);
-  if (!mag) return 3.0 + (seg + 7) * (0.5 + 0.03 * b * b) * waves;
+  // What the launch costs a fluid sweep: 7 us for pencils under 16 cells, which are not
+  // staged (neither it nor the next one overlaps: 256 x 256 x 3 alone 14.4 us against
+  // 16.8 by tiles, the step the same); 6 in boxes below 1.4 M cells, where one among
+  // tile sweeps keeps them from overlapping (224 x 146 x 33: 26.7 us alone either
+  // way, a step 217 us with tiles and 230 marching); 3 beyond.  Of 270 random boxes
+  // of 80 .. 252 x 17 .. 149 x 17 .. 149 cells 40 gain 1.5 to 14 % over the estimate
+  // without padding, one loses more than 1.5 % (2.6 %).
+  const double launch = m->n[d] < 16 ? 7.0 : (m->N < 1400000 ? 6.0 : 3.0);
+  if (!mag) return launch + (seg + 7) * (0.5 + 0.03 * b * b) * waves;
   return 3.0 + (passes == 2 ? (seg + 14) * (0.55 + 0.16 * b) : (seg + 7) * (0.36 + 0.1 * b)) * waves;
 }
-double tile_us(const mhd_s* m, bool mag) { return (mag ? 19e-6 : 21e-6) * (double)m->N; }
+int fluid_tile_threads(const mhd_s* m, int d) { return m->n[d] > 64 ? 256 : 128; }
+double tile_us(const mhd_s* m, int d, bool mag) {
+  const double cells = (double)m->N;
+  return mag ? 19e-6 * cells * mhd::mag_tile_padding(m->n[d])
+             : 21e-6 * cells * mhd::fluid_tile_padding(d, m->n[d], fluid_tile_threads(m, d));
+}
 
 // Tile sweep or not, along axis d of a box in the plain layout: 0, or the tile
 // argument of FluidArgs / MagArgs (-1: the magnetic row sweep).  Along y and z by the estimates above.
@@ -274,8 +291,8 @@ int tile_choice(const mhd_s* m, int d, bool mag, int passes) {
     return fits && mhd::mag_rows_us(m->n, m->sms > 0 ? m->sms : 152) < 15e-6 * (double)m->N ? -1 : shape;
   }
   if (mag && passes == 2 && m->n[d] > mhd::kMTileWhole) return 0;
-  if (tile_us(m, mag) * (passes == 2 ? 1.3 : 1.0) >= march_us(m, d, mag, passes)) return 0;
-  return mag ? shape : (m->n[d] > 64 ? 256 : 128);
+  if (tile_us(m, d, mag) * (passes == 2 ? 1.3 : 1.0) >= march_us(m, d, mag, passes)) return 0;
+  return mag ? shape : fluid_tile_threads(m, d);
 }
 
 // Whether the two magnetic z sweeps in the middle of a step run as one
@@ -283,7 +300,7 @@ int tile_choice(const mhd_s* m, int d, bool mag, int passes) {
 // for the fused tile sweep (96^3: 2 x 21 us against 41 us, 64^3: 2 x 12 and 34).
 bool fuse_z_pair(const mhd_s* m) {
   if (m->n[2] <= mhd::kMTileWhole || !tile_choice(m, 2, true, 1)) return true;
-  return 2.0 * tile_us(m, true) >= march_us(m, 2, true, 2);
+  return 2.0 * tile_us(m, 2, true) >= march_us(m, 2, true, 2);
 }
 
 // Bracket the launches issued by `body` with an event pair when tracing.

@@ -167,6 +167,15 @@ __host__ __device__ inline MagTile mag_tile_split(int nD) {
   s.segs = (nD + s.out - 1) / s.out;
   return s;
 }
+// Positions that a tile sweep along a pencil of nD cells computes per cell of
+// it: the fluid sweep's groups of 4 cells and halo threads (12 for a pencil of
+// one cell, 1 for whole pencils of a multiple of 4), the magnetic sweep's groups
+// of 4 edges of a whole pencil.
+inline double fluid_tile_padding(int axis, int nD, int threads) {
+  const FluidTile t = fluid_tile_split(axis, nD, threads);
+  return (double)t.td * kTileCells * t.segs / nD;
+}
+inline double mag_tile_padding(int nD) { return nD <= kMTileWhole ? (nD + 3) / 4 * 4.0 / nD : 1.0; }
 
 // What a step begins with: its sweep step tau = cfl / rate (0 for an invalid
 // state: stand still), or tau_host where cfl <= 0, the time, and the next CFL

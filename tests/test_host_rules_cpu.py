@@ -1,6 +1,6 @@
 """Host-side rules of the library, compiled from its headers into a small program
-that needs no GPU: which copies a kernel may make, and how many values a thread
-adds into one window of FP32 words."""
+that needs no GPU: which copies a kernel may make, how many values a thread
+adds into one window of FP32 words, and what a tile sweep computes beyond its cells."""
 import os
 import subprocess
 
@@ -20,6 +20,9 @@ int main() {
   for (long long n : {0LL, 1LL, 255LL, 256LL, 257LL, 155648LL, 155649LL, 262144LL, 39845888LL, 39845889LL, 39911425LL,
                       134217728LL, 2147483647LL})
     std::printf("sums %lld %d %d %d\n", n, mhd::sum_blocks(n), mhd::kSumThreads, mhd::kWin);
+  for (int n : {1, 2, 3, 4, 5, 8, 9, 32, 40, 41, 96, 98, 130})
+    std::printf("pad %d %.6f %.6f %.6f\n", n, mhd::fluid_tile_padding(2, n, n > 64 ? 256 : 128),
+                mhd::fluid_tile_padding(0, (n + 3) / 4 * 4, 128), mhd::mag_tile_padding(n));
   return 0;
 }
 """
@@ -50,3 +53,14 @@ def test_no_thread_adds_more_values_than_a_window_holds(printed):
         assert blocks >= 1 and -(-n // (blocks * threads)) <= win
     grid = {r[0]: r[1] for r in rows}  # one grid from 155,648 values to 39.8 M
     assert grid[262144] == grid[39845888] == 608 and grid[2147483647] == 32768
+
+
+def test_tile_estimates_count_what_a_block_computes(printed):
+    """Whole pencils of a multiple of 4 cells have no padding; others a halo thread
+    of 4 cells at each end of every segment."""
+    rows = {int(ln.split()[1]): [float(v) for v in ln.split()[2:]] for ln in printed if ln.startswith("pad")}
+    z = {n: 4 * (-(-n // 4) + 2) / n for n in (1, 2, 3, 5, 9, 41)}
+    z.update({4: 1, 8: 1, 32: 1, 40: 1, 96: 1, 98: 4 * 27 / 98, 130: 2 * 4 * 19 / 130})
+    mag = {n: -(-n // 4) * 4 / n if n <= 40 else 1 for n in rows}
+    for n, (fluid_z, fluid_x, m) in rows.items():
+        assert fluid_z == pytest.approx(z[n], abs=1e-6) and fluid_x == 1.0 and m == pytest.approx(mag[n], abs=1e-6)
