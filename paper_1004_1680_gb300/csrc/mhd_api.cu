@@ -115,16 +115,23 @@ struct mhd_s {
 
 namespace {
 
-// x sweeps run directly along x (row or tile sweeps) wherever staged sweeps
+// x sweeps run directly along x (row or tile sweeps) where staged sweeps
 // are on, the freezing speed is one of its own per cell, and either no segment
 // length of x is given (which keeps tiles off) or the rows are whole for both row
 // sweeps; otherwise they go through the exchanged layout once the state no longer
 // fits in L2 (the pencil sweeps along x read 32 different lines per warp and
 // position, which only L2 can absorb: 200^3 in x segments of 100 cells 2739 us per
 // step along x, 1255 exchanged; 132 x 132 x 128 918 and 582).
+// Rows of more than 1024 cells have no row sweep, only tiles: large boxes of them go
+// through the exchanged layout too where its magnetic sweep is staged (ms per step
+// along x and exchanged: 1280 x 256 x 256 9.30 and 8.81, 2048 x 256 x 256 14.5 and
+// 14.0, 2048 x 128 x 128 3.86 and 3.75, 4096 x 256 x 256 28.3 and 27.3, 8192 x 32 x 32
+// 1.17 and 1.16; but 2048 x 64 x 32 0.603 and 0.611, 1500 x 300 x 200 10.5 and 10.6,
+// 2048 x 2048 x 2 3.28 and 3.54).
 int auto_xpath(const mhd_s* m) {
   const bool rows = m->n[0] % 128 == 0 && m->n[0] <= 1024 && m->n[1] % mhd::mag_row_tile(m->n[0]) == 0 && m->n[2] >= 2;
-  if (m->tma && m->fast != 2 && (rows || !m->seg_set[0])) return 1;
+  const bool exchanged = m->n[0] > 1024 && m->n[1] % 32 == 0 && m->n[2] % mhd::kMagWarps == 0 && m->N >= (8LL << 20);
+  if (m->tma && m->fast != 2 && (rows || !m->seg_set[0])) return exchanged ? 2 : 1;
   return m->N * 32LL > (64LL << 20) ? 2 : 1;
 }
 
