@@ -435,8 +435,6 @@ template <int LIM>
 cudaError_t launch_mag_t(int axis, const MagArgs& a, cudaStream_t s);
 template <int LIM>
 cudaError_t prepare_mag_t();
-template <int LIM, int FRZ>
-cudaError_t prepare_fluid_t();
 extern template cudaError_t launch_fluid_t<0, 0>(int, bool, const FluidArgs&, cudaStream_t);
 extern template cudaError_t launch_fluid_t<1, 0>(int, bool, const FluidArgs&, cudaStream_t);
 extern template cudaError_t launch_fluid_t<2, 0>(int, bool, const FluidArgs&, cudaStream_t);
@@ -445,10 +443,6 @@ extern template cudaError_t launch_fluid_t<0, 2>(int, bool, const FluidArgs&, cu
 extern template cudaError_t launch_mag_t<0>(int, const MagArgs&, cudaStream_t);
 extern template cudaError_t launch_mag_t<1>(int, const MagArgs&, cudaStream_t);
 extern template cudaError_t launch_mag_t<2>(int, const MagArgs&, cudaStream_t);
-extern template cudaError_t prepare_fluid_t<0, 0>();
-extern template cudaError_t prepare_fluid_t<1, 0>();
-extern template cudaError_t prepare_fluid_t<2, 0>();
-extern template cudaError_t prepare_fluid_t<0, 1>();
 extern template cudaError_t prepare_mag_t<0>();
 extern template cudaError_t prepare_mag_t<1>();
 extern template cudaError_t prepare_mag_t<2>();

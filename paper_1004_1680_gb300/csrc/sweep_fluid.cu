@@ -80,7 +80,6 @@ bool make_fluid_maps(int axis, const FluidArgs& a, FluidMaps* out) {
 }
 
 template cudaError_t launch_fluid_t<0, 0>(int, bool, const FluidArgs&, cudaStream_t);
-template cudaError_t prepare_fluid_t<0, 0>();
 
 cudaError_t launch_fluid(int axis, bool rate, const FluidArgs& a, cudaStream_t s) {
   if (a.fast == 1) return launch_fluid_t<0, 1>(axis, rate, a, s);

@@ -481,12 +481,4 @@ cudaError_t launch_fluid_t(int axis, bool rate, const FluidArgs& a, cudaStream_t
   return cudaGetLastError();
 }
 
-// The tile kernels' shared-memory limits (once per device, before any launch).
-template <int LIM, int FRZ>
-cudaError_t prepare_fluid_t() {
-  cudaError_t e = prepare_fluid_tile<LIM, FRZ, true>();
-  if (e == cudaSuccess) e = prepare_fluid_tile<LIM, FRZ, false>();
-  return e;
-}
-
 }  // namespace mhd

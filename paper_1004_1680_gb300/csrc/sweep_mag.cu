@@ -96,10 +96,6 @@ template cudaError_t prepare_mag_t<0>();
 
 cudaError_t prepare_sweep_kernels() {
   cudaError_t e = prepare_mag_t<0>();
-  if (e == cudaSuccess) e = prepare_fluid_t<0, 0>();
-  if (e == cudaSuccess) e = prepare_fluid_t<1, 0>();
-  if (e == cudaSuccess) e = prepare_fluid_t<2, 0>();
-  if (e == cudaSuccess) e = prepare_fluid_t<0, 1>();
   if (e == cudaSuccess) e = prepare_mag_t<1>();
   if (e == cudaSuccess) e = prepare_mag_t<2>();
   return e;

@@ -5,6 +5,5 @@
 namespace mhd {
 
 template cudaError_t launch_fluid_t<0, 1>(int, bool, const FluidArgs&, cudaStream_t);
-template cudaError_t prepare_fluid_t<0, 1>();
 
 }  // namespace mhd
