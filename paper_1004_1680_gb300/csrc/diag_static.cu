@@ -16,12 +16,11 @@
 
 namespace {
 
-// The diagnostics grid never has more blocks than kDiagMaxBlocks (diag_blocks
-// caps it), so the partials of any box fit; the last 16 doubles take the 10
-// results.
-constexpr int kStaticDiagBlocks = mhd::kDiagMaxBlocks;
+// The diagnostics grid never has more blocks than kDiagGrid (diag_blocks caps
+// it), so the partials of any box fit; the last 16 doubles take the 10 results.
+constexpr int kStaticDiagBlocks = mhd::kDiagGrid;
 constexpr int kStaticDiagDoubles = kStaticDiagBlocks * mhd::kDiagSlots + 16;
-__device__ __align__(256) double g_diag_scratch[kStaticDiagDoubles];  // 194 KiB per GPU
+__device__ __align__(256) double g_diag_scratch[kStaticDiagDoubles];  // 48 KiB per GPU
 
 // Device address of g_diag_scratch in the context current on this thread.
 // In host code the name g_diag_scratch is only a host-side stand-in, not a

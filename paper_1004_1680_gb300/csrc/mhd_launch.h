@@ -493,7 +493,6 @@ cudaError_t launch_set_tau(float* tau, double value, cudaStream_t s);
 // doubles), then a fixed-order final reduction into out[10] (device).
 constexpr int kDiagSlots = 20;  // 8 (sum, compensation) pairs + max|div b| + min p
 constexpr int kDiagGrid = 152 * 2;       // cap of the diagnostics grid (diag_blocks): the blocks that fit at once
-constexpr int kDiagMaxBlocks = 152 * 8;  // blocks that mhd_diagnostics_static's scratch has room for
 int diag_blocks(const Box& box);
 cudaError_t launch_diagnostics(const float* const f[8], const Box& box, double gamma, double* partial,
                                double* out, cudaStream_t s);
