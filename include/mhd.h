@@ -476,7 +476,8 @@ int mhd_cnn_project_backward(int nx, int ny, int nz, const float *const g[8], co
  * (divergence-free, never scaled); the density correction is clipped at
  * -rho/2; the cell correction (rho, m, e) is scaled by the largest of 1,
  * 1/2, 1/4, 0 that keeps the thermal energy above half its uncorrected value,
- * and if none does e is raised to that bound.  scratch: nx*ny*nz floats;
+ * and if none does e is raised to that bound.  scratch: any non-NULL pointer, not
+ * accessed (it held the uncorrected thermal energies of an earlier algorithm);
  * nclip (device int, may be NULL) counts the cells where a limit acted. */
 int mhd_correct(int nx, int ny, int nz, float *const s[8], const float *const d[8], float *scratch,
                 int *nclip, void *stream);

@@ -109,7 +109,6 @@ class Corrector:
         self.x = torch.empty((cells, 8), dtype=torch.bfloat16, device=dev)
         self.d = torch.empty((8, n[2], n[1], n[0]), dtype=torch.float32, device=dev)
         self.sums = torch.empty(5, dtype=torch.float64, device=dev)
-        self.scratch = torch.empty(cells, dtype=torch.float32, device=dev)
 
     def predict(self, state: torch.Tensor) -> torch.Tensor:
         """Correction for the coarse step that starts from `state` (the
@@ -120,7 +119,7 @@ class Corrector:
 
     def apply(self, stepped: torch.Tensor, d: torch.Tensor, nclip=None):
         """Add a predicted correction to the state after the coarse step."""
-        mhd.correct(stepped, d, scratch=self.scratch, nclip=nclip)
+        mhd.correct(stepped, d, nclip=nclip)
 
 
 # --------------------------------------------------------------------------

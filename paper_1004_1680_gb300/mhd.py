@@ -636,7 +636,7 @@ def correct(state, d, scratch=None, nclip=None, stream=None):
     lib = load()
     nz, ny, nx = state.shape[1:]
     if scratch is None:
-        scratch = torch.empty(nx * ny * nz, dtype=torch.float32, device=state.device)
+        scratch = state  # (must not be null; not accessed)
     _check(lib.mhd_correct(nx, ny, nz, _fields(state), _fields(d), _ptr(scratch), _ptr(nclip), _stream(stream)))
 
 
