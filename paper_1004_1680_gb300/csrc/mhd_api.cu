@@ -181,7 +181,7 @@ void rate_window(const mhd_s* m, int p, int* lo, int* hi) {
 // 0.6 + 0.4 (b - 1) / 3 per cell, and a tenth of the last block's length is
 // added (blocks do not end together: short last ones fill the gaps).  Within
 // 1.1 % of the best length on average (3 % at most, 256^3 and 384^3), e.g.
-// 200^3 139 -> 117 us with 140 + 60 cells, 256^3 196 -> 188 with 228 + 28
+// 200^3 139 -> 117 us with 140 + 60 cells, 256^3 196 -> 188 with 224 + 32
 // (equal segments: 190), 512^3 1312 -> 1288.
 int choose_seg(const mhd_s* m, int d, int kind) {
   const int nd = m->n[d], nA = m->n[d == 0 ? 1 : 0], nO = m->n[d == 2 ? 1 : 2];

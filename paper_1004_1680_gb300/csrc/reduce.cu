@@ -294,7 +294,8 @@ __device__ __forceinline__ void p_ff2(float2 rho, float2 m1, float2 m2, float2 m
   err = __ffma2_rn(f2(0x1p-38f * g_hi), U, f2(1e-37f));
 }
 
-// n / d for 0 <= n < 2^31 by a multiplication: the quotient rounded down.
+// n / d for 0 <= n < 2^31 by a multiplication: the quotient rounded down (Granlund
+// and Montgomery, "Division by invariant integers using multiplication", 1994).
 struct FastDiv {
   unsigned mul, shift, d;
 };
