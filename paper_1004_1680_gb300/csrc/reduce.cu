@@ -252,9 +252,16 @@ __device__ __forceinline__ void div_ff2(float2 xl, float2 xh, float2 yl, float2 
   err = __ffma2_rn(f2(0x1p-22f), dabs, __ffma2_rn(f2(0x1p-40f), dT, f2(1e-37f)));
 }
 
+// What an estimate of p may lose to underflow: the momenta's squares and their
+// error words, a dozen terms that may each be off by 2^-149, over rho (at densities
+// and momenta of 1e-25 that is most of p), and the other terms.
+__device__ __forceinline__ float2 underflow2(float2 rr, float g_hi) {
+  return __ffma2_rn(f2(0x1p-142f * g_hi), abs2(rr), f2(1e-37f));
+}
+
 // Float-float estimate ph + pl of the pressure of two cells on packed FP32,
-// within 2^-42 (gamma - 1) U of p (U below); err covers it with a margin of 16.
-// rr: an approximate reciprocal of rho.
+// within 2^-42 (gamma - 1) U of p (U below) and what underflows (underflow2); err
+// covers it with a margin of 16.  rr: an approximate reciprocal of rho.
 __device__ __forceinline__ void p_ff2(float2 rho, float2 m1, float2 m2, float2 m3, float2 e, float2 xl, float2 xh,
                                       float2 yl, float2 yh, float2 zl, float2 zh, float2 rr, float g_hi, float g_lo,
                                       float2 U, float2& ph, float2& pl, float2& err) {
@@ -291,7 +298,7 @@ __device__ __forceinline__ void p_ff2(float2 rho, float2 m1, float2 m2, float2 m
   float2 phe;
   two_prod2(f2(g_hi), d2, ph, phe);
   pl = __fadd2_rn(phe, __ffma2_rn(f2(g_hi), dlo, __fmul2_rn(f2(g_lo), d2)));
-  err = __ffma2_rn(f2(0x1p-38f * g_hi), U, f2(1e-37f));
+  err = __ffma2_rn(f2(0x1p-38f * g_hi), U, underflow2(rr, g_hi));
 }
 
 // n / d for 0 <= n < 2^31 by a multiplication: the quotient rounded down (Granlund
@@ -430,7 +437,7 @@ diag_partial_kernel(const float* __restrict__ rho, const float* __restrict__ mx,
                  a2 = __fadd2_rn(abs2(pair(7)), abs2(zh));
     const float2 U = __ffma2_rn(f2(0.125f), __ffma2_rn(a0, a0, __ffma2_rn(a1, a1, __fmul2_rn(a2, a2))),
                                 __fadd2_rn(abs2(pair(4)), abs2(kin)));
-    const float2 perr = __ffma2_rn(f2(0x1p-17f * g_hi), U, f2(1e-37f));
+    const float2 perr = __ffma2_rn(f2(0x1p-17f * g_hi), U, underflow2(rr, g_hi));
     const float2 p32 = __fmul2_rn(f2(g_hi), sub2(__ffma2_rn(f2(-0.125f), b2, pair(4)), kin));
     auto el = [](const float2& x, int e) { return e & 1 ? x.y : x.x; };
     if (!seeded) {  // the block's first thresholds
