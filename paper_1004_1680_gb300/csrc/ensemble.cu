@@ -151,20 +151,24 @@ int even_segment(int n, int want) {
 int segment_target(const mhd_ens_s* e, int kind, int d, int layout, int sms) {
   const int ka = kernel_axis(layout, d), resident = kind ? 2 : 4, warm = kind && d == 2 ? 14 : 7;
   const long long slots = (long long)sms * resident;
-  int longest = 0;
-  for (auto& b : e->boxes) longest = std::max(longest, b.n[d]);
+  // blocks per segment of all boxes with pencils of one length
+  std::map<int, long long> tiles_of;
+  for (auto& b : e->boxes) {
+    const int n[3] = {layout ? b.n[1] : b.n[0], layout ? b.n[0] : b.n[1], b.n[2]};
+    const Tiles t = sweep_tiles(kind, ka, n);
+    tiles_of[b.n[d]] += (long long)t.x * t.y;
+  }
+  const int longest = tiles_of.rbegin()->first;
   int best = longest;
   double best_end = 0.0;
   for (int want = longest; want >= 24; want -= std::max(4, want / 12)) {
     std::map<int, long long, std::greater<int>> jobs;  // cells marched -> blocks
     double work = 0.0;
-    for (auto& b : e->boxes) {
-      const int n[3] = {layout ? b.n[1] : b.n[0], layout ? b.n[0] : b.n[1], b.n[2]};
-      const Tiles t = sweep_tiles(kind, ka, n);
-      const int seg = even_segment(b.n[d], want), rest = b.n[d] % seg;
-      jobs[seg + warm] += (long long)t.x * t.y * (b.n[d] / seg);
-      if (rest) jobs[rest + warm] += (long long)t.x * t.y;
-      work += (double)t.x * t.y * (b.n[d] + warm * (b.n[d] / seg + (rest > 0)));
+    for (auto& [nd, tiles] : tiles_of) {
+      const int seg = even_segment(nd, want), rest = nd % seg;
+      jobs[seg + warm] += tiles * (nd / seg);
+      if (rest) jobs[rest + warm] += tiles;
+      work += (double)tiles * (nd + warm * (nd / seg + (rest > 0)));
     }
     std::map<int, long long> running;  // cell at which they end -> blocks
     long long active = 0;
@@ -221,25 +225,32 @@ int build_lists(mhd_ens_s* e) {
   for (int kind = 0; kind < 2; kind++) {
     for (int d = 0; d < 3; d++) {
       const int L = sweep_layout(e, d), ka = kernel_axis(L, d);
-      std::vector<int4> items;
-      int minext = 1 << 30;
-      for (int bi = 0; bi < e->nbox; bi++) {
-        const mhd::EnsBox& b = e->boxes[bi];
-        const int n[3] = {L ? b.n[1] : b.n[0], L ? b.n[0] : b.n[1], b.n[2]};
-        minext = std::min(minext, n[ka]);
-        const Tiles t = sweep_tiles(kind, ka, n);
-        const int gz = (n[ka] + b.seg[kind][d] - 1) / b.seg[kind][d];
-        for (int z = 0; z < gz; z++)
-          for (int y = 0; y < t.y; y++)
-            for (int x = 0; x < t.x; x++) items.push_back(make_int4(bi, x, y, z));
-      }
-      // the longest blocks first, otherwise in box order
-      auto length = [&](const int4& it) {
-        const mhd::EnsBox& b = e->boxes[it.x];
-        return std::min(b.seg[kind][d], b.n[d] - it.w * b.seg[kind][d]);
+      int minext = 1 << 30, longest = 0;
+      // each(box, its tiles, segment, the segment's cells) in box order
+      auto segments = [&](auto each) {
+        for (int bi = 0; bi < e->nbox; bi++) {
+          const mhd::EnsBox& b = e->boxes[bi];
+          const int n[3] = {L ? b.n[1] : b.n[0], L ? b.n[0] : b.n[1], b.n[2]}, seg = b.seg[kind][d];
+          const Tiles t = sweep_tiles(kind, ka, n);
+          for (int z = 0; z * seg < n[ka]; z++) each(bi, t, z, std::min(seg, n[ka] - z * seg));
+        }
       };
-      std::stable_sort(items.begin(), items.end(),
-                       [&](const int4& p, const int4& q) { return length(p) > length(q); });
+      for (auto& b : e->boxes) {
+        minext = std::min(minext, b.n[d]);
+        longest = std::max(longest, b.seg[kind][d]);
+      }
+      // the longest blocks first, otherwise in box order: where the blocks of each
+      // length begin (5000 uneven boxes: 16.6 ms to create with a sort of the blocks
+      // and a pass over the boxes for every length that segment_target tries)
+      std::vector<size_t> at(longest + 2, 0);
+      segments([&](int, Tiles t, int, int len) { at[len] += (size_t)t.x * t.y; });
+      for (int len = longest; len >= 0; len--) at[len] += at[len + 1];
+      std::vector<int4> items(at[0]);
+      segments([&](int bi, Tiles t, int z, int len) {
+        size_t& to = at[len + 1];
+        for (int y = 0; y < t.y; y++)
+          for (int x = 0; x < t.x; x++) items[to++] = make_int4(bi, x, y, z);
+      });
       int rc = upload(kind == 0 ? &e->fluid[d] : &e->mag[d], items, minext);
       if (rc) return rc;
     }
