@@ -206,8 +206,9 @@ int mhd_set_fusion(mhd_t *m, int on);
  * register loads.  With on = 1, boxes whose pencils are few or short, and x
  * sweeps of boxes that the row sweeps do not take, run tile sweeps instead: a
  * block holds its pencils' whole stencil on chip and each thread updates 4
- * cells, with bitwise the result of the sweep they replace.  Ensembles, pencils shorter than 16 cells and boxes that do
- * not qualify use register loads.  If staged data does not arrive within the
+ * cells, with bitwise the result of a marching sweep along that axis with the
+ * same square root.  Ensembles, and pencils shorter than 16 cells and boxes that
+ * do not qualify where they are not swept by tiles, use register loads.  If staged data does not arrive within the
  * bounded wait (about half a second), the block records the failure and
  * stops; mhd_cfl_dt then returns MHD_E_TIMEOUT until the next mhd_set_state.
  * MHD_E_ARG unless on is 0 or 1, or for an FP64 box. */
@@ -282,10 +283,12 @@ int mhd_set_segments(mhd_t *m, int seg_x, int seg_y, int seg_z);
  * warp stages 8-cell row pieces of its 32 pencils), 2 = through a copy with x
  * and y exchanged (all 8 fields transposed once before a group of x sweeps
  * and once after; consecutive steps share one group, so a run of steps costs
- * two transposes per step), 0 = automatic: 1 with mhd_set_tma on (row or tile
- * sweeps) unless the freezing speed is per pencil, else 2 once the state
- * exceeds 64 MiB, else 1.  3 = the paper's data flow,
- * as an ablation: every sweep runs along the contiguous axis of a copy
+ * two transposes per step), 0 = automatic.  Automatic with mhd_set_tma on is
+ * 1 (row or tile sweeps), but 2 for boxes of 2^23 cells or more with rows of
+ * more than 1024, ny a multiple of 32 and nz of 8.  Register loads, the
+ * per-pencil freezing speed, and given x segments (mhd_set_segments) on rows
+ * that the row sweeps do not take have 2 once the state exceeds 64 MiB, else 1.
+ * 3 = the paper's data flow, as an ablation: every sweep runs along the contiguous axis of a copy
  * transposed so that its axis is fastest (x<->y around the y sweeps, x<->z
  * around the z sweeps; six transposes per step); needs every extent a
  * multiple of 4.  All paths compute the same update; results differ by FP32

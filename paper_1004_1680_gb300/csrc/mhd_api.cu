@@ -116,7 +116,7 @@ struct mhd_s {
 namespace {
 
 // x sweeps run directly along x (row or tile sweeps) where staged sweeps
-// are on, the freezing speed is one of its own per cell, and either no segment
+// are on, the freezing speed is one per cell, and either no segment
 // length of x is given (which keeps tiles off) or the rows are whole for both row
 // sweeps; otherwise they go through the exchanged layout once the state no longer
 // fits in L2 (the pencil sweeps along x read 32 different lines per warp and
