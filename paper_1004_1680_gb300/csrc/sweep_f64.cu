@@ -55,8 +55,13 @@ __device__ __forceinline__ void movers64(const double u[5], const double b[3], d
 }
 
 // Threads of a block and split of a pencil of nD cells: one thread per cell,
-// np pencils, the whole periodic pencil (`whole`) or a segment of `out`
-// cells with 3 halo cells at each end (the reach of both sweeps' stencils).
+// np pencils, the whole periodic pencil (`whole`, up to 512 cells) or a segment of
+// `out` cells with 3 halo cells at each end (the reach of both sweeps' stencils).
+// Few pencils per block, down to one, cost less across the contiguous axis (their
+// 8 np-byte pieces come from L2, which has time) than halo cells do in the FP64
+// pipe: with at least 4 pencils a block, and segments beyond 128 cells, 256^3 took
+// 106 ms per step, now 82, 384^3 336 and 282, 512^3 827 and 671 (a thread per pencil,
+// marching: 106, 321, 740), 132^3 14.6 and 12.2.
 constexpr int kThreads64 = 512;
 struct Tile64 {
   int threads, np, td, out, segs;
@@ -64,13 +69,12 @@ struct Tile64 {
 };
 __host__ __device__ inline Tile64 tile64(int nD) {
   Tile64 t;
-  const int most = kThreads64 / 4;  // at least 4 pencils: 32-byte pieces across the pencils
-  t.whole = nD <= most;
-  t.segs = t.whole ? 1 : (nD + most - 7) / (most - 6);
+  t.whole = nD <= kThreads64;
+  t.segs = t.whole ? 1 : (nD + kThreads64 - 7) / (kThreads64 - 6);
   t.out = (nD + t.segs - 1) / t.segs;
   t.td = t.out + (t.whole ? 0 : 6);
-  t.threads = t.td <= 64 ? 256 : kThreads64;
-  t.np = t.threads / t.td;
+  t.np = (t.td <= 64 ? 256 : kThreads64) / t.td;
+  t.threads = (t.np * t.td + 31) / 32 * 32;
   return t;
 }
 
@@ -112,12 +116,12 @@ __device__ __forceinline__ Cell64 cell64(const int n[3]) {
 }
 
 // Fluid sweep, one thread per cell.  FP64 arithmetic bounds it (350 operations
-// per cell, 16 cycles of an SM per warp instruction: its pipe is 85 % busy), so nothing is
+// per cell, 16 cycles of an SM per warp instruction: its pipe is 83 % busy), so nothing is
 // computed twice but a few subtractions: the movers of both stages and the
 // limited values are exchanged through shared memory, [component][thread], in
 // two alternating sets.  (Marching whole pencils with one thread each left
 // the FP64 pipe idle below about 150,000 pencils: 64^3 1050 us a sweep, now
-// 175; 256^3 111 ms a step, now 101.)
+// 180; at 512^3 740 ms a step, now 671.)
 template <int D>
 __global__ void __launch_bounds__(kThreads64, 1) fluid64_kernel(const __grid_constant__ Fluid64Args a) {
   wait_for_previous();
