@@ -7,6 +7,8 @@ import sys
 
 import pytest
 
+from paper_1004_1680_gb300.build import ROOT
+
 pytestmark = pytest.mark.gpu
 
 PROGRAM = """
@@ -27,7 +29,7 @@ assert b.time() > 0.0 and bool(torch.isfinite(s).all())
                                                       ("superbee", "bound", 0.0), ("vanleer", "fast", 1e-3),
                                                       ("vanleer", "pencil", 0.0)])
 def test_variant_in_a_fresh_process(limiter, freezing, floor):
-    subprocess.run([sys.executable, "-c", PROGRAM.format(limiter=limiter, freezing=freezing, floor=floor)], check=True)
+    subprocess.run([sys.executable, "-c", PROGRAM.format(limiter=limiter, freezing=freezing, floor=floor)], check=True, cwd=ROOT)
 
 
 ENSEMBLE = """
@@ -46,4 +48,4 @@ assert (e.times() > 0.0).all() and all(bool(torch.isfinite(e.get_state(b)).all()
 
 @pytest.mark.parametrize("xpath, segdiv", [(1, 1), (1, 2), (2, 1), (2, 4)])
 def test_ensemble_in_a_fresh_process(xpath, segdiv):
-    subprocess.run([sys.executable, "-c", ENSEMBLE.format(xpath=xpath, segdiv=segdiv)], check=True)
+    subprocess.run([sys.executable, "-c", ENSEMBLE.format(xpath=xpath, segdiv=segdiv)], check=True, cwd=ROOT)
